@@ -241,8 +241,8 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
     TVS_CUDA(launch_rowmap(d_dir, 1, v.R, d_lo, d_hi, s), "rowmap launch");
     TVS_CUDA(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned), s), "reset work counter");
     TVS_CUDA(launch_sweep(d_dir, d_jobs, reinterpret_cast<const int*>(ws + L.istart), 1, c.items, d_lo, d_hi, d_cv,
-                          d_cb, v.W, v.K, h->tuning.prune, !h->tuning.fp32_decisions, d_cnt, nullptr, nullptr, 0,
-                          h->num_sms, h->smem_optin, h->tuning.sweep_max_warps, s),
+                          d_cb, v.W, v.K, h->tuning.prune, !h->tuning.fp32_decisions, d_cnt,
+                          reinterpret_cast<int4*>(ws + L.flags), d_cnt + 16, (int)L.flag_cap, h->num_sms, h->smem_optin, h->tuning.sweep_max_warps, s),
              "sweep launch");
     std::vector<int> slab(c.slab_elems), slabb(c.slab_elems), lo(v.R), hi(v.R);
     TVS_CUDA(cudaMemcpyAsync(slab.data(), d_cv, c.slab_elems * 4, cudaMemcpyDeviceToHost, s), "copy cv");
@@ -475,8 +475,13 @@ extern "C" int tvs_total_viewshed_device_noalloc(const float* d_dem, int rows, i
     const size_t o_slabs = o_chunk + 2 * align256(max_rows * 4);
     int* d_cvf = reinterpret_cast<int*>(base + o_slabs);
     int* d_cvb = reinterpret_cast<int*>(base + o_slabs + align256(max_slab * 4));
-    if (o_slabs + 2 * align256(max_slab * 4) > kNoAllocScratchBytes)
+    const size_t o_flags = o_slabs + 2 * align256(max_slab * 4);
+    if (o_flags > kNoAllocScratchBytes)
         return fail(TVS_ERR_OOM, "the job's layout does not fit the 64 MiB no-allocation scratch");
+    // what is left holds flagged walks; without room for one they are marked
+    // in the measures and found by the scan
+    int4* d_flags = reinterpret_cast<int4*>(base + o_flags);
+    const int flag_cap = (int)((kNoAllocScratchBytes - o_flags) / FLAG_ENTRY_BYTES);
 
     // Copies from pageable host memory: the runtime has staged the tables
     // before each call returns, so the next call may reuse them.
@@ -501,8 +506,8 @@ extern "C" int tvs_total_viewshed_device_noalloc(const float* d_dem, int rows, i
         // the shared array keeps the previous call's contents: the work counter must start at zero
         TVS_CUDA(cudaMemsetAsync(d_counter, 0, sizeof(unsigned), s), "reset work counter");
         TVS_CUDA(launch_sweep(cd, d_job, d_istart + at, nd, istart[at + nd], d_rowlo, d_rowhi, d_cvf, d_cvb, wmax,
-                              dmax, tn.prune, !tn.fp32_decisions, d_counter, nullptr, nullptr, 0, num_sms,
-                              smem_optin, tn.sweep_max_warps, s),
+                              dmax, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_counter + 16, flag_cap,
+                              num_sms, smem_optin, tn.sweep_max_warps, s),
                  "sweep launch");
         TVS_CUDA(launch_unskew(d_cvf, d_cvb, d_job, cd, d_cj + c, 1, tiles, cjs[c].nsplit, d_part, s),
                  "unskew launch");
@@ -614,7 +619,7 @@ int tvs_batch_create(tvs_handle h, const tvs_job* jobs, int njobs, size_t hbm_bu
     if (e != cudaSuccess) { tvs_batch_destroy(b); return cuda_fail(e, "end capture"); }
     e = cudaGraphInstantiate(&b->exec, b->graph, 0);
     if (e != cudaSuccess) { b->exec = nullptr; tvs_batch_destroy(b); return cuda_fail(e, "instantiate graph"); }
-    for (const Chunk& c : b->plan.chunks) b->kernels += 4 + (c.max_split > 1 ? 1 : 0);
+    for (const Chunk& c : b->plan.chunks) b->kernels += (h->tuning.fp32_decisions ? 3 : 5) + (c.max_split > 1 ? 1 : 0);
     *out = b;
     return TVS_OK;
 }

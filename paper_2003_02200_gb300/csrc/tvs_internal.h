@@ -129,10 +129,10 @@ cudaError_t launch_colmap(const DirDev* d_dir, int* dest, unsigned* frac, cudaSt
 // direction (items 2p and 2p + 1 of a direction are row p forward and
 // backward), its row gathered from the job's DEM; `prune` turns exact horizon
 // pruning on, `cert` certified (exact) visibility decisions instead of FP32
-// ones.  With cert and a flag buffer (flag_cap entries, flag_count two
-// counters) the walks the sweep cannot certify are walked exactly by a second
-// kernel on the same stream; without one (or once it is full) the sweep's
-// warps walk them themselves.
+// ones.  With cert the walks the sweep cannot certify go to the flag buffer
+// (flag_cap entries, possibly none; flag_count three counters) and are walked
+// exactly by a second kernel on the same stream; those that find it full are
+// marked in their measures and found by a third.
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
                          int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
                          int dmax, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,

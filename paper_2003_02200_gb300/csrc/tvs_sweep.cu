@@ -70,8 +70,8 @@ struct SweepParams {
     int* cv_fwd;       // forward measure of every sample (slab layout)
     int* cv_bwd;       // backward measure of every sample (slab layout)
     unsigned* counter;
-    int4* flag_buf;    // certified: flagged walks for the exact pass (NULL: walked in the sweep)
-    unsigned* flag_count;
+    int4* flag_buf;    // certified: flagged walks for the exact pass
+    unsigned* flag_count;   // its fill, the exact pass's claims, and whether a walk found it full
     int flag_cap;
     int ndir;
     int total_items;
@@ -81,7 +81,7 @@ struct SweepParams {
     int half;          // floats of one staged row array (multiple of 4)
     int per_pair;      // floats of a warp pair's shared area (certified)
     int zs_len;        // floats of the row's suffix maxima (0 without pruning)
-    int fl_cap;        // entries of the flagged-POV list (certified only)
+    int wm_len;        // floats of the row's window maxima (certified pruned launches, else 0)
     int per_warp;      // floats of a warp's shared area
 };
 
@@ -117,20 +117,14 @@ struct ItemRow {
     bool rev;
 };
 
-// Decodes item into its row; false when the row is empty.
-__device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* istart, int item, ItemRow* it)
+// Skewed row p of direction `dir`, walked forward or backward; false when the
+// row is empty.
+__device__ __forceinline__ bool decode_row(const SweepParams& sp, int dir, int p, bool rev, ItemRow* it)
 {
-    int lo = 0, hi = sp.ndir - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (istart[mid] <= item) lo = mid; else hi = mid - 1;
-    }
-    const DirDev& d = sp.dirs[lo];
-    const int rem = item - istart[lo];
-    const int p = rem >> 1;
-    it->rev = (rem & 1) != 0;
+    const DirDev& d = sp.dirs[dir];
+    it->rev = rev;
     const int jlo = sp.rowlo[d.row_off + p], jhi = sp.rowhi[d.row_off + p];
-    it->dir = lo;
+    it->dir = dir;
     it->p = p;
     it->jlo = jlo;
     it->L = jhi - jlo + 1;
@@ -139,6 +133,18 @@ __device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* is
     it->pov = row_pov(it->L, d.K, d.pov, d.p4_pct);
     it->rowbase = d.slab + (long long)p * d.Wp + jlo;
     return it->L > 0;
+}
+
+// Decodes item into its row; false when the row is empty.
+__device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* istart, int item, ItemRow* it)
+{
+    int lo = 0, hi = sp.ndir - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (istart[mid] <= item) lo = mid; else hi = mid - 1;
+    }
+    const int rem = item - istart[lo];
+    return decode_row(sp, lo, rem >> 1, (rem & 1) != 0, it);
 }
 
 // Stages the item's row from the DEM: FP32 heights into Fh, or with CERT hi
@@ -430,30 +436,57 @@ __device__ __forceinline__ void suffix_max(const float* __restrict__ F, float* _
     }
 }
 
-// Prefix maxima of the staged row F (row order, certified backward walks) at
-// every ZS_STRIDE-th sample: ZP[j] = max F[x] over x <= ZS_STRIDE * j +
-// ZS_STRIDE - 1, for j <= (L - 1) / ZS_STRIDE.  Lane l scans its own segment,
-// a warp scan joins the segments.
-__device__ __forceinline__ void prefix_max(const float* __restrict__ F, float* __restrict__ ZP, int L, int lane)
+// Maximum of the four samples 4 q .. 4 q + 3 of the staged row (ROW_PADL
+// keeps them 16-byte aligned).
+__device__ __forceinline__ float quad_max(const float* __restrict__ F, int q)
 {
-    const float NEG = neg_inf();
-    const int seglen = ((L + 31) / 32 + ZS_STRIDE - 1) / ZS_STRIDE * ZS_STRIDE;
-    const int a = lane * seglen, b = min(a + seglen, L);
-    float m = NEG;
-    for (int x = a; x < b; ++x) m = fmaxf(m, F[ROW_PADL + x]);
-    // inclusive prefix scan of the segment maxima over the lanes
-    float s = m;
+    const float4 v = *reinterpret_cast<const float4*>(F + ROW_PADL + 4 * q);
+    return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
+}
+
+// The maxima a pruned certified walk tests its blocks against, one entry per
+// ZS_STRIDE samples of the staged row F (L samples, -inf beyond them).
+// warp-scans of 32 quads at a time: consecutive lanes read consecutive quads.
+//
+// Suffix maxima ZS[q] = max F[x >= 4 q], or prefix maxima ZS[q] = max
+// F[x <= 4 q + 3] (PREFIX, backward walks), q <= (L - 1) / 4.
+template <bool PREFIX>
+__device__ __forceinline__ void end_max(const float* __restrict__ F, float* __restrict__ ZS, int L, int lane)
+{
+    static_assert(ZS_STRIDE == 4, "quads");
+    const unsigned FULL = 0xffffffffu;
+    const int nq = (L + 3) / 4;
+    float carry = neg_inf();
+    const int chunks = (nq + 31) / 32;
+    for (int c = 0; c < chunks; ++c) {
+        const int q = (PREFIX ? c : chunks - 1 - c) * 32 + lane;
+        float m = q < nq ? quad_max(F, q) : neg_inf();
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s = fmaxf(s, t);
+        for (int o = 1; o < 32; o <<= 1) {
+            const float t = PREFIX ? __shfl_up_sync(FULL, m, o) : __shfl_down_sync(FULL, m, o);
+            if (PREFIX ? lane >= o : lane + o < 32) m = fmaxf(m, t);
+        }
+        m = fmaxf(m, carry);
+        if (q < nq) ZS[q] = m;
+        carry = __shfl_sync(FULL, m, PREFIX ? 31 : 0);
     }
-    float before = __shfl_up_sync(0xffffffffu, s, 1);   // maximum of the earlier segments
-    if (lane == 0) before = NEG;
-    float run = before;
-    for (int x = a; x < b; ++x) {
-        run = fmaxf(run, F[ROW_PADL + x]);
-        if (x % ZS_STRIDE == ZS_STRIDE - 1 || x == L - 1) ZP[x / ZS_STRIDE] = run;
+}
+
+// Window maxima WM[j] = max F[x] over the P + U samples from 4 j - U on, the
+// window of one block of a pruned walk that starts at sample 4 j - U, for
+// j < (L + U + 3) / 4 (backward windows start up to U samples before the
+// row).  `part` of `parts` warps each fill their share.
+template <int P, int U>
+__device__ __forceinline__ void window_max(const float* __restrict__ F, float* __restrict__ WM, int L, int lane,
+                                           int part = 0, int parts = 1)
+{
+    static_assert(P % 4 == 0 && U % 4 == 0 && U <= ROW_PADL, "quads");
+    const int n = (L + U + 3) / 4;
+    for (int j = lane + 32 * part; j < n; j += 32 * parts) {
+        float m = quad_max(F, j - U / 4);
+#pragma unroll
+        for (int k = 1; k < (P + U) / 4; ++k) m = fmaxf(m, quad_max(F, j - U / 4 + k));
+        WM[j] = m;
     }
 }
 
@@ -515,6 +548,32 @@ constexpr int CERT_UNROLL_SINGLE = TVS_CERT_UNROLL_SINGLE;   // one-row-per-warp
 constexpr int CERT_POV = TVS_CERT_POV;
 static_assert(CERT_POV + CERT_UNROLL <= ROW_PADR && CERT_POV + CERT_UNROLL_SINGLE <= ROW_PADR,
               "a forward block's window reads up to P + U samples on");
+#ifndef TVS_SKIP_READY
+#define TVS_SKIP_READY 24
+#endif
+constexpr int SKIP_READY = TVS_SKIP_READY;   // lanes with a block before a pruned walk evaluates
+#ifndef TVS_SKIP_RESTART
+#define TVS_SKIP_RESTART 4
+#endif
+constexpr int SKIP_RESTART = TVS_SKIP_RESTART;   // finished lanes before a pruned walk replaces groups
+#ifndef TVS_SKIP_TESTS
+#define TVS_SKIP_TESTS 4
+#endif
+constexpr int SKIP_TESTS = TVS_SKIP_TESTS;       // blocks a searching lane tests at a time
+#ifndef TVS_SKIP_CHUNK
+#define TVS_SKIP_CHUNK 8
+#endif
+constexpr int SKIP_CHUNK = TVS_SKIP_CHUNK;       // steps per pass of a block's evaluation loop
+#ifndef TVS_SKIP_WARPS
+#define TVS_SKIP_WARPS 16
+#endif
+constexpr int SKIP_WARPS = TVS_SKIP_WARPS;       // most warps of a pruned certified CTA
+#ifndef TVS_SKIP_UNROLL
+#define TVS_SKIP_UNROLL 16
+#endif
+constexpr int SKIP_UNROLL = TVS_SKIP_UNROLL;   // steps per block of a pruned walk
+static_assert(SKIP_UNROLL <= ROW_PADL && CERT_POV + SKIP_UNROLL <= ROW_PADR && FLUSH_STEPS % SKIP_UNROLL == 0,
+              "pads and flushes of a pruned walk");
 static_assert(CERT_UNROLL <= ROW_PADL, "a backward block's window starts up to U samples before the row");
 static_assert(FLUSH_STEPS % CERT_UNROLL == 0, "long walks flush on block boundaries");
 // A certified kernel with U-step blocks stores distance entry m at slot m +
@@ -524,8 +583,9 @@ static_assert(FLUSH_STEPS % CERT_UNROLL == 0, "long walks flush on block boundar
 // 16-byte bank groups.  Skewed, entry u of block k sits in bank group
 // ((U + 1) k + u) mod 8 (U a multiple of 8), which spreads blocks k over all
 // eight.  Tables are sized for the shorter block, which needs the most slots.
-constexpr int TAB_SKEW_MIN = CERT_UNROLL < CERT_UNROLL_SINGLE ? CERT_UNROLL : CERT_UNROLL_SINGLE;
+constexpr int TAB_SKEW_MIN = std::min({CERT_UNROLL, CERT_UNROLL_SINGLE, SKIP_UNROLL});
 static_assert(CERT_UNROLL % 8 == 0 && CERT_UNROLL_SINGLE % 8 == 0, "skewed blocks cover the eight bank groups");
+static_assert(SKIP_UNROLL % 8 == 0, "as above");
 __host__ __device__ constexpr int tab_slots_for(int entries, bool skew)
 {
     return skew ? ((entries + entries / TAB_SKEW_MIN + 1 + 1) & ~1) : entries;
@@ -558,8 +618,6 @@ constexpr int CERT_NEAR = TVS_CERT_NEAR;
 constexpr int CERT_FAR = TVS_CERT_FAR;
 constexpr int CERT_FAR2 = TVS_CERT_FAR2;
 
-// Entries of a warp's flagged-POV list (at least 32 lanes x LARGE_POV).
-constexpr int FLAG_CAP = 256;
 // Targets per lane per chunk of an exact walk.
 constexpr int XW_KPL = 8;
 
@@ -572,81 +630,157 @@ __device__ __forceinline__ float sat_pos(float s)
     return v;
 }
 
-// What the exact walks of a row need.
-struct ExactCtx {
+// The measure the sweep writes for a flagged walk that found the flag buffer
+// full: the scan after the exact pass looks for negative measures.
+constexpr int CV_FLAGGED = (int)0x80000000;
+
+// A staged row as its certified walks see it.
+struct CertRow {
     const float* H;      // staged hi parts (index 0 = first sample)
     const float* Lo;     // staged lo parts
     int L, K;
-    float h0h, h0l;      // h0 = h0h + h0l (to 2^-48)
-    float eta;           // bound of the staged heights' error, plus h0's split
-    int* cvrow;
-    bool bwd;            // walks go toward lower sample indices
-    bool from_dem;       // samples blended from the DEM as needed (no staged row)
-    bool rev_staged;     // the staged row is reversed: staged x is row sample L - 1 - x
+    float h0;
     float eh0, el0;      // hi and lo parts of the first sample (a sentinel in H, Lo)
     float ehL, elL;      // and of the last one
-    const DirDev* dir;
-    const JobDev* job;
-    int p, jlo;
-    int half;            // floats of a staged row array (index bound, with ROW_PADL)
-    int zs_len;          // entries of the suffix maxima
-    const float4* tab;   // the distance table (skewed: entry m at m + m / tskew)
-    int tabn;            // its entries
-    int tskew;           // its skew: the block length of the kernel that built it
+    float eg0;           // 2.01u |h0| + |h0 - float(h0)| + 4 eta: the parts of Eg common to the row's groups
+    float zmax;          // the row's largest |elevation|
+    int* cvrow;
+    int item;            // the row's work item
+    bool rev_staged;     // the staged row is reversed: staged x is row sample L - 1 - x
 };
 
-// fl(1/d), correctly rounded: from the distance table while it reaches d.
-__device__ __forceinline__ float inv_d(const ExactCtx& c, int d)
+// The certified row of a staged item.  eta bounds the staged heights' error,
+// plus h0's split (h0 = float(h0) + h0_lo to 2^-48).
+__device__ __forceinline__ CertRow cert_row(const SweepParams& sp, const ItemRow& it, int item, const float* Fh,
+                                            const float* Fl, const float* ends, float zmax, int* cv, bool rev_staged)
 {
-    const int m = d - 1;
-    return m < c.tabn ? c.tab[m + m / c.tskew].x : __frcp_rn((float)d);
-}
-
-// Hi and lo parts of sample xs (row order) blended from the DEM, as the
-// staging forms them.
-__device__ __forceinline__ void dem_hl(const ExactCtx& c, int xs, float& hi, float& lo)
-{
-    const DirDev& d = *c.dir;
-    const int j = c.jlo + (c.rev_staged ? c.L - 1 - xs : xs);
-    const unsigned long long y = (unsigned long long)j * d.t_fx;
-    const int a = c.p - d.D + (int)(y >> 32);
-    const unsigned fr = (unsigned)y;
-    int st;
-    const long long idx = view_index(d, c.job->cols, a, j, &st);
-    const long long cells = (long long)c.job->rows * c.job->cols;
-    const float va = in_range(idx, cells, 16) ? c.job->dem[idx] : 0.f;
-    const float vb = fr != 0u ? (in_range(idx + st, cells, 17) ? c.job->dem[idx + st] : 0.f) : va;
-    df::df_blend(va, vb, fr, hi, lo);
+    const float eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
+    CertRow r;
+    r.H = Fh + ROW_PADL;
+    r.Lo = Fl + ROW_PADL;
+    r.L = it.L;
+    r.K = it.K;
+    r.h0 = it.h0;
+    r.eh0 = ends[0];
+    r.el0 = ends[1];
+    r.ehL = ends[2];
+    r.elL = ends[3];
+    r.eg0 = 2.01f * 0x1p-24f * fabsf(it.h0) + fabsf(sp.dirs[it.dir].h0_lo) * 1.0001f + 4.04f * eta;
+    r.zmax = zmax;
+    r.cvrow = cv + it.rowbase;
+    r.item = item;
+    r.rev_staged = rev_staged;
+    return r;
 }
 
 // Hi and lo parts of POV x's ground height (the end samples are sentinels in
 // the staged arrays; their real parts are kept aside).
-__device__ __forceinline__ void pov_hl(const ExactCtx& c, int x, float& hi, float& lo)
+__device__ __forceinline__ void pov_hl(const CertRow& r, int x, float& hi, float& lo)
 {
-    if (c.from_dem) dem_hl(c, x, hi, lo);
-    else if (x == 0) { hi = c.eh0; lo = c.el0; }
-    else if (x == c.L - 1) { hi = c.ehL; lo = c.elL; }
-    else { hi = c.H[x]; lo = c.Lo[x]; }
+    if (x == 0) { hi = r.eh0; lo = r.el0; }
+    else if (x == r.L - 1) { hi = r.ehL; lo = r.elL; }
+    else { hi = r.H[x]; lo = r.Lo[x]; }
 }
 
-// FP64 height of staged sample xs (row order) exactly as the FP64 definition
-// forms it: (1 - r) * a + r * b with r = fr / 2^32, every operation rounded.
-__device__ __forceinline__ double z64_at(const ExactCtx& c, int xs)
+// Hands the flagged walks of one group (bits of fm, staged samples x0 + bit)
+// to the exact pass; returns the bits that found the buffer full.
+__device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const CertRow& r, unsigned fm, int x0)
+{
+    // a full buffer's fill no longer counts, so it cannot wrap
+    const unsigned cap = (unsigned)sp.flag_cap;
+    unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
+    if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)__popc(fm));
+    for (; fm && at < cap; fm &= fm - 1, ++at) {
+        const int xs = x0 + __ffs(fm) - 1;   // staged sample; the entry holds the row's
+        sp.flag_buf[at] = make_int4(r.item, r.rev_staged ? r.L - 1 - xs : xs, __float_as_int(r.zmax), 0);
+    }
+    if (fm) sp.flag_count[2] = 1u;
+    return fm;
+}
+
+// Writes the measures of a finished group of P POVs (pov_x(q): staged sample
+// of POV q; mask: its flagged POVs).
+template <int P, bool LONG, bool BWD, class X, class N, class S>
+__device__ __forceinline__ void finish_group(const SweepParams& sp, const CertRow& r, int x0, unsigned mask,
+                                             X pov_x, N walk_n, S measure, const int* spill)
+{
+    unsigned full = 0u;                      // bits by sample
+    if (mask) full = flag_walks(sp, r, BWD ? __brev(mask) >> (32 - P) : mask, x0);
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        const int x = pov_x(q);
+        if (x >= r.L) continue;
+        const bool lost = (full >> (x - x0)) & 1u;
+        if (((mask >> q) & 1u) && !lost) continue;   // the exact pass writes it
+        const int cv = walk_n(x) >= 1 ? 1 + (int)measure(q) + (LONG ? spill[32 * q] : 0) : 0;
+        r.cvrow[r.rev_staged ? r.L - 1 - x : x] = lost ? CV_FLAGGED : cv;
+    }
+}
+
+// What the exact walk of a sample needs.
+struct ExactCtx {
+    int L, K;
+    float h0h, h0l;      // h0 = h0h + h0l (to 2^-48)
+    float eta;           // bound of the blended heights' error, plus h0's split
+    int* cvrow;
+    bool bwd;            // walks go toward lower sample indices
+    const DirDev* dir;
+    const JobDev* job;
+    int p, jlo;
+};
+
+__device__ __forceinline__ ExactCtx exact_ctx(const SweepParams& sp, const ItemRow& it, float zmax)
+{
+    ExactCtx c;
+    c.dir = sp.dirs + it.dir;
+    c.job = sp.jobs + c.dir->job;
+    c.L = it.L;
+    c.K = it.K;
+    c.h0h = it.h0;
+    c.h0l = c.dir->h0_lo;
+    c.eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
+    c.cvrow = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
+    c.bwd = it.rev;
+    c.p = it.p;
+    c.jlo = it.jlo;
+    return c;
+}
+
+// Elevations that sample xs of the row blends (row a, row a + 1) and the
+// weight's fraction.
+__device__ __forceinline__ void dem_pair(const ExactCtx& c, int xs, float& va, float& vb, unsigned& fr)
 {
     const DirDev& d = *c.dir;
-    const int j = c.jlo + (c.rev_staged ? c.L - 1 - xs : xs);
+    const int j = c.jlo + xs;
     const unsigned long long y = (unsigned long long)j * d.t_fx;
     const int a = c.p - d.D + (int)(y >> 32);
-    const unsigned fr = (unsigned)y;
+    fr = (unsigned)y;
     int st;
     const long long idx = view_index(d, c.job->cols, a, j, &st);
     const long long cells = (long long)c.job->rows * c.job->cols;
-    if (!in_range(idx, cells, 16) || (fr != 0u && !in_range(idx + st, cells, 17))) return 0.0;
-    const double lo = (double)c.job->dem[idx];
-    if (fr == 0u) return lo;
-    const double hi = (double)c.job->dem[idx + st];
+    va = in_range(idx, cells, 16) ? c.job->dem[idx] : 0.f;
+    vb = fr != 0u ? (in_range(idx + st, cells, 17) ? c.job->dem[idx + st] : 0.f) : va;
+}
+
+// Hi and lo parts of sample xs, as the staging forms them.
+__device__ __forceinline__ void dem_hl(const ExactCtx& c, int xs, float& hi, float& lo)
+{
+    float va, vb;
+    unsigned fr;
+    dem_pair(c, xs, va, vb, fr);
+    df::df_blend(va, vb, fr, hi, lo);
+}
+
+// FP64 height of sample xs exactly as the FP64 definition forms it:
+// (1 - r) * a + r * b with r = fr / 2^32, every operation rounded.
+__device__ __forceinline__ double z64_at(const ExactCtx& c, int xs)
+{
+    float va, vb;
+    unsigned fr;
+    dem_pair(c, xs, va, vb, fr);
+    if (fr == 0u) return (double)va;
     const double r = __dmul_rn((double)fr, 0x1p-32);
-    return __dadd_rn(__dmul_rn(__dsub_rn(1.0, r), lo), __dmul_rn(r, hi));
+    return __dadd_rn(__dmul_rn(__dsub_rn(1.0, r), (double)va), __dmul_rn(r, (double)vb));
 }
 
 __device__ __forceinline__ int warp_sum(int v)
@@ -707,7 +841,7 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
     float hh, hl;
     {
         float zh, zl;
-        pov_hl(c, x, zh, zl);
+        dem_hl(c, x, zh, zl);
         float s, e;
         df::two_sum(zh, c.h0h, s, e);
         e = __fadd_rn(e, __fadd_rn(zl, c.h0l));
@@ -726,11 +860,10 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
         for (int k = 0; k < XW_KPL; ++k) {
             const int d = d0 + k;
             th[k] = NEG; tl[k] = 0.f; iv[k] = 1.f;
-            if (d <= last && (c.from_dem || in_range(ROW_PADL + x + dir * d, c.half, 15))) {
-                iv[k] = inv_d(c, d);
+            if (d <= last) {
+                iv[k] = __frcp_rn((float)d);
                 float zh, zl;
-                if (c.from_dem) dem_hl(c, x + dir * d, zh, zl);
-                else { zh = c.H[x + dir * d]; zl = c.Lo[x + dir * d]; }
+                dem_hl(c, x + dir * d, zh, zl);
                 df::df_slope_iv(zh, zl, hh, hl, d, iv[k], th[k], tl[k]);
                 if (df::df_gt(th[k], tl[k], mh, ml)) { mh = th[k]; ml = tl[k]; md = d; }
             }
@@ -749,7 +882,7 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
         float cl = __shfl_up_sync(0xffffffffu, pl, 1);
         int cd = __shfl_up_sync(0xffffffffu, pd, 1);
         if (lane == 0 || df::df_gt(rh, rl, ch, cl)) { ch = rh; cl = rl; cd = rd; }
-        float icd = inv_d(c, cd);
+        float icd = __frcp_rn((float)cd);
 #pragma unroll
         for (int k = 0; k < XW_KPL; ++k) {
             const int d = d0 + k;
@@ -776,7 +909,7 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
     return warp_sum(acc);
 }
 
-// Exact measure of POV x of the staged row, written by lane 0.
+// Exact measure of POV x of the row, written by lane 0.
 __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
@@ -792,70 +925,7 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
             if (esc) atomicAdd(&g_sweep_stats[1], 1ull);
         }
     }
-    if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[c.rev_staged ? c.L - 1 - x : x] = cv;
-}
-
-// The warp's list of flagged POVs (positions in the staged row).
-struct FlagList {
-    int* list;
-    int count;
-    int4* gbuf;          // the launch's flagged-walk buffer (NULL: walk every flag here)
-    unsigned* gcount;    // its fill counter
-    int gcap;            // its capacity
-    int item;            // the current row's work item
-    float zmax;          // and its largest |elevation| (for the staged heights' error bound)
-};
-
-__device__ __noinline__ void drain_flags(FlagList& fl, const ExactCtx& c, int lane)
-{
-    __syncwarp();
-    const long long t0 = clock64();
-    for (int i = 0; i < fl.count; ++i) exact_walk(c, fl.list[i], lane);
-    fl.count = 0;
-    if (lane == 0) atomicAdd(&g_sweep_stats[2], (unsigned long long)(clock64() - t0));
-    __syncwarp();
-}
-
-// Warp-collective: appends every lane's flagged POVs (bits of fm, positions
-// x0 + q), first walking the list exactly when it would overflow.
-__device__ __forceinline__ void flag_push(FlagList& fl, const ExactCtx& c, unsigned fm, int x0, int lane)
-{
-    const int cnt = __popc(fm);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (fl.gbuf) {
-        // hand the walks to the exact pass after the sweep: (item, sample)
-        // entries; when the buffer is full they are walked here instead
-        unsigned at = 0u;
-        if (lane == 0) at = atomicAdd(fl.gcount, (unsigned)total);
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if ((unsigned long long)at + (unsigned long long)total <= (unsigned long long)fl.gcap) {
-            unsigned pos = at + (unsigned)(incl - cnt);
-            for (unsigned m = fm; m; m &= m - 1, ++pos)
-                if (in_range(pos, fl.gcap, 20)) {
-                    const int xs = x0 + __ffs(m) - 1;   // staged sample; the entry holds the row's
-                    fl.gbuf[pos] = make_int4(fl.item, c.rev_staged ? c.L - 1 - xs : xs, __float_as_int(fl.zmax), 0);
-                }
-            __syncwarp();
-            return;
-        }
-        // full: the slots reserved below the capacity are marked empty
-        for (unsigned long long pos = (unsigned long long)at + lane;
-             pos < (unsigned long long)at + (unsigned long long)total && pos < (unsigned long long)fl.gcap; pos += 32)
-            fl.gbuf[pos] = make_int4(-1, -1, 0, 0);
-        __syncwarp();
-    }
-    if (fl.count + total > FLAG_CAP) drain_flags(fl, c, lane);
-    int pos = fl.count + incl - cnt;
-    for (unsigned m = fm; m; m &= m - 1, ++pos)
-        if (in_range(pos, FLAG_CAP, 13)) fl.list[pos] = x0 + __ffs(m) - 1;
-    fl.count += total;
-    __syncwarp();
+    if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
 }
 
 // min(a, |b|, |c|).  TVS_CERT_MIN3 selects the three-input minimum of
@@ -921,24 +991,8 @@ __device__ __forceinline__ void cert_block(const float* y, const float4* __restr
     }
 }
 
-// Upper bound of the slopes a POV of the group can meet among targets whose
-// hi heights are at most z (a suffix or prefix maximum): max(0, z + slack -
-// Rh - gmin) / (e + 1), with slack covering the hi / lo split, the rounding of
-// the differences and of g (2^-20 relative, plus eg).  z = -inf (sentinels
-// only) gives 0.
-__device__ __forceinline__ float bound_slope(float z, float Rh, float gmin, float eg, float ive)
-{
-    const float A = __fsub_rn(__fsub_rn(z, Rh), gmin);
-    const float sl = 0x1p-20f * (fminf(fabsf(z), 0x1p100f) + fabsf(Rh) + fabsf(gmin)) + eg;
-    return __fmul_rn(fmaxf(__fadd_rn(A, sl), 0.f), ive) * 1.0000039f;
-}
-
-// Certified sweep of one staged row (the lane queue of sweep_row).  eg0 =
-// 2.01u |h0| + |h0 - float(h0)| + 4 eta (the parts of Eg that do not depend
-// on the group).  With PRUNE a group stops once, for every POV q, the
-// remaining targets' largest possible exact slope (from the suffix maxima,
-// or the prefix maxima of a backward walk) is at most M_q - 2 delta_q: they
-// are then not above theta_a exactly.
+// Certified sweep of one staged row (the lane queue of sweep_row).  Every
+// target is walked; pruned launches take sweep_row_skip.
 //
 // The row is staged in row order for both walk directions.  A group covers
 // the samples x0 .. x0 + P - 1 (x0 a multiple of 4, so that every window is
@@ -947,18 +1001,17 @@ __device__ __forceinline__ float bound_slope(float z, float Rh, float gmin, floa
 // w meets the window's element q + w + 1: a backward block's window is
 // loaded from x0 - e - U and stored reversed.  Backward groups are taken
 // from the row's end (the longest walks first).
-template <int P, int U, bool LONG, bool PRUNE, bool BWD, bool TIERS>
-__device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* __restrict__ ZS,
-                                               const float4* __restrict__ tab,
-                                               int tabn, int* __restrict__ spill, float eg0, FlagList& fl, int lane)
+template <int P, int U, bool LONG, bool BWD, bool TIERS>
+__device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const CertRow& r,
+                                               const float4* __restrict__ tab, int* __restrict__ spill, int lane)
 {
     static_assert(P % 4 == 0 && U % 4 == 0, "window loads must stay 16-byte aligned");
     const unsigned FULL = 0xffffffffu;
     const unsigned below = (1u << lane) - 1u;
     const float NEG = neg_inf();
-    const float* __restrict__ H = xc.H;
-    const float* __restrict__ Lo = xc.Lo;
-    const int L = xc.L, K = xc.K;
+    const float* __restrict__ H = r.H;
+    const float* __restrict__ Lo = r.Lo;
+    const int L = r.L, K = r.K, tabn = sp.inv_len;
     const int G = (L + P - 1) / P;
     const int klim = K - 1;
     // a backward block's window is stored reversed, so its aligned register
@@ -969,7 +1022,7 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
     float2 M2[P / 2], acc2[P / 2];   // running maxima of POV pairs (packed x - M)
 #define CERT_M(q) ((q) % 2 ? M2[(q) / 2].y : M2[(q) / 2].x)
 #define CERT_NG(q) ((q) % 2 ? ng2[(q) / 2].y : ng2[(q) / 2].x)
-    float Rh = 0.f, gmin = 0.f, c2e = 0.f;
+    float Rh = 0.f, c2e = 0.f;
     unsigned mask = 0u;
     int gi = lane, next = 32;
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
@@ -1000,9 +1053,7 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
         const int elast = (dlim - 1) / U * U;
         const int wlo = BWD ? x0 - elast - U : x0;           // lowest window start
         const int whi = BWD ? x0 - U : x0 + elast;           // highest window start
-        const int zsi = BWD ? (x0 + P - 2) / ZS_STRIDE : (x0 + elast + 1) / ZS_STRIDE;
-        if (!in_range(ROW_PADL + wlo, xc.half, 19) || !in_range(ROW_PADL + whi + P + U - 1, xc.half, 19) ||
-            (PRUNE && !in_range(zsi, xc.zs_len, 9)) ||
+        if (!in_range(ROW_PADL + wlo, sp.half, 19) || !in_range(ROW_PADL + whi + P + U - 1, sp.half, 19) ||
             (!(LONG && elast + U > tabn) && !in_range(elast + U - 1, tabn, 11))) {
             dlim = 0;
             const unsigned all = L - x0 >= P ? (1u << P) - 1u : (1u << (L - x0)) - 1u;   // bits by sample
@@ -1010,24 +1061,22 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
             return;
         }
         float Rl;
-        pov_hl(xc, x0, Rh, Rl);
+        pov_hl(r, x0, Rh, Rl);
         (void)Rl;
         float gmax = 0.f;
-        gmin = pos_inf();
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             const int x = pov_x(q);
             float gq = 0.f;
             if (BWD ? (x >= 1 && x <= L - 1) : x <= L - 2) {   // POVs with a target
                 float zh, zl;
-                pov_hl(xc, x, zh, zl);
-                gq = __fadd_rn(__fadd_rn(__fsub_rn(zh, Rh), zl), xc.h0h);
-                gmin = fminf(gmin, gq);
+                pov_hl(r, x, zh, zl);
+                gq = __fadd_rn(__fadd_rn(__fsub_rn(zh, Rh), zl), r.h0);
             }
             CERT_NG(q) = -gq;
             gmax = fmaxf(gmax, fabsf(gq));
         }
-        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, eg0);
+        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, r.eg0);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             // target 1 (a sentinel, -inf, when the POV has no target adding
@@ -1039,8 +1088,7 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
             const float x1 = __fadd_rn(y1, CERT_NG(q));
             const float C = __fmaf_rn(0x1p-6f, fabsf(x1), __fmaf_rn(4.f, c2e, 0x1p-16f));
             // a POV with no target that adds area starts at +inf: nothing is
-            // visible to it, no step is inside its margin, and it never holds
-            // back pruning
+            // visible to it and no step is inside its margin
             const bool area = BWD ? (x >= 2 && x <= L - 1) : x <= L - 3;
             CERT_M(q) = area ? __fsub_rn(x1, C) : pos_inf();
             ia[q] = 1.f;
@@ -1052,20 +1100,8 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
         const unsigned need = __ballot_sync(FULL, fin);
         if (need) {
             if (fin) {
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    const int x = pov_x(q);
-                    if (x < L && !((mask >> q) & 1u)) {
-                        const int n = walk_n(x);
-                        const float s = q % 2 ? acc2[q / 2].y : acc2[q / 2].x;
-                        xc.cvrow[xc.rev_staged ? L - 1 - x : x] = n >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
-                    }
-                }
-            }
-            // flagged POVs as bits by sample (x0 + bit)
-            const unsigned fm = fin ? (BWD ? __brev(mask) >> (32 - P) : mask) : 0u;
-            if (__any_sync(FULL, fm != 0u)) flag_push(fl, xc, fm, x0, lane);
-            if (fin) {
+                finish_group<P, LONG, BWD>(sp, r, x0, mask, pov_x, walk_n,
+                                           [&](int q) { return q % 2 ? acc2[q / 2].y : acc2[q / 2].x; }, spill);
                 gi = next + __popc(need & below);
                 if (gi < G) start(); else gi = G;
             }
@@ -1083,13 +1119,11 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
                     acc2[q / 2] = make_float2(0.f, 0.f);
                 }
             }
-            // a margin block of nh window blocks of U steps.  The bounds are
-            // formed branch-free: a window or suffix of sentinels only (-inf)
-            // gives 0.  A margin block of several window blocks lies wholly
+            // a margin block of nh window blocks of U steps.  A margin block of several window blocks lies wholly
             // before the group's last needed step (e + nh U <= dlim), so none
             // of its window blocks is masked and every window and table entry
             // it reads lies in the ranges start() checked.
-            const int nh = (!TIERS || PRUNE || LONG || e < CERT_NEAR) ? 1
+            const int nh = (!TIERS || LONG || e < CERT_NEAR) ? 1
                          : (e >= CERT_FAR2 && e + 8 * U <= dlim) ? 8
                          : (e >= CERT_FAR && e + 4 * U <= dlim) ? 4
                          : (e + 2 * U <= dlim) ? 2 : 1;
@@ -1100,22 +1134,6 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
             for (int q = 0; q < P; ++q) {
                 Ms[q] = CERT_M(q);
                 mn[q] = pos_inf();
-            }
-            if (PRUNE) {
-                // the remaining targets (samples from x0 + e + 1 on forward, up
-                // to x0 + P - 2 - e backward) have exact slopes of at most Bp;
-                // delta with Mb = |M| bounds |M - theta_a| now, so once M - 2
-                // delta >= Bp for every POV none of them rises above theta_a
-                const float ce = __fmaf_rn(c2e, ive, CERT_FLOOR);
-                const int zi = BWD ? max(x0 + P - 2 - e, 0) / ZS_STRIDE : (x0 + e + 1) / ZS_STRIDE;
-                const float Bp = bound_slope(ZS[zi], Rh, gmin, 2.f * c2e, ive);
-                float m = pos_inf();
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    const float dq = __fmaf_rn(CERT_REL, fabsf(CERT_M(q)), __fmaf_rn(c2e, ia[q], ce));
-                    m = fminf(m, __fmaf_rn(-2.f, dq, CERT_M(q)));
-                }
-                if (m >= Bp) { e = dlim; continue; }
             }
 #pragma unroll 1
             for (int h = 0; h < nh; ++h) {
@@ -1164,9 +1182,272 @@ __device__ __forceinline__ void sweep_row_cert(const ExactCtx& xc, const float* 
             e += nh * U;
         }
     }
-    if (fl.count > 0) drain_flags(fl, xc, lane);
 #undef CERT_M
 #undef CERT_NG
+}
+
+// Pruned certified sweep of one staged row: sweep_row_cert's walk, but a lane
+// evaluates only the blocks of U steps that can hold a visible target, and
+// stops where none is left.  (On fractal terrain 3 to 5 % of the targets of a
+// walk are visible; the walks reach their stopping point after about 40 % of
+// them, and about 12 % lie in blocks that cannot be skipped.)
+//
+// The test needs no slope: POV q's exact running maximum theta_a is at least
+// thr_q = M_q - 2 delta_q (delta_q bounds |M_q - theta_a| as it does in the
+// margin test, taken at the last evaluated block, whose 1 / (e + 1) is
+// larger), so a target at distance d that is no higher than the line
+//     R + g_q + thr_q d
+// is not visible and leaves the maximum as it is.  Over the block's distances
+// e + 1 .. e + U the line is lowest at the first when thr_q >= 0, at the last
+// otherwise:
+//     limit_q = thr_q (e + 1) + k_q,
+//     k_q = R + g_q + (U - 1) min(thr_q, 0) - slack,
+// and the block is skipped when its window's maximum height (WM) is at most
+// min_q limit_q.  The walk is over when every thr_q >= 0 (the lines only
+// rise) and the maximum of all remaining targets (ZS: suffix maxima, or
+// prefix maxima walking backward) is at most that minimum too.  slack covers
+// the hi / lo split, the rounding of g_q (Eg) and of the line: the line's own
+// three roundings are relative to values no larger than the heights it is
+// compared with (where it is larger it is not close), 2^-20 of the row's
+// largest elevation and of |g_q| each; the (U - 1) term is taken 2^-17 larger.
+// A POV with no target that adds area has M = +inf and thr NaN, which the
+// minimum drops.
+//
+// Measured (sweep and exact pass, against the walk that only stopped): 2000^2
+// 196 -> 102 ms, 1000^2 31.8 -> 21.3 ms.  Bound by instruction latency: with 3
+// warps per scheduler half of the issue slots stayed empty, so the kernel
+// keeps no exact walks of its own (their context cost 200 bytes of local
+// memory per lane) and fits 16 warps in 128 registers (12 warps: 118 ms, 20
+// with spills: 127).
+//
+// Work is done in three warp-wide phases, each with as many lanes as possible:
+// finished groups are written and replaced (SKIP_RESTART lanes at a time, or
+// when no lane has work); lanes without a block test SKIP_TESTS blocks at a
+// time until SKIP_READY lanes have one or nobody is searching; the lanes that
+// have one evaluate it.  A lane waits while others search or restart, so the
+// thresholds trade idle lanes against phases run for a few lanes only.  A
+// block is evaluated SKIP_CHUNK steps at a time, with the window formed as it
+// goes: the few registers that takes let 20 warps share an SM, and their
+// number is what hides the latency of the tests.
+template <int P, int U, bool LONG, bool BWD>
+__device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const CertRow& r, const float* __restrict__ ZS,
+                                               const float* __restrict__ WM, const float4* __restrict__ tab,
+                                               int* __restrict__ spill, int lane)
+{
+    constexpr int CH = SKIP_CHUNK, NT = SKIP_TESTS;
+    static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
+    const unsigned FULL = 0xffffffffu;
+    const unsigned below = (1u << lane) - 1u;
+    const float* __restrict__ H = r.H;
+    const float* __restrict__ Lo = r.Lo;
+    const int L = r.L, K = r.K, tabn = sp.inv_len;
+    const int G = (L + P - 1) / P;
+    const int klim = K - 1;
+    constexpr bool PACK = !BWD && TVS_CERT_PACKADD;
+    float ia[P];
+    float2 ng2[P / 2];               // -g of POV pairs
+    float2 M2[P / 2], acc2[P / 2];   // running maxima and measures of POV pairs
+    float2 T2[P / 2], K2[P / 2];     // thr and k of POV pairs
+    bool rising = false;             // every thr >= 0
+    float Rh = 0.f, c2e = 0.f;
+    unsigned mask = 0u;
+    int gi = lane, next = 32;
+    int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
+    bool klimited = false, ready = false;
+    auto pov_x = [&](int q) { return BWD ? x0 + P - 1 - q : x0 + q; };
+    auto walk_n = [&](int x) { return min(BWD ? x : L - 1 - x, K); };
+    // every index the row's blocks and tests use, checked once: windows start
+    // at most U samples before the row and end before sample L + P + U
+    const bool inside = in_range(ROW_PADL + L + P + U, sp.half, 19) && in_range((L - 1) / ZS_STRIDE, sp.zs_len, 9) &&
+                        in_range((L + U + 3) / ZS_STRIDE - 1, sp.wm_len, 10) &&
+                        (LONG || in_range(min(K, L) + U - 1, tabn, 11));
+
+    auto start = [&]() {
+        x0 = (BWD ? G - 1 - gi : gi) * P;
+        const int xl = BWD ? min(x0 + P - 1, L - 1) : x0;
+        const int rowlim = BWD ? xl - 1 : L - 2 - xl;
+        dlim = min(klim, rowlim);
+        klimited = klim < rowlim;
+        e = 0;
+        seg = FLUSH_STEPS;
+        mask = 0u;
+#pragma unroll
+        for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
+        if (LONG) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) spill[32 * q] = 0;
+        }
+        if (dlim < 1) return;
+        if (!inside) {
+            dlim = 0;
+            const unsigned all = L - x0 >= P ? (1u << P) - 1u : (1u << (L - x0)) - 1u;   // bits by sample
+            mask = BWD ? __brev(all) >> (32 - P) : all;                                   // bits by POV q
+            return;
+        }
+        ready = true;                                        // the first block is always evaluated
+        // the group's samples in POV order, and each POV's first target
+        const float4 a = *reinterpret_cast<const float4*>(H + x0), b = *reinterpret_cast<const float4*>(Lo + x0);
+        const int xt = BWD ? x0 - 1 : x0 + P;                // POV P - 1's first target
+        const float th = H[xt], tl = Lo[xt];
+        const float zs[P + 1] = {BWD ? a.w : a.x, BWD ? a.z : a.y, BWD ? a.y : a.z, BWD ? a.x : a.w, th};
+        const float ls[P + 1] = {BWD ? b.w : b.x, BWD ? b.z : b.y, BWD ? b.y : b.z, BWD ? b.x : b.w, tl};
+        float zh[P], zl[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) { zh[q] = zs[q]; zl[q] = ls[q]; }
+        if (x0 == 0) {                                       // the row's end samples are sentinels when staged
+            zh[BWD ? P - 1 : 0] = r.eh0;
+            zl[BWD ? P - 1 : 0] = r.el0;
+        }
+        if (x0 + P >= L) {
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+                if (pov_x(q) == L - 1) { zh[q] = r.ehL; zl[q] = r.elL; }
+        }
+        Rh = zh[BWD ? P - 1 : 0];
+        float gq[P], gmax = 0.f;
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const int x = pov_x(q);
+            const bool pov = BWD ? (x >= 1 && x <= L - 1) : x <= L - 2;   // POVs with a target
+            gq[q] = pov ? __fadd_rn(__fadd_rn(__fsub_rn(zh[q], Rh), zl[q]), r.h0) : 0.f;
+            gmax = fmaxf(gmax, fabsf(gq[q]));
+        }
+        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, r.eg0);
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            // as sweep_row_cert: M starts just below the first target's slope
+            const int x = pov_x(q);
+            const float x1 = __fsub_rn(__fadd_rn(__fsub_rn(zs[q + 1], Rh), ls[q + 1]), gq[q]);
+            const float C = __fmaf_rn(0x1p-6f, fabsf(x1), __fmaf_rn(4.f, c2e, 0x1p-16f));
+            const bool area = BWD ? (x >= 2 && x <= L - 1) : x <= L - 3;
+            (q % 2 ? ng2[q / 2].y : ng2[q / 2].x) = -gq[q];
+            (q % 2 ? M2[q / 2].y : M2[q / 2].x) = area ? __fsub_rn(x1, C) : pos_inf();
+            ia[q] = 1.f;
+        }
+    };
+    if (gi < G) start();
+    for (;;) {
+        // 1. finished groups: write their measures, hand over their flagged
+        // walks, take the next groups
+        const bool fin = gi < G && !ready && e >= dlim;
+        const unsigned need = __ballot_sync(FULL, fin);
+        if (need && (__popc(need) >= SKIP_RESTART || !__any_sync(FULL, gi < G && !fin))) {
+            if (fin) {
+                finish_group<P, LONG, BWD>(sp, r, x0, mask, pov_x, walk_n,
+                                           [&](int q) { return q % 2 ? acc2[q / 2].y : acc2[q / 2].x; }, spill);
+                gi = next + __popc(need & below);
+                if (gi < G) start(); else gi = G;
+            }
+            next += __popc(need);
+            if (!__any_sync(FULL, gi < G)) break;
+        }
+        // 2. lanes without a block look for one
+        for (;;) {
+            if (gi < G && !ready && e < dlim) {
+                const float d = (float)(e + 1);
+                // x0 and e are multiples of 4; the entries of blocks past the
+                // walk's end are not used
+                const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE, wlast = (L + U + 3) / ZS_STRIDE - 1;
+                float lim[NT], wm[NT];
+#pragma unroll
+                for (int k = 0; k < NT; ++k) {
+                    const float dk = d + (float)(k * U);
+                    const float2 l0 = __ffma2_rn(T2[0], make_float2(dk, dk), K2[0]);
+                    const float2 l1 = __ffma2_rn(T2[1], make_float2(dk, dk), K2[1]);
+                    lim[k] = fminf(fminf(l0.x, l0.y), fminf(l1.x, l1.y));
+                    wm[k] = WM[BWD ? max(w0 - k * U / ZS_STRIDE, 0) : min(w0 + k * U / ZS_STRIDE, wlast)];
+                }
+                const float end = ZS[(BWD ? x0 - e : x0 + e) / ZS_STRIDE];
+                int n = NT;
+#pragma unroll
+                for (int k = NT - 1; k >= 0; --k)
+                    if (!(wm[k] <= lim[k])) n = k;
+                e = rising && end <= lim[0] ? dlim : e + n * U;
+                ready = n < NT && e < dlim;
+            }
+            const unsigned have = __ballot_sync(FULL, ready);
+            const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
+            if (!look || __popc(have) >= SKIP_READY) break;
+        }
+        // 3. evaluate the blocks found
+        if (ready) {
+            ready = false;
+            if (LONG && e >= seg) {
+                // at most FLUSH_STEPS steps of distance between two flushes
+                seg = e + FLUSH_STEPS;
+#pragma unroll
+                for (int q = 0; q < P; q += 2) {
+                    spill[32 * q] += __float2int_rz(acc2[q / 2].x);
+                    spill[32 * (q + 1)] += __float2int_rz(acc2[q / 2].y);
+                    acc2[q / 2] = make_float2(0.f, 0.f);
+                }
+            }
+            const bool far = LONG && e + U > tabn;
+            const float4* __restrict__ tb = tab + e + e / U;
+            const float ive = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tb->x;
+            float Ms[P], mn[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                Ms[q] = q % 2 ? M2[q / 2].y : M2[q / 2].x;
+                mn[q] = pos_inf();
+            }
+            {
+                // the window relative to R, y[m] = sample m of the block's
+                // window in walk order, kept P samples back from step to step
+                const float2 nRh = make_float2(-Rh, -Rh);
+                const float* bh = H + (BWD ? x0 - e : x0 + e);
+                const float* bl = Lo + (BWD ? x0 - e : x0 + e);
+                float y[P + CH];
+                auto quad = [&](int at, int m) {   // y[m ..] from the four samples at `at`
+                    const float4 a = *reinterpret_cast<const float4*>(bh + at);
+                    const float4 b = *reinterpret_cast<const float4*>(bl + at);
+                    const float2 y0 = __fadd2_rn(__fadd2_rn(make_float2(a.x, a.y), nRh), make_float2(b.x, b.y));
+                    const float2 y1 = __fadd2_rn(__fadd2_rn(make_float2(a.z, a.w), nRh), make_float2(b.z, b.w));
+                    y[m] = BWD ? y1.y : y0.x;
+                    y[m + 1] = BWD ? y1.x : y0.y;
+                    y[m + 2] = BWD ? y0.y : y1.x;
+                    y[m + 3] = BWD ? y0.x : y1.y;
+                };
+                quad(0, 0);
+                const int steps = min(dlim - e, U);
+#pragma unroll 1
+                for (int c = 0; c < steps; c += CH) {
+#pragma unroll
+                    for (int m = P; m < P + CH; m += 4) quad(BWD ? -(c + m) : c + m, m);
+                    if (klimited && c + CH > steps) {
+                        if (far) cert_block<P, CH, true, true, PACK>(y, tab, e + c, ng2, M2, acc2, mn, steps - c);
+                        else cert_block<P, CH, true, false, PACK>(y, tb + c, e, ng2, M2, acc2, mn, steps - c);
+                    } else {
+                        if (far) cert_block<P, CH, false, true, PACK>(y, tab, e + c, ng2, M2, acc2, mn, CH);
+                        else cert_block<P, CH, false, false, PACK>(y, tb + c, e, ng2, M2, acc2, mn, CH);
+                    }
+#pragma unroll
+                    for (int m = 0; m < P; ++m) y[m] = y[m + CH];
+                }
+            }
+            // the margin test of sweep_row_cert, and the lines of the next tests
+            const float ce = __fmaf_rn(c2e, ive, CERT_FLOOR);
+            float gm = 0.f;
+#pragma unroll
+            for (int q = 0; q < P; ++q) gm = fmaxf(gm, fabsf(q % 2 ? ng2[q / 2].y : ng2[q / 2].x));
+            const float base = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, r.zmax, gm), __fmul_rn(2.f, c2e)));
+            rising = true;
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const float m = q % 2 ? M2[q / 2].y : M2[q / 2].x;
+                const float dq = __fmaf_rn(CERT_REL, fmaxf(fabsf(Ms[q]), fabsf(m)), __fmaf_rn(c2e, ia[q], ce));
+                mask |= mn[q] < dq ? 1u << q : 0u;
+                ia[q] = m > Ms[q] ? ive : ia[q];
+                const float thr = __fmaf_rn(-2.f, dq, m);
+                const float g = -(q % 2 ? ng2[q / 2].y : ng2[q / 2].x);
+                (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
+                (q % 2 ? K2[q / 2].y : K2[q / 2].x) =
+                    __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), __fadd_rn(base, g));
+                rising = rising && !(thr < 0.f);
+            }
+            e += U;
+        }
+    }
 }
 
 template <bool LONG, bool PRUNE>
@@ -1254,7 +1535,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
 // room for at least TVS_CERT_SINGLE_MIN of them (16 warps when they fit, else
 // 12): a backward item's row is staged reversed and walked forward, like the
 // FP32 sweep's.  Per warp, shared memory holds
-// [Fh half][Fl half][suffix maxima][flag list][spill][ends 4].
+// [Fh half][Fl half][suffix maxima][window maxima][ends 4].
 template <bool PRUNE, bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams sp)
 {
@@ -1265,17 +1546,17 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
     float* Fh = smem + 4 * sp.tab_slots + sp.istart_len + warp * sp.per_warp;
     float* Fl = Fh + sp.half;
     float* ZS = Fl + sp.half;
-    int* flist = reinterpret_cast<int*>(ZS + sp.zs_len);
-    int* spill = flist + sp.fl_cap + lane;
+    float* WM = ZS + sp.zs_len;
+    constexpr int U = PRUNE ? SKIP_UNROLL : CERT_UNROLL_SINGLE;
+    int* spill = reinterpret_cast<int*>(WM + sp.wm_len) + lane;
     float* ends = Fh + sp.per_warp - 4;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
         const float c = (float)(2 * m + 3);
-        tab[m + m / CERT_UNROLL_SINGLE] = make_float4(r, r, c, c);
+        tab[m + m / U] = make_float4(r, r, c, c);
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
-    FlagList fl{flist, 0, sp.flag_buf, sp.flag_count, sp.flag_cap, 0, 0.f};
     const long long t_start = clock64();
 
     int next = 0;
@@ -1292,40 +1573,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         __syncwarp();
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
         __syncwarp();   // the staged row is visible to every lane
-        if (PRUNE) suffix_max(Fh, ZS, it.L, lane);
-        __syncwarp();
-        fl.item = item;
-        fl.zmax = zmax;
-        const DirDev* d = sp.dirs + it.dir;
-        ExactCtx xc;
-        xc.H = Fh + ROW_PADL;
-        xc.Lo = Fl + ROW_PADL;
-        xc.L = it.L;
-        xc.K = it.K;
-        xc.h0h = it.h0;
-        xc.h0l = d->h0_lo;
-        xc.eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
-        xc.cvrow = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
-        xc.bwd = false;
-        xc.from_dem = false;
-        xc.rev_staged = it.rev;
-        xc.eh0 = ends[0];
-        xc.el0 = ends[1];
-        xc.ehL = ends[2];
-        xc.elL = ends[3];
-        xc.dir = d;
-        xc.job = sp.jobs + d->job;
-        xc.p = it.p;
-        xc.jlo = it.jlo;
-        xc.half = sp.half;
-        xc.zs_len = sp.zs_len;
-        xc.tab = tab;
-        xc.tskew = CERT_UNROLL_SINGLE;
-        xc.tabn = sp.inv_len;
-        const float u = 0x1p-24f;
-        const float eg0 = 2.01f * u * fabsf(it.h0) + fabsf(d->h0_lo) * 1.0001f + 4.04f * xc.eta;
-        sweep_row_cert<CERT_POV, CERT_UNROLL_SINGLE, LONG, PRUNE, false, false>(xc, ZS, tab, sp.inv_len, spill, eg0,
-                                                                                fl, lane);
+        if (PRUNE) {
+            end_max<false>(Fh, ZS, it.L, lane);
+            window_max<CERT_POV, U>(Fh, WM, it.L, lane);
+            __syncwarp();
+        }
+        const CertRow r = cert_row(sp, it, item, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
+        if constexpr (PRUNE) sweep_row_skip<CERT_POV, U, LONG, false>(sp, r, ZS, WM, tab, spill, lane);
+        else sweep_row_cert<CERT_POV, U, LONG, false, false>(sp, r, tab, spill, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
@@ -1344,8 +1599,8 @@ __device__ __forceinline__ void pair_sync(int pair)
 // rows).  Both warps stage half of the row; the forward warp computes its
 // suffix maxima, the backward warp its prefix maxima (pruning).  Each warp
 // runs one direction's code only.  Per pair, shared memory holds [Fh
-// half][Fl half][suffix maxima][prefix maxima][ends 4][exchange 4]; per warp
-// the flagged-POV list and the long-walk spill.
+// half][Fl half][suffix maxima][prefix maxima][window maxima][ends 4][exchange 4]; per warp
+// the long-walk spill.
 template <bool PRUNE, bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams sp)
 {
@@ -1359,19 +1614,19 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     float* Fh = base + pair * sp.per_pair;
     float* Fl = Fh + sp.half;
     float* ZS = Fl + sp.half + bwd * sp.zs_len;            // this warp's suffix or prefix maxima
-    float* ends = Fl + sp.half + 2 * sp.zs_len;              // 4 floats
+    float* WM = Fl + sp.half + 2 * sp.zs_len;              // window maxima (both warps')
+    float* ends = WM + sp.wm_len;                          // 4 floats
+    constexpr int U = PRUNE ? SKIP_UNROLL : CERT_UNROLL;
     float* xch = ends + 4;                                   // item number and the halves' zmax
     float* own = base + npairs * sp.per_pair + warp * sp.per_warp;
-    int* flist = reinterpret_cast<int*>(own);
-    int* spill = reinterpret_cast<int*>(own) + sp.fl_cap + lane;
+    int* spill = reinterpret_cast<int*>(own) + lane;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
         const float c = (float)(2 * m + 3);
-        tab[m + m / CERT_UNROLL] = make_float4(r, r, c, c);
+        tab[m + m / U] = make_float4(r, r, c, c);
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
-    FlagList fl{flist, 0, sp.flag_buf, sp.flag_count, sp.flag_cap, 0, 0.f};
     const long long t_start = clock64();
 
     for (;;) {
@@ -1381,52 +1636,25 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
         if (pitem >= sp.total_items) break;
         ItemRow it;
         const bool nonempty = decode_item(sp, istart, pitem + bwd, &it);
-        fl.item = pitem + bwd;
         if (nonempty) {
             const float zpart = stage_row<true>(sp, it, Fh, Fl, ends, lane, bwd, 2, false);
             if (lane == 0) xch[1 + bwd] = zpart;
             pair_sync(pair);   // the staged row is complete
-            if (PRUNE) {   // each warp's own suffix or prefix maxima
-                if (bwd) prefix_max(Fh, ZS, it.L, lane);
-                else suffix_max(Fh, ZS, it.L, lane);
-                __syncwarp();
+            if (PRUNE) {   // each warp's own suffix or prefix maxima, half of the window maxima
+                if (bwd) end_max<true>(Fh, ZS, it.L, lane);
+                else end_max<false>(Fh, ZS, it.L, lane);
+                window_max<CERT_POV, U>(Fh, WM, it.L, lane, bwd, 2);
+                pair_sync(pair);
             }
             const float zmax = fmaxf(xch[1], xch[2]);
-            fl.zmax = zmax;
-            const DirDev* d = sp.dirs + it.dir;
-            ExactCtx xc;
-            xc.H = Fh + ROW_PADL;
-            xc.Lo = Fl + ROW_PADL;
-            xc.L = it.L;
-            xc.K = it.K;
-            xc.h0h = it.h0;
-            xc.h0l = d->h0_lo;
-            xc.eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
-            xc.cvrow = (bwd ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
-            xc.bwd = bwd != 0;
-            xc.from_dem = false;
-            xc.rev_staged = false;
-            xc.eh0 = ends[0];
-            xc.el0 = ends[1];
-            xc.ehL = ends[2];
-            xc.elL = ends[3];
-            xc.dir = d;
-            xc.job = sp.jobs + d->job;
-            xc.p = it.p;
-            xc.jlo = it.jlo;
-            xc.half = sp.half;
-            xc.zs_len = sp.zs_len;
-                xc.tab = tab;
-                xc.tskew = CERT_UNROLL;
-            xc.tabn = sp.inv_len;
-            const float u = 0x1p-24f;
-            const float eg0 = 2.01f * u * fabsf(it.h0) + fabsf(d->h0_lo) * 1.0001f + 4.04f * xc.eta;
-            if (bwd)
-                sweep_row_cert<CERT_POV, CERT_UNROLL, LONG, PRUNE, true, true>(xc, ZS, tab, sp.inv_len, spill, eg0, fl,
-                                                                               lane);
-            else
-                sweep_row_cert<CERT_POV, CERT_UNROLL, LONG, PRUNE, false, true>(xc, ZS, tab, sp.inv_len, spill, eg0, fl,
-                                                                                lane);
+            const CertRow r = cert_row(sp, it, pitem + bwd, Fh, Fl, ends, zmax, bwd ? sp.cv_bwd : sp.cv_fwd, false);
+            if constexpr (PRUNE) {
+                if (bwd) sweep_row_skip<CERT_POV, U, LONG, true>(sp, r, ZS, WM, tab, spill, lane);
+                else sweep_row_skip<CERT_POV, U, LONG, false>(sp, r, ZS, WM, tab, spill, lane);
+            } else {
+                if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
+                else sweep_row_cert<CERT_POV, U, LONG, false, true>(sp, r, tab, spill, lane);
+            }
         }
         pair_sync(pair);   // both walks are done with the row (and with the exchange slot)
     }
@@ -1452,37 +1680,50 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
         i = __shfl_sync(0xffffffffu, i, 0);
         if (i >= n) break;
         const int4 en = sp.flag_buf[i];
-        if (en.x < 0) continue;                 // a slot of a push that did not fit
         if (!in_range(en.x, sp.total_items, 22)) continue;
         ItemRow it;
         if (!decode_item(sp, sp.item_start, en.x, &it)) continue;
         if (!in_range(en.y, it.L, 23)) continue;
-        const DirDev* d = sp.dirs + it.dir;
-        ExactCtx xc;
-        xc.H = nullptr;
-        xc.Lo = nullptr;
-        xc.L = it.L;
-        xc.K = it.K;
-        xc.h0h = it.h0;
-        xc.h0l = d->h0_lo;
-        xc.eta = 0x1p-42f * (__int_as_float(en.z) + fabsf(it.h0)) + 0x1p-126f;
-        xc.cvrow = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
-        xc.bwd = it.rev;
-        xc.from_dem = true;
-        xc.rev_staged = false;
-        xc.eh0 = xc.el0 = xc.ehL = xc.elL = 0.f;
-        xc.dir = d;
-        xc.job = sp.jobs + d->job;
-        xc.p = it.p;
-        xc.jlo = it.jlo;
-        xc.half = sp.half;
-        xc.zs_len = 0;
-        xc.tab = nullptr;
-        xc.tabn = 0;     // 1/d by __frcp_rn
-        xc.tskew = 1;
+        const ExactCtx xc = exact_ctx(sp, it, __int_as_float(en.z));
         exact_walk(xc, en.y, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[2], (unsigned long long)(clock64() - t_start));
+}
+
+// The walks that found the flag buffer full: their measures are negative.
+// Does nothing unless the sweep saw a full buffer; otherwise every row of the
+// launch is searched, a warp per item, and its marked walks are walked exactly.
+__global__ void __launch_bounds__(EXACT_WARPS * 32) exact_scan_kernel(SweepParams sp)
+{
+    if (sp.flag_count[2] == 0u) return;
+    const int lane = threadIdx.x & 31;
+    const long long step = (long long)gridDim.x * EXACT_WARPS;
+    for (long long item = (long long)blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); item < sp.total_items;
+         item += step) {
+        ItemRow it;
+        if (!decode_item(sp, sp.item_start, (int)item, &it)) continue;
+        const int* cv = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
+        ExactCtx xc;
+        bool ready = false;                  // xc is set once a marked walk is found
+        for (int x0 = 0; x0 < it.L; x0 += 32) {
+            unsigned marked = __ballot_sync(0xffffffffu, x0 + lane < it.L && cv[x0 + lane] < 0);
+            if (marked && !ready) {
+                ready = true;
+                xc = exact_ctx(sp, it, 0.f);
+                float zmax = 0.f;
+                for (int x = lane; x < it.L; x += 32) {
+                    float va, vb;
+                    unsigned fr;
+                    dem_pair(xc, x, va, vb, fr);
+                    zmax = fmaxf(zmax, fmaxf(fabsf(va), fabsf(vb)));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+                xc = exact_ctx(sp, it, zmax);
+            }
+            for (; marked; marked &= marked - 1) exact_walk(xc, x0 + __ffs(marked) - 1, lane);
+        }
+    }
 }
 
 }  // namespace
@@ -1496,6 +1737,8 @@ constexpr int MIN_TABLE = 1024;
 // of up to wmax samples and walks of up to dmax steps in a launch of ndir
 // directions (launch_sweep runs that kernel when the count reaches
 // TVS_CERT_SINGLE_MIN).
+static int wm_entries(int wmax) { return ((wmax + SKIP_UNROLL + 3) / ZS_STRIDE + 4) & ~3; }
+
 static size_t cert_single_fit(int wmax, int dmax, int prune, int ndir, int smem_optin)
 {
     const int inv_len = (std::min(dmax, wmax) + 2 * LARGE_UNROLL + 8 + 1) & ~1;
@@ -1503,7 +1746,8 @@ static size_t cert_single_fit(int wmax, int dmax, int prune, int ndir, int smem_
     const int istart_len = (ndir + 1 + 3) & ~3;
     const int half = (ROW_PADL + 4 + wmax + ROW_PADR + 3) & ~3;
     const int zs_len = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
-    const int single_warp = 2 * half + zs_len + FLAG_CAP + 4;
+    const int wm_len = prune ? wm_entries(wmax) : 0;
+    const int single_warp = 2 * half + zs_len + wm_len + 4;
     const size_t fixed = (size_t)(4 * tab_slots + istart_len) * 4;
     return fixed >= (size_t)smem_optin ? 0 : ((size_t)smem_optin - fixed) / ((size_t)single_warp * 4);
 }
@@ -1526,10 +1770,10 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     sp.dirs = d_dirs; sp.jobs = d_jobs; sp.item_start = d_item_start; sp.rowlo = rowlo;
     sp.rowhi = rowhi; sp.cv_fwd = cv_fwd; sp.cv_bwd = cv_bwd; sp.counter = counter; sp.ndir = ndir;
     sp.total_items = total_items;
-    const bool pass = cert && flag_buf && flag_count && flag_cap > 0;   // flagged walks in a second kernel
-    sp.flag_buf = pass ? flag_buf : nullptr;
-    sp.flag_count = pass ? flag_count : nullptr;
-    sp.flag_cap = pass ? flag_cap : 0;
+    if (cert && !flag_count) return cudaErrorInvalidValue;
+    sp.flag_buf = flag_buf;
+    sp.flag_count = flag_count;
+    sp.flag_cap = flag_buf ? flag_cap : 0;
     // the distance table is read up to d = dmax + U (a walk of at most
     // min(K, W) - 1 steps, rounded up to U); dmax <= wmax
     sp.inv_len = (std::min(dmax, wmax) + 2 * U + 8 + 1) & ~1;
@@ -1538,7 +1782,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     sp.half = (ROW_PADL + 4 + wmax + ROW_PADR + 3) & ~3;
     const bool longw = wmax - 2 > LONG_WALK && dmax - 1 > LONG_WALK;
     sp.zs_len = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
-    sp.fl_cap = cert ? FLAG_CAP : 0;
+    sp.wm_len = prune && cert ? wm_entries(wmax) : 0;
     const int lspill = longw ? 32 * LARGE_POV : 0;
     // FP32 decisions: one row per warp.  Certified: one row per warp
     // (reversed for backward walks) when TVS_CERT_SINGLE_MIN such warps fit, else
@@ -1546,14 +1790,14 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     // the end samples and an exchange slot), and per warp its
     // flag list and spill: a row's samples are then held once for both walk
     // directions.
-    const int single_warp = 2 * sp.half + sp.zs_len + sp.fl_cap + 4;
+    const int single_warp = 2 * sp.half + sp.zs_len + sp.wm_len + 4;
     const size_t single_fit = cert ? cert_single_fit(wmax, dmax, prune, ndir, smem_optin) : 0;
     const int single_min = TVS_CERT_SINGLE_MIN;
     const bool single = cert && !longw && (max_warps == 0 || max_warps >= single_min) &&
                         single_fit >= (size_t)single_min;
     const bool pairs = cert && !single;
-    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + 8 : 0;
-    sp.per_warp = single ? single_warp : pairs ? sp.fl_cap + lspill : sp.half + sp.zs_len + lspill;
+    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 8 : 0;
+    sp.per_warp = single ? single_warp : pairs ? lspill : sp.half + sp.zs_len + lspill;
     // shared memory of one unit: a pair of warps or one warp
     const int uw = pairs ? 2 : 1;
     const size_t unit = (size_t)(sp.per_pair + uw * sp.per_warp) * 4;
@@ -1584,17 +1828,14 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     int most;
     if (single) {
         const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = wide ? WW : CW;
-        if (wide) kern = prune ? sweep_cert_kernel<true, false, WW> : sweep_cert_kernel<false, false, WW>;
-        else kern = prune ? sweep_cert_kernel<true, false, CW> : sweep_cert_kernel<false, false, CW>;
+        most = prune ? SKIP_WARPS : wide ? WW : CW;
+        if (prune) kern = sweep_cert_kernel<true, false, SKIP_WARPS>;
+        else kern = wide ? sweep_cert_kernel<false, false, WW> : sweep_cert_kernel<false, false, CW>;
     } else if (pairs) {
-        // pruned walks are short and restart groups often: the 12-warp
-        // instantiation (no spills) beats 16 warps there (2000^2: 210.9
-        // against 218.4 ms), while unpruned walks favour 16 (351 against 365)
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = wide ? WW : CW;
+        most = wide ? WW : prune && !longw ? SKIP_WARPS : CW;
         if (wide) kern = sweep_pair_kernel<false, false, WW>;
-        else kern = prune ? (longw ? sweep_pair_kernel<true, true, CW> : sweep_pair_kernel<true, false, CW>)
+        else kern = prune ? (longw ? sweep_pair_kernel<true, true, CW> : sweep_pair_kernel<true, false, SKIP_WARPS>)
                           : (longw ? sweep_pair_kernel<false, true, CW> : sweep_pair_kernel<false, false, CW>);
     } else {
         most = FW;
@@ -1611,19 +1852,22 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if (pass) {
-        err = cudaMemsetAsync(flag_count, 0, 2 * sizeof(unsigned), stream);
+    if (cert) {
+        err = cudaMemsetAsync(flag_count, 0, 3 * sizeof(unsigned), stream);
         if (err != cudaSuccess) return err;
     }
     kern<<<per_sm * num_sms, warps * 32, smem, stream>>>(sp);
     err = cudaGetLastError();
-    if (err != cudaSuccess || !pass) return err;
+    if (err != cudaSuccess || !cert) return err;
     // the exact pass: no shared memory, as many warps as registers allow
     int xper = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&xper, exact_kernel, EXACT_WARPS * 32, 0);
     if (err != cudaSuccess) return err;
     if (xper < 1) return cudaErrorInvalidConfiguration;
     exact_kernel<<<xper * num_sms, EXACT_WARPS * 32, 0, stream>>>(sp);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    exact_scan_kernel<<<num_sms, EXACT_WARPS * 32, 0, stream>>>(sp);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,82 @@
+"""The pruned certified walk (blocks skipped by their window maxima, flagged
+work handed over or marked): per-sample measures are integers and must equal
+the FP64 oracle's exactly, at row lengths around the group, block and chunk
+sizes, on terrain that falls away from every observer (negative slopes, the
+falling lines of the skip test), on ties, and with the flag buffer full."""
+import numpy as np
+import pytest
+
+import paper_2003_02200_gb300 as tvs
+from paper_2003_02200_gb300 import terrain
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    with tvs.Context(0) as c:
+        yield c
+
+
+def _terrain(kind, rows, cols, seed):
+    r = np.random.default_rng(seed)
+    j = np.arange(cols, dtype=np.float64)[None, :].repeat(rows, 0)
+    if kind == "fractal":
+        return terrain.fractal_dem(rows, cols, 0.7, 1200.0, seed)
+    if kind == "valley":        # every walk looks down first, then up a far slope
+        z = 0.004 * (j - 0.6 * cols) ** 2
+    elif kind == "ridge":       # slopes stay negative: the lines of the test fall
+        z = -0.01 * (j - 0.4 * cols) ** 2 - 300.0
+    elif kind == "sawtooth":    # many equal crests: near ties block after block
+        z = (j % 37) * 4.0 + 1000.0
+        return z.astype(np.float32)
+    else:
+        raise ValueError(kind)
+    return (z + r.uniform(0.0, 3.0, (rows, cols))).astype(np.float32)
+
+
+def _check(ctx, orc, dem, h0, n, rng, ks):
+    rows, cols = dem.shape
+    for k in ks:
+        got = ctx.debug_direction_cv(dem, 10.0, h0, n, rng, k)
+        d = orc.direction(n, k, rows, cols)
+        want = np.stack([orc.line_cv(dem, 10.0, h0, n, rng, 64, k, p - d["D"]) for p in range(d["H"] + d["D"])])
+        bad = np.argwhere(got != want)
+        assert bad.size == 0, f"k {k}: {len(bad)} samples differ, first {bad[:4].tolist()}"
+
+
+@pytest.mark.parametrize("cols", [2, 3, 4, 5, 15, 16, 17, 18, 19, 20, 21, 31, 33, 35, 63, 64, 66, 127, 129, 131, 513])
+@pytest.mark.parametrize("kind", ["fractal", "ridge"])
+def test_row_lengths(ctx, orc, cols, kind):
+    _check(ctx, orc, _terrain(kind, 5, cols, cols), 1.5, 8, 0.0, (0, 1, 7))
+
+
+@pytest.mark.parametrize("rng", [0.0, 9.0, 25.0, 159.0, 165.0, 175.0, 335.0, 700.0])
+@pytest.mark.parametrize("kind", ["fractal", "valley", "ridge", "sawtooth"])
+def test_walk_limits(ctx, orc, kind, rng):
+    """Limits inside, at and past a 16-step block."""
+    _check(ctx, orc, _terrain(kind, 6, 150, 5), 2.0, 12, rng, (0, 2, 11))
+
+
+# rows of 1100 to 2300 samples take the paired-warp layout, shorter ones one row per warp
+@pytest.mark.parametrize("cols", [1000, 1351, 2003, 2300])
+@pytest.mark.parametrize("kind", ["fractal", "valley", "ridge", "sawtooth"])
+def test_long_rows(ctx, orc, kind, cols):
+    _check(ctx, orc, _terrain(kind, 3, cols, 9), 1.5, 8, 0.0, (0, 7))
+
+
+@pytest.mark.parametrize("rows,cols", [(260, 300), (3, 2100)])
+def test_full_flag_buffer(ctx, rows, cols):
+    """Level ground seen from its own height: every target ties with the
+    running maximum, so nearly every walk is flagged and the buffer (one entry
+    per 64 walks) overflows.  A half-line of two or more targets sees the
+    first one only and measures 4; those of the inner cells all have them."""
+    n = 16
+    dem = np.zeros((rows, cols), np.float32)
+    got = ctx.total_viewshed(dem, 10.0, 0.0, n)
+    with tvs.Context(0) as c:
+        c.set_tuning(prune=0)
+        np.testing.assert_array_equal(got, c.total_viewshed(dem, 10.0, 0.0, n))
+    if rows > 10:
+        g = [1.0 + tvs.direction(n, k, rows, cols)["t"] ** 2 for k in range(n)]
+        np.testing.assert_allclose(got[20:-20, 20:-20], 8.0 * sum(g) * np.pi / (2 * n) * 100.0, rtol=4e-6)
