@@ -698,6 +698,26 @@ __device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const Cert
     return fm;
 }
 
+// The sample field of a flag entry holds the entry's kind above bit 16: a
+// whole walk to take again, or one block of a walk whose running maximum
+// before it lies in one earlier block, or anywhere before it.  The fourth
+// field of a block entry is its first step e0 and that earlier block's.
+constexpr int FLAG_WALK = 0, FLAG_BLOCK = 1, FLAG_PREFIX = 2;
+static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
+
+// Hands block e0 of staged sample x's walk to the exact pass, p0 the block of
+// its last rise; false when the buffer is full.
+__device__ __forceinline__ bool flag_block(const SweepParams& sp, const CertRow& r, int x, int e0, int p0, int kind)
+{
+    const unsigned cap = (unsigned)sp.flag_cap;
+    unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
+    if (at < cap) at = atomicAdd(sp.flag_count, 1u);
+    if (at >= cap) return false;
+    sp.flag_buf[at] = make_int4(r.item, (r.rev_staged ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax),
+                                e0 | p0 << 14);
+    return true;
+}
+
 // Writes the measures of a finished group of P POVs (pov_x(q): staged sample
 // of POV q; mask: its flagged POVs).
 template <int P, bool LONG, bool BWD, class X, class N, class S>
@@ -792,10 +812,10 @@ __device__ __forceinline__ int warp_sum(int v)
 
 // The FP64 walk of POV x (Alg. 8 in double precision: theta = (z - h) / d
 // rounded once, strict comparison with the running maximum): sum of 2d + 1
-// over the visible targets d = 1 .. last.  Warp-cooperative: 32 x XW_KPL
+// over the visible targets d = from + 1 .. last.  Warp-cooperative: 32 x XW_KPL
 // targets per chunk, a warp max-scan gives each lane the running maximum
 // before its first target.
-__device__ __noinline__ int fp64_walk(const ExactCtx& c, int x, int last, int lane)
+__device__ __noinline__ int fp64_walk(const ExactCtx& c, int x, int from, int last, int lane)
 {
     const double h = __dadd_rn(z64_at(c, x), c.job->h0);
     const int dir = c.bwd ? -1 : 1;
@@ -824,20 +844,26 @@ __device__ __noinline__ int fp64_walk(const ExactCtx& c, int x, int last, int la
         for (int k = 0; k < XW_KPL; ++k) {
             const int d = d0 + k;
             if (d > last) break;
-            if (th[k] > cur) { acc += 2 * d + 1; cur = th[k]; }
+            if (th[k] > cur) { acc += d > from ? 2 * d + 1 : 0; cur = th[k]; }
         }
         run = fmax(run, __shfl_sync(0xffffffffu, incl, 31));
     }
     return warp_sum(acc);
 }
 
-// The double-float walk of POV x: the same sum, with every decision proved by
-// a margin (slope error <= 2^-45 |theta| + eta / d each); a decision inside
-// its margin sets *esc and the FP64 walk decides instead.
-__device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane, bool* esc_out)
+// The double-float walk of POV x over the targets a0 < d <= a1 and then
+// b0 < d <= b1: the sum of 2d + 1 over the second span's visible targets,
+// given that the largest slope before it lies in the first (a1 == a0: no
+// earlier target).  32 x KPL targets per chunk.  Every comparison is proved by
+// a margin (slope error <= 2^-45 |theta| + eta / d each); one inside its
+// margin sets *esc and the FP64 walk decides instead.
+template <int KPL>
+__device__ __forceinline__ int df_walk(const ExactCtx& c, int x, int a0, int a1, int b0, int b1, int lane,
+                                       bool* esc_out)
 {
     const float NEG = neg_inf();
     const int dir = c.bwd ? -1 : 1;
+    const int na = a1 - a0, total = na + b1 - b0;
     float hh, hl;
     {
         float zh, zl;
@@ -851,16 +877,17 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
     int rd = 1;
     int acc = 0;
     bool esc = false;
-    for (int base = 1; base <= last; base += 32 * XW_KPL) {
-        float th[XW_KPL], tl[XW_KPL], iv[XW_KPL];
+    for (int base = 0; base < total; base += 32 * KPL) {
+        float th[KPL], tl[KPL], iv[KPL];
         float mh = NEG, ml = 0.f;
         int md = 1;
-        const int d0 = base + lane * XW_KPL;
+        const int i0 = base + lane * KPL;
+        auto dist = [&](int i) { return i < na ? a0 + 1 + i : b0 + 1 + i - na; };
 #pragma unroll
-        for (int k = 0; k < XW_KPL; ++k) {
-            const int d = d0 + k;
+        for (int k = 0; k < KPL; ++k) {
+            const int i = i0 + k, d = dist(i);
             th[k] = NEG; tl[k] = 0.f; iv[k] = 1.f;
-            if (d <= last) {
+            if (i < total) {
                 iv[k] = __frcp_rn((float)d);
                 float zh, zl;
                 dem_hl(c, x + dir * d, zh, zl);
@@ -884,9 +911,9 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
         if (lane == 0 || df::df_gt(rh, rl, ch, cl)) { ch = rh; cl = rl; cd = rd; }
         float icd = __frcp_rn((float)cd);
 #pragma unroll
-        for (int k = 0; k < XW_KPL; ++k) {
-            const int d = d0 + k;
-            if (d > last) break;
+        for (int k = 0; k < KPL; ++k) {
+            const int i = i0 + k, d = dist(i);
+            if (i >= total) break;
             bool v = true;                           // the first target (no earlier one) is visible
             if (ch > NEG) {
                 float s, e;
@@ -897,7 +924,7 @@ __device__ __noinline__ int df_walk(const ExactCtx& c, int x, int last, int lane
                 if (!(fabsf(dh) > marg)) esc = true;
                 v = dh > 0.f;
             }
-            if (v) acc += 2 * d + 1;
+            if (v && i >= na) acc += 2 * d + 1;
             if (df::df_gt(th[k], tl[k], ch, cl)) { ch = th[k]; cl = tl[k]; cd = d; icd = iv[k]; }
         }
         const float lh = __shfl_sync(0xffffffffu, ph, 31);
@@ -918,14 +945,33 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
         cv = n < 1 ? 0 : 1;
     } else {
         bool esc = false;
-        const int s = df_walk(c, x, n - 1, lane, &esc);
-        cv = 1 + (esc ? fp64_walk(c, x, n - 1, lane) : s);
+        const int s = df_walk<XW_KPL>(c, x, 0, 0, 0, n - 1, lane, &esc);
+        cv = 1 + (esc ? fp64_walk(c, x, 0, n - 1, lane) : s);
         if (lane == 0) {
             atomicAdd(&g_sweep_stats[0], 1ull);
             if (esc) atomicAdd(&g_sweep_stats[1], 1ull);
         }
     }
     if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
+}
+
+// Adds to POV x's measure what the targets of block e0 (U steps) add, decided
+// exactly; kind and p0 as in the flag entry.
+template <int U>
+__device__ __forceinline__ void exact_block(const ExactCtx& c, int x, int e0, int p0, int kind, int lane)
+{
+    const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
+    const int last = min(n - 1, e0 + U);
+    if (last <= e0) return;
+    bool esc = false;
+    const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, 0, e0, e0, last, lane, &esc)
+                                      : df_walk<1>(c, x, p0, min(p0 + U, e0), e0, last, lane, &esc);
+    const int add = esc ? fp64_walk(c, x, e0, last, lane) : s;
+    if (lane == 0 && in_range(x, c.L, 14)) {
+        if (add) atomicAdd(c.cvrow + x, add);
+        atomicAdd(&g_sweep_stats[0], 1ull);
+        if (esc) atomicAdd(&g_sweep_stats[1], 1ull);
+    }
 }
 
 // min(a, |b|, |c|).  TVS_CERT_MIN3 selects the three-input minimum of
@@ -1250,7 +1296,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
     float2 T2[P / 2], K2[P / 2];     // thr and k of POV pairs
     bool rising = false;             // every thr >= 0
     float Rh = 0.f, c2e = 0.f;
-    unsigned mask = 0u;
+    unsigned lost = 0u, again = 0u;  // POVs whose walk is taken again; with an earlier flagged block
     int gi = lane, next = 32;
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
     bool klimited = false, ready = false;
@@ -1270,7 +1316,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
         klimited = klim < rowlim;
         e = 0;
         seg = FLUSH_STEPS;
-        mask = 0u;
+        lost = again = 0u;
 #pragma unroll
         for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
         if (LONG) {
@@ -1280,8 +1326,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
         if (dlim < 1) return;
         if (!inside) {
             dlim = 0;
-            const unsigned all = L - x0 >= P ? (1u << P) - 1u : (1u << (L - x0)) - 1u;   // bits by sample
-            mask = BWD ? __brev(all) >> (32 - P) : all;                                   // bits by POV q
+            lost = (1u << P) - 1u;
             return;
         }
         ready = true;                                        // the first block is always evaluated
@@ -1333,8 +1378,15 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
         const unsigned need = __ballot_sync(FULL, fin);
         if (need && (__popc(need) >= SKIP_RESTART || !__any_sync(FULL, gi < G && !fin))) {
             if (fin) {
-                finish_group<P, LONG, BWD>(sp, r, x0, mask, pov_x, walk_n,
-                                           [&](int q) { return q % 2 ? acc2[q / 2].y : acc2[q / 2].x; }, spill);
+                if (lost) sp.flag_count[2] = 1u;
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int x = pov_x(q);
+                    if (x >= L) continue;
+                    const float s = q % 2 ? acc2[q / 2].y : acc2[q / 2].x;
+                    const int cv = walk_n(x) >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
+                    r.cvrow[r.rev_staged ? L - 1 - x : x] = (lost >> q) & 1u ? CV_FLAGGED : cv;
+                }
                 gi = next + __popc(need & below);
                 if (gi < G) start(); else gi = G;
             }
@@ -1386,6 +1438,9 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
             const float4* __restrict__ tb = tab + e + e / U;
             const float ive = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tb->x;
             float Ms[P], mn[P];
+            float2 blk2[P / 2];      // the block's share of the measures
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) blk2[q] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < P; ++q) {
                 Ms[q] = q % 2 ? M2[q / 2].y : M2[q / 2].x;
@@ -1415,11 +1470,11 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
 #pragma unroll
                     for (int m = P; m < P + CH; m += 4) quad(BWD ? -(c + m) : c + m, m);
                     if (klimited && c + CH > steps) {
-                        if (far) cert_block<P, CH, true, true, PACK>(y, tab, e + c, ng2, M2, acc2, mn, steps - c);
-                        else cert_block<P, CH, true, false, PACK>(y, tb + c, e, ng2, M2, acc2, mn, steps - c);
+                        if (far) cert_block<P, CH, true, true, PACK>(y, tab, e + c, ng2, M2, blk2, mn, steps - c);
+                        else cert_block<P, CH, true, false, PACK>(y, tb + c, e, ng2, M2, blk2, mn, steps - c);
                     } else {
-                        if (far) cert_block<P, CH, false, true, PACK>(y, tab, e + c, ng2, M2, acc2, mn, CH);
-                        else cert_block<P, CH, false, false, PACK>(y, tb + c, e, ng2, M2, acc2, mn, CH);
+                        if (far) cert_block<P, CH, false, true, PACK>(y, tab, e + c, ng2, M2, blk2, mn, CH);
+                        else cert_block<P, CH, false, false, PACK>(y, tb + c, e, ng2, M2, blk2, mn, CH);
                     }
 #pragma unroll
                     for (int m = 0; m < P; ++m) y[m] = y[m + CH];
@@ -1432,12 +1487,33 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
             for (int q = 0; q < P; ++q) gm = fmaxf(gm, fabsf(q % 2 ? ng2[q / 2].y : ng2[q / 2].x));
             const float base = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, r.zmax, gm), __fmul_rn(2.f, c2e)));
             rising = true;
+            unsigned fm = 0u;
+            float dqs[P];
 #pragma unroll
             for (int q = 0; q < P; ++q) {
                 const float m = q % 2 ? M2[q / 2].y : M2[q / 2].x;
-                const float dq = __fmaf_rn(CERT_REL, fmaxf(fabsf(Ms[q]), fabsf(m)), __fmaf_rn(c2e, ia[q], ce));
-                mask |= mn[q] < dq ? 1u << q : 0u;
-                ia[q] = m > Ms[q] ? ive : ia[q];
+                dqs[q] = __fmaf_rn(CERT_REL, fmaxf(fabsf(Ms[q]), fabsf(m)), __fmaf_rn(c2e, ia[q], ce));
+                fm |= mn[q] < dqs[q] ? 1u << q : 0u;
+            }
+            if (fm) {
+                // flagged POVs leave the block to the exact pass
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    if (!((fm >> q) & 1u)) continue;
+                    (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
+                    const int p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
+                    if (!flag_block(sp, r, pov_x(q), e, p0, (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                        lost |= 1u << q;
+                }
+                again |= fm;
+            }
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) acc2[q] = __fadd2_rn(acc2[q], blk2[q]);
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const float m = q % 2 ? M2[q / 2].y : M2[q / 2].x;
+                const float dq = dqs[q];
+                ia[q] = m > Ms[q] && !((fm >> q) & 1u) ? ive : ia[q];
                 const float thr = __fmaf_rn(-2.f, dq, m);
                 const float g = -(q % 2 ? ng2[q / 2].y : ng2[q / 2].x);
                 (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
@@ -1674,18 +1750,16 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
     const int lane = threadIdx.x & 31;
     const unsigned n = min(sp.flag_count[0], (unsigned)sp.flag_cap);
     const long long t_start = clock64();
-    for (;;) {
-        unsigned i = 0u;
-        if (lane == 0) i = atomicAdd(sp.flag_count + 1, 1u);
-        i = __shfl_sync(0xffffffffu, i, 0);
-        if (i >= n) break;
+    for (unsigned i = blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * EXACT_WARPS) {
         const int4 en = sp.flag_buf[i];
         if (!in_range(en.x, sp.total_items, 22)) continue;
         ItemRow it;
         if (!decode_item(sp, sp.item_start, en.x, &it)) continue;
-        if (!in_range(en.y, it.L, 23)) continue;
+        const int x = en.y & 0xffff, kind = en.y >> 16;
+        if (!in_range(x, it.L, 23)) continue;
         const ExactCtx xc = exact_ctx(sp, it, __int_as_float(en.z));
-        exact_walk(xc, en.y, lane);
+        if (kind == FLAG_WALK) exact_walk(xc, x, lane);
+        else exact_block<SKIP_UNROLL>(xc, x, en.w & 0x3fff, en.w >> 14, kind, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[2], (unsigned long long)(clock64() - t_start));
 }
