@@ -54,7 +54,8 @@ struct PointsParams {
     float h0;
     float h0_lo;            // h0 - (double)h0 above, rounded
     double h0d;             // h0 (the FP64 walks)
-    int cert;               // certified (exact) visibility decisions
+    const float* tiles;     // tile maxima of the DEM, or NULL (walks visit every target)
+    int tpitch;             // tiles per DEM row
 };
 
 // View value V[i][j] of the direction's D4 view, read from the row-major DEM.
@@ -475,10 +476,193 @@ __device__ __noinline__ int walk_df(const LineRef& L, float hh, float hl, float 
     return n >= 1 ? 1 + sum - (lastvis ? 2 * n + 1 : 0) : 0;
 }
 
+// ------------------------------------------------- certified walks by tiles --
+// Most targets of a half-line are hidden by a wide margin.  With the maximum
+// elevation of every TILE x TILE block of DEM cells at hand, a walk bounds the
+// slopes of the TILE targets inside one tile column (or row) of its walk axis
+// from the two or three tiles they cross, 32 such spans at a time (a lane
+// each), and evaluates only the spans that can hold a visible target.  The
+// walks are bound by the latency of their dependent gathers and scans, so
+// fewer of them and more warps in flight are what counts.
+constexpr int TILE = 16;
+
+// Maximum of every TILE x TILE block of the DEM (smaller at the edges): a CTA
+// of 256 threads takes TILE rows of 256 columns.  Reads the DEM once.
+__global__ void __launch_bounds__(256) tile_max_kernel(const float* __restrict__ dem, int rows, int cols,
+                                                       float* __restrict__ tiles, int tpitch)
+{
+    const int j = blockIdx.x * 256 + threadIdx.x, i0 = blockIdx.y * TILE;
+    float m = __int_as_float(0xff800000);
+    if (j < cols) {
+#pragma unroll
+        for (int k = 0; k < TILE; ++k)
+            if (i0 + k < rows) m = fmaxf(m, dem[(long long)(i0 + k) * cols + j]);
+    }
+#pragma unroll
+    for (int o = TILE / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x % TILE == 0 && j < cols) tiles[(long long)blockIdx.y * tpitch + j / TILE] = m;
+}
+
+// Targets of the half-line: its usable samples on that side, at most K (the
+// samples with 0 <= base + y(j) 2^-32 <= H - 1 are a contiguous range of j).
+__device__ __forceinline__ int line_targets(const LineRef& L)
+{
+    const DirDev& d = L.d;
+    int n = L.dir > 0 ? d.W - 1 - L.j0 : L.j0;
+    if (d.t_fx != 0ull) {
+        if (L.dir > 0) {
+            // rows grow with j; count them from the POV's column (DIRECT) or from column 0
+            const unsigned long long top = (unsigned long long)(d.H - 1 - L.base) << 32;
+            const long long j = (long long)(top / d.t_fx);
+            n = (int)min((long long)n, L.direct ? j : j - L.j0);
+        } else if (L.direct) {
+            n = (int)min((long long)n, (long long)(((unsigned long long)L.base << 32) / d.t_fx));
+        } else if (L.base < 0) {
+            const unsigned long long low = (unsigned long long)(-L.base) << 32;
+            n = (int)min((long long)n, L.j0 - (long long)((low + d.t_fx - 1ull) / d.t_fx));
+        }
+    }
+    return min(n, d.K);
+}
+
+// The walk of walk_df (same slopes, margins and result) over the spans that
+// the tile maxima leave: the first 32 targets, then one tile's targets at a
+// time, two spans per pass.  A span is left out when its largest possible
+// slope, rounded up and with the running maximum's own error allowed for
+// (run = rh + rl at distance rd: eta / rd, and 2^-21 |rh| for rl and the
+// rounding of the test), is at most the running maximum: its targets are then
+// not visible, by more than walk_df's margin, and leave the maximum as it is.
+__device__ __noinline__ int walk_tiles(const LineRef& L, const float* __restrict__ tiles, int tpitch, float hh,
+                                       float hl, float zobs, float h0abs, unsigned char* flags, int cap, int lane,
+                                       bool* esc_out)
+{
+    const unsigned FULL = 0xffffffffu;
+    const float NEG = __int_as_float(0xff800000);
+    const DirDev& dd = L.d;
+    const int n = line_targets(L);
+    const ViewAddr va = view_addr(dd, L.cols);
+    const int H = dd.H, W = dd.W, frame = dd.frame, j0 = L.j0, dir = L.dir, base = (int)L.base;
+    const long long t_fx = (long long)dd.t_fx;
+    const bool direct = L.direct;
+    const float* __restrict__ dem = L.dem;
+    // view row of the target at distance d, and its 32-bit fraction
+    auto row_of = [&](int d, unsigned* fr) {
+        const long long y = (long long)(direct ? dir * d : j0 + dir * d) * t_fx;
+        *fr = (unsigned)y;
+        return base + (int)(y >> 32);
+    };
+    float rh = NEG, rl = 0.f;
+    int rd = 1;
+    float zmax = zobs, eta = 0.f;
+    int sum = 0;
+    bool esc = false;
+
+    // decides the lanes' targets (distance d, 0: none), which increase with the lane
+    auto evaluate = [&](int d) {
+        float th = NEG, tl = 0.f, iv = 1.f, za = 0.f;
+        if (d > 0) {
+            unsigned fr;
+            const int at = va.o + row_of(d, &fr) * va.sa + (j0 + dir * d) * va.sj;
+            const float z0 = dem[at];
+            const float z1 = fr ? dem[at + va.sa] : z0;
+            float zh, zl;
+            df::df_blend(z0, z1, fr, zh, zl);
+            za = fmaxf(fabsf(z0), fabsf(z1));
+            iv = __frcp_rn((float)d);
+            df::df_slope_iv(zh, zl, hh, hl, d, iv, th, tl);
+        }
+        // the largest |elevation| so far (floats >= 0 order like their bits)
+        zmax = fmaxf(zmax, __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(za))));
+        eta = 0x1p-42f * (zmax + h0abs) + 0x1p-126f;
+        float ph = th, pl = tl;
+        int pd = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float qh = __shfl_up_sync(FULL, ph, o);
+            const float ql = __shfl_up_sync(FULL, pl, o);
+            const int qd = __shfl_up_sync(FULL, pd, o);
+            if (lane >= o && df::df_gt(qh, ql, ph, pl)) { ph = qh; pl = ql; pd = qd; }
+        }
+        float ch = __shfl_up_sync(FULL, ph, 1);
+        float cl = __shfl_up_sync(FULL, pl, 1);
+        int cd = __shfl_up_sync(FULL, pd, 1);
+        if (lane == 0 || df::df_gt(rh, rl, ch, cl)) { ch = rh; cl = rl; cd = rd; }
+        if (d > 0) {
+            bool vis = true;                   // the first target (no earlier one) is visible
+            if (ch > NEG) {
+                float s, e;
+                df::two_sum(th, -ch, s, e);
+                const float dh = __fadd_rn(s, __fadd_rn(e, __fsub_rn(tl, cl)));
+                const float marg = __fmaf_rn(0x1p-40f, fabsf(th) + fabsf(ch),
+                                             4.04f * eta * (iv + __frcp_rn((float)cd))) + 0x1p-120f;
+                if (!(fabsf(dh) > marg)) esc = true;
+                vis = dh > 0.f;
+            }
+            if (vis) {
+                if (d < n) sum += 2 * d + 1;   // the last target only closes a segment
+                if (flags && d < cap) flags[d] = 1;
+            }
+        }
+        const float lh = __shfl_sync(FULL, ph, 31), ll = __shfl_sync(FULL, pl, 31);
+        const int ld = __shfl_sync(FULL, pd, 31);
+        if (df::df_gt(lh, ll, rh, rl)) { rh = lh; rl = ll; rd = ld; }
+    };
+
+    evaluate(lane < n ? lane + 1 : 0);
+    // DEM coordinate along the walk: w0 + sw d; across it, c = c0 + sc a
+    const int w0 = frame == 2 ? W - 1 - j0 : j0;
+    const int sw = frame == 2 ? -dir : dir;
+    const bool down = frame == 1 || frame == 2;            // the walk runs along DEM columns' length (rows vary)
+    const int far = n - 32;                                // targets past the first pass
+    const int t0 = w0 / TILE;
+    const int spans = far > 0 ? (sw > 0 ? (w0 + n) / TILE - t0 : t0 - (w0 - n) / TILE) + 1 : 0;
+    for (int m0 = sw > 0 ? (w0 + 33) / TILE - t0 : t0 - max(w0 - 33, 0) / TILE; m0 < spans; m0 += 32) {
+        const int t = t0 + sw * (m0 + lane);
+        int dlo = 1, dhi = 0;
+        float up = NEG;                                    // bound of the span's slopes
+        if (m0 + lane < spans) {
+            dlo = max(sw > 0 ? t * TILE - w0 : w0 - t * TILE - (TILE - 1), 33);
+            dhi = min(sw > 0 ? t * TILE + (TILE - 1) - w0 : w0 - t * TILE, n);
+        }
+        if (dlo <= dhi) {
+            unsigned fr;
+            const int a0 = row_of(dlo, &fr), a1 = row_of(dhi, &fr);
+            const int alo = min(a0, a1), ahi = min(max(a0, a1) + 1, H - 1);
+            // a span of TILE targets covers at most TILE + 1 rows: 2 or 3 tiles
+            const int c0 = (frame == 3 ? H - 1 - ahi : alo) / TILE;
+            const int c1 = (frame == 3 ? H - 1 - alo : ahi) / TILE;
+            const int cs = down ? 1 : tpitch, at = down ? t * tpitch : t;
+            const float z = fmaxf(fmaxf(tiles[at + c0 * cs], tiles[at + min(c0 + 1, c1) * cs]), tiles[at + c1 * cs]);
+            const float A = __fadd_rn(__fsub_rn(z, hh), 0x1p-21f * (fabsf(z) + fabsf(hh)));
+            const float rlo = __frcp_rn((float)dlo);
+            up = fmaxf(A * rlo * 1.0000019f, A * __frcp_rn((float)dhi) * 0.9999981f) + 4.04f * eta * rlo;
+        }
+        unsigned left = FULL;                              // spans not yet passed
+        for (;;) {
+            const float run = rh - 0x1p-21f * fabsf(rh) - 4.04f * eta * __frcp_rn((float)rd);
+            const unsigned cand = __ballot_sync(FULL, dlo <= dhi && up > run) & left;
+            if (!cand) break;
+            const int s0 = __ffs(cand) - 1;
+            const unsigned rest = cand & (cand - 1);
+            const int s1 = rest ? __ffs(rest) - 1 : 32;
+            const int src = lane < TILE ? s0 : min(s1, 31);
+            const int d0 = __shfl_sync(FULL, dlo, src), d1 = __shfl_sync(FULL, dhi, src);
+            const int d = d0 + lane % TILE;
+            evaluate(d <= d1 && (lane < TILE || s1 < 32) ? d : 0);
+            left = s1 >= 31 ? 0u : ~0u << (s1 + 1);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+    *esc_out = __any_sync(FULL, esc);
+    return n >= 1 ? 1 + sum : 0;
+}
+
 // Certified measure of a half-line whose observer stands on the sample
 // (a0, fr0) of view column j0 (DIRECT: the cell itself, fr0 = 0).
 __device__ __forceinline__ int walk_exact(const LineRef& L, long long a0, unsigned fr0, float h0, float h0_lo,
-                                          double h0d, unsigned char* flags, int cap, int lane)
+                                          double h0d, const float* tiles, int tpitch, unsigned char* flags, int cap,
+                                          int lane)
 {
     const float va = view_at(L.dem, L.cols, L.d, a0, L.j0);
     const float vb = fr0 ? view_at(L.dem, L.cols, L.d, a0 + 1, L.j0) : va;
@@ -491,25 +675,35 @@ __device__ __forceinline__ int walk_exact(const LineRef& L, long long a0, unsign
         df::two_sum(s, e, hh, hl);
     }
     bool esc = false;
-    const int cv = walk_df(L, hh, hl, fmaxf(fabsf(va), fabsf(vb)), fabsf(h0), flags, cap, lane, &esc);
+    const float zobs = fmaxf(fabsf(va), fabsf(vb));
+    const int cv = tiles ? walk_tiles(L, tiles, tpitch, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc)
+                         : walk_df(L, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc);
     if (!esc) return cv;
     return walk_fp64(L, __dadd_rn(z64_of(L, a0, fr0, L.j0), h0d), flags, cap, lane);
 }
 
 // Directions per CTA of the points kernel (4 warps each: 2 lines x 2 sides).
 constexpr int POINTS_DIRS = 2;
+// CTAs of 8 warps per SM that a certified walk kernel's registers leave room
+// for: the walks wait on their gathers one after another, so warps in flight
+// decide (2000 POVs on 2000^2: 4.5, 3.6, 3.1 and 2.8 ms with 24, 32, 40 and 48
+// warps, the last at 40 registers with a few spills).
+constexpr int POINTS_MIN_CTAS = 6;
 
 // One CTA of 4 POINTS_DIRS warps per (POV q, POINTS_DIRS consecutive
 // directions): warp 4 kk + 2 v + s walks direction k0 + kk, virtual POV v
 // (hi / lo; DIRECT uses v = 0 only), forward (s = 0) or backward (s = 1).
 // Then one thread per direction blends its lines' measures (Kernel-3) and
 // stores the direction's term g * blend.
-__global__ void __launch_bounds__(128 * POINTS_DIRS) points_kernel(PointsParams pp)
+template <bool CERT>
+__global__ void __launch_bounds__(128 * POINTS_DIRS, CERT ? POINTS_MIN_CTAS : 1) points_kernel(PointsParams pp)
 {
     __shared__ int cvs[4 * POINTS_DIRS];
-    extern __shared__ float rtab[];   // rcp(d), d = 1 .. max(rows, cols)
-    fill_rcp(rtab, max(pp.rows, pp.cols));
-    __syncthreads();
+    extern __shared__ float rtab[];   // rcp(d), d = 1 .. max(rows, cols) (FP32 decisions)
+    if (!CERT) {
+        fill_rcp(rtab, max(pp.rows, pp.cols));
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int per_pov = (pp.n + POINTS_DIRS - 1) / POINTS_DIRS;
     const int q = (int)(blockIdx.x / (unsigned)per_pov);
@@ -523,9 +717,9 @@ __global__ void __launch_bounds__(128 * POINTS_DIRS) points_kernel(PointsParams 
             long long a;
             unsigned fr;
             line_pos(L.d, direct, L.base, L.j0, L.j0, &a, &fr);
-            if (pp.cert) {
+            if constexpr (CERT) {
                 const LineRef R{pp.dem, pp.cols, L.d, L.base, L.j0, s ? -1 : 1, direct};
-                cv = walk_exact(R, a, fr, pp.h0, pp.h0_lo, pp.h0d, nullptr, 0, lane);
+                cv = walk_exact(R, a, fr, pp.h0, pp.h0_lo, pp.h0d, pp.tiles, pp.tpitch, nullptr, 0, lane);
             } else {
                 const float h = __fadd_rn(direct ? view_at(pp.dem, pp.cols, L.d, L.i, L.j0)
                                                  : sample_at(pp.dem, pp.cols, L.d, a, fr, L.j0), pp.h0);
@@ -588,15 +782,19 @@ struct MapParams {
     float h0;
     float h0_lo;
     double h0d;
-    int cert;
+    const float* tiles;     // as PointsParams
+    int tpitch;
 };
 
 // One warp per (POV, slot), walking the half-line as the points kernel does.
-__global__ void __launch_bounds__(256) map_flags_kernel(MapParams mp)
+template <bool CERT>
+__global__ void __launch_bounds__(256, CERT ? POINTS_MIN_CTAS : 1) map_flags_kernel(MapParams mp)
 {
-    extern __shared__ float rtab[];   // rcp(d), d = 1 .. max(rows, cols)
-    fill_rcp(rtab, max(mp.rows, mp.cols));
-    __syncthreads();
+    extern __shared__ float rtab[];   // rcp(d), d = 1 .. max(rows, cols) (FP32 decisions)
+    if (!CERT) {
+        fill_rcp(rtab, max(mp.rows, mp.cols));
+        __syncthreads();
+    }
     const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // (q, slot)
     const int lane = threadIdx.x & 31;
     if (t >= (long long)mp.npov * 2 * mp.n) return;                                // warp-uniform
@@ -611,23 +809,12 @@ __global__ void __launch_bounds__(256) map_flags_kernel(MapParams mp)
     case 2:  i = jD; j0 = d.W - 1 - iD; break;
     default: i = d.H - 1 - iD; j0 = jD; break;
     }
-    if (mp.cert) {
+    if constexpr (CERT) {
         const LineRef R{mp.dem, mp.cols, d, i, j0, dir, true};
-        walk_exact(R, i, 0u, mp.h0, mp.h0_lo, mp.h0d, mp.flags + t * mp.cap, mp.cap, lane);
-        return;
-    }
-    const float h = __fadd_rn(view_at(mp.dem, mp.cols, d, i, j0), mp.h0);
-    walk_half_line(mp.dem, mp.cols, d, rtab, i, j0, true, dir, h, mp.flags + t * mp.cap, mp.cap, lane);
-}
-
-// View coordinates of DEM cell (iD, jD) in direction d's view.
-__device__ __forceinline__ void to_view(const DirDev& d, int iD, int jD, int* i, int* j)
-{
-    switch (d.frame) {
-    case 0:  *i = iD; *j = jD; break;
-    case 1:  *i = jD; *j = iD; break;
-    case 2:  *i = jD; *j = d.W - 1 - iD; break;
-    default: *i = d.H - 1 - iD; *j = jD; break;
+        walk_exact(R, i, 0u, mp.h0, mp.h0_lo, mp.h0d, mp.tiles, mp.tpitch, mp.flags + t * mp.cap, mp.cap, lane);
+    } else {
+        const float h = __fadd_rn(view_at(mp.dem, mp.cols, d, i, j0), mp.h0);
+        walk_half_line(mp.dem, mp.cols, d, rtab, i, j0, true, dir, h, mp.flags + t * mp.cap, mp.cap, lane);
     }
 }
 
@@ -639,41 +826,85 @@ __device__ __forceinline__ void to_view(const DirDev& d, int iD, int jD, int* i,
 // within a few ulp of the angle (|angle| <= pi, ulp 2^-22), so with the three
 // roundings of q = angle (n / pi) + 1/2 the single-precision q is within
 // about 4.1e-7 n of the double one; a cell whose q lies within
-// 4e-6 n + 1e-6 of a boundary takes the double-precision angle instead.
-__global__ void map_raster_kernel(MapParams mp)
+// 1e-6 n + 1e-6 of a boundary takes the double-precision angle instead (a
+// warp takes that path, hundreds of FP64 instructions, when one of its 32
+// cells does, so the margin is kept tight: 4e-6 n sent 4.5 % of the warps
+// there at n = 180).
+// A warp takes 8 x 4 cells and a CTA RASTER_X x RASTER_Y: seen from a POV such a
+// patch lies in a few sectors and a few distances, so the flags its cells
+// read fall in a few 32-byte sectors (a row of 32 cells reads up to 32 of
+// them).  Bound by instructions, the angle's above all: 10 POVs on 2000^2 take
+// 0.167 ms (0.174 a row of cells per warp; 0.26 with the margin of 4e-6 n;
+// 0.42 before, with the direction table read and 64-bit remainders per cell).
+constexpr int RASTER_X = 32, RASTER_Y = 8;
+
+__global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapParams mp)
 {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= (long long)mp.rows * mp.cols) return;
-    const int iD = (int)(c / mp.cols), jD = (int)(c % mp.cols);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int jD = blockIdx.x * RASTER_X + (warp & 3) * 8 + (lane & 7);
+    const int iD = blockIdx.y * RASTER_Y + (warp >> 2) * 4 + (lane >> 3);
+    if (iD >= mp.rows || jD >= mp.cols) return;
+    const long long c = (long long)iD * mp.cols + jD;
     const float scale = (float)((double)mp.n / 3.141592653589793);
-    const float margin = 4e-6f * (float)mp.n + 1e-6f;
+    const float margin = 1e-6f * (float)mp.n + 1e-6f;
     int seen = 0;
     for (int q = 0; q < mp.npov; ++q) {
         const int i0 = mp.pov[2 * q], j0 = mp.pov[2 * q + 1];
         if (iD == i0 && jD == j0) { ++seen; continue; }
-        const float x = __fadd_rn(__fmul_rn(atan2f((float)(iD - i0), (float)(jD - j0)), scale), 0.5f);
+        const int di = iD - i0, dj = jD - j0;
+        const float x = __fadd_rn(__fmul_rn(atan2f((float)di, (float)dj), scale), 0.5f);
         const float fl = floorf(x);
         const float fx = x - fl;                  // exact
-        long long kp;
+        int kp;
         if (fx > margin && fx < 1.0f - margin) {
-            kp = (long long)fl;
+            kp = (int)fl;
         } else {
-            const double qq = atan2((double)(iD - i0), (double)(jD - j0)) * (double)mp.n / 3.141592653589793;
-            kp = (long long)floor(qq + 0.5);
+            const double qq = atan2((double)di, (double)dj) * (double)mp.n / 3.141592653589793;
+            kp = (int)floor(qq + 0.5);
         }
-        kp = ((kp % (2 * mp.n)) + 2 * mp.n) % (2 * mp.n);
-        const int k = (int)(kp % mp.n);
-        const DirDev d = mp.dirs[k];
-        // +j of the view points along theta_k in views 0 and 1, along theta_k + pi in views 2 and 3
-        const bool plus = (d.frame <= 1) == (kp < mp.n);
-        int iv, jv, iv0, jv0;
-        to_view(d, iD, jD, &iv, &jv);
-        to_view(d, i0, j0, &iv0, &jv0);
-        const int dd = plus ? jv - jv0 : jv0 - jv;
-        const long long slot = plus ? k : mp.n + k;
-        if (dd >= 1 && dd < mp.cap) seen += mp.flags[((long long)q * 2 * mp.n + slot) * mp.cap + dd];
+        // kp mod 2n: the angle lies in [-pi, pi], so kp in [-n, n]
+        if (kp < 0) kp += 2 * mp.n;
+        const bool half = kp < mp.n;
+        const int k = half ? kp : kp - mp.n;
+        // direction k's view (the integer tests of the direction table) decides
+        // which DEM axis the half-line walks and which way: the walk axis is
+        // the column in views 0 and 3, the row in view 1 and the reversed row in
+        // view 2; +j of the view points along theta_k in views 0 and 1, along
+        // theta_k + pi in views 2 and 3
+        const long long k4 = 4ll * k;
+        const bool first2 = k4 < 2ll * mp.n;
+        const bool along_cols = k4 < mp.n || k4 >= 3ll * mp.n;
+        const bool plus = first2 == half;
+        int dd = along_cols ? dj : first2 ? di : -di;
+        if (!plus) dd = -dd;
+        if (dd >= 1 && dd < mp.cap)
+            seen += mp.flags[((long long)q * 2 * mp.n + (plus ? k : mp.n + k)) * mp.cap + dd];
     }
     mp.count[c] = seen;
+}
+
+// Whether a call's certified walks go by tile maxima.  The tile kernel reads
+// the DEM once (6 us on 2000^2, of memory bandwidth beyond), the walks then
+// skip most targets: 10 POVs on 2000^2 take 72 us instead of 113, 2000 POVs
+// 2.8 ms instead of 15.7.  Walks of fewer than 128 targets have little to
+// skip, and the DEM may be larger than what the walks save: a walk_df pass
+// (256 targets) takes some 15 us, the time to read 2^24 cells, so a call has to
+// walk at least one target per 2^16 cells.
+bool use_tiles(bool cert, int rows, int cols, const std::vector<DirDev>& dirs)
+{
+    int reach = 0;
+    for (const DirDev& d : dirs) reach = std::max(reach, std::min(d.K, d.W));
+    return cert && reach >= 128 && (long long)rows * cols <= (long long)reach << 16;
+}
+
+int tile_pitch(int cols) { return (cols + TILE - 1) / TILE; }
+size_t tile_bytes(int rows, int cols) { return align256((size_t)tile_pitch(cols) * ((rows + TILE - 1) / TILE) * 4); }
+
+cudaError_t launch_tile_max(const float* dem, int rows, int cols, float* tiles, cudaStream_t s)
+{
+    const dim3 grid((cols + 255) / 256, (rows + TILE - 1) / TILE);
+    tile_max_kernel<<<grid, 256, 0, s>>>(dem, rows, cols, tiles, tile_pitch(cols));
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -759,7 +990,9 @@ extern "C" int tvs_visibility_map(tvs_handle h, const float* d_dem, int rows, in
     const size_t o_dirs = 0, o_pov = align256((size_t)n_sectors * sizeof(DirDev));
     const size_t hdr = o_pov + align256((size_t)npov * 8);
     const size_t o_flags = hdr;
-    const size_t total = o_flags + align256(flag_bytes);
+    const size_t o_tiles = o_flags + align256(flag_bytes);
+    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs);
+    const size_t total = o_tiles + (tiles ? tile_bytes(rows, cols) : 0);
     rc = ensure_scratch(h, total);
     if (rc) return rc;
     std::vector<char> img(hdr, 0);
@@ -778,23 +1011,31 @@ extern "C" int tvs_visibility_map(tvs_handle h, const float* d_dem, int rows, in
     mp.h0 = (float)obs_height_m;
     mp.h0_lo = (float)(obs_height_m - (double)mp.h0);
     mp.h0d = obs_height_m;
-    mp.cert = !h->tuning.fp32_decisions;
+    const bool cert = !h->tuning.fp32_decisions;
+    if (tiles) {
+        mp.tiles = reinterpret_cast<const float*>(h->ws + o_tiles);
+        mp.tpitch = tile_pitch(cols);
+    }
     const long long walks = (long long)npov * 2 * n_sectors;
-    const size_t rtab_bytes = ((size_t)std::max(rows, cols) + 1) * sizeof(float);
-    TVS_CUDA(cudaFuncSetAttribute(map_flags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rtab_bytes),
+    const size_t rtab_bytes = cert ? 0 : ((size_t)std::max(rows, cols) + 1) * sizeof(float);
+    const auto flags_kernel = cert ? map_flags_kernel<true> : map_flags_kernel<false>;
+    TVS_CUDA(cudaFuncSetAttribute(flags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rtab_bytes),
              "visibility flags shared memory");
     {
         const double evals = h->profiling ? (double)tvs_count_point_evals(rows, cols, n_sectors, step_m, max_range_m,
                                                                           pov_ij, npov, TVS_POINTS_DIRECT)
                                           : 0.0;
         Timer t(h, K_MAP_FLAGS, s, evals);
-        map_flags_kernel<<<(unsigned)((walks * 32 + 255) / 256), 256, rtab_bytes, s>>>(mp);
+        if (tiles)
+            TVS_CUDA(launch_tile_max(d_dem, rows, cols, reinterpret_cast<float*>(h->ws + o_tiles), s), "tile maxima");
+        flags_kernel<<<(unsigned)((walks * 32 + 255) / 256), 256, rtab_bytes, s>>>(mp);
     }
     TVS_CUDA(cudaGetLastError(), "visibility flags launch");
     const long long cells = (long long)rows * cols;
     {
         Timer t(h, K_MAP_RASTER, s, (double)cells * npov);
-        map_raster_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, s>>>(mp);
+        const dim3 grid((cols + RASTER_X - 1) / RASTER_X, (rows + RASTER_Y - 1) / RASTER_Y);
+        map_raster_kernel<<<grid, RASTER_X * RASTER_Y, 0, s>>>(mp);
     }
     TVS_CUDA(cudaGetLastError(), "visibility raster launch");
     return TVS_OK;
@@ -831,7 +1072,9 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
     const size_t hdr = o_pov + align256((size_t)npov * 8);
     const size_t o_part = hdr;
     const size_t o_term = o_part + align256((size_t)npov * ngroups * 16);
-    const size_t total = o_term + align256((size_t)npov * n_sectors * 4);
+    const size_t o_tiles = o_term + align256((size_t)npov * n_sectors * 4);
+    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs);
+    const size_t total = o_tiles + (tiles ? tile_bytes(rows, cols) : 0);
     rc = ensure_scratch(h, total);
     if (rc) return rc;
     std::vector<char> img(hdr, 0);
@@ -851,17 +1094,24 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
     pp.h0 = (float)obs_height_m;
     pp.h0_lo = (float)(obs_height_m - (double)pp.h0);
     pp.h0d = obs_height_m;
-    pp.cert = !h->tuning.fp32_decisions;
-    const size_t rtab_bytes = ((size_t)std::max(rows, cols) + 1) * sizeof(float);
-    TVS_CUDA(cudaFuncSetAttribute(points_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rtab_bytes),
+    const bool cert = !h->tuning.fp32_decisions;
+    if (tiles) {
+        pp.tiles = reinterpret_cast<const float*>(h->ws + o_tiles);
+        pp.tpitch = tile_pitch(cols);
+    }
+    const size_t rtab_bytes = cert ? 0 : ((size_t)std::max(rows, cols) + 1) * sizeof(float);
+    const auto walk_kernel = cert ? points_kernel<true> : points_kernel<false>;
+    TVS_CUDA(cudaFuncSetAttribute(walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rtab_bytes),
              "points shared memory");
     {
         const double evals = h->profiling ? (double)tvs_count_point_evals(rows, cols, n_sectors, step_m, max_range_m,
                                                                           pov_ij, npov, mode)
                                           : 0.0;
         Timer t(h, K_POINTS, s, evals);
+        if (tiles)
+            TVS_CUDA(launch_tile_max(d_dem, rows, cols, reinterpret_cast<float*>(h->ws + o_tiles), s), "tile maxima");
         const long long ctas = (long long)npov * ((n_sectors + POINTS_DIRS - 1) / POINTS_DIRS);
-        points_kernel<<<(unsigned)ctas, 128 * POINTS_DIRS, rtab_bytes, s>>>(pp);
+        walk_kernel<<<(unsigned)ctas, 128 * POINTS_DIRS, rtab_bytes, s>>>(pp);
         const long long groups = (long long)npov * ngroups;
         points_groups<<<(unsigned)((groups + 127) / 128), 128, 0, s>>>(pp);
         points_finalize<<<(npov + 127) / 128, 128, 0, s>>>(pp);
