@@ -81,7 +81,7 @@ struct SweepParams {
     int half;          // floats of one staged row array (multiple of 4)
     int per_pair;      // floats of a warp pair's shared area (certified)
     int zs_len;        // floats of the row's suffix maxima (0 without pruning)
-    int wm_len;        // floats of the row's window maxima (certified pruned launches, else 0)
+    int wm_len;        // floats of the row's window maxima (0 without pruning)
     int per_warp;      // floats of a warp's shared area
 };
 
@@ -154,8 +154,8 @@ __device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* is
 // a sentinel that is never visible.  With CERT the first sample and the
 // ROW_PADL samples before it are sentinels too (the last target of a backward
 // walk), and the real hi and lo parts of the two end samples, which are POVs,
-// go to ends[0..3] (first hi, first lo, last hi, last lo).  Returns (CERT) the
-// row's largest |elevation| read, for the blend's error bound.
+// go to ends[0..3] (first hi, first lo, last hi, last lo).  Returns the row's
+// largest |elevation| read, for the error bounds.
 template <bool CERT>
 __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow& it, float* Fh, float* Fl,
                                            float* ends, int lane, int part = 0, int parts = 1, bool rev_ok = true)
@@ -203,6 +203,7 @@ __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow&
                 zmax = fmaxf(zmax, fmaxf(fabsf(va[k]), fabsf(vb[k])));
             } else {
                 Fh[ROW_PADL + x] = x == it.L - 1 ? NEG : blend32(va[k], vb[k], fr[k]);
+                zmax = fmaxf(zmax, fmaxf(fabsf(va[k]), fabsf(vb[k])));
             }
         }
     }
@@ -213,9 +214,11 @@ __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow&
     }
     if (CERT) {
         if (part == 0 && lane < ROW_PADL) { Fh[lane] = NEG; Fl[lane] = 0.f; }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+    } else if (lane < ROW_PADL) {
+        Fh[lane] = NEG;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
     return zmax;
 }
 
@@ -275,10 +278,9 @@ __device__ __forceinline__ void sweep_block(const float* w, const float4* __rest
 // flush (the LONG = false instantiation).
 constexpr int LONG_WALK = 4000;
 constexpr int FLUSH_STEPS = 336;   // a multiple of SMALL_UNROLL, LARGE_UNROLL and 24
-// Suffix maxima of a staged row are kept at every ZS_STRIDE-th sample; pruning
-// checks every PRUNE_EVERY blocks.
+// The maxima of a staged row that pruned walks test are kept at every
+// ZS_STRIDE-th sample.
 constexpr int ZS_STRIDE = 4;
-constexpr int PRUNE_EVERY = 1;
 
 // A warp item is one skewed row and one walk direction.  Its G groups of P
 // consecutive POVs are taken in order (longest walks first) from a warp-local
@@ -290,20 +292,11 @@ constexpr int PRUNE_EVERY = 1;
 // cv = 1 + sum_{d=1}^{n-1} v_d (2d + 1) for n >= 1 targets, which is Alg. 8's
 // sum of d^2 - open^2 over its closed segments plus the segment still open at
 // the end (closed at the last target).
-//
-// PRUNE (exact horizon pruning): every PRUNE_EVERY blocks a lane stops its
-// group's walks once min_q M_q >= B, B = fl(A * (1/d)) if A >= 0 else 0, where
-// d is the next target distance and A = fl(Zmax - min_q h_q) with Zmax an upper
-// bound of every remaining target (the suffix maximum ZS).  Rounding to nearest
-// is monotone, so every remaining slope fl(fl(z - h_q) * fl(1/d')) is at most
-// fl(A * fl(1/d)) when A >= 0 (d' >= d) and at most 0 when A < 0: no remaining
-// target can be strictly above its POV's running maximum, and the walk's
-// measure is already complete.  The result is bit for bit the same.
+// Every target is walked; pruned launches take sweep_row_skip32.
 //
 // With LONG, `spill` is the lane's column (stride 32) of P integers.
-template <int P, int U, bool LONG, bool PRUNE>
-__device__ __forceinline__ void sweep_row(const float* __restrict__ F, const float* __restrict__ ZS,
-                                          const float4* __restrict__ tab, int tabn, int* __restrict__ cvrow,
+template <int P, int U, bool LONG>
+__device__ __forceinline__ void sweep_row(const float* __restrict__ F, const float4* __restrict__ tab, int tabn, int* __restrict__ cvrow,
                                           int* __restrict__ spill, int L, int K, float h0, bool rev, int lane)
 {
     // the window is read as float4 from F + ROW_PADL + x0 + e (x0 = g P, e a
@@ -316,10 +309,8 @@ __device__ __forceinline__ void sweep_row(const float* __restrict__ F, const flo
     const int klim = K - 1;          // last target distance that still adds area
     float h[P], M[P];
     float2 acc2[P / 2];
-    float hmin = 0.f;
     int g = lane, next = 32;         // the lane's group; the first group nobody has taken
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
-    int pc = 1;                      // blocks until the next pruning check
     bool klimited = false;
 
     auto start = [&]() {
@@ -329,16 +320,10 @@ __device__ __forceinline__ void sweep_row(const float* __restrict__ F, const flo
         klimited = klim < rowlim;
         e = 0;
         seg = FLUSH_STEPS;
-        pc = 1;
 #pragma unroll
         for (int q = 0; q < P; ++q) { h[q] = __fadd_rn(F[ROW_PADL + x0 + q], h0); M[q] = NEG; }
 #pragma unroll
         for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
-        if (PRUNE) {
-            hmin = h[0];
-#pragma unroll
-            for (int q = 1; q < P; ++q) hmin = fminf(hmin, h[q]);
-        }
         if (LONG) {
 #pragma unroll
             for (int q = 0; q < P; ++q) spill[32 * q] = 0;
@@ -378,16 +363,6 @@ __device__ __forceinline__ void sweep_row(const float* __restrict__ F, const flo
                     acc2[q / 2] = make_float2(0.f, 0.f);
                 }
             }
-            if (PRUNE && --pc < 0) {
-                pc = PRUNE_EVERY - 1;
-                const float A = __fsub_rn(ZS[(x0 + e + 1) / ZS_STRIDE], hmin);
-                const float rd = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tab[e].x;
-                const float B = A >= 0.f ? __fmul_rn(A, rd) : 0.f;
-                float m = M[0];
-#pragma unroll
-                for (int q = 1; q < P; ++q) m = fminf(m, M[q]);
-                if (m >= B) { e = dlim; continue; }
-            }
             const float* base = F + ROW_PADL + x0 + e;
             float w[P + U];
 #pragma unroll
@@ -409,33 +384,6 @@ __device__ __forceinline__ void sweep_row(const float* __restrict__ F, const flo
     }
 }
 
-// Suffix maxima of the staged row F (L samples, -inf from L - 1 on) at every
-// ZS_STRIDE-th sample: ZS[j] = max F[x] over x >= ZS_STRIDE * j, for
-// j <= (L - 1) / ZS_STRIDE.  Lane l scans its own segment, a warp scan joins
-// the segments.
-__device__ __forceinline__ void suffix_max(const float* __restrict__ F, float* __restrict__ ZS, int L, int lane)
-{
-    const float NEG = neg_inf();
-    const int seglen = ((L + 31) / 32 + ZS_STRIDE - 1) / ZS_STRIDE * ZS_STRIDE;
-    const int a = lane * seglen, b = min(a + seglen, L);
-    float m = NEG;
-    for (int x = b - 1; x >= a; --x) m = fmaxf(m, F[ROW_PADL + x]);
-    // inclusive suffix scan of the segment maxima over the lanes
-    float s = m;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float t = __shfl_down_sync(0xffffffffu, s, o);
-        if (lane + o < 32) s = fmaxf(s, t);
-    }
-    float after = __shfl_down_sync(0xffffffffu, s, 1);   // maximum of the following segments
-    if (lane == 31) after = NEG;
-    float run = after;
-    for (int x = b - 1; x >= a; --x) {
-        run = fmaxf(run, F[ROW_PADL + x]);
-        if (x % ZS_STRIDE == 0) ZS[x / ZS_STRIDE] = run;   // x / ZS_STRIDE <= (L - 1) / ZS_STRIDE < zs_len
-    }
-}
-
 // Maximum of the four samples 4 q .. 4 q + 3 of the staged row (ROW_PADL
 // keeps them 16-byte aligned).
 __device__ __forceinline__ float quad_max(const float* __restrict__ F, int q)
@@ -444,7 +392,7 @@ __device__ __forceinline__ float quad_max(const float* __restrict__ F, int q)
     return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
 }
 
-// The maxima a pruned certified walk tests its blocks against, one entry per
+// The maxima a pruned walk tests its blocks against, one entry per
 // ZS_STRIDE samples of the staged row F (L samples, -inf beyond them).
 // warp-scans of 32 quads at a time: consecutive lanes read consecutive quads.
 //
@@ -1232,6 +1180,39 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
 #undef CERT_NG
 }
 
+// One round of a searching lane: tests SKIP_TESTS blocks from step e on
+// against the lines T d + K of its four POVs (see sweep_row_skip) and returns
+// the first step that may hold a visible target (*ready), the walk's end when
+// no remaining target can be visible, or the step after the tested blocks.
+// x0 and e are multiples of 4.
+template <int U, bool BWD>
+__device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, bool rising, int x0, int e, int dlim,
+                                           int L, const float* __restrict__ WM, const float* __restrict__ ZS,
+                                           bool* ready)
+{
+    constexpr int NT = SKIP_TESTS;
+    const float d = (float)(e + 1);
+    // the entries of blocks past the walk's end are not used
+    const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE, wlast = (L + U + 3) / ZS_STRIDE - 1;
+    float lim[NT], wm[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const float dk = d + (float)(k * U);
+        const float2 l0 = __ffma2_rn(T2[0], make_float2(dk, dk), K2[0]);
+        const float2 l1 = __ffma2_rn(T2[1], make_float2(dk, dk), K2[1]);
+        lim[k] = fminf(fminf(l0.x, l0.y), fminf(l1.x, l1.y));
+        wm[k] = WM[BWD ? max(w0 - k * U / ZS_STRIDE, 0) : min(w0 + k * U / ZS_STRIDE, wlast)];
+    }
+    const float end = ZS[(BWD ? x0 - e : x0 + e) / ZS_STRIDE];
+    int n = NT;
+#pragma unroll
+    for (int k = NT - 1; k >= 0; --k)
+        if (!(wm[k] <= lim[k])) n = k;
+    e = rising && end <= lim[0] ? dlim : e + n * U;
+    *ready = n < NT && e < dlim;
+    return e;
+}
+
 // Pruned certified sweep of one staged row: sweep_row_cert's walk, but a lane
 // evaluates only the blocks of U steps that can hold a visible target, and
 // stops where none is left.  (On fractal terrain 3 to 5 % of the targets of a
@@ -1280,7 +1261,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                                                const float* __restrict__ WM, const float4* __restrict__ tab,
                                                int* __restrict__ spill, int lane)
 {
-    constexpr int CH = SKIP_CHUNK, NT = SKIP_TESTS;
+    constexpr int CH = SKIP_CHUNK;
     static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
     const unsigned FULL = 0xffffffffu;
     const unsigned below = (1u << lane) - 1u;
@@ -1396,26 +1377,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
         // 2. lanes without a block look for one
         for (;;) {
             if (gi < G && !ready && e < dlim) {
-                const float d = (float)(e + 1);
-                // x0 and e are multiples of 4; the entries of blocks past the
-                // walk's end are not used
-                const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE, wlast = (L + U + 3) / ZS_STRIDE - 1;
-                float lim[NT], wm[NT];
-#pragma unroll
-                for (int k = 0; k < NT; ++k) {
-                    const float dk = d + (float)(k * U);
-                    const float2 l0 = __ffma2_rn(T2[0], make_float2(dk, dk), K2[0]);
-                    const float2 l1 = __ffma2_rn(T2[1], make_float2(dk, dk), K2[1]);
-                    lim[k] = fminf(fminf(l0.x, l0.y), fminf(l1.x, l1.y));
-                    wm[k] = WM[BWD ? max(w0 - k * U / ZS_STRIDE, 0) : min(w0 + k * U / ZS_STRIDE, wlast)];
-                }
-                const float end = ZS[(BWD ? x0 - e : x0 + e) / ZS_STRIDE];
-                int n = NT;
-#pragma unroll
-                for (int k = NT - 1; k >= 0; --k)
-                    if (!(wm[k] <= lim[k])) n = k;
-                e = rising && end <= lim[0] ? dlim : e + n * U;
-                ready = n < NT && e < dlim;
+                e = skip_blocks<U, BWD>(T2, K2, rising, x0, e, dlim, L, WM, ZS, &ready);
             }
             const unsigned have = __ballot_sync(FULL, ready);
             const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
@@ -1526,16 +1488,144 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
     }
 }
 
-template <bool LONG, bool PRUNE>
-__device__ __forceinline__ void sweep_item(const ItemRow& it, const float* F, const float* ZS, const float4* tab,
-                                           int tabn, int* cvrow, int* spill, int lane)
+// Pruned FP32-decision sweep of one staged row (backward rows staged
+// reversed), in the phases of sweep_row_skip.  A skipped target must be one
+// whose single-precision slope fl(fl(z - h) fl(1/d)) is at most M_q, which the
+// maximum then keeps: three roundings move a slope by less than 2^-22 of
+// itself, so with thr_q = M_q - 2^-21 |M_q| every target no higher than
+// h_q + thr_q d qualifies; slack covers the line's own rounding as there.
+// Every measure is bit for bit the unpruned walk's.  A POV without targets
+// has thr = -inf, which keeps its (short) group from skipping.
+// 1201 x 777, 180 directions: 19.5 -> 13.5 ms against the walk that only
+// stopped (8 POVs and 28 steps per block: larger blocks hold a visible target
+// more often).
+template <int P, int U, bool LONG>
+__device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const float* __restrict__ F,
+                                                 const float* __restrict__ ZS, const float* __restrict__ WM,
+                                                 const float4* __restrict__ tab, int* __restrict__ cvrow,
+                                                 int* __restrict__ spill, int L, int K, float h0, float zmax,
+                                                 bool rev, int lane)
+{
+    constexpr int CH = SKIP_CHUNK;
+    static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
+    const unsigned FULL = 0xffffffffu;
+    const unsigned below = (1u << lane) - 1u;
+    const float NEG = neg_inf();
+    const int G = (L + P - 1) / P;
+    const int klim = K - 1, tabn = sp.inv_len;
+    float h[P], M[P];
+    float2 acc2[P / 2], T2[P / 2], K2[P / 2];
+    bool rising = false, ready = false, klimited = false;
+    int gi = lane, next = 32;
+    int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
+    const bool inside = in_range(ROW_PADL + L + P + U, sp.half, 6) && in_range((L - 1) / ZS_STRIDE, sp.zs_len, 7) &&
+                        in_range((L + U + 3) / ZS_STRIDE - 1, sp.wm_len, 8) &&
+                        (LONG || in_range(min(K, L) + U - 1, tabn, 12));
+    if (!inside) return;
+
+    auto start = [&]() {
+        x0 = gi * P;
+        const int rowlim = L - 2 - x0;
+        dlim = min(klim, rowlim);
+        klimited = klim < rowlim;
+        e = 0;
+        seg = FLUSH_STEPS;
+        ready = dlim > 0;                                    // the first block is always evaluated
+        const float4 a = *reinterpret_cast<const float4*>(F + ROW_PADL + x0);
+        h[0] = __fadd_rn(a.x, h0); h[1] = __fadd_rn(a.y, h0);
+        h[2] = __fadd_rn(a.z, h0); h[3] = __fadd_rn(a.w, h0);
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            M[q] = NEG;
+            if (LONG) spill[32 * q] = 0;
+        }
+#pragma unroll
+        for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
+    };
+    if (gi < G) start();
+    for (;;) {
+        const bool fin = gi < G && !ready && e >= dlim;
+        const unsigned need = __ballot_sync(FULL, fin);
+        if (need && (__popc(need) >= SKIP_RESTART || !__any_sync(FULL, gi < G && !fin))) {
+            if (fin) {
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int x = x0 + q;
+                    if (x >= L) continue;
+                    const float s = q % 2 ? acc2[q / 2].y : acc2[q / 2].x;
+                    cvrow[rev ? L - 1 - x : x] =
+                        min(L - 1 - x, K) >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
+                }
+                gi = next + __popc(need & below);
+                if (gi < G) start(); else gi = G;
+            }
+            next += __popc(need);
+            if (!__any_sync(FULL, gi < G)) break;
+        }
+        for (;;) {
+            if (gi < G && !ready && e < dlim) e = skip_blocks<U, false>(T2, K2, rising, x0, e, dlim, L, WM, ZS, &ready);
+            const unsigned have = __ballot_sync(FULL, ready);
+            const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
+            if (!look || __popc(have) >= SKIP_READY) break;
+        }
+        if (ready) {
+            ready = false;
+            if (LONG && e >= seg) {
+                seg = e + FLUSH_STEPS;
+#pragma unroll
+                for (int q = 0; q < P; q += 2) {
+                    spill[32 * q] += __float2int_rz(acc2[q / 2].x);
+                    spill[32 * (q + 1)] += __float2int_rz(acc2[q / 2].y);
+                    acc2[q / 2] = make_float2(0.f, 0.f);
+                }
+            }
+            const bool far = LONG && e + U > tabn;
+            const float4* __restrict__ tb = tab + e + e / U;
+            const float* base = F + ROW_PADL + x0 + e;
+            float w[P + CH];
+            auto quad = [&](int at, int m) {
+                const float4 v = *reinterpret_cast<const float4*>(base + at);
+                w[m] = v.x; w[m + 1] = v.y; w[m + 2] = v.z; w[m + 3] = v.w;
+            };
+            quad(0, 0);
+            const int steps = min(dlim - e, U);
+#pragma unroll 1
+            for (int c = 0; c < steps; c += CH) {
+#pragma unroll
+                for (int m = P; m < P + CH; m += 4) quad(c + m, m);
+                if (klimited && c + CH > steps) {
+                    if (far) sweep_block<P, CH, true, true>(w, tab, e + c, h, M, acc2, steps - c);
+                    else sweep_block<P, CH, true, false>(w, tb + c, e, h, M, acc2, steps - c);
+                } else {
+                    if (far) sweep_block<P, CH, false, true>(w, tab, e + c, h, M, acc2, CH);
+                    else sweep_block<P, CH, false, false>(w, tb + c, e, h, M, acc2, CH);
+                }
+#pragma unroll
+                for (int m = 0; m < P; ++m) w[m] = w[m + CH];
+            }
+            rising = true;
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const float thr = __fmaf_rn(-0x1p-21f, fabsf(M[q]), M[q]);
+                const float base0 = __fsub_rn(h[q], 0x1p-20f * __fmaf_rn(3.f, zmax, fabsf(h[q])));
+                (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
+                (q % 2 ? K2[q / 2].y : K2[q / 2].x) =
+                    __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), base0);
+                rising = rising && thr >= 0.f;
+            }
+            e += U;
+        }
+    }
+}
+
+template <bool LONG>
+__device__ __forceinline__ void sweep_item(const ItemRow& it, const float* F, const float4* tab, int tabn, int* cvrow,
+                                           int* spill, int lane)
 {
     if (it.pov == SMALL_POV)
-        sweep_row<SMALL_POV, SMALL_UNROLL, LONG, PRUNE>(F, ZS, tab, tabn, cvrow, spill, it.L, it.K, it.h0, it.rev,
-                                                       lane);
+        sweep_row<SMALL_POV, SMALL_UNROLL, LONG>(F, tab, tabn, cvrow, spill, it.L, it.K, it.h0, it.rev, lane);
     else
-        sweep_row<LARGE_POV, LARGE_UNROLL, LONG, PRUNE>(F, ZS, tab, tabn, cvrow, spill, it.L, it.K, it.h0, it.rev,
-                                                       lane);
+        sweep_row<LARGE_POV, LARGE_UNROLL, LONG>(F, tab, tabn, cvrow, spill, it.L, it.K, it.h0, it.rev, lane);
 }
 
 
@@ -1574,12 +1664,13 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* Fh = smem + 4 * sp.tab_slots + sp.istart_len + warp * sp.per_warp;
     float* ZS = Fh + sp.half;
-    int* spill = reinterpret_cast<int*>(ZS + sp.zs_len) + lane;
+    float* WM = ZS + sp.zs_len;
+    int* spill = reinterpret_cast<int*>(WM + sp.wm_len) + lane;
     // per distance d = m + 1: (1/d, 1/d, 2d + 1, 2d + 1); 1/d correctly rounded
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
         const float c = (float)(2 * m + 3);
-        tab[m] = make_float4(r, r, c, c);
+        tab[PRUNE ? m + m / SKIP_UNROLL : m] = make_float4(r, r, c, c);
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
@@ -1596,14 +1687,18 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
         next = __shfl_sync(0xffffffffu, next, 0);
         if (!nonempty) continue;
         __syncwarp();
-        stage_row<false>(sp, it, Fh, nullptr, nullptr, lane);
+        const float zmax = stage_row<false>(sp, it, Fh, nullptr, nullptr, lane);
         __syncwarp();   // the staged row is visible to every lane
-        if (PRUNE) {
-            suffix_max(Fh, ZS, it.L, lane);
-            __syncwarp();
-        }
         int* cvrow = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
-        sweep_item<LONG, PRUNE>(it, Fh, ZS, tab, sp.inv_len, cvrow, spill, lane);
+        if constexpr (PRUNE) {
+            end_max<false>(Fh, ZS, it.L, lane);
+            window_max<SMALL_POV, SKIP_UNROLL>(Fh, WM, it.L, lane);
+            __syncwarp();
+            sweep_row_skip32<SMALL_POV, SKIP_UNROLL, LONG>(sp, Fh, ZS, WM, tab, cvrow, spill, it.L, it.K, it.h0, zmax,
+                                                           it.rev, lane);
+        } else {
+            sweep_item<LONG>(it, Fh, tab, sp.inv_len, cvrow, spill, lane);
+        }
     }
 }
 
@@ -1851,12 +1946,13 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     // the distance table is read up to d = dmax + U (a walk of at most
     // min(K, W) - 1 steps, rounded up to U); dmax <= wmax
     sp.inv_len = (std::min(dmax, wmax) + 2 * U + 8 + 1) & ~1;
-    sp.tab_slots = tab_slots_for(sp.inv_len, cert != 0);
+    const bool skewed = cert || prune;
+    sp.tab_slots = tab_slots_for(sp.inv_len, skewed);
     sp.istart_len = (ndir + 1 + 3) & ~3;
     sp.half = (ROW_PADL + 4 + wmax + ROW_PADR + 3) & ~3;
     const bool longw = wmax - 2 > LONG_WALK && dmax - 1 > LONG_WALK;
     sp.zs_len = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
-    sp.wm_len = prune && cert ? wm_entries(wmax) : 0;
+    sp.wm_len = prune ? wm_entries(wmax) : 0;
     const int lspill = longw ? 32 * LARGE_POV : 0;
     // FP32 decisions: one row per warp.  Certified: one row per warp
     // (reversed for backward walks) when TVS_CERT_SINGLE_MIN such warps fit, else
@@ -1871,7 +1967,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
                         single_fit >= (size_t)single_min;
     const bool pairs = cert && !single;
     sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 8 : 0;
-    sp.per_warp = single ? single_warp : pairs ? lspill : sp.half + sp.zs_len + lspill;
+    sp.per_warp = single ? single_warp : pairs ? lspill : sp.half + sp.zs_len + sp.wm_len + lspill;
     // shared memory of one unit: a pair of warps or one warp
     const int uw = pairs ? 2 : 1;
     const size_t unit = (size_t)(sp.per_pair + uw * sp.per_warp) * 4;
@@ -1883,14 +1979,14 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         // entries); the long-walk sweep computes the entries past its end.
         const size_t base = (size_t)sp.istart_len * 4;
         int w = LONG_MIN_WARPS / uw;
-        const size_t min_tab = (size_t)tab_slots_for(MIN_TABLE, cert != 0) * 16;
+        const size_t min_tab = (size_t)tab_slots_for(MIN_TABLE, skewed) * 16;
         while (w > 1 && base + min_tab + (size_t)w * unit > (size_t)smem_optin) --w;
         if (base + 16 * 4 + (size_t)w * unit >= (size_t)smem_optin) return cudaErrorInvalidConfiguration;
         // slots that fit, and the most entries whose slots do
         const size_t room = ((size_t)smem_optin - base - (size_t)w * unit) / 16;
-        const size_t fit = cert ? (room - 2) * TAB_SKEW_MIN / (TAB_SKEW_MIN + 1) : room;
+        const size_t fit = skewed ? (room - 2) * TAB_SKEW_MIN / (TAB_SKEW_MIN + 1) : room;
         sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, fit) & ~1;
-        sp.tab_slots = tab_slots_for(sp.inv_len, cert != 0);
+        sp.tab_slots = tab_slots_for(sp.inv_len, skewed);
         fixed = (size_t)(4 * sp.tab_slots + sp.istart_len) * 4;
     }
     if (fixed + unit > (size_t)smem_optin) return cudaErrorInvalidConfiguration;
