@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace tvs {
 
@@ -75,10 +76,13 @@ struct SweepParams {
     int flag_cap;
     int ndir;
     int total_items;
-    int inv_len;       // entries of the per-distance table (float4 each)
-    int tab_slots;     // float4 slots the table takes (the certified kernels skew it)
+    int inv_len;       // entries of the per-distance table
+    int tab_floats;    // floats it takes (a multiple of 4)
     int istart_len;    // ints of the item-start table (multiple of 4)
     int half;          // floats of one staged row array (multiple of 4)
+    int padr;          // of them after the row's samples
+    int lgna;          // packed kernel: log2 of the staged rows per warp
+    int per_row;       // packed kernel: floats of a staged row's arrays
     int per_pair;      // floats of a warp pair's shared area (certified)
     int zs_len;        // floats of the row's suffix maxima (0 without pruning)
     int wm_len;        // floats of the row's window maxima (0 without pruning)
@@ -149,7 +153,8 @@ __device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* is
 
 // Stages the item's row from the DEM: FP32 heights into Fh, or with CERT hi
 // parts into Fh and lo parts into Fl, reversed for backward items unless
-// rev_ok is false (rows that both walk directions share stay in row order).  The last sample and ROW_PADR samples after
+// rev_ok is false (rows that both walk directions share stay in row order);
+// with mirror arrays also reversed into those.  The last sample and sp.padr samples after
 // it hold -inf (lo 0): the last target of a walk never adds area, so it may be
 // a sentinel that is never visible.  With CERT the first sample and the
 // ROW_PADL samples before it are sentinels too (the last target of a backward
@@ -158,7 +163,8 @@ __device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* is
 // largest |elevation| read, for the error bounds.
 template <bool CERT>
 __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow& it, float* Fh, float* Fl,
-                                           float* ends, int lane, int part = 0, int parts = 1, bool rev_ok = true)
+                                           float* ends, int lane, int part = 0, int parts = 1, bool rev_ok = true,
+                                           float* mirror_h = nullptr, float* mirror_l = nullptr)
 {
     const DirDev& d = sp.dirs[it.dir];
     const float* __restrict__ dem = sp.jobs[d.job].dem;
@@ -200,6 +206,10 @@ __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow&
                 if (x == it.L - 1) { ends[2] = zh; ends[3] = zl; }
                 Fh[ROW_PADL + x] = end ? NEG : zh;
                 Fl[ROW_PADL + x] = end ? 0.f : zl;
+                if (mirror_h) {
+                    mirror_h[ROW_PADL + it.L - 1 - x] = end ? NEG : zh;
+                    mirror_l[ROW_PADL + it.L - 1 - x] = end ? 0.f : zl;
+                }
                 zmax = fmaxf(zmax, fmaxf(fabsf(va[k]), fabsf(vb[k])));
             } else {
                 Fh[ROW_PADL + x] = x == it.L - 1 ? NEG : blend32(va[k], vb[k], fr[k]);
@@ -207,13 +217,15 @@ __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow&
             }
         }
     }
-    for (int m = lane; part == 0 && m < ROW_PADR; m += 32) {
+    for (int m = lane; part == 0 && m < sp.padr; m += 32) {
         if (!in_range(ROW_PADL + it.L + m, sp.half, 4)) continue;
         Fh[ROW_PADL + it.L + m] = NEG;
         if (CERT) Fl[ROW_PADL + it.L + m] = 0.f;
+        if (CERT && mirror_h) { mirror_h[ROW_PADL + it.L + m] = NEG; mirror_l[ROW_PADL + it.L + m] = 0.f; }
     }
     if (CERT) {
         if (part == 0 && lane < ROW_PADL) { Fh[lane] = NEG; Fl[lane] = 0.f; }
+        if (part == 0 && mirror_h && lane < ROW_PADL) { mirror_h[lane] = NEG; mirror_l[lane] = 0.f; }
     } else if (lane < ROW_PADL) {
         Fh[lane] = NEG;
     }
@@ -239,6 +251,35 @@ __device__ __forceinline__ float4 dist_entry(int d)
     return make_float4(r, r, c, c);
 }
 
+// (1/d, 1/d) and (2d + 1, 2d + 1) of step u of a block that starts at step e
+// (d = e + 1 + u), tab at the block's first entry.  Unpruned walks keep both in
+// the table (float4).  Pruned walks keep (1/d, 1/d) alone: their lanes stand at
+// 32 different steps, so an entry of 16 bytes costs four passes over the
+// shared-memory banks per step, the largest part of a pipe that was 68 % busy;
+// 2d + 1 is then one packed add.  That alone measured the same (2000^2 92.8 and
+// 92.1 ms); the room it frees holds more warps and packed rows.
+template <bool FAR>
+__device__ __forceinline__ void dist_pair(const float4* __restrict__ tab, int e, int u, float2& iv, float2& c)
+{
+    const float4 t = FAR ? dist_entry(e + u + 1) : tab[u];
+    iv = make_float2(t.x, t.y);
+    c = make_float2(t.z, t.w);
+}
+template <bool FAR>
+__device__ __forceinline__ void dist_pair(const float2* __restrict__ tab, int e, int u, float2& iv, float2& c)
+{
+    if (FAR) {
+        const float r = __frcp_rn((float)(e + u + 1));
+        iv = make_float2(r, r);
+    } else {
+        // two entries per 16-byte load (the compiler keeps one of the two)
+        const float4 t = *reinterpret_cast<const float4*>(tab + (u & ~1));
+        iv = u % 2 ? make_float2(t.z, t.w) : make_float2(t.x, t.y);
+    }
+    const float b = (float)(2 * e + 3);
+    c = __fadd2_rn(make_float2(b, b), make_float2((float)(2 * u), (float)(2 * u)));
+}
+
 // U steps of one lane's P POVs.  POV q at step u (distance d = e + 1 + u)
 // sees target w[q + u + 1]; its slope is (target - h_q) * (1/d) in single
 // precision, it is visible iff that slope is strictly above the running
@@ -247,16 +288,16 @@ __device__ __forceinline__ float4 dist_entry(int d)
 // the maximum are scalar.  tab[u] holds (1/d, 1/d, 2d + 1, 2d + 1); a
 // range-limited walk's last block counts only its first `nvalid` steps.
 // With FAR the block's entries are computed (distances e + 1 .. e + U, past
-// the end of a capped table) instead of read from tab[0 .. U).
-template <int P, int U, bool MASKED, bool FAR>
-__device__ __forceinline__ void sweep_block(const float* w, const float4* __restrict__ tab, int e, const float* h,
+// the end of a capped table) instead of read from tab[0 .. U).  T is the
+// table's entry type (see dist_pair).
+template <int P, int U, bool MASKED, bool FAR, class T>
+__device__ __forceinline__ void sweep_block(const float* w, const T* __restrict__ tab, int e, const float* h,
                                             float* M, float2* acc2, int nvalid)
 {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const float4 t4 = FAR ? dist_entry(e + u + 1) : tab[u];
-        const float2 iv = make_float2(t4.x, t4.y);
-        float2 cpair = make_float2(t4.z, t4.w);
+        float2 iv, cpair;
+        dist_pair<FAR>(tab, e, u, iv, cpair);
         if (MASKED && u >= nvalid) cpair = make_float2(0.f, 0.f);
 #pragma unroll
         for (int q = 0; q < P; q += 2) {
@@ -497,7 +538,7 @@ constexpr int CERT_POV = TVS_CERT_POV;
 static_assert(CERT_POV + CERT_UNROLL <= ROW_PADR && CERT_POV + CERT_UNROLL_SINGLE <= ROW_PADR,
               "a forward block's window reads up to P + U samples on");
 #ifndef TVS_SKIP_READY
-#define TVS_SKIP_READY 24
+#define TVS_SKIP_READY 22
 #endif
 constexpr int SKIP_READY = TVS_SKIP_READY;   // lanes with a block before a pruned walk evaluates
 #ifndef TVS_SKIP_RESTART
@@ -512,13 +553,19 @@ constexpr int SKIP_TESTS = TVS_SKIP_TESTS;       // blocks a searching lane test
 #define TVS_SKIP_CHUNK 8
 #endif
 constexpr int SKIP_CHUNK = TVS_SKIP_CHUNK;       // steps per pass of a block's evaluation loop
-#ifndef TVS_SKIP_WARPS
-#define TVS_SKIP_WARPS 16
-#endif
-constexpr int SKIP_WARPS = TVS_SKIP_WARPS;       // most warps of a pruned certified CTA
 #ifndef TVS_SKIP_UNROLL
 #define TVS_SKIP_UNROLL 16
 #endif
+// Samples after a staged row that a pruned walk's windows read.
+constexpr int SKIP_PADR = CERT_POV + TVS_SKIP_UNROLL + 8;
+#ifndef TVS_SKIP_WARPS
+#define TVS_SKIP_WARPS 16
+#endif
+constexpr int SKIP_WARPS = TVS_SKIP_WARPS;       // most warps of a pruned certified CTA of warp pairs
+#ifndef TVS_PACK_WARPS
+#define TVS_PACK_WARPS 20
+#endif
+constexpr int PACK_WARPS = TVS_PACK_WARPS;       // and of packed rows
 constexpr int SKIP_UNROLL = TVS_SKIP_UNROLL;   // steps per block of a pruned walk
 static_assert(SKIP_UNROLL <= ROW_PADL && CERT_POV + SKIP_UNROLL <= ROW_PADR && FLUSH_STEPS % SKIP_UNROLL == 0,
               "pads and flushes of a pruned walk");
@@ -531,12 +578,22 @@ static_assert(FLUSH_STEPS % CERT_UNROLL == 0, "long walks flush on block boundar
 // 16-byte bank groups.  Skewed, entry u of block k sits in bank group
 // ((U + 1) k + u) mod 8 (U a multiple of 8), which spreads blocks k over all
 // eight.  Tables are sized for the shorter block, which needs the most slots.
-constexpr int TAB_SKEW_MIN = std::min({CERT_UNROLL, CERT_UNROLL_SINGLE, SKIP_UNROLL});
-static_assert(CERT_UNROLL % 8 == 0 && CERT_UNROLL_SINGLE % 8 == 0, "skewed blocks cover the eight bank groups");
-static_assert(SKIP_UNROLL % 8 == 0, "as above");
-__host__ __device__ constexpr int tab_slots_for(int entries, bool skew)
+static_assert(SKIP_UNROLL % 8 == 0 && CERT_UNROLL % 8 == 0 && CERT_UNROLL_SINGLE % 8 == 0,
+              "skewed blocks cover the eight bank groups");
+// A pruned kernel's 8-byte entry m sits at slot m + 2 (m / SKIP_UNROLL) (two
+// slots: the blocks stay 16-byte aligned), which spreads the blocks alike.
+constexpr int TAB_SKEW_MIN = std::min(CERT_UNROLL, CERT_UNROLL_SINGLE);
+// Floats of a table of `entries` distances, a multiple of 4, and the most
+// entries that fit `floats`.
+int tab_floats_for(int entries, bool prune, bool cert)
 {
-    return skew ? ((entries + entries / TAB_SKEW_MIN + 1 + 1) & ~1) : entries;
+    if (prune) return 2 * ((entries + 2 * (entries / SKIP_UNROLL) + 2 + 1) & ~1);
+    return 4 * (cert ? (entries + entries / TAB_SKEW_MIN + 1 + 1) & ~1 : entries);
+}
+size_t tab_entries_fit(size_t floats, bool prune, bool cert)
+{
+    if (prune) return floats / 2 < 4 ? 0 : (floats / 2 - 4) * SKIP_UNROLL / (SKIP_UNROLL + 2);
+    return cert ? (floats / 4 < 2 ? 0 : (floats / 4 - 2) * TAB_SKEW_MIN / (TAB_SKEW_MIN + 1)) : floats / 4;
 }
 // Far from the POV one margin serves several window blocks: from step
 // CERT_NEAR on a margin block is 2 window blocks long, from CERT_FAR on 4 and
@@ -653,17 +710,62 @@ __device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const Cert
 constexpr int FLAG_WALK = 0, FLAG_BLOCK = 1, FLAG_PREFIX = 2;
 static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 
+// A staged row as the pruned certified walks see it (in shared memory, so that
+// the lanes of a warp may be on different rows).
+struct __align__(16) SkipRow {
+    int L, K;
+    int item;            // its work item
+    int rev;             // staged x is row sample L - 1 - x
+    float ends[4];       // hi and lo parts of the first and of the last sample (sentinels when staged)
+    float h0;
+    float eg0;           // as CertRow
+    float zmax;          // the row's largest |elevation|
+    int pad;
+    int* cv;             // the row's measures
+    long long pad2;
+};
+static_assert(sizeof(SkipRow) == 64, "16 floats");
+constexpr int SKIP_ROW_FLOATS = 16;
+#ifndef TVS_PACK_MAX_LG
+#define TVS_PACK_MAX_LG 3
+#endif
+constexpr int PACK_MAX_LG = TVS_PACK_MAX_LG;           // at most 8 staged rows per warp
+#ifndef TVS_PACK_MIN_CLAIMS
+#define TVS_PACK_MIN_CLAIMS 3
+#endif
+constexpr int PACK_MIN_CLAIMS = TVS_PACK_MIN_CLAIMS;   // packs per warp that packing must leave
+
 // Hands block e0 of staged sample x's walk to the exact pass, p0 the block of
 // its last rise; false when the buffer is full.
-__device__ __forceinline__ bool flag_block(const SweepParams& sp, const CertRow& r, int x, int e0, int p0, int kind)
+__device__ __forceinline__ bool flag_block(const SweepParams& sp, const SkipRow& r, int x, int e0, int p0, int kind)
 {
     const unsigned cap = (unsigned)sp.flag_cap;
     unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
     if (at < cap) at = atomicAdd(sp.flag_count, 1u);
     if (at >= cap) return false;
-    sp.flag_buf[at] = make_int4(r.item, (r.rev_staged ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax),
-                                e0 | p0 << 14);
+    sp.flag_buf[at] = make_int4(r.item, (r.rev ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax), e0 | p0 << 14);
     return true;
+}
+
+// Fills a staged item's row (the ends are there already); false when a walk of
+// the row could leave its arrays or the distance table (windows start at most
+// SKIP_UNROLL samples before the row and end before sample L + P + U).
+__device__ __forceinline__ bool skip_row(const SweepParams& sp, const ItemRow& it, int item, float zmax, int* cv,
+                                         bool rev, bool longw, SkipRow* r)
+{
+    const float eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
+    r->L = it.L;
+    r->K = it.K;
+    r->item = item;
+    r->rev = rev;
+    r->h0 = it.h0;
+    r->eg0 = 2.01f * 0x1p-24f * fabsf(it.h0) + fabsf(sp.dirs[it.dir].h0_lo) * 1.0001f + 4.04f * eta;
+    r->zmax = zmax;
+    r->cv = cv + it.rowbase;
+    return in_range(ROW_PADL + it.L + CERT_POV + SKIP_UNROLL, sp.half, 19) &&
+           in_range((it.L - 1) / ZS_STRIDE, sp.zs_len, 9) &&
+           in_range((it.L + SKIP_UNROLL + 3) / ZS_STRIDE - 1, sp.wm_len, 10) &&
+           (longw || in_range(min(it.K, it.L) + SKIP_UNROLL - 1, sp.inv_len, 11));
 }
 
 // Writes the measures of a finished group of P POVs (pov_x(q): staged sample
@@ -946,8 +1048,8 @@ __device__ __forceinline__ float min_abs2(float a, float b, float c)
 // go through one packed add wherever their two targets form an aligned pair
 // of the window (y[2j], y[2j + 1]: every other step); y - g and y + (-g)
 // round alike.
-template <int P, int U, bool MASKED, bool FAR, bool PACK>
-__device__ __forceinline__ void cert_block(const float* y, const float4* __restrict__ tab, int e, const float2* ng2,
+template <int P, int U, bool MASKED, bool FAR, bool PACK, class T>
+__device__ __forceinline__ void cert_block(const float* y, const T* __restrict__ tab, int e, const float2* ng2,
                                            float2* M2, float2* acc2, float* mn, int nvalid)
 {
     static_assert(U % 2 == 0, "steps go in pairs");
@@ -957,9 +1059,8 @@ __device__ __forceinline__ void cert_block(const float* y, const float4* __restr
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int w = u + k;
-            const float4 t4 = FAR ? dist_entry(e + w + 1) : tab[w + w / U];
-            const float2 iv = make_float2(t4.x, t4.y);
-            float2 cp = make_float2(t4.z, t4.w);
+            float2 iv, cp;
+            dist_pair<FAR>(tab, e, w, iv, cp);
             if (MASKED && w >= nvalid) cp = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < P; q += 2) {
@@ -1187,13 +1288,13 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
 // x0 and e are multiples of 4.
 template <int U, bool BWD>
 __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, bool rising, int x0, int e, int dlim,
-                                           int L, const float* __restrict__ WM, const float* __restrict__ ZS,
+                                           int wlast, const float* __restrict__ WM, const float* __restrict__ ZS,
                                            bool* ready)
 {
     constexpr int NT = SKIP_TESTS;
     const float d = (float)(e + 1);
     // the entries of blocks past the walk's end are not used
-    const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE, wlast = (L + U + 3) / ZS_STRIDE - 1;
+    const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE;
     float lim[NT], wm[NT];
 #pragma unroll
     for (int k = 0; k < NT; ++k) {
@@ -1213,7 +1314,8 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
     return e;
 }
 
-// Pruned certified sweep of one staged row: sweep_row_cert's walk, but a lane
+// Pruned certified sweep of a warp's staged rows (2^lgna of them, sp.per_row
+// floats apart; `groups` is the most groups of any): sweep_row_cert's walk, but a lane
 // evaluates only the blocks of U steps that can hold a visible target, and
 // stops where none is left.  (On fractal terrain 3 to 5 % of the targets of a
 // walk are visible; the walks reach their stopping point after about 40 % of
@@ -1257,19 +1359,18 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // goes: the few registers that takes let 20 warps share an SM, and their
 // number is what hides the latency of the tests.
 template <int P, int U, bool LONG, bool BWD>
-__device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const CertRow& r, const float* __restrict__ ZS,
-                                               const float* __restrict__ WM, const float4* __restrict__ tab,
-                                               int* __restrict__ spill, int lane)
+__device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const SkipRow* __restrict__ rows,
+                                                const float* H0, int lgna, int groups, int zs_off, int wm_off,
+                                                const float2* __restrict__ tab, int* __restrict__ spill, int lane)
 {
     constexpr int CH = SKIP_CHUNK;
     static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
     const unsigned FULL = 0xffffffffu;
     const unsigned below = (1u << lane) - 1u;
-    const float* __restrict__ H = r.H;
-    const float* __restrict__ Lo = r.Lo;
-    const int L = r.L, K = r.K, tabn = sp.inv_len;
-    const int G = (L + P - 1) / P;
-    const int klim = K - 1;
+    const int tabn = sp.inv_len;
+    // the group's staged row (the lanes of a warp may be on different ones)
+    const SkipRow* r = rows;
+    const float* H = H0;             // its hi parts; lo parts, end and window maxima at fixed offsets
     constexpr bool PACK = !BWD && TVS_CERT_PACKADD;
     float ia[P];
     float2 ng2[P / 2];               // -g of POV pairs
@@ -1277,20 +1378,23 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
     float2 T2[P / 2], K2[P / 2];     // thr and k of POV pairs
     bool rising = false;             // every thr >= 0
     float Rh = 0.f, c2e = 0.f;
+    float level = 0.f;               // R - slack
     unsigned lost = 0u, again = 0u;  // POVs whose walk is taken again; with an earlier flagged block
-    int gi = lane, next = 32;
+    const int tasks = groups << lgna;  // group t >> lgna of row t & (rows - 1), longest walks first
+    int next = 32;
+    bool has = lane < tasks;
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
     bool klimited = false, ready = false;
     auto pov_x = [&](int q) { return BWD ? x0 + P - 1 - q : x0 + q; };
-    auto walk_n = [&](int x) { return min(BWD ? x : L - 1 - x, K); };
-    // every index the row's blocks and tests use, checked once: windows start
-    // at most U samples before the row and end before sample L + P + U
-    const bool inside = in_range(ROW_PADL + L + P + U, sp.half, 19) && in_range((L - 1) / ZS_STRIDE, sp.zs_len, 9) &&
-                        in_range((L + U + 3) / ZS_STRIDE - 1, sp.wm_len, 10) &&
-                        (LONG || in_range(min(K, L) + U - 1, tabn, 11));
 
-    auto start = [&]() {
+    auto start = [&](int task) {
+        r = rows + (task & ((1 << lgna) - 1));
+        H = H0 + (task & ((1 << lgna) - 1)) * sp.per_row;
+        const int L = r->L, gi = task >> lgna, G = (L + P - 1) / P;
+        const float* Lo = H + sp.half;
         x0 = (BWD ? G - 1 - gi : gi) * P;
+        if (gi >= G) { x0 = L; e = 0; dlim = -1; return; }   // a shorter row of the pack
+        const int klim = r->K - 1;
         const int xl = BWD ? min(x0 + P - 1, L - 1) : x0;
         const int rowlim = BWD ? xl - 1 : L - 2 - xl;
         dlim = min(klim, rowlim);
@@ -1305,11 +1409,6 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
             for (int q = 0; q < P; ++q) spill[32 * q] = 0;
         }
         if (dlim < 1) return;
-        if (!inside) {
-            dlim = 0;
-            lost = (1u << P) - 1u;
-            return;
-        }
         ready = true;                                        // the first block is always evaluated
         // the group's samples in POV order, and each POV's first target
         const float4 a = *reinterpret_cast<const float4*>(H + x0), b = *reinterpret_cast<const float4*>(Lo + x0);
@@ -1321,13 +1420,13 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
 #pragma unroll
         for (int q = 0; q < P; ++q) { zh[q] = zs[q]; zl[q] = ls[q]; }
         if (x0 == 0) {                                       // the row's end samples are sentinels when staged
-            zh[BWD ? P - 1 : 0] = r.eh0;
-            zl[BWD ? P - 1 : 0] = r.el0;
+            zh[BWD ? P - 1 : 0] = r->ends[0];
+            zl[BWD ? P - 1 : 0] = r->ends[1];
         }
         if (x0 + P >= L) {
 #pragma unroll
             for (int q = 0; q < P; ++q)
-                if (pov_x(q) == L - 1) { zh[q] = r.ehL; zl[q] = r.elL; }
+                if (pov_x(q) == L - 1) { zh[q] = r->ends[2]; zl[q] = r->ends[3]; }
         }
         Rh = zh[BWD ? P - 1 : 0];
         float gq[P], gmax = 0.f;
@@ -1335,10 +1434,11 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
         for (int q = 0; q < P; ++q) {
             const int x = pov_x(q);
             const bool pov = BWD ? (x >= 1 && x <= L - 1) : x <= L - 2;   // POVs with a target
-            gq[q] = pov ? __fadd_rn(__fadd_rn(__fsub_rn(zh[q], Rh), zl[q]), r.h0) : 0.f;
+            gq[q] = pov ? __fadd_rn(__fadd_rn(__fsub_rn(zh[q], Rh), zl[q]), r->h0) : 0.f;
             gmax = fmaxf(gmax, fabsf(gq[q]));
         }
-        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, r.eg0);
+        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, r->eg0);
+        level = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, r->zmax, gmax), __fmul_rn(2.f, c2e)));
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             // as sweep_row_cert: M starts just below the first target's slope
@@ -1351,36 +1451,41 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
             ia[q] = 1.f;
         }
     };
-    if (gi < G) start();
+    if (tasks == 0) return;
+    if (has) start(lane);
     for (;;) {
         // 1. finished groups: write their measures, hand over their flagged
         // walks, take the next groups
-        const bool fin = gi < G && !ready && e >= dlim;
+        const bool fin = has && !ready && e >= dlim;
         const unsigned need = __ballot_sync(FULL, fin);
-        if (need && (__popc(need) >= SKIP_RESTART || !__any_sync(FULL, gi < G && !fin))) {
+        if (need && (__popc(need) >= SKIP_RESTART || !__any_sync(FULL, has && !fin))) {
             if (fin) {
+                const int L = r->L, K = r->K;
+                int* cvrow = r->cv;
+                const bool rev = r->rev != 0;
                 if (lost) sp.flag_count[2] = 1u;
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     const int x = pov_x(q);
                     if (x >= L) continue;
                     const float s = q % 2 ? acc2[q / 2].y : acc2[q / 2].x;
-                    const int cv = walk_n(x) >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
-                    r.cvrow[r.rev_staged ? L - 1 - x : x] = (lost >> q) & 1u ? CV_FLAGGED : cv;
+                    const int n = min(BWD ? x : L - 1 - x, K);
+                    const int cv = n >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
+                    cvrow[rev ? L - 1 - x : x] = (lost >> q) & 1u ? CV_FLAGGED : cv;
                 }
-                gi = next + __popc(need & below);
-                if (gi < G) start(); else gi = G;
+                const int task = next + __popc(need & below);
+                has = task < tasks;
+                if (has) start(task);
             }
             next += __popc(need);
-            if (!__any_sync(FULL, gi < G)) break;
+            if (!__any_sync(FULL, has)) break;
         }
         // 2. lanes without a block look for one
         for (;;) {
-            if (gi < G && !ready && e < dlim) {
-                e = skip_blocks<U, BWD>(T2, K2, rising, x0, e, dlim, L, WM, ZS, &ready);
-            }
+            if (has && !ready && e < dlim)
+                e = skip_blocks<U, BWD>(T2, K2, rising, x0, e, dlim, sp.wm_len - 1, H + wm_off, H + zs_off, &ready);
             const unsigned have = __ballot_sync(FULL, ready);
-            const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
+            const unsigned look = __ballot_sync(FULL, has && !ready && e < dlim);
             if (!look || __popc(have) >= SKIP_READY) break;
         }
         // 3. evaluate the blocks found
@@ -1397,7 +1502,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                 }
             }
             const bool far = LONG && e + U > tabn;
-            const float4* __restrict__ tb = tab + e + e / U;
+            const float2* __restrict__ tb = tab + e + 2 * (e / U);
             const float ive = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tb->x;
             float Ms[P], mn[P];
             float2 blk2[P / 2];      // the block's share of the measures
@@ -1413,7 +1518,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                 // window in walk order, kept P samples back from step to step
                 const float2 nRh = make_float2(-Rh, -Rh);
                 const float* bh = H + (BWD ? x0 - e : x0 + e);
-                const float* bl = Lo + (BWD ? x0 - e : x0 + e);
+                const float* bl = bh + sp.half;
                 float y[P + CH];
                 auto quad = [&](int at, int m) {   // y[m ..] from the four samples at `at`
                     const float4 a = *reinterpret_cast<const float4*>(bh + at);
@@ -1433,10 +1538,10 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                     for (int m = P; m < P + CH; m += 4) quad(BWD ? -(c + m) : c + m, m);
                     if (klimited && c + CH > steps) {
                         if (far) cert_block<P, CH, true, true, PACK>(y, tab, e + c, ng2, M2, blk2, mn, steps - c);
-                        else cert_block<P, CH, true, false, PACK>(y, tb + c, e, ng2, M2, blk2, mn, steps - c);
+                        else cert_block<P, CH, true, false, PACK>(y, tb + c, e + c, ng2, M2, blk2, mn, steps - c);
                     } else {
                         if (far) cert_block<P, CH, false, true, PACK>(y, tab, e + c, ng2, M2, blk2, mn, CH);
-                        else cert_block<P, CH, false, false, PACK>(y, tb + c, e, ng2, M2, blk2, mn, CH);
+                        else cert_block<P, CH, false, false, PACK>(y, tb + c, e + c, ng2, M2, blk2, mn, CH);
                     }
 #pragma unroll
                     for (int m = 0; m < P; ++m) y[m] = y[m + CH];
@@ -1444,10 +1549,6 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
             }
             // the margin test of sweep_row_cert, and the lines of the next tests
             const float ce = __fmaf_rn(c2e, ive, CERT_FLOOR);
-            float gm = 0.f;
-#pragma unroll
-            for (int q = 0; q < P; ++q) gm = fmaxf(gm, fabsf(q % 2 ? ng2[q / 2].y : ng2[q / 2].x));
-            const float base = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, r.zmax, gm), __fmul_rn(2.f, c2e)));
             rising = true;
             unsigned fm = 0u;
             float dqs[P];
@@ -1464,7 +1565,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                     if (!((fm >> q) & 1u)) continue;
                     (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
                     const int p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
-                    if (!flag_block(sp, r, pov_x(q), e, p0, (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                    if (!flag_block(sp, *r, pov_x(q), e, p0, (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
                 }
                 again |= fm;
@@ -1480,7 +1581,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
                 const float g = -(q % 2 ? ng2[q / 2].y : ng2[q / 2].x);
                 (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
                 (q % 2 ? K2[q / 2].y : K2[q / 2].x) =
-                    __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), __fadd_rn(base, g));
+                    __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), __fadd_rn(level, g));
                 rising = rising && !(thr < 0.f);
             }
             e += U;
@@ -1502,7 +1603,7 @@ __device__ __forceinline__ void sweep_row_skip(const SweepParams& sp, const Cert
 template <int P, int U, bool LONG>
 __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const float* __restrict__ F,
                                                  const float* __restrict__ ZS, const float* __restrict__ WM,
-                                                 const float4* __restrict__ tab, int* __restrict__ cvrow,
+                                                 const float2* __restrict__ tab, int* __restrict__ cvrow,
                                                  int* __restrict__ spill, int L, int K, float h0, float zmax,
                                                  bool rev, int lane)
 {
@@ -1563,7 +1664,7 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
             if (!__any_sync(FULL, gi < G)) break;
         }
         for (;;) {
-            if (gi < G && !ready && e < dlim) e = skip_blocks<U, false>(T2, K2, rising, x0, e, dlim, L, WM, ZS, &ready);
+            if (gi < G && !ready && e < dlim) e = skip_blocks<U, false>(T2, K2, rising, x0, e, dlim, sp.wm_len - 1, WM, ZS, &ready);
             const unsigned have = __ballot_sync(FULL, ready);
             const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
             if (!look || __popc(have) >= SKIP_READY) break;
@@ -1580,7 +1681,7 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
                 }
             }
             const bool far = LONG && e + U > tabn;
-            const float4* __restrict__ tb = tab + e + e / U;
+            const float2* __restrict__ tb = tab + e + 2 * (e / U);
             const float* base = F + ROW_PADL + x0 + e;
             float w[P + CH];
             auto quad = [&](int at, int m) {
@@ -1595,10 +1696,10 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
                 for (int m = P; m < P + CH; m += 4) quad(c + m, m);
                 if (klimited && c + CH > steps) {
                     if (far) sweep_block<P, CH, true, true>(w, tab, e + c, h, M, acc2, steps - c);
-                    else sweep_block<P, CH, true, false>(w, tb + c, e, h, M, acc2, steps - c);
+                    else sweep_block<P, CH, true, false>(w, tb + c, e + c, h, M, acc2, steps - c);
                 } else {
                     if (far) sweep_block<P, CH, false, true>(w, tab, e + c, h, M, acc2, CH);
-                    else sweep_block<P, CH, false, false>(w, tb + c, e, h, M, acc2, CH);
+                    else sweep_block<P, CH, false, false>(w, tb + c, e + c, h, M, acc2, CH);
                 }
 #pragma unroll
                 for (int m = 0; m < P; ++m) w[m] = w[m + CH];
@@ -1659,18 +1760,19 @@ template <bool PRUNE, bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
-    float4* tab = reinterpret_cast<float4*>(smem);
-    int* istart = reinterpret_cast<int*>(smem + 4 * sp.tab_slots);
+    using Entry = std::conditional_t<PRUNE, float2, float4>;
+    Entry* tab = reinterpret_cast<Entry*>(smem);
+    int* istart = reinterpret_cast<int*>(smem + sp.tab_floats);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* Fh = smem + 4 * sp.tab_slots + sp.istart_len + warp * sp.per_warp;
+    float* Fh = smem + sp.tab_floats + sp.istart_len + warp * sp.per_warp;
     float* ZS = Fh + sp.half;
     float* WM = ZS + sp.zs_len;
     int* spill = reinterpret_cast<int*>(WM + sp.wm_len) + lane;
     // per distance d = m + 1: (1/d, 1/d, 2d + 1, 2d + 1); 1/d correctly rounded
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
-        const float c = (float)(2 * m + 3);
-        tab[PRUNE ? m + m / SKIP_UNROLL : m] = make_float4(r, r, c, c);
+        if constexpr (PRUNE) tab[m + 2 * (m / SKIP_UNROLL)] = make_float2(r, r);
+        else tab[m] = make_float4(r, r, (float)(2 * m + 3), (float)(2 * m + 3));
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
@@ -1702,29 +1804,26 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
     }
 }
 
-// The certified sweep with one row per warp, for launches whose rows leave
+// The unpruned certified sweep with one row per warp, for launches whose rows leave
 // room for at least TVS_CERT_SINGLE_MIN of them (16 warps when they fit, else
 // 12): a backward item's row is staged reversed and walked forward, like the
 // FP32 sweep's.  Per warp, shared memory holds
-// [Fh half][Fl half][suffix maxima][window maxima][ends 4].
-template <bool PRUNE, bool LONG, int WARPS>
+// [Fh half][Fl half][ends 4].
+template <bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
     float4* tab = reinterpret_cast<float4*>(smem);
-    int* istart = reinterpret_cast<int*>(smem + 4 * sp.tab_slots);
+    int* istart = reinterpret_cast<int*>(smem + sp.tab_floats);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* Fh = smem + 4 * sp.tab_slots + sp.istart_len + warp * sp.per_warp;
+    float* Fh = smem + sp.tab_floats + sp.istart_len + warp * sp.per_warp;
     float* Fl = Fh + sp.half;
-    float* ZS = Fl + sp.half;
-    float* WM = ZS + sp.zs_len;
-    constexpr int U = PRUNE ? SKIP_UNROLL : CERT_UNROLL_SINGLE;
-    int* spill = reinterpret_cast<int*>(WM + sp.wm_len) + lane;
+    constexpr int U = CERT_UNROLL_SINGLE;
+    int* spill = reinterpret_cast<int*>(Fl + sp.half) + lane;
     float* ends = Fh + sp.per_warp - 4;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
-        const float c = (float)(2 * m + 3);
-        tab[m + m / U] = make_float4(r, r, c, c);
+        tab[m + m / U] = make_float4(r, r, (float)(2 * m + 3), (float)(2 * m + 3));
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
@@ -1744,14 +1843,93 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         __syncwarp();
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
         __syncwarp();   // the staged row is visible to every lane
-        if (PRUNE) {
-            end_max<false>(Fh, ZS, it.L, lane);
-            window_max<CERT_POV, U>(Fh, WM, it.L, lane);
-            __syncwarp();
-        }
         const CertRow r = cert_row(sp, it, item, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
-        if constexpr (PRUNE) sweep_row_skip<CERT_POV, U, LONG, false>(sp, r, ZS, WM, tab, spill, lane);
-        else sweep_row_cert<CERT_POV, U, LONG, false, false>(sp, r, tab, spill, lane);
+        sweep_row_cert<CERT_POV, U, LONG, false, false>(sp, r, tab, spill, lane);
+    }
+    if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
+}
+
+// The pruned certified sweep of rows that leave room for a warp's own: a warp
+// stages 2^lgna walks' rows at a time, walked forward.  With lgna = 0 that is
+// one work item (a backward item's row reversed); with more, both walk
+// directions of 2^(lgna - 1) consecutive rows, gathered once and stored in
+// either order.  The groups of all of them share the lanes' queue: a row of
+// 100 samples alone has 25 groups for 32 lanes, and its lanes would wait for
+// the longest walk of every row and for its gathers.  60 tiles of 64 to 256
+// cells a side: 21.6 -> 14.9 ms, 100 x 100: 309 -> 232 us (packs of one row
+// at 20 warps instead of 16: 1000^2 21.9 -> 20.5 ms).  Per warp, shared memory
+// holds the rows' SkipRows and per row [Fh half][Fl half][suffix maxima]
+// [window maxima].
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams sp)
+{
+    extern __shared__ __align__(16) float smem[];
+    float2* tab = reinterpret_cast<float2*>(smem);
+    int* istart = reinterpret_cast<int*>(smem + sp.tab_floats);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int na = 1 << sp.lgna;
+    SkipRow* rows = reinterpret_cast<SkipRow*>(smem + sp.tab_floats + sp.istart_len + warp * sp.per_warp);
+    float* arrays = reinterpret_cast<float*>(rows + na);
+    const int zs_off = 2 * sp.half - ROW_PADL, wm_off = zs_off + sp.zs_len;   // from the hi parts
+    constexpr int U = SKIP_UNROLL;
+    for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
+        const float r = __frcp_rn((float)(m + 1));
+        tab[m + 2 * (m / U)] = make_float2(r, r);
+    }
+    for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
+    __syncthreads();
+    const long long t_start = clock64();
+
+    int next = 0;
+    if (lane == 0) next = (int)atomicAdd(sp.counter, (unsigned)na);
+    next = __shfl_sync(0xffffffffu, next, 0);
+    while (next < sp.total_items) {
+        const int base = next;
+        if (lane == 0) next = (int)atomicAdd(sp.counter, (unsigned)na);
+        next = __shfl_sync(0xffffffffu, next, 0);
+        __syncwarp();
+        int longest = 0;
+        for (int a = 0; a < na; a += 2) {      // items base + a and base + a + 1 are one row, both directions
+            ItemRow it;
+            SkipRow* r = rows + a;
+            if (base + a >= sp.total_items || !decode_item(sp, istart, base + a, &it)) {
+                if (lane == 0) {
+                    r->L = 0;
+                    if (na > 1) r[1].L = 0;
+                }
+                continue;
+            }
+            float* Fh = arrays + a * sp.per_row;
+            float* Fb = Fh + sp.per_row;
+            const bool both = na > 1;
+            const float zmax = stage_row<true>(sp, it, Fh, Fh + sp.half, r->ends, lane, 0, 1, true,
+                                               both ? Fb : nullptr, Fb + sp.half);
+            __syncwarp();   // the staged rows are visible to every lane
+            if (lane == 0) {
+                const bool ok = skip_row(sp, it, base + a, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev, false, r);
+                if (both) {
+                    skip_row(sp, it, base + a + 1, zmax, sp.cv_bwd, true, false, r + 1);
+                    r[1].ends[0] = r->ends[2]; r[1].ends[1] = r->ends[3];
+                    r[1].ends[2] = r->ends[0]; r[1].ends[3] = r->ends[1];
+                }
+                if (!ok) {
+                    r->L = 0;
+                    if (both) r[1].L = 0;
+                }
+            }
+            longest = max(longest, it.L);
+            for (int b = 0; b <= (both ? 1 : 0); ++b) {
+                const float* F = Fh + b * sp.per_row;
+                float* ZS = Fh + b * sp.per_row + 2 * sp.half;
+                end_max<false>(F, ZS, it.L, lane);
+                window_max<CERT_POV, U>(F, ZS + sp.zs_len, it.L, lane);
+            }
+        }
+        __syncwarp();
+        if (longest > 0)
+            sweep_rows_skip<CERT_POV, U, false, false>(sp, rows, arrays + ROW_PADL, sp.lgna,
+                                                       (longest + CERT_POV - 1) / CERT_POV, zs_off, wm_off, tab,
+                                                       nullptr, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
@@ -1770,18 +1948,20 @@ __device__ __forceinline__ void pair_sync(int pair)
 // rows).  Both warps stage half of the row; the forward warp computes its
 // suffix maxima, the backward warp its prefix maxima (pruning).  Each warp
 // runs one direction's code only.  Per pair, shared memory holds [Fh
-// half][Fl half][suffix maxima][prefix maxima][window maxima][ends 4][exchange 4]; per warp
+// half][Fl half][suffix maxima][prefix maxima][window maxima][ends 4][exchange
+// 4][SkipRow per warp]; per warp
 // the long-walk spill.
 template <bool PRUNE, bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
-    float4* tab = reinterpret_cast<float4*>(smem);
-    int* istart = reinterpret_cast<int*>(smem + 4 * sp.tab_slots);
+    using Entry = std::conditional_t<PRUNE, float2, float4>;
+    Entry* tab = reinterpret_cast<Entry*>(smem);
+    int* istart = reinterpret_cast<int*>(smem + sp.tab_floats);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int pair = warp >> 1, bwd = warp & 1;
     const int npairs = blockDim.x >> 6;
-    float* base = smem + 4 * sp.tab_slots + sp.istart_len;
+    float* base = smem + sp.tab_floats + sp.istart_len;
     float* Fh = base + pair * sp.per_pair;
     float* Fl = Fh + sp.half;
     float* ZS = Fl + sp.half + bwd * sp.zs_len;            // this warp's suffix or prefix maxima
@@ -1789,12 +1969,13 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     float* ends = WM + sp.wm_len;                          // 4 floats
     constexpr int U = PRUNE ? SKIP_UNROLL : CERT_UNROLL;
     float* xch = ends + 4;                                   // item number and the halves' zmax
+    SkipRow* row = reinterpret_cast<SkipRow*>(xch + 4) + bwd;   // this warp's view of the row (pruned)
     float* own = base + npairs * sp.per_pair + warp * sp.per_warp;
     int* spill = reinterpret_cast<int*>(own) + lane;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
         const float r = __frcp_rn((float)(m + 1));
-        const float c = (float)(2 * m + 3);
-        tab[m + m / U] = make_float4(r, r, c, c);
+        if constexpr (PRUNE) tab[m + 2 * (m / U)] = make_float2(r, r);
+        else tab[m + m / U] = make_float4(r, r, (float)(2 * m + 3), (float)(2 * m + 3));
     }
     for (int m = threadIdx.x; m <= sp.ndir; m += blockDim.x) istart[m] = sp.item_start[m];
     __syncthreads();
@@ -1818,11 +1999,25 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                 pair_sync(pair);
             }
             const float zmax = fmaxf(xch[1], xch[2]);
-            const CertRow r = cert_row(sp, it, pitem + bwd, Fh, Fl, ends, zmax, bwd ? sp.cv_bwd : sp.cv_fwd, false);
+            int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
             if constexpr (PRUNE) {
-                if (bwd) sweep_row_skip<CERT_POV, U, LONG, true>(sp, r, ZS, WM, tab, spill, lane);
-                else sweep_row_skip<CERT_POV, U, LONG, false>(sp, r, ZS, WM, tab, spill, lane);
+                bool ok = true;
+                if (lane == 0) {
+                    ok = skip_row(sp, it, pitem + bwd, zmax, cv, false, LONG, row);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) row->ends[m] = ends[m];
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                __syncwarp();
+                const float* H = Fh + ROW_PADL;
+                const int groups = ok ? (it.L + CERT_POV - 1) / CERT_POV : 0;
+                const int zs_off = (int)(ZS - H), wm_off = (int)(WM - H);
+                if (bwd)
+                    sweep_rows_skip<CERT_POV, U, LONG, true>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
+                else
+                    sweep_rows_skip<CERT_POV, U, LONG, false>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
             } else {
+                const CertRow r = cert_row(sp, it, pitem + bwd, Fh, Fl, ends, zmax, cv, false);
                 if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
                 else sweep_row_cert<CERT_POV, U, LONG, false, true>(sp, r, tab, spill, lane);
             }
@@ -1902,30 +2097,57 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_scan_kernel(SweepParam
 constexpr int LONG_MIN_WARPS = 2;
 constexpr int MIN_TABLE = 1024;
 
-// Certified one-row-per-warp sweep warps that shared memory holds for rows
-// of up to wmax samples and walks of up to dmax steps in a launch of ndir
-// directions (launch_sweep runs that kernel when the count reaches
-// TVS_CERT_SINGLE_MIN).
-static int wm_entries(int wmax) { return ((wmax + SKIP_UNROLL + 3) / ZS_STRIDE + 4) & ~3; }
+// Shared-memory sizes of a launch (floats), for rows of up to wmax samples and
+// walks of up to dmax steps in a launch of ndir directions.
+struct SweepSizes {
+    int inv_len, tab, istart;   // distance table (entries, floats) and item table
+    int padr, half, zs, wm;     // right pad, one staged array, end maxima, window maxima
+    int row;                    // a packed row's arrays
+    size_t room;                // what the tables leave (0 if they do not fit)
+};
 
-static size_t cert_single_fit(int wmax, int dmax, int prune, int ndir, int smem_optin)
+static SweepSizes sweep_sizes(int wmax, int dmax, bool prune, bool cert, int ndir, int smem_optin)
 {
-    const int inv_len = (std::min(dmax, wmax) + 2 * LARGE_UNROLL + 8 + 1) & ~1;
-    const int tab_slots = tab_slots_for(inv_len, true);
-    const int istart_len = (ndir + 1 + 3) & ~3;
-    const int half = (ROW_PADL + 4 + wmax + ROW_PADR + 3) & ~3;
-    const int zs_len = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
-    const int wm_len = prune ? wm_entries(wmax) : 0;
-    const int single_warp = 2 * half + zs_len + wm_len + 4;
-    const size_t fixed = (size_t)(4 * tab_slots + istart_len) * 4;
-    return fixed >= (size_t)smem_optin ? 0 : ((size_t)smem_optin - fixed) / ((size_t)single_warp * 4);
+    SweepSizes z;
+    // the distance table is read up to d = dmax + U (a walk of at most
+    // min(K, W) - 1 steps, rounded up to U); dmax <= wmax
+    z.inv_len = (std::min(dmax, wmax) + 2 * LARGE_UNROLL + 8 + 1) & ~1;
+    z.tab = tab_floats_for(z.inv_len, prune, cert);
+    z.istart = (ndir + 1 + 3) & ~3;
+    z.padr = prune ? SKIP_PADR : ROW_PADR;
+    z.half = (ROW_PADL + 4 + wmax + z.padr + 3) & ~3;
+    z.zs = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
+    z.wm = prune ? ((wmax + SKIP_UNROLL + 3) / ZS_STRIDE + 4) & ~3 : 0;
+    z.row = 2 * z.half + z.zs + z.wm;
+    const size_t total = (size_t)smem_optin / 4, fixed = (size_t)z.tab + z.istart;
+    z.room = fixed >= total ? 0 : total - fixed;
+    return z;
+}
+
+// Certified warps that hold a row of their own in shared memory (launch_sweep
+// gives them one when there are at least TVS_CERT_SINGLE_MIN, else rows go to
+// pairs of warps).
+static size_t cert_single_fit(const SweepSizes& z, bool prune)
+{
+    return z.room / (size_t)(prune ? SKIP_ROW_FLOATS + z.row : 2 * z.half + 4);
+}
+
+// log2 of the rows that PACK_WARPS warps of a packed launch can each stage.
+static int pack_fit(const SweepSizes& z)
+{
+    int lg = 0;
+    while (lg < PACK_MAX_LG && (size_t)PACK_WARPS * (size_t)(SKIP_ROW_FLOATS + z.row) * (2u << lg) <= z.room) ++lg;
+    return lg;
 }
 
 int cert_sweep_class(int wmax, int dmax, int prune, int ndir, int smem_optin)
 {
     if (wmax - 2 > LONG_WALK && dmax - 1 > LONG_WALK) return 0;
-    const size_t fit = cert_single_fit(wmax, dmax, prune, ndir, smem_optin);
-    return fit >= (size_t)CERT_WIDE_WARPS ? CERT_WIDE_WARPS : fit >= (size_t)TVS_CERT_SINGLE_MIN ? CERT_MAX_WARPS : 0;
+    const SweepSizes z = sweep_sizes(wmax, dmax, prune != 0, true, ndir, smem_optin);
+    const size_t fit = cert_single_fit(z, prune != 0);
+    if (fit < (size_t)TVS_CERT_SINGLE_MIN) return 0;
+    if (fit < (size_t)CERT_WIDE_WARPS) return CERT_MAX_WARPS;
+    return CERT_WIDE_WARPS << (prune ? pack_fit(z) : 0);
 }
 
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
@@ -1934,7 +2156,6 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
                          int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream)
 {
     if (ndir <= 0 || total_items <= 0) return cudaSuccess;
-    constexpr int U = LARGE_UNROLL;
     SweepParams sp;
     sp.dirs = d_dirs; sp.jobs = d_jobs; sp.item_start = d_item_start; sp.rowlo = rowlo;
     sp.rowhi = rowhi; sp.cv_fwd = cv_fwd; sp.cv_bwd = cv_bwd; sp.counter = counter; sp.ndir = ndir;
@@ -1943,35 +2164,46 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     sp.flag_buf = flag_buf;
     sp.flag_count = flag_count;
     sp.flag_cap = flag_buf ? flag_cap : 0;
-    // the distance table is read up to d = dmax + U (a walk of at most
-    // min(K, W) - 1 steps, rounded up to U); dmax <= wmax
-    sp.inv_len = (std::min(dmax, wmax) + 2 * U + 8 + 1) & ~1;
-    const bool skewed = cert || prune;
-    sp.tab_slots = tab_slots_for(sp.inv_len, skewed);
-    sp.istart_len = (ndir + 1 + 3) & ~3;
-    sp.half = (ROW_PADL + 4 + wmax + ROW_PADR + 3) & ~3;
+    const SweepSizes z = sweep_sizes(wmax, dmax, prune != 0, cert != 0, ndir, smem_optin);
+    sp.inv_len = z.inv_len;
+    sp.tab_floats = z.tab;
+    sp.istart_len = z.istart;
+    sp.padr = z.padr;
+    sp.half = z.half;
+    sp.zs_len = z.zs;
+    sp.wm_len = z.wm;
+    sp.per_row = z.row;
+    sp.lgna = 0;
     const bool longw = wmax - 2 > LONG_WALK && dmax - 1 > LONG_WALK;
-    sp.zs_len = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
-    sp.wm_len = prune ? wm_entries(wmax) : 0;
     const int lspill = longw ? 32 * LARGE_POV : 0;
-    // FP32 decisions: one row per warp.  Certified: one row per warp
-    // (reversed for backward walks) when TVS_CERT_SINGLE_MIN such warps fit, else
-    // one row per pair of warps (both staged arrays, suffix and prefix maxima,
-    // the end samples and an exchange slot), and per warp its
-    // flag list and spill: a row's samples are then held once for both walk
-    // directions.
-    const int single_warp = 2 * sp.half + sp.zs_len + sp.wm_len + 4;
-    const size_t single_fit = cert ? cert_single_fit(wmax, dmax, prune, ndir, smem_optin) : 0;
+    // FP32 decisions: one row per warp.  Certified: rows of a warp's own (one,
+    // reversed for backward walks, or when pruned up to 2^PACK_MAX_LG) when
+    // TVS_CERT_SINGLE_MIN such warps fit, else one row per pair of warps (both
+    // staged arrays, the maxima, the end samples, an exchange slot and pruned
+    // each warp's SkipRow), and per warp its spill: a row's samples are then
+    // held once for both walk directions.
+    const size_t single_fit = cert ? cert_single_fit(z, prune != 0) : 0;
     const int single_min = TVS_CERT_SINGLE_MIN;
     const bool single = cert && !longw && (max_warps == 0 || max_warps >= single_min) &&
                         single_fit >= (size_t)single_min;
     const bool pairs = cert && !single;
-    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 8 : 0;
-    sp.per_warp = single ? single_warp : pairs ? lspill : sp.half + sp.zs_len + sp.wm_len + lspill;
+    if (single && prune) {
+        // as many rows as fit, while every warp still finds several packs to
+        // claim: the last packs of a launch run alone (100 x 100, 180
+        // directions: 232 us with at least 3 packs per warp, 255 with 1)
+        const int cap = max_warps == 0 || max_warps >= PACK_WARPS ? pack_fit(z) : 0;
+        while (sp.lgna < cap && (long long)total_items >> (sp.lgna + 1) >=
+                                    (long long)PACK_MIN_CLAIMS * num_sms * PACK_WARPS)
+            ++sp.lgna;
+    }
+    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 8 + (prune ? 2 * SKIP_ROW_FLOATS : 0) : 0;
+    sp.per_warp = single ? (prune ? (SKIP_ROW_FLOATS + z.row) << sp.lgna : 2 * sp.half + 4)
+                : pairs ? lspill
+                        : sp.half + sp.zs_len + sp.wm_len + lspill;
     // shared memory of one unit: a pair of warps or one warp
     const int uw = pairs ? 2 : 1;
     const size_t unit = (size_t)(sp.per_pair + uw * sp.per_warp) * 4;
-    size_t fixed = (size_t)(4 * sp.tab_slots + sp.istart_len) * 4;
+    size_t fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4;
     if (longw && fixed + (size_t)(LONG_MIN_WARPS / uw) * unit > (size_t)smem_optin) {
         // Rows of more than about 10^4 samples: the whole table and several
         // staged rows do not fit together.  Keep LONG_MIN_WARPS warps (or as
@@ -1979,15 +2211,14 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         // entries); the long-walk sweep computes the entries past its end.
         const size_t base = (size_t)sp.istart_len * 4;
         int w = LONG_MIN_WARPS / uw;
-        const size_t min_tab = (size_t)tab_slots_for(MIN_TABLE, skewed) * 16;
+        const size_t min_tab = (size_t)tab_floats_for(MIN_TABLE, prune != 0, cert != 0) * 4;
         while (w > 1 && base + min_tab + (size_t)w * unit > (size_t)smem_optin) --w;
         if (base + 16 * 4 + (size_t)w * unit >= (size_t)smem_optin) return cudaErrorInvalidConfiguration;
-        // slots that fit, and the most entries whose slots do
-        const size_t room = ((size_t)smem_optin - base - (size_t)w * unit) / 16;
-        const size_t fit = skewed ? (room - 2) * TAB_SKEW_MIN / (TAB_SKEW_MIN + 1) : room;
-        sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, fit) & ~1;
-        sp.tab_slots = tab_slots_for(sp.inv_len, skewed);
-        fixed = (size_t)(4 * sp.tab_slots + sp.istart_len) * 4;
+        // floats that fit, and the most entries whose slots do
+        const size_t room = ((size_t)smem_optin - base - (size_t)w * unit) / 16 * 4;
+        sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, tab_entries_fit(room, prune != 0, cert != 0)) & ~1;
+        sp.tab_floats = tab_floats_for(sp.inv_len, prune != 0, cert != 0);
+        fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4;
     }
     if (fixed + unit > (size_t)smem_optin) return cudaErrorInvalidConfiguration;
     // As many resident units as shared memory and registers allow, in one CTA
@@ -1998,9 +2229,9 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     int most;
     if (single) {
         const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = prune ? SKIP_WARPS : wide ? WW : CW;
-        if (prune) kern = sweep_cert_kernel<true, false, SKIP_WARPS>;
-        else kern = wide ? sweep_cert_kernel<false, false, WW> : sweep_cert_kernel<false, false, CW>;
+        most = prune ? PACK_WARPS : wide ? WW : CW;
+        if (prune) kern = sweep_pack_kernel<PACK_WARPS>;
+        else kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
     } else if (pairs) {
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
         most = wide ? WW : prune && !longw ? SKIP_WARPS : CW;

@@ -80,3 +80,17 @@ def test_full_flag_buffer(ctx, rows, cols):
     if rows > 10:
         g = [1.0 + tvs.direction(n, k, rows, cols)["t"] ** 2 for k in range(n)]
         np.testing.assert_allclose(got[20:-20, 20:-20], 8.0 * sum(g) * np.pi / (2 * n) * 100.0, rtol=4e-6)
+
+
+@pytest.mark.parametrize("rows,cols,n,rng", [(33, 41, 1500, 0.0), (64, 97, 720, 0.0), (130, 61, 360, 333.0),
+                                             (5, 300, 500, 0.0), (16, 16, 4096, 45.0), (250, 250, 90, 0.0)])
+@pytest.mark.parametrize("kind", ["fractal", "ridge", "sawtooth"])
+def test_packed_rows(ctx, kind, rows, cols, n, rng):
+    """Launches with enough short rows pack several of them, of both walk
+    directions and across direction boundaries, into a warp: every area equals
+    the unpruned sweep's, which takes one row per warp."""
+    dem = _terrain(kind, rows, cols, 21)
+    got = ctx.total_viewshed(dem, 10.0, 2.5, n, rng)
+    with tvs.Context(0) as c:
+        c.set_tuning(prune=0)
+        np.testing.assert_array_equal(got, c.total_viewshed(dem, 10.0, 2.5, n, rng))
