@@ -635,6 +635,10 @@ __device__ __forceinline__ float sat_pos(float s)
     return v;
 }
 
+// What names a walk's row in the flag buffer: direction (< 4096), skewed row
+// (< 32768) and walk direction.
+__device__ __forceinline__ int row_key(int dir, int p, bool back) { return dir << 16 | p << 1 | (back ? 1 : 0); }
+
 // The measure the sweep writes for a flagged walk that found the flag buffer
 // full: the scan after the exact pass looks for negative measures.
 constexpr int CV_FLAGGED = (int)0x80000000;
@@ -650,13 +654,13 @@ struct CertRow {
     float eg0;           // 2.01u |h0| + |h0 - float(h0)| + 4 eta: the parts of Eg common to the row's groups
     float zmax;          // the row's largest |elevation|
     int* cvrow;
-    int item;            // the row's work item
+    int key;             // row_key of the row's walks
     bool rev_staged;     // the staged row is reversed: staged x is row sample L - 1 - x
 };
 
 // The certified row of a staged item.  eta bounds the staged heights' error,
 // plus h0's split (h0 = float(h0) + h0_lo to 2^-48).
-__device__ __forceinline__ CertRow cert_row(const SweepParams& sp, const ItemRow& it, int item, const float* Fh,
+__device__ __forceinline__ CertRow cert_row(const SweepParams& sp, const ItemRow& it, const float* Fh,
                                             const float* Fl, const float* ends, float zmax, int* cv, bool rev_staged)
 {
     const float eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
@@ -673,7 +677,7 @@ __device__ __forceinline__ CertRow cert_row(const SweepParams& sp, const ItemRow
     r.eg0 = 2.01f * 0x1p-24f * fabsf(it.h0) + fabsf(sp.dirs[it.dir].h0_lo) * 1.0001f + 4.04f * eta;
     r.zmax = zmax;
     r.cvrow = cv + it.rowbase;
-    r.item = item;
+    r.key = row_key(it.dir, it.p, it.rev);
     r.rev_staged = rev_staged;
     return r;
 }
@@ -697,7 +701,7 @@ __device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const Cert
     if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)__popc(fm));
     for (; fm && at < cap; fm &= fm - 1, ++at) {
         const int xs = x0 + __ffs(fm) - 1;   // staged sample; the entry holds the row's
-        sp.flag_buf[at] = make_int4(r.item, r.rev_staged ? r.L - 1 - xs : xs, __float_as_int(r.zmax), 0);
+        sp.flag_buf[at] = make_int4(r.key, r.rev_staged ? r.L - 1 - xs : xs, __float_as_int(r.zmax), 0);
     }
     if (fm) sp.flag_count[2] = 1u;
     return fm;
@@ -714,7 +718,7 @@ static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 // the lanes of a warp may be on different rows).
 struct __align__(16) SkipRow {
     int L, K;
-    int item;            // its work item
+    int key;             // row_key of its walks
     int rev;             // staged x is row sample L - 1 - x
     float ends[4];       // hi and lo parts of the first and of the last sample (sentinels when staged)
     float h0;
@@ -743,20 +747,21 @@ __device__ __forceinline__ bool flag_block(const SweepParams& sp, const SkipRow&
     unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
     if (at < cap) at = atomicAdd(sp.flag_count, 1u);
     if (at >= cap) return false;
-    sp.flag_buf[at] = make_int4(r.item, (r.rev ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax), e0 | p0 << 14);
+    sp.flag_buf[at] = make_int4(r.key, (r.rev ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax), e0 | p0 << 14);
     return true;
 }
 
-// Fills a staged item's row (the ends are there already); false when a walk of
+// Fills a staged row's SkipRow (the ends are there already), walked backward
+// with `back`, staged reversed with `rev`; false when a walk of
 // the row could leave its arrays or the distance table (windows start at most
 // SKIP_UNROLL samples before the row and end before sample L + P + U).
-__device__ __forceinline__ bool skip_row(const SweepParams& sp, const ItemRow& it, int item, float zmax, int* cv,
+__device__ __forceinline__ bool skip_row(const SweepParams& sp, const ItemRow& it, bool back, float zmax, int* cv,
                                          bool rev, bool longw, SkipRow* r)
 {
     const float eta = 0x1p-42f * (zmax + fabsf(it.h0)) + 0x1p-126f;
     r->L = it.L;
     r->K = it.K;
-    r->item = item;
+    r->key = row_key(it.dir, it.p, back);
     r->rev = rev;
     r->h0 = it.h0;
     r->eg0 = 2.01f * 0x1p-24f * fabsf(it.h0) + fabsf(sp.dirs[it.dir].h0_lo) * 1.0001f + 4.04f * eta;
@@ -986,8 +991,9 @@ __device__ __forceinline__ int df_walk(const ExactCtx& c, int x, int a0, int a1,
     return warp_sum(acc);
 }
 
-// Exact measure of POV x of the row, written by lane 0.
-__device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
+// Exact measure of POV x of the row, written by lane 0.  count[0] and count[1]
+// are the warp's exact and FP64 walks so far.
+__device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane, unsigned* count)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
     int cv;
@@ -997,10 +1003,8 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
         bool esc = false;
         const int s = df_walk<XW_KPL>(c, x, 0, 0, 0, n - 1, lane, &esc);
         cv = 1 + (esc ? fp64_walk(c, x, 0, n - 1, lane) : s);
-        if (lane == 0) {
-            atomicAdd(&g_sweep_stats[0], 1ull);
-            if (esc) atomicAdd(&g_sweep_stats[1], 1ull);
-        }
+        ++count[0];
+        if (esc) ++count[1];
     }
     if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
 }
@@ -1008,7 +1012,8 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane)
 // Adds to POV x's measure what the targets of block e0 (U steps) add, decided
 // exactly; kind and p0 as in the flag entry.
 template <int U>
-__device__ __forceinline__ void exact_block(const ExactCtx& c, int x, int e0, int p0, int kind, int lane)
+__device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int p0, int kind, int lane,
+                                         unsigned* count)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
     const int last = min(n - 1, e0 + U);
@@ -1017,11 +1022,78 @@ __device__ __forceinline__ void exact_block(const ExactCtx& c, int x, int e0, in
     const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, 0, e0, e0, last, lane, &esc)
                                       : df_walk<1>(c, x, p0, min(p0 + U, e0), e0, last, lane, &esc);
     const int add = esc ? fp64_walk(c, x, e0, last, lane) : s;
-    if (lane == 0 && in_range(x, c.L, 14)) {
-        if (add) atomicAdd(c.cvrow + x, add);
-        atomicAdd(&g_sweep_stats[0], 1ull);
-        if (esc) atomicAdd(&g_sweep_stats[1], 1ull);
+    if (lane == 0 && in_range(x, c.L, 14) && add) atomicAdd(c.cvrow + x, add);
+    ++count[0];
+    if (esc) ++count[1];
+}
+
+// The same for one FLAG_BLOCK entry per half-warp (h: the lane's place in its
+// half; valid: the half has an entry): one target of the earlier block and one
+// of the flagged block per lane.  The maximum of the earlier block is one of
+// its near-tied largest slopes, so its error is taken at that block's first
+// distance.  Returns whether the half's decisions need the FP64 walk (nothing
+// is added then).
+template <int U>
+__device__ __forceinline__ bool exact_half(const ExactCtx& c, bool valid, int x, int e0, int p0, int lane)
+{
+    static_assert(U <= 16, "a lane per target");
+    const unsigned FULL = 0xffffffffu;
+    const float NEG = neg_inf();
+    const int h = lane & 15, dir = c.bwd ? -1 : 1;
+    int da = 0, db = 0;
+    if (valid) {
+        const int last = min(min(c.bwd ? x : c.L - 1 - x, c.K) - 1, e0 + U);
+        if (p0 + 1 + h <= min(p0 + U, e0)) da = p0 + 1 + h;
+        if (e0 + 1 + h <= last) db = e0 + 1 + h;
     }
+    float ah = NEG, al = 0.f, bh = NEG, bl = 0.f, iv = 1.f;
+    if (valid) {
+        float zh, zl, hh, hl, s, e;
+        dem_hl(c, x, zh, zl);
+        df::two_sum(zh, c.h0h, s, e);
+        e = __fadd_rn(e, __fadd_rn(zl, c.h0l));
+        df::two_sum(s, e, hh, hl);
+        if (da) {
+            dem_hl(c, x + dir * da, zh, zl);
+            df::df_slope(zh, zl, hh, hl, da, ah, al);
+        }
+        if (db) {
+            iv = __frcp_rn((float)db);
+            dem_hl(c, x + dir * db, zh, zl);
+            df::df_slope_iv(zh, zl, hh, hl, db, iv, bh, bl);
+        }
+    }
+    // the maximum before the block, and before each of its targets
+    float ph = bh, pl = bl;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const float qh = __shfl_xor_sync(FULL, ah, o), ql = __shfl_xor_sync(FULL, al, o);
+        if (df::df_gt(qh, ql, ah, al)) { ah = qh; al = ql; }
+        const float rh = __shfl_up_sync(FULL, ph, o, 16), rl = __shfl_up_sync(FULL, pl, o, 16);
+        if (h >= o && df::df_gt(rh, rl, ph, pl)) { ph = rh; pl = rl; }
+    }
+    float ch = __shfl_up_sync(FULL, ph, 1, 16), cl = __shfl_up_sync(FULL, pl, 1, 16);
+    if (h == 0 || df::df_gt(ah, al, ch, cl)) { ch = ah; cl = al; }
+    bool esc = false;
+    int add = 0;
+    if (db) {
+        bool v = true;                       // the first target (no earlier one) is visible
+        if (ch > NEG) {
+            float s, e;
+            df::two_sum(bh, -ch, s, e);
+            const float dh = __fadd_rn(s, __fadd_rn(e, __fsub_rn(bl, cl)));
+            const float marg = __fmaf_rn(0x1p-40f, fabsf(bh) + fabsf(ch),
+                                         4.04f * c.eta * (iv + __frcp_rn((float)(p0 + 1)))) + 0x1p-120f;
+            esc = !(fabsf(dh) > marg);
+            v = dh > 0.f;
+        }
+        if (v) add = 2 * db + 1;
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) add += __shfl_xor_sync(FULL, add, o);
+    const bool any = (__ballot_sync(FULL, esc) >> (lane & 16) & 0xffffu) != 0u;
+    if (valid && !any && h == 0 && add && in_range(x, c.L, 14)) atomicAdd(c.cvrow + x, add);
+    return any;
 }
 
 // min(a, |b|, |c|).  TVS_CERT_MIN3 selects the three-input minimum of
@@ -1843,7 +1915,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         __syncwarp();
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
         __syncwarp();   // the staged row is visible to every lane
-        const CertRow r = cert_row(sp, it, item, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
+        const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
         sweep_row_cert<CERT_POV, U, LONG, false, false>(sp, r, tab, spill, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
@@ -1906,9 +1978,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
                                                both ? Fb : nullptr, Fb + sp.half);
             __syncwarp();   // the staged rows are visible to every lane
             if (lane == 0) {
-                const bool ok = skip_row(sp, it, base + a, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev, false, r);
+                const bool ok = skip_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev, false, r);
                 if (both) {
-                    skip_row(sp, it, base + a + 1, zmax, sp.cv_bwd, true, false, r + 1);
+                    skip_row(sp, it, true, zmax, sp.cv_bwd, true, false, r + 1);
                     r[1].ends[0] = r->ends[2]; r[1].ends[1] = r->ends[3];
                     r[1].ends[2] = r->ends[0]; r[1].ends[3] = r->ends[1];
                 }
@@ -2003,7 +2075,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
             if constexpr (PRUNE) {
                 bool ok = true;
                 if (lane == 0) {
-                    ok = skip_row(sp, it, pitem + bwd, zmax, cv, false, LONG, row);
+                    ok = skip_row(sp, it, bwd != 0, zmax, cv, false, LONG, row);
 #pragma unroll
                     for (int m = 0; m < 4; ++m) row->ends[m] = ends[m];
                 }
@@ -2017,7 +2089,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                 else
                     sweep_rows_skip<CERT_POV, U, LONG, false>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
             } else {
-                const CertRow r = cert_row(sp, it, pitem + bwd, Fh, Fl, ends, zmax, cv, false);
+                const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, cv, false);
                 if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
                 else sweep_row_cert<CERT_POV, U, LONG, false, true>(sp, r, tab, spill, lane);
             }
@@ -2027,12 +2099,17 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
 
-// The exact pass of a certified launch: every walk the sweep flagged and
-// handed over (an (item, sample, row |elevation| bound) entry of the flag
-// buffer) is walked again exactly (double-float, FP64 past its margin) by one
-// warp, which blends the walk's samples from the DEM as the staging does
-// (the DEM is L2-resident while the sweep runs).  Warps claim one entry at a
-// time; flag_count[0] is the buffer's fill, flag_count[1] the claim counter.
+// The exact pass of a certified launch: every walk or block the sweep flagged
+// (a row key, the sample and its entry's kind, the row's |elevation| bound and
+// the blocks) is decided again exactly, double-float or FP64 past its margin,
+// on samples blended from the DEM as the staging does (the DEM is L2-resident
+// while the sweep runs).  Bound by the latency of those gathers.  A warp takes
+// two entries at a time: two FLAG_BLOCK entries in one go, a half-warp each,
+// what else there is (whole walks, walks with an earlier flagged block, FP64)
+// with all 32 lanes.  An entry names its row directly (no search of the item
+// table) and the counters stay in registers: 12 mixed tiles (7.3 million
+// blocks) 214 -> 204 ms, 2000^2 (1.26 million) 95.5 -> 92.6 ms.
+// flag_count[0] is the buffer's fill.
 constexpr int EXACT_WARPS = 16;
 
 __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
@@ -2040,18 +2117,44 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
     const int lane = threadIdx.x & 31;
     const unsigned n = min(sp.flag_count[0], (unsigned)sp.flag_cap);
     const long long t_start = clock64();
-    for (unsigned i = blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * EXACT_WARPS) {
-        const int4 en = sp.flag_buf[i];
-        if (!in_range(en.x, sp.total_items, 22)) continue;
+    unsigned count[2] = {0u, 0u};
+    for (unsigned i = 2 * (blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5)); i < n; i += 2 * gridDim.x * EXACT_WARPS) {
+        const unsigned at = i + (lane >> 4);
+        int4 en = make_int4(0, 0, 0, 0);
         ItemRow it;
-        if (!decode_item(sp, sp.item_start, en.x, &it)) continue;
-        const int x = en.y & 0xffff, kind = en.y >> 16;
-        if (!in_range(x, it.L, 23)) continue;
-        const ExactCtx xc = exact_ctx(sp, it, __int_as_float(en.z));
-        if (kind == FLAG_WALK) exact_walk(xc, x, lane);
-        else exact_block<SKIP_UNROLL>(xc, x, en.w & 0x3fff, en.w >> 14, kind, lane);
+        bool ok = at < n;
+        if (ok) {
+            en = sp.flag_buf[at];
+            ok = in_range(en.x >> 16, sp.ndir, 22) && in_range(en.x >> 1 & 0x7fff, sp.dirs[en.x >> 16].R, 24) &&
+                 decode_row(sp, en.x >> 16, en.x >> 1 & 0x7fff, (en.x & 1) != 0, &it) &&
+                 in_range(en.y & 0xffff, it.L, 23);
+        }
+        ExactCtx c{};
+        if (ok) c = exact_ctx(sp, it, __int_as_float(en.z));
+        const int x = en.y & 0xffff, kind = en.y >> 16, e0 = en.w & 0x3fff, p0 = en.w >> 14;
+        const bool half = ok && kind == FLAG_BLOCK;
+        bool left = ok;                       // the half's entry is still to do
+        if (__any_sync(0xffffffffu, half)) {
+            const bool esc = exact_half<SKIP_UNROLL>(c, half, x, e0, p0, lane);
+            if (half && !esc) left = false;
+            count[0] += __popc(__ballot_sync(0xffffffffu, half && !esc) & 0x00010001u);
+        }
+        const unsigned todo = __ballot_sync(0xffffffffu, left) & 0x00010001u;
+        for (unsigned m = todo; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const int key = __shfl_sync(0xffffffffu, en.x, src), y = __shfl_sync(0xffffffffu, en.y, src);
+            const int z = __shfl_sync(0xffffffffu, en.z, src), w = __shfl_sync(0xffffffffu, en.w, src);
+            decode_row(sp, key >> 16, key >> 1 & 0x7fff, (key & 1) != 0, &it);
+            const ExactCtx cc = exact_ctx(sp, it, __int_as_float(z));
+            if (y >> 16 == FLAG_WALK) exact_walk(cc, y & 0xffff, lane, count);
+            else exact_block<SKIP_UNROLL>(cc, y & 0xffff, w & 0x3fff, w >> 14, y >> 16, lane, count);
+        }
     }
-    if (lane == 0) atomicAdd(&g_sweep_stats[2], (unsigned long long)(clock64() - t_start));
+    if (lane == 0) {
+        if (count[0]) atomicAdd(&g_sweep_stats[0], (unsigned long long)count[0]);
+        if (count[1]) atomicAdd(&g_sweep_stats[1], (unsigned long long)count[1]);
+        atomicAdd(&g_sweep_stats[2], (unsigned long long)(clock64() - t_start));
+    }
 }
 
 // The walks that found the flag buffer full: their measures are negative.
@@ -2062,6 +2165,7 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_scan_kernel(SweepParam
     if (sp.flag_count[2] == 0u) return;
     const int lane = threadIdx.x & 31;
     const long long step = (long long)gridDim.x * EXACT_WARPS;
+    unsigned count[2] = {0u, 0u};
     for (long long item = (long long)blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); item < sp.total_items;
          item += step) {
         ItemRow it;
@@ -2085,8 +2189,12 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_scan_kernel(SweepParam
                 for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
                 xc = exact_ctx(sp, it, zmax);
             }
-            for (; marked; marked &= marked - 1) exact_walk(xc, x0 + __ffs(marked) - 1, lane);
+            for (; marked; marked &= marked - 1) exact_walk(xc, x0 + __ffs(marked) - 1, lane, count);
         }
+    }
+    if (lane == 0) {
+        if (count[0]) atomicAdd(&g_sweep_stats[0], (unsigned long long)count[0]);
+        if (count[1]) atomicAdd(&g_sweep_stats[1], (unsigned long long)count[1]);
     }
 }
 
