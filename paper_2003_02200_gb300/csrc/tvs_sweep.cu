@@ -545,10 +545,18 @@ constexpr int SKIP_READY = TVS_SKIP_READY;   // lanes with a block before a prun
 #define TVS_SKIP_RESTART 4
 #endif
 constexpr int SKIP_RESTART = TVS_SKIP_RESTART;   // finished lanes before a pruned walk replaces groups
+// Blocks a searching lane tests at a time: on long rows most tests pass and
+// their latency is shared by more of them, on packed short rows few blocks
+// are left (2000^2 89.1 ms with 4, 88.0 with 6; 60 small tiles 14.7 with 3,
+// 15.0 with 4, 15.3 with 6).
 #ifndef TVS_SKIP_TESTS
-#define TVS_SKIP_TESTS 4
+#define TVS_SKIP_TESTS 6
 #endif
-constexpr int SKIP_TESTS = TVS_SKIP_TESTS;       // blocks a searching lane tests at a time
+#ifndef TVS_PACK_TESTS
+#define TVS_PACK_TESTS 3
+#endif
+constexpr int SKIP_TESTS = TVS_SKIP_TESTS;
+constexpr int PACK_TESTS = TVS_PACK_TESTS;
 #ifndef TVS_SKIP_CHUNK
 #define TVS_SKIP_CHUNK 8
 #endif
@@ -562,10 +570,16 @@ constexpr int SKIP_PADR = CERT_POV + TVS_SKIP_UNROLL + 8;
 #define TVS_SKIP_WARPS 16
 #endif
 constexpr int SKIP_WARPS = TVS_SKIP_WARPS;       // most warps of a pruned certified CTA of warp pairs
-#ifndef TVS_PACK_WARPS
-#define TVS_PACK_WARPS 20
+// and of rows of a warp's own: 20 when each warp holds one (1000^2 20.5 ms with
+// 16), 16 when that leaves room for two or more (60 small tiles 15.0 ms with
+// 20 warps, 14.5 with 16 and more rows in each).
+#ifndef TVS_SINGLE_WARPS
+#define TVS_SINGLE_WARPS 20
 #endif
-constexpr int PACK_WARPS = TVS_PACK_WARPS;       // and of packed rows
+#ifndef TVS_PACK_WARPS
+#define TVS_PACK_WARPS 16
+#endif
+constexpr int SINGLE_WARPS = TVS_SINGLE_WARPS, PACK_WARPS = TVS_PACK_WARPS;
 constexpr int SKIP_UNROLL = TVS_SKIP_UNROLL;   // steps per block of a pruned walk
 static_assert(SKIP_UNROLL <= ROW_PADL && CERT_POV + SKIP_UNROLL <= ROW_PADR && FLUSH_STEPS % SKIP_UNROLL == 0,
               "pads and flushes of a pruned walk");
@@ -1353,19 +1367,31 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
 #undef CERT_NG
 }
 
-// One round of a searching lane: tests SKIP_TESTS blocks from step e on
+// min(a, b, c), one instruction; a NaN is dropped.
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Floats that a search may read past the last row's window maxima.
+constexpr int WM_SLACK = std::max(SKIP_TESTS, PACK_TESTS) * SKIP_UNROLL / ZS_STRIDE;
+
+// One round of a searching lane: tests NT blocks from step e on
 // against the lines T d + K of its four POVs (see sweep_row_skip) and returns
 // the first step that may hold a visible target (*ready), the walk's end when
 // no remaining target can be visible, or the step after the tested blocks.
-// x0 and e are multiples of 4.
-template <int U, bool BWD>
+// x0 and e are multiples of 4.  Blocks past the walk's end are tested against
+// what lies up to WM_SLACK entries past the window maxima (or before them,
+// walking backward: the end maxima); whatever the outcome, e is then past the
+// end and the walk is over.
+template <int U, bool BWD, int NT>
 __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, bool rising, int x0, int e, int dlim,
-                                           int wlast, const float* __restrict__ WM, const float* __restrict__ ZS,
+                                           const float* __restrict__ WM, const float* __restrict__ ZS,
                                            bool* ready)
 {
-    constexpr int NT = SKIP_TESTS;
     const float d = (float)(e + 1);
-    // the entries of blocks past the walk's end are not used
     const int w0 = (BWD ? x0 - e : x0 + e + U) / ZS_STRIDE;
     float lim[NT], wm[NT];
 #pragma unroll
@@ -1373,8 +1399,8 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
         const float dk = d + (float)(k * U);
         const float2 l0 = __ffma2_rn(T2[0], make_float2(dk, dk), K2[0]);
         const float2 l1 = __ffma2_rn(T2[1], make_float2(dk, dk), K2[1]);
-        lim[k] = fminf(fminf(l0.x, l0.y), fminf(l1.x, l1.y));
-        wm[k] = WM[BWD ? max(w0 - k * U / ZS_STRIDE, 0) : min(w0 + k * U / ZS_STRIDE, wlast)];
+        lim[k] = min3(fminf(l0.x, l0.y), l1.x, l1.y);
+        wm[k] = WM[BWD ? w0 - k * U / ZS_STRIDE : w0 + k * U / ZS_STRIDE];
     }
     const float end = ZS[(BWD ? x0 - e : x0 + e) / ZS_STRIDE];
     int n = NT;
@@ -1414,23 +1440,24 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // A POV with no target that adds area has M = +inf and thr NaN, which the
 // minimum drops.
 //
-// Measured (sweep and exact pass, against the walk that only stopped): 2000^2
-// 196 -> 102 ms, 1000^2 31.8 -> 21.3 ms.  Bound by instruction latency: with 3
-// warps per scheduler half of the issue slots stayed empty, so the kernel
-// keeps no exact walks of its own (their context cost 200 bytes of local
-// memory per lane) and fits 16 warps in 128 registers (12 warps: 118 ms, 20
-// with spills: 127).
+// Measured (whole maps, against the walk that only stopped): 2000^2 199 ->
+// 88.0 ms, 1000^2 32.7 -> 19.4 ms.  Bound by the FMA and ALU pipes and by what
+// the lanes wait for each other (22 of 32 active, issue slots 67 to 75 %
+// used): registers decide how many warps hide the tests' latency, so the
+// kernels keep no exact walks of their own (their context cost 200 bytes of
+// local memory per lane; 16 warps then lost to 12), form the window as they
+// go, and treat the inner groups of a row apart from its ends (92.6 -> 89.1).
 //
 // Work is done in three warp-wide phases, each with as many lanes as possible:
 // finished groups are written and replaced (SKIP_RESTART lanes at a time, or
-// when no lane has work); lanes without a block test SKIP_TESTS blocks at a
+// when no lane has work); lanes without a block test NT blocks at a
 // time until SKIP_READY lanes have one or nobody is searching; the lanes that
 // have one evaluate it.  A lane waits while others search or restart, so the
 // thresholds trade idle lanes against phases run for a few lanes only.  A
 // block is evaluated SKIP_CHUNK steps at a time, with the window formed as it
 // goes: the few registers that takes let 20 warps share an SM, and their
 // number is what hides the latency of the tests.
-template <int P, int U, bool LONG, bool BWD>
+template <int P, int U, bool LONG, bool BWD, int NT>
 __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const SkipRow* __restrict__ rows,
                                                 const float* H0, int lgna, int groups, int zs_off, int wm_off,
                                                 const float2* __restrict__ tab, int* __restrict__ spill, int lane)
@@ -1444,7 +1471,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
     const SkipRow* r = rows;
     const float* H = H0;             // its hi parts; lo parts, end and window maxima at fixed offsets
     constexpr bool PACK = !BWD && TVS_CERT_PACKADD;
-    float ia[P];
+    float2 ia2[P / 2];
     float2 ng2[P / 2];               // -g of POV pairs
     float2 M2[P / 2], acc2[P / 2];   // running maxima and measures of POV pairs
     float2 T2[P / 2], K2[P / 2];     // thr and k of POV pairs
@@ -1463,64 +1490,74 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
         r = rows + (task & ((1 << lgna) - 1));
         H = H0 + (task & ((1 << lgna) - 1)) * sp.per_row;
         const int L = r->L, gi = task >> lgna, G = (L + P - 1) / P;
-        const float* Lo = H + sp.half;
         x0 = (BWD ? G - 1 - gi : gi) * P;
-        if (gi >= G) { x0 = L; e = 0; dlim = -1; return; }   // a shorter row of the pack
+        e = 0;
+        dlim = -1;
+        lost = again = 0u;
+        if (gi >= G) { x0 = L; return; }                     // a shorter row of the pack
         const int klim = r->K - 1;
         const int xl = BWD ? min(x0 + P - 1, L - 1) : x0;
         const int rowlim = BWD ? xl - 1 : L - 2 - xl;
         dlim = min(klim, rowlim);
         klimited = klim < rowlim;
-        e = 0;
         seg = FLUSH_STEPS;
-        lost = again = 0u;
 #pragma unroll
-        for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
+        for (int q = 0; q < P / 2; ++q) {
+            acc2[q] = make_float2(0.f, 0.f);
+            ia2[q] = make_float2(1.f, 1.f);
+        }
         if (LONG) {
 #pragma unroll
             for (int q = 0; q < P; ++q) spill[32 * q] = 0;
         }
         if (dlim < 1) return;
         ready = true;                                        // the first block is always evaluated
-        // the group's samples in POV order, and each POV's first target
-        const float4 a = *reinterpret_cast<const float4*>(H + x0), b = *reinterpret_cast<const float4*>(Lo + x0);
-        const int xt = BWD ? x0 - 1 : x0 + P;                // POV P - 1's first target
-        const float th = H[xt], tl = Lo[xt];
-        const float zs[P + 1] = {BWD ? a.w : a.x, BWD ? a.z : a.y, BWD ? a.y : a.z, BWD ? a.x : a.w, th};
-        const float ls[P + 1] = {BWD ? b.w : b.x, BWD ? b.z : b.y, BWD ? b.y : b.z, BWD ? b.x : b.w, tl};
-        float zh[P], zl[P];
-#pragma unroll
-        for (int q = 0; q < P; ++q) { zh[q] = zs[q]; zl[q] = ls[q]; }
-        if (x0 == 0) {                                       // the row's end samples are sentinels when staged
-            zh[BWD ? P - 1 : 0] = r->ends[0];
-            zl[BWD ? P - 1 : 0] = r->ends[1];
+        // the group's samples and its last POV's first target, relative to R
+        const float4 a = *reinterpret_cast<const float4*>(H + x0);
+        const float4 b = *reinterpret_cast<const float4*>(H + sp.half + x0);
+        const float* ht = H + (BWD ? x0 - 1 : x0 + P);
+        // all but a row's first and last groups stand on samples staged as
+        // they are, and all of their POVs see targets that add area
+        const bool inner = x0 > 0 && x0 + P <= L - 2;
+        Rh = a.x;
+        if (!inner) {                                        // the row's end samples are sentinels when staged
+            if (x0 == 0) Rh = r->ends[0];
+            else if (x0 == L - 1) Rh = r->ends[2];
         }
-        if (x0 + P >= L) {
-#pragma unroll
-            for (int q = 0; q < P; ++q)
-                if (pov_x(q) == L - 1) { zh[q] = r->ends[2]; zl[q] = r->ends[3]; }
-        }
-        Rh = zh[BWD ? P - 1 : 0];
-        float gq[P], gmax = 0.f;
+        const float2 nRh = make_float2(-Rh, -Rh);
+        const float2 y0 = __fadd2_rn(__fadd2_rn(make_float2(a.x, a.y), nRh), make_float2(b.x, b.y));
+        const float2 y1 = __fadd2_rn(__fadd2_rn(make_float2(a.z, a.w), nRh), make_float2(b.z, b.w));
+        const float yt = __fadd_rn(__fsub_rn(ht[0], Rh), ht[sp.half]);
+        const float ys[P + 1] = {BWD ? y1.y : y0.x, BWD ? y1.x : y0.y, BWD ? y0.y : y1.x, BWD ? y0.x : y1.y, yt};
+        const float4 rh = *reinterpret_cast<const float4*>(&r->h0);   // h0, eg0, zmax
+        float gq[P];
+        bool area[P];
 #pragma unroll
         for (int q = 0; q < P; ++q) {
-            const int x = pov_x(q);
-            const bool pov = BWD ? (x >= 1 && x <= L - 1) : x <= L - 2;   // POVs with a target
-            gq[q] = pov ? __fadd_rn(__fadd_rn(__fsub_rn(zh[q], Rh), zl[q]), r->h0) : 0.f;
-            gmax = fmaxf(gmax, fabsf(gq[q]));
+            gq[q] = __fadd_rn(ys[q], rh.x);
+            area[q] = true;
         }
-        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, r->eg0);
-        level = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, r->zmax, gmax), __fmul_rn(2.f, c2e)));
+        if (!inner) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int x = pov_x(q);
+                if (x == 0) gq[q] = __fadd_rn(__fadd_rn(__fsub_rn(r->ends[0], Rh), r->ends[1]), rh.x);
+                if (x == L - 1) gq[q] = __fadd_rn(__fadd_rn(__fsub_rn(r->ends[2], Rh), r->ends[3]), rh.x);
+                if (!(BWD ? (x >= 1 && x <= L - 1) : x <= L - 2)) gq[q] = 0.f;   // no target
+                area[q] = BWD ? (x >= 2 && x <= L - 1) : x <= L - 3;
+            }
+        }
+        const float gmax = fmaxf(fmaxf(fabsf(gq[0]), fabsf(gq[1])), fmaxf(fabsf(gq[2]), fabsf(gq[3])));
+        c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, rh.y);
+        level = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, rh.z, gmax), __fmul_rn(2.f, c2e)));
+        const float c0 = __fmaf_rn(4.f, c2e, 0x1p-16f);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             // as sweep_row_cert: M starts just below the first target's slope
-            const int x = pov_x(q);
-            const float x1 = __fsub_rn(__fadd_rn(__fsub_rn(zs[q + 1], Rh), ls[q + 1]), gq[q]);
-            const float C = __fmaf_rn(0x1p-6f, fabsf(x1), __fmaf_rn(4.f, c2e, 0x1p-16f));
-            const bool area = BWD ? (x >= 2 && x <= L - 1) : x <= L - 3;
+            const float x1 = __fsub_rn(ys[q + 1], gq[q]);
+            const float m = area[q] ? __fsub_rn(x1, __fmaf_rn(0x1p-6f, fabsf(x1), c0)) : pos_inf();
             (q % 2 ? ng2[q / 2].y : ng2[q / 2].x) = -gq[q];
-            (q % 2 ? M2[q / 2].y : M2[q / 2].x) = area ? __fsub_rn(x1, C) : pos_inf();
-            ia[q] = 1.f;
+            (q % 2 ? M2[q / 2].y : M2[q / 2].x) = m;
         }
     };
     if (tasks == 0) return;
@@ -1535,14 +1572,26 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                 const int L = r->L, K = r->K;
                 int* cvrow = r->cv;
                 const bool rev = r->rev != 0;
-                if (lost) sp.flag_count[2] = 1u;
+                int add[P];                                  // by sample
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
+                    const int i = BWD ? P - 1 - q : q;
+                    add[i] = (int)(q % 2 ? acc2[q / 2].y : acc2[q / 2].x) + (LONG ? spill[32 * q] : 0);
+                }
+                if (dlim >= 1 && x0 > 0 && x0 + P <= L - 2 && !lost) {
+                    // every POV has a target
+                    int* at = cvrow + (rev ? L - 1 - x0 : x0);
+                    const int st = rev ? -1 : 1;
+#pragma unroll
+                    for (int i = 0; i < P; ++i, at += st) *at = 1 + add[i];
+                } else
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    if (q == 0 && lost) sp.flag_count[2] = 1u;
                     const int x = pov_x(q);
                     if (x >= L) continue;
-                    const float s = q % 2 ? acc2[q / 2].y : acc2[q / 2].x;
                     const int n = min(BWD ? x : L - 1 - x, K);
-                    const int cv = n >= 1 ? 1 + (int)s + (LONG ? spill[32 * q] : 0) : 0;
+                    const int cv = n >= 1 ? 1 + add[BWD ? P - 1 - q : q] : 0;
                     cvrow[rev ? L - 1 - x : x] = (lost >> q) & 1u ? CV_FLAGGED : cv;
                 }
                 const int task = next + __popc(need & below);
@@ -1555,7 +1604,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
         // 2. lanes without a block look for one
         for (;;) {
             if (has && !ready && e < dlim)
-                e = skip_blocks<U, BWD>(T2, K2, rising, x0, e, dlim, sp.wm_len - 1, H + wm_off, H + zs_off, &ready);
+                e = skip_blocks<U, BWD, NT>(T2, K2, rising, x0, e, dlim, H + wm_off, H + zs_off, &ready);
             const unsigned have = __ballot_sync(FULL, ready);
             const unsigned look = __ballot_sync(FULL, has && !ready && e < dlim);
             if (!look || __popc(have) >= SKIP_READY) break;
@@ -1576,14 +1625,14 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
             const bool far = LONG && e + U > tabn;
             const float2* __restrict__ tb = tab + e + 2 * (e / U);
             const float ive = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tb->x;
-            float Ms[P], mn[P];
+            float mn[P];
+            float2 Ms2[P / 2];
             float2 blk2[P / 2];      // the block's share of the measures
 #pragma unroll
-            for (int q = 0; q < P / 2; ++q) blk2[q] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < P; ++q) {
-                Ms[q] = q % 2 ? M2[q / 2].y : M2[q / 2].x;
-                mn[q] = pos_inf();
+            for (int q = 0; q < P / 2; ++q) {
+                blk2[q] = make_float2(0.f, 0.f);
+                Ms2[q] = M2[q];
+                mn[2 * q] = mn[2 * q + 1] = pos_inf();
             }
             {
                 // the window relative to R, y[m] = sample m of the block's
@@ -1621,41 +1670,41 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
             }
             // the margin test of sweep_row_cert, and the lines of the next tests
             const float ce = __fmaf_rn(c2e, ive, CERT_FLOOR);
-            rising = true;
-            unsigned fm = 0u;
-            float dqs[P];
+            float2 dq2[P / 2], ex2[P / 2];               // delta, and mn - delta
 #pragma unroll
-            for (int q = 0; q < P; ++q) {
-                const float m = q % 2 ? M2[q / 2].y : M2[q / 2].x;
-                dqs[q] = __fmaf_rn(CERT_REL, fmaxf(fabsf(Ms[q]), fabsf(m)), __fmaf_rn(c2e, ia[q], ce));
-                fm |= mn[q] < dqs[q] ? 1u << q : 0u;
+            for (int q = 0; q < P / 2; ++q) {
+                const float2 mb = make_float2(fmaxf(fabsf(Ms2[q].x), fabsf(M2[q].x)),
+                                              fmaxf(fabsf(Ms2[q].y), fabsf(M2[q].y)));
+                dq2[q] = __ffma2_rn(make_float2(CERT_REL, CERT_REL), mb,
+                                    __ffma2_rn(make_float2(c2e, c2e), ia2[q], make_float2(ce, ce)));
+                ex2[q] = __ffma2_rn(make_float2(-1.f, -1.f), dq2[q], make_float2(mn[2 * q], mn[2 * q + 1]));
             }
-            if (fm) {
+            unsigned fm = 0u;
+            if (min3(fminf(ex2[0].x, ex2[0].y), ex2[1].x, ex2[1].y) < 0.f) {
                 // flagged POVs leave the block to the exact pass
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
-                    if (!((fm >> q) & 1u)) continue;
+                    if (!((q % 2 ? ex2[q / 2].y : ex2[q / 2].x) < 0.f)) continue;
+                    fm |= 1u << q;
                     (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
-                    const int p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
+                    const int p0 = __float2int_rn(__frcp_rn(q % 2 ? ia2[q / 2].y : ia2[q / 2].x)) - 1;
                     if (!flag_block(sp, *r, pov_x(q), e, p0, (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
                 }
                 again |= fm;
             }
 #pragma unroll
-            for (int q = 0; q < P / 2; ++q) acc2[q] = __fadd2_rn(acc2[q], blk2[q]);
-#pragma unroll
-            for (int q = 0; q < P; ++q) {
-                const float m = q % 2 ? M2[q / 2].y : M2[q / 2].x;
-                const float dq = dqs[q];
-                ia[q] = m > Ms[q] && !((fm >> q) & 1u) ? ive : ia[q];
-                const float thr = __fmaf_rn(-2.f, dq, m);
-                const float g = -(q % 2 ? ng2[q / 2].y : ng2[q / 2].x);
-                (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
-                (q % 2 ? K2[q / 2].y : K2[q / 2].x) =
-                    __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), __fadd_rn(level, g));
-                rising = rising && !(thr < 0.f);
+            for (int q = 0; q < P / 2; ++q) {
+                acc2[q] = __fadd2_rn(acc2[q], blk2[q]);
+                // (the last rise of a flagged POV stays where it was)
+                ia2[q].x = M2[q].x > Ms2[q].x && !((fm >> 2 * q) & 1u) ? ive : ia2[q].x;
+                ia2[q].y = M2[q].y > Ms2[q].y && !((fm >> (2 * q + 1)) & 1u) ? ive : ia2[q].y;
+                T2[q] = __ffma2_rn(make_float2(-2.f, -2.f), dq2[q], M2[q]);
+                const float2 lv = __ffma2_rn(make_float2(-1.f, -1.f), ng2[q], make_float2(level, level));
+                K2[q] = __ffma2_rn(make_float2((float)(U - 1) * 1.00001f, (float)(U - 1) * 1.00001f),
+                                   make_float2(fminf(T2[q].x, 0.f), fminf(T2[q].y, 0.f)), lv);
             }
+            rising = !(min3(fminf(T2[0].x, T2[0].y), T2[1].x, T2[1].y) < 0.f);
             e += U;
         }
     }
@@ -1736,7 +1785,7 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
             if (!__any_sync(FULL, gi < G)) break;
         }
         for (;;) {
-            if (gi < G && !ready && e < dlim) e = skip_blocks<U, false>(T2, K2, rising, x0, e, dlim, sp.wm_len - 1, WM, ZS, &ready);
+            if (gi < G && !ready && e < dlim) e = skip_blocks<U, false, SKIP_TESTS>(T2, K2, rising, x0, e, dlim, WM, ZS, &ready);
             const unsigned have = __ballot_sync(FULL, ready);
             const unsigned look = __ballot_sync(FULL, gi < G && !ready && e < dlim);
             if (!look || __popc(have) >= SKIP_READY) break;
@@ -1932,7 +1981,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
 // at 20 warps instead of 16: 1000^2 21.9 -> 20.5 ms).  Per warp, shared memory
 // holds the rows' SkipRows and per row [Fh half][Fl half][suffix maxima]
 // [window maxima].
-template <int WARPS>
+template <int WARPS, int NT>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1999,7 +2048,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
         }
         __syncwarp();
         if (longest > 0)
-            sweep_rows_skip<CERT_POV, U, false, false>(sp, rows, arrays + ROW_PADL, sp.lgna,
+            sweep_rows_skip<CERT_POV, U, false, false, NT>(sp, rows, arrays + ROW_PADL, sp.lgna,
                                                        (longest + CERT_POV - 1) / CERT_POV, zs_off, wm_off, tab,
                                                        nullptr, lane);
     }
@@ -2085,9 +2134,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                 const int groups = ok ? (it.L + CERT_POV - 1) / CERT_POV : 0;
                 const int zs_off = (int)(ZS - H), wm_off = (int)(WM - H);
                 if (bwd)
-                    sweep_rows_skip<CERT_POV, U, LONG, true>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
+                    sweep_rows_skip<CERT_POV, U, LONG, true, SKIP_TESTS>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
                 else
-                    sweep_rows_skip<CERT_POV, U, LONG, false>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
+                    sweep_rows_skip<CERT_POV, U, LONG, false, SKIP_TESTS>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
             } else {
                 const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, cv, false);
                 if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
@@ -2227,7 +2276,7 @@ static SweepSizes sweep_sizes(int wmax, int dmax, bool prune, bool cert, int ndi
     z.zs = prune ? ((wmax + ZS_STRIDE - 1) / ZS_STRIDE + 4) & ~3 : 0;
     z.wm = prune ? ((wmax + SKIP_UNROLL + 3) / ZS_STRIDE + 4) & ~3 : 0;
     z.row = 2 * z.half + z.zs + z.wm;
-    const size_t total = (size_t)smem_optin / 4, fixed = (size_t)z.tab + z.istart;
+    const size_t total = (size_t)smem_optin / 4, fixed = (size_t)z.tab + z.istart + (prune ? WM_SLACK : 0);
     z.room = fixed >= total ? 0 : total - fixed;
     return z;
 }
@@ -2311,13 +2360,14 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     // shared memory of one unit: a pair of warps or one warp
     const int uw = pairs ? 2 : 1;
     const size_t unit = (size_t)(sp.per_pair + uw * sp.per_warp) * 4;
-    size_t fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4;
+    const size_t slack = prune ? WM_SLACK * 4 : 0;   // past the last warp's window maxima
+    size_t fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4 + slack;
     if (longw && fixed + (size_t)(LONG_MIN_WARPS / uw) * unit > (size_t)smem_optin) {
         // Rows of more than about 10^4 samples: the whole table and several
         // staged rows do not fit together.  Keep LONG_MIN_WARPS warps (or as
         // many as fit) and a table of what is left (at least MIN_TABLE
         // entries); the long-walk sweep computes the entries past its end.
-        const size_t base = (size_t)sp.istart_len * 4;
+        const size_t base = (size_t)sp.istart_len * 4 + slack;
         int w = LONG_MIN_WARPS / uw;
         const size_t min_tab = (size_t)tab_floats_for(MIN_TABLE, prune != 0, cert != 0) * 4;
         while (w > 1 && base + min_tab + (size_t)w * unit > (size_t)smem_optin) --w;
@@ -2326,7 +2376,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         const size_t room = ((size_t)smem_optin - base - (size_t)w * unit) / 16 * 4;
         sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, tab_entries_fit(room, prune != 0, cert != 0)) & ~1;
         sp.tab_floats = tab_floats_for(sp.inv_len, prune != 0, cert != 0);
-        fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4;
+        fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4 + slack;
     }
     if (fixed + unit > (size_t)smem_optin) return cudaErrorInvalidConfiguration;
     // As many resident units as shared memory and registers allow, in one CTA
@@ -2337,8 +2387,9 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     int most;
     if (single) {
         const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = prune ? PACK_WARPS : wide ? WW : CW;
-        if (prune) kern = sweep_pack_kernel<PACK_WARPS>;
+        const bool pack = sp.lgna > 0;
+        most = prune ? (pack ? PACK_WARPS : SINGLE_WARPS) : wide ? WW : CW;
+        if (prune) kern = pack ? sweep_pack_kernel<PACK_WARPS, PACK_TESTS> : sweep_pack_kernel<SINGLE_WARPS, SKIP_TESTS>;
         else kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
     } else if (pairs) {
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
