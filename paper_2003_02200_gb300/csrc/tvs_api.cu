@@ -154,7 +154,7 @@ int tvs_debug_rowmap(tvs_handle h, int rows, int cols, int n_sectors, int k, int
     cudaStream_t s = h->stream;
     TVS_CUDA(cudaMemcpyAsync(d_dir, &v, sizeof(v), cudaMemcpyHostToDevice, s), "copy direction");
     TVS_CUDA(launch_colmap(d_dir, d_dest, d_frac, s), "colmap launch");
-    TVS_CUDA(launch_rowmap(d_dir, 1, d.R, d_lo, d_hi, s), "rowmap launch");
+    TVS_CUDA(launch_rowmap(d_dir, 1, d.R, d_lo, d_hi, nullptr, s), "rowmap launch");
     TVS_CUDA(cudaMemcpyAsync(dest, d_dest, (size_t)d.W * 4, cudaMemcpyDeviceToHost, s), "copy dest");
     TVS_CUDA(cudaMemcpyAsync(frac, d_frac, (size_t)d.W * 4, cudaMemcpyDeviceToHost, s), "copy frac");
     TVS_CUDA(cudaMemcpyAsync(jlo, d_lo, (size_t)d.R * 4, cudaMemcpyDeviceToHost, s), "copy jlo");
@@ -238,11 +238,10 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
     int* d_cv = reinterpret_cast<int*>(ws + L.cvf);
     int* d_cb = reinterpret_cast<int*>(ws + L.cvb);
     unsigned* d_cnt = reinterpret_cast<unsigned*>(ws + L.counter);
-    TVS_CUDA(launch_rowmap(d_dir, 1, v.R, d_lo, d_hi, s), "rowmap launch");
-    TVS_CUDA(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned), s), "reset work counter");
+    TVS_CUDA(launch_rowmap(d_dir, 1, v.R, d_lo, d_hi, d_cnt, s), "rowmap launch");
     TVS_CUDA(launch_sweep(d_dir, d_jobs, reinterpret_cast<const int*>(ws + L.istart), 1, c.items, d_lo, d_hi, d_cv,
                           d_cb, v.W, v.K, h->tuning.prune, !h->tuning.fp32_decisions, d_cnt,
-                          reinterpret_cast<int4*>(ws + L.flags), d_cnt + 16, (int)L.flag_cap, h->num_sms, h->smem_optin, h->tuning.sweep_max_warps, s),
+                          reinterpret_cast<int4*>(ws + L.flags), d_cnt + FLAG_COUNT, (int)L.flag_cap, h->num_sms, h->smem_optin, h->tuning.sweep_max_warps, s),
              "sweep launch");
     std::vector<int> slab(c.slab_elems), slabb(c.slab_elems), lo(v.R), hi(v.R);
     TVS_CUDA(cudaMemcpyAsync(slab.data(), d_cv, c.slab_elems * 4, cudaMemcpyDeviceToHost, s), "copy cv");
@@ -502,11 +501,9 @@ extern "C" int tvs_total_viewshed_device_noalloc(const float* d_dem, int rows, i
             wmax = std::max(wmax, dirs[q].W);
         }
         const DirDev* cd = d_dirs + k0;
-        TVS_CUDA(launch_rowmap(cd, nd, max_R, d_rowlo, d_rowhi, s), "rowmap launch");
-        // the shared array keeps the previous call's contents: the work counter must start at zero
-        TVS_CUDA(cudaMemsetAsync(d_counter, 0, sizeof(unsigned), s), "reset work counter");
+        TVS_CUDA(launch_rowmap(cd, nd, max_R, d_rowlo, d_rowhi, d_counter, s), "rowmap launch");
         TVS_CUDA(launch_sweep(cd, d_job, d_istart + at, nd, istart[at + nd], d_rowlo, d_rowhi, d_cvf, d_cvb, wmax,
-                              dmax, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_counter + 16, flag_cap,
+                              dmax, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_counter + FLAG_COUNT, flag_cap,
                               num_sms, smem_optin, tn.sweep_max_warps, s),
                  "sweep launch");
         TVS_CUDA(launch_unskew(d_cvf, d_cvb, d_job, cd, d_cj + c, 1, tiles, cjs[c].nsplit, d_part, s),

@@ -122,7 +122,11 @@ struct ChunkJob {
 };
 
 // Launchers (tvs_kernels.cu).  All are asynchronous on `stream`.
-cudaError_t launch_rowmap(const DirDev* d_dirs, int ndir, int max_R, int* rowlo, int* rowhi,
+// The row tables of a chunk; also clears the COUNTER_WORDS counters of the
+// chunk's other kernels (the sweep's work counter, at FLAG_COUNT its flag
+// counters) unless `counters` is NULL: one launch instead of three.
+constexpr int COUNTER_WORDS = 32, FLAG_COUNT = 16;
+cudaError_t launch_rowmap(const DirDev* d_dirs, int ndir, int max_R, int* rowlo, int* rowhi, unsigned* counters,
                           cudaStream_t stream);
 cudaError_t launch_colmap(const DirDev* d_dir, int* dest, unsigned* frac, cudaStream_t stream);
 // Sweep of a chunk (tvs_sweep.cu): one warp item per skewed row and walk
@@ -130,7 +134,8 @@ cudaError_t launch_colmap(const DirDev* d_dir, int* dest, unsigned* frac, cudaSt
 // backward), its row gathered from the job's DEM; `prune` turns exact horizon
 // pruning on, `cert` certified (exact) visibility decisions instead of FP32
 // ones.  With cert the walks the sweep cannot certify go to the flag buffer
-// (flag_cap entries, possibly none; flag_count three counters) and are walked
+// (flag_cap entries, possibly none; flag_count three counters; these and
+// `counter` are zero before the launch) and are walked
 // exactly by a second kernel on the same stream; those that find it full are
 // marked in their measures and found by a third.
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,

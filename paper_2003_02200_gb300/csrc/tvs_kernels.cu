@@ -28,8 +28,9 @@ __device__ __forceinline__ int dest_of(unsigned long long t_fx, int j)
 // row b + j*t (t = t_fx / 2^32) and is usable iff 0 <= b + j*t <= H - 1,
 // i.e. j*t_fx >= -b*2^32 and j*t_fx <= (H-1-b)*2^32 (exact integers).
 __global__ void rowmap_kernel(const DirDev* __restrict__ dirs, int* __restrict__ rowlo,
-                              int* __restrict__ rowhi)
+                              int* __restrict__ rowhi, unsigned* __restrict__ counters)
 {
+    if (counters && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < COUNTER_WORDS) counters[threadIdx.x] = 0u;
     const DirDev d = dirs[blockIdx.y];
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < d.R; p += gridDim.x * blockDim.x) {
         const long long b = (long long)p - d.D;
@@ -67,8 +68,8 @@ __global__ void colmap_kernel(const DirDev* __restrict__ dir, int* __restrict__ 
 // ---------------------------------------------------------------- unskew --
 // CTA = UNSKEW_TI x UNSKEW_TJ DEM cells and one range of the chunk's
 // directions; for each direction the skewed rows those cells blend (both
-// virtual POVs of every cell) are staged in shared memory with coalesced row
-// reads, then every cell takes g * ((1-r) cv_hi + r cv_lo) (Kernel-3 weights;
+// virtual POVs of every cell) are read in 16-byte pieces, forward and backward
+// measure added, and staged in shared memory as floats, then every cell takes g * ((1-r) cv_hi + r cv_lo) (Kernel-3 weights;
 // a virtual POV whose sample falls outside the DEM is dropped and the other
 // takes weight 1), cv being the forward plus the backward measure.  Partial
 // sums are FP32 over groups of FP32_GROUP consecutive directions; each group
@@ -79,7 +80,7 @@ __global__ void colmap_kernel(const DirDev* __restrict__ dir, int* __restrict__ 
 // unskew_finalize adds.  Integer addition being exact, the result does not
 // depend on the ranges, the chunking or the other jobs of a chunk.
 constexpr int UNSKEW_ROWS = UNSKEW_TI + UNSKEW_TJ + 4;
-constexpr int UNSKEW_PITCH = UNSKEW_TJ + 1;
+constexpr int UNSKEW_PITCH = UNSKEW_TJ + 4;
 constexpr int UNSKEW_THREADS = 256;
 constexpr int UNSKEW_CELLS = UNSKEW_TI * UNSKEW_TJ / UNSKEW_THREADS;
 
@@ -135,35 +136,19 @@ __device__ __forceinline__ int find_chunk_job(const ChunkJob* __restrict__ cj, i
     return lo;
 }
 
-// Asynchronous global -> shared copies of 4 bytes and of 16 bytes (both
-// addresses 16-byte aligned).
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(sa), "l"(gmem) : "memory");
-}
-
-// Row pitch of a staged window.  In views 0 and 3 a warp's lanes blend 32
-// consecutive view columns of one view row, whose skewed rows step down with
-// the column: pitch 32 keeps each lane on its own bank, and rows of 128 bytes
-// take 16-byte copies (the window starts at a tile column, a multiple of 32,
-// in rows padded to a multiple of 4).  In views 1 and 2 the lanes blend 32
-// consecutive view rows at one column: pitch 33 keeps them on distinct banks
-// (4-byte copies).
+// Row pitch of a staged window, in floats.  In views 0 and 3 a warp's lanes
+// blend 32 consecutive view columns of one view row, whose skewed rows step
+// down with the column: pitch 32 keeps each lane on its own bank (the window
+// starts at a tile column, a multiple of 32).  In views 1 and 2 the lanes blend
+// 32 consecutive view rows at one column: with rows of 16-byte pieces four
+// lanes share a bank whatever the pitch.  View 2's window starts at any column,
+// rounded down to a multiple of 4: up to 36 columns, 9 pieces.
 __device__ __forceinline__ int unskew_pitch(int frame) { return frame == 0 || frame == 3 ? 32 : UNSKEW_PITCH; }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
 // The staged window of one direction for a tile: skewed rows pmin.. (np of
 // them) and view columns vj0.. (nj of them) of the direction's slabs.
 struct UnskewWin {
-    int pmin, np, vj0, nj;
+    int pmin, np, vj0, nq;   // vj0 a multiple of 4, nq pieces of 4 columns
 };
 
 __device__ __forceinline__ UnskewWin unskew_window(const DirDev& d, int iD0, int iD1, int jD0, int jD1)
@@ -179,46 +164,66 @@ __device__ __forceinline__ UnskewWin unskew_window(const DirDev& d, int iD0, int
     w.pmin = max(vi0 - dest_of(d.t_fx, vj1) + d.D - 1, 0);
     const int pmax = min(vi1 - dest_of(d.t_fx, vj0) + d.D, d.R - 1);
     w.np = pmax - w.pmin + 1;
-    w.vj0 = vj0;
-    w.nj = vj1 - vj0 + 1;
+    w.vj0 = vj0 & ~3;
+    w.nq = (vj1 - w.vj0) / 4 + 1;
     return w;
 }
 
-// Copies (asynchronously) the forward and backward measures of a window.
-__device__ __forceinline__ void unskew_stage(const UnskewParams& up, const DirDev& d, const UnskewWin& w, int* SF,
-                                             int* SB)
+// A thread's pieces of a window (4 columns of a row each): at most
+// ceil(UNSKEW_ROWS * 9 / UNSKEW_THREADS).
+constexpr int UNSKEW_PIECES = (UNSKEW_ROWS * 9 + UNSKEW_THREADS - 1) / UNSKEW_THREADS;
+
+// Row and piece of the window's k-th piece of this thread; false past its end.
+__device__ __forceinline__ bool unskew_piece(const UnskewWin& w, int frame, int k, int* r, int* q)
+{
+    const int idx = threadIdx.x + k * UNSKEW_THREADS;
+    *r = frame == 2 ? idx / 9 : idx >> 3;
+    *q = frame == 2 ? idx - 9 * *r : idx & 7;
+    return *r < w.np && *q < w.nq;
+}
+
+// Loads the forward and backward measures of a window into registers.  The
+// last piece of a row may read up to 3 padding columns (rows are padded to a
+// multiple of 4).
+__device__ __forceinline__ void unskew_load(const UnskewParams& up, const DirDev& d, const UnskewWin& w, int4* f,
+                                            int4* b)
 {
     const long long off = d.slab + (long long)w.pmin * d.Wp + w.vj0;
-    if (d.frame == 0 || d.frame == 3) {
-        // 8 chunks of 4 columns per row; the last may read up to 3 padding
-        // columns of the row (vj0 + 4 ceil(nj / 4) <= Wp)
-        for (int idx = threadIdx.x; idx < w.np * 8; idx += UNSKEW_THREADS) {
-            const int r = idx >> 3, q4 = (idx & 7) * 4;
-            if (q4 < w.nj) {
-                const long long a = off + (long long)r * d.Wp + q4;
-                cp_async16(SF + r * 32 + q4, up.cvf + a);
-                cp_async16(SB + r * 32 + q4, up.cvb + a);
-            }
-        }
-    } else {
-        for (int idx = threadIdx.x; idx < w.np * 32; idx += UNSKEW_THREADS) {
-            const int r = idx >> 5, cc = idx & 31;
-            if (cc < w.nj) {
-                const long long a = off + (long long)r * d.Wp + cc;
-                cp_async4(SF + r * UNSKEW_PITCH + cc, up.cvf + a);
-                cp_async4(SB + r * UNSKEW_PITCH + cc, up.cvb + a);
-            }
-        }
+#pragma unroll
+    for (int k = 0; k < UNSKEW_PIECES; ++k) {
+        int r, q;
+        if (!unskew_piece(w, d.frame, k, &r, &q)) continue;
+        const long long a = off + (long long)(r * d.Wp + 4 * q);
+        f[k] = __ldg(reinterpret_cast<const int4*>(up.cvf + a));
+        b[k] = __ldg(reinterpret_cast<const int4*>(up.cvb + a));
+    }
+}
+
+// Stores their sums as floats.
+__device__ __forceinline__ void unskew_store(const DirDev& d, const UnskewWin& w, const int4* f, const int4* b,
+                                             float* S)
+{
+    const int pitch = unskew_pitch(d.frame);
+    // (samples outside the DEM hold anything: their sums are never used, or times 0)
+    auto sum = [](int x, int y) { return (float)(int)((unsigned)x + (unsigned)y); };
+#pragma unroll
+    for (int k = 0; k < UNSKEW_PIECES; ++k) {
+        int r, q;
+        if (!unskew_piece(w, d.frame, k, &r, &q)) continue;
+        *reinterpret_cast<float4*>(S + r * pitch + 4 * q) =
+            make_float4(sum(f[k].x, b[k].x), sum(f[k].y, b[k].y), sum(f[k].z, b[k].z), sum(f[k].w, b[k].w));
     }
 }
 
 // Directions are double-buffered: while the cells of a tile blend one
-// direction's staged rows, the next direction's rows are in flight.
+// direction's staged rows, the next direction's rows are on their way to
+// registers; one barrier per direction.  Bound by instruction issue: with
+// 4-byte asynchronous copies of both slabs and the sums taken per cell a warp
+// spent 425 instructions per direction.  2000^2, 180 directions: 2.64 -> 2.19
+// ms; 100^2, whose 368 CTAs wait on their loads: 31 -> 24 us.
 __global__ void __launch_bounds__(UNSKEW_THREADS, 4) unskew_kernel(UnskewParams up)
 {
-    __shared__ __align__(16) int SF[2][UNSKEW_ROWS * UNSKEW_PITCH];
-    __shared__ __align__(16) int SB[2][UNSKEW_ROWS * UNSKEW_PITCH];
-    static_assert((UNSKEW_ROWS * UNSKEW_PITCH * 4) % 16 == 0, "second buffers stay 16-byte aligned");
+    __shared__ __align__(16) float S[2][UNSKEW_ROWS * UNSKEW_PITCH];
     const ChunkJob c = up.cj[find_chunk_job(up.cj, up.ncj, blockIdx.x, false)];
     if ((int)blockIdx.z >= c.nsplit) return;
     const JobDev J = up.jobs[c.job];
@@ -235,77 +240,76 @@ __global__ void __launch_bounds__(UNSKEW_THREADS, 4) unskew_kernel(UnskewParams 
 #pragma unroll
     for (int m = 0; m < UNSKEW_CELLS; ++m) { acc32[m] = 0.f; accx[m] = 0; }
     int group = kbeg < kend ? up.dirs[kbeg].gidx / FP32_GROUP : 0;
+    const int iD = iD0 + ly, jD = jD0 + lx;      // the thread's cells: iD + 8 m, jD
 
     DirDev d_next;
     UnskewWin w_next{0, 0, 0, 0};
+    int4 f[UNSKEW_PIECES], b[UNSKEW_PIECES];
     if (kbeg < kend) {
         d_next = up.dirs[kbeg];
         w_next = unskew_window(d_next, iD0, iD1, jD0, jD1);
-        unskew_stage(up, d_next, w_next, SF[0], SB[0]);
+        unskew_load(up, d_next, w_next, f, b);
     }
-    cp_async_commit();
     for (int kk = kbeg; kk < kend; ++kk) {
-        const int buf = (kk - kbeg) & 1;
+        float* V = S[(kk - kbeg) & 1];
         const DirDev d = d_next;
         const UnskewWin w = w_next;
+        unskew_store(d, w, f, b, V);
         if (kk + 1 < kend) {
             d_next = up.dirs[kk + 1];
             w_next = unskew_window(d_next, iD0, iD1, jD0, jD1);
-            unskew_stage(up, d_next, w_next, SF[buf ^ 1], SB[buf ^ 1]);
+            unskew_load(up, d_next, w_next, f, b);
         }
-        cp_async_commit();
-        cp_async_wait<1>();          // every group but the one just issued has landed
+        // the buffer stored next was last read before this barrier
         __syncthreads();
         if (d.gidx / FP32_GROUP != group) {
 #pragma unroll
             for (int m = 0; m < UNSKEW_CELLS; ++m) { accx[m] += acc_of(acc32[m]); acc32[m] = 0.f; }
             group = d.gidx / FP32_GROUP;
         }
-        const int* F = SF[buf];
-        const int* B = SB[buf];
-        const int pitch = unskew_pitch(d.frame);
+        // cell value g (wa hi + wb lo): weights 1 - r and r, or 1 and 0 where one
+        // line is the sample or the other leaves the DEM (a finite value times 0
+        // leaves the sum as it is)
+        auto blend = [&](int m, int i, int hi, int pitch, float r, bool whole) {
+            const bool lo_only = !whole && i > d.H - 2;
+            const bool hi_only = whole || i < 1;
+            const float wa = lo_only ? 0.f : hi_only ? 1.f : __fsub_rn(1.0f, r);
+            const float wb = lo_only ? 1.f : hi_only ? 0.f : r;
+            const float val = __fadd_rn(__fmul_rn(wa, V[hi]), __fmul_rn(wb, V[max(hi - pitch, 0)]));
+            acc32[m] = __fadd_rn(acc32[m], __fmul_rn(d.g, val));
+        };
+        if (jD <= jD1) {
+            if (d.frame == 0 || d.frame == 3) {
+                // one view column: the sample's position is the same for all cells
+                const unsigned long long y = (unsigned long long)jD * d.t_fx;
+                const unsigned fr = (unsigned)y;
+                const float r = __fmul_rn(__uint2float_rn(fr), 0x1p-32f);
+                const int base = (d.D - (int)(y >> 32) - w.pmin) * 32 + (jD - w.vj0);
 #pragma unroll
-        for (int m = 0; m < UNSKEW_CELLS; ++m) {
-            const int iD = iD0 + ly + 8 * m, jD = jD0 + lx;
-            if (iD > iD1 || jD > jD1) continue;
-            int i, j;
-            switch (d.frame) {
-            case 0:  i = iD; j = jD; break;
-            case 1:  i = jD; j = iD; break;
-            case 2:  i = jD; j = d.W - 1 - iD; break;
-            default: i = d.H - 1 - iD; j = jD; break;
-            }
-            const unsigned long long y = (unsigned long long)j * d.t_fx;
-            const int dest = (int)(y >> 32);
-            const unsigned fr = (unsigned)(y & 0xFFFFFFFFull);
-            const int hi = (i - dest + d.D - w.pmin) * pitch + (j - w.vj0);   // line through i + r
-            const int lo = hi - pitch;                                       // line through i - 1 + r
-            float val;
-            if (fr == 0u) {
-                val = (float)(F[hi] + B[hi]);
+                for (int m = 0; m < UNSKEW_CELLS; ++m) {
+                    if (iD + 8 * m > iD1) break;
+                    const int i = d.frame == 0 ? iD + 8 * m : d.H - 1 - (iD + 8 * m);
+                    blend(m, i, base + i * 32, 32, r, fr == 0u);
+                }
             } else {
-                const bool hi_ok = i <= d.H - 2, lo_ok = i >= 1;
-                if (hi_ok && lo_ok) {
+#pragma unroll
+                for (int m = 0; m < UNSKEW_CELLS; ++m) {
+                    if (iD + 8 * m > iD1) break;
+                    const int j = d.frame == 1 ? iD + 8 * m : d.W - 1 - (iD + 8 * m);
+                    const unsigned long long y = (unsigned long long)j * d.t_fx;
+                    const unsigned fr = (unsigned)y;
                     const float r = __fmul_rn(__uint2float_rn(fr), 0x1p-32f);
-                    val = __fadd_rn(__fmul_rn(__fsub_rn(1.0f, r), (float)(F[hi] + B[hi])),
-                                    __fmul_rn(r, (float)(F[lo] + B[lo])));
-                } else if (hi_ok) {
-                    val = (float)(F[hi] + B[hi]);
-                } else {
-                    val = (float)(F[lo] + B[lo]);
+                    blend(m, jD, (jD + d.D - (int)(y >> 32) - w.pmin) * UNSKEW_PITCH + (j - w.vj0), UNSKEW_PITCH, r,
+                          fr == 0u);
                 }
             }
-            acc32[m] = __fadd_rn(acc32[m], __fmul_rn(d.g, val));
         }
-        __syncthreads();             // the buffer is refilled two directions later
     }
-    cp_async_wait<0>();
     const long long cells = (long long)rows * cols;
 #pragma unroll
     for (int m = 0; m < UNSKEW_CELLS; ++m) {
-        const int iD = iD0 + ly + 8 * m, jD = jD0 + lx;
-        if (iD > iD1 || jD > jD1) continue;
-        const long long idx = (long long)iD * cols + jD;
+        if (iD + 8 * m > iD1 || jD > jD1) continue;
+        const long long idx = (long long)(iD + 8 * m) * cols + jD;
         __int128 tot = accx[m] + acc_of(acc32[m]);
         if (c.nsplit > 1) {
             up.part[c.part_off + (long long)blockIdx.z * cells + idx] = tot;
@@ -337,12 +341,12 @@ __global__ void unskew_finalize(UnskewParams up)
 }  // namespace
 
 // -------------------------------------------------------------- launchers --
-cudaError_t launch_rowmap(const DirDev* d_dirs, int ndir, int max_R, int* rowlo, int* rowhi,
+cudaError_t launch_rowmap(const DirDev* d_dirs, int ndir, int max_R, int* rowlo, int* rowhi, unsigned* counters,
                           cudaStream_t stream)
 {
     if (ndir <= 0) return cudaSuccess;
     dim3 grid((max_R + 255) / 256, ndir);
-    rowmap_kernel<<<grid, 256, 0, stream>>>(d_dirs, rowlo, rowhi);
+    rowmap_kernel<<<grid, 256, 0, stream>>>(d_dirs, rowlo, rowhi, counters);
     return cudaGetLastError();
 }
 

@@ -582,7 +582,7 @@ int enqueue_chunks(tvs_ctx* h, const BatchPlan& plan, const Layout& L, char* bas
     const ChunkJob* d_cj = reinterpret_cast<const ChunkJob*>(base + L.cj);
     const int* d_istart = reinterpret_cast<const int*>(base + L.istart);
     unsigned* d_counter = reinterpret_cast<unsigned*>(base + L.counter);
-    unsigned* d_fcount = reinterpret_cast<unsigned*>(base + L.counter + 64);
+    unsigned* d_fcount = d_counter + FLAG_COUNT;
     int4* d_flags = reinterpret_cast<int4*>(base + L.flags);
     __int128* d_part = reinterpret_cast<__int128*>(base + L.part);
     int* d_rowlo = reinterpret_cast<int*>(base + L.rowlo);
@@ -595,9 +595,8 @@ int enqueue_chunks(tvs_ctx* h, const BatchPlan& plan, const Layout& L, char* bas
         const DirDev* cd = d_dirs + c.i0;
         {
             Timer t(h, K_ROWMAP, s, c.rowmap_bytes);
-            TVS_CUDA(launch_rowmap(cd, nd, c.max_R, d_rowlo, d_rowhi, s), "rowmap launch");
+            TVS_CUDA(launch_rowmap(cd, nd, c.max_R, d_rowlo, d_rowhi, d_counter, s), "rowmap launch");
         }
-        TVS_CUDA(cudaMemsetAsync(d_counter, 0, sizeof(unsigned), s), "reset work counter");
         {
             Timer t(h, K_SWEEP, s, c.evals);
             TVS_CUDA(launch_sweep(cd, d_jobs, d_istart + c.istart_at, nd, c.items, d_rowlo, d_rowhi, d_cvf, d_cvb,

@@ -2412,10 +2412,6 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if (cert) {
-        err = cudaMemsetAsync(flag_count, 0, 3 * sizeof(unsigned), stream);
-        if (err != cudaSuccess) return err;
-    }
     kern<<<per_sm * num_sms, warps * 32, smem, stream>>>(sp);
     err = cudaGetLastError();
     if (err != cudaSuccess || !cert) return err;
