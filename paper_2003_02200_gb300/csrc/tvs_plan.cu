@@ -494,16 +494,19 @@ int plan_batch(const std::vector<JobSpec>& jobs, size_t avail, int num_sms, cons
     return TVS_OK;
 }
 
-// Entries of the flagged-walk buffer for these jobs: 1 in 64 of their walks
-// (flags run between 1 in 700 and 1 in 250 on fractal terrain; walks beyond
-// the buffer are walked in the sweep itself, at a cost), at least 4096, at
-// most `cap` and FLAG_BUF_ENTRIES.
+// Entries of the flagged-walk buffer for these jobs: 1 in 64 of their walks,
+// more in proportion where they are longer than 1024 samples (flagged blocks
+// run between 1 in 700 and 1 in 250 walks on fractal terrain at 1000 to 2000
+// samples and to 1 in 10 at 8000; what finds the buffer full is searched for
+// and walked whole, at a cost), at least 4096, at most `cap` and
+// FLAG_BUF_ENTRIES.
 size_t flag_entries(const std::vector<JobSpec>& jobs, size_t cap)
 {
     double walks = 0.0;
     for (const JobSpec& J : jobs) {
         const int nd = J.k1 > J.k0 ? J.k1 - J.k0 : J.n;   // the job's directions in this call
-        walks += 2.0 * (double)J.rows * (double)J.cols * (double)nd;
+        walks += 2.0 * (double)J.rows * (double)J.cols * (double)nd *
+                 std::max(1.0, (double)std::max(J.rows, J.cols) / 1024.0);
     }
     return (size_t)std::min<double>((double)std::min<size_t>(cap, FLAG_BUF_ENTRIES), std::max(4096.0, walks / 64.0));
 }

@@ -76,6 +76,7 @@ struct SweepParams {
     int flag_cap;
     int ndir;
     int total_items;
+    int scan_blocks;   // 32-sample blocks of the longest row
     int inv_len;       // entries of the per-distance table
     int tab_floats;    // floats it takes (a multiple of 4)
     int istart_len;    // ints of the item-start table (multiple of 4)
@@ -83,7 +84,8 @@ struct SweepParams {
     int padr;          // of them after the row's samples
     int lgna;          // packed kernel: log2 of the staged rows per warp
     int per_row;       // packed kernel: floats of a staged row's arrays
-    int per_pair;      // floats of a warp pair's shared area (certified)
+    int lgw;           // log2 of the warps that share a row (certified, long rows)
+    int per_pair;      // floats of their shared area
     int zs_len;        // floats of the row's suffix maxima (0 without pruning)
     int wm_len;        // floats of the row's window maxima (0 without pruning)
     int per_warp;      // floats of a warp's shared area
@@ -722,9 +724,11 @@ __device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const Cert
 }
 
 // The sample field of a flag entry holds the entry's kind above bit 16: a
-// whole walk to take again, or one block of a walk whose running maximum
-// before it lies in one earlier block, or anywhere before it.  The fourth
-// field of a block entry is its first step e0 and that earlier block's.
+// whole walk to take again, or one block of a walk.  The fourth field of a
+// block entry is the block's first step e0 and p0, the first step of the block
+// in which the maximum last rose for certain: the walk's running maximum
+// before e0 lies in that block, or (FLAG_PREFIX, when a block after it was
+// flagged) anywhere from there on.
 constexpr int FLAG_WALK = 0, FLAG_BLOCK = 1, FLAG_PREFIX = 2;
 static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 
@@ -1033,7 +1037,7 @@ __device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int p
     const int last = min(n - 1, e0 + U);
     if (last <= e0) return;
     bool esc = false;
-    const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, 0, e0, e0, last, lane, &esc)
+    const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, p0, e0, e0, last, lane, &esc)
                                       : df_walk<1>(c, x, p0, min(p0 + U, e0), e0, last, lane, &esc);
     const int add = esc ? fp64_walk(c, x, e0, last, lane) : s;
     if (lane == 0 && in_range(x, c.L, 14) && add) atomicAdd(c.cvrow + x, add);
@@ -1413,7 +1417,8 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 }
 
 // Pruned certified sweep of a warp's staged rows (2^lgna of them, sp.per_row
-// floats apart; `groups` is the most groups of any): sweep_row_cert's walk, but a lane
+// floats apart; `groups` is the most groups of any), or of its share of a row's
+// groups (every 2^lgs-th from gsub on): sweep_row_cert's walk, but a lane
 // evaluates only the blocks of U steps that can hold a visible target, and
 // stops where none is left.  (On fractal terrain 3 to 5 % of the targets of a
 // walk are visible; the walks reach their stopping point after about 40 % of
@@ -1459,7 +1464,8 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // number is what hides the latency of the tests.
 template <int P, int U, bool LONG, bool BWD, int NT>
 __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const SkipRow* __restrict__ rows,
-                                                const float* H0, int lgna, int groups, int zs_off, int wm_off,
+                                                const float* H0, int lgna, int groups, int lgs, int gsub, int zs_off,
+                                                int wm_off,
                                                 const float2* __restrict__ tab, int* __restrict__ spill, int lane)
 {
     constexpr int CH = SKIP_CHUNK;
@@ -1478,8 +1484,9 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
     bool rising = false;             // every thr >= 0
     float Rh = 0.f, c2e = 0.f;
     float level = 0.f;               // R - slack
-    unsigned lost = 0u, again = 0u;  // POVs whose walk is taken again; with an earlier flagged block
-    const int tasks = groups << lgna;  // group t >> lgna of row t & (rows - 1), longest walks first
+    unsigned lost = 0u, again = 0u;  // POVs whose walk is taken again; with a flagged block since the last certain rise
+    // group (t >> lgna) 2^lgs + gsub of row t & (rows - 1), longest walks first
+    const int tasks = (groups - gsub + (1 << lgs) - 1) >> lgs << lgna;
     int next = 32;
     bool has = lane < tasks;
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
@@ -1489,7 +1496,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
     auto start = [&](int task) {
         r = rows + (task & ((1 << lgna) - 1));
         H = H0 + (task & ((1 << lgna) - 1)) * sp.per_row;
-        const int L = r->L, gi = task >> lgna, G = (L + P - 1) / P;
+        const int L = r->L, gi = ((task >> lgna) << lgs) + gsub, G = (L + P - 1) / P;
         x0 = (BWD ? G - 1 - gi : gi) * P;
         e = 0;
         dlim = -1;
@@ -1560,7 +1567,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
             (q % 2 ? M2[q / 2].y : M2[q / 2].x) = m;
         }
     };
-    if (tasks == 0) return;
+    if (tasks <= 0) return;
     if (has) start(lane);
     for (;;) {
         // 1. finished groups: write their measures, hand over their flagged
@@ -1696,9 +1703,10 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
 #pragma unroll
             for (int q = 0; q < P / 2; ++q) {
                 acc2[q] = __fadd2_rn(acc2[q], blk2[q]);
-                // (the last rise of a flagged POV stays where it was)
-                ia2[q].x = M2[q].x > Ms2[q].x && !((fm >> 2 * q) & 1u) ? ive : ia2[q].x;
-                ia2[q].y = M2[q].y > Ms2[q].y && !((fm >> (2 * q + 1)) & 1u) ? ive : ia2[q].y;
+                // (the last rise of a flagged POV stays where it was; a certain
+                // rise lies above every earlier target, flagged or not)
+                if (M2[q].x > Ms2[q].x && !((fm >> 2 * q) & 1u)) { ia2[q].x = ive; again &= ~(1u << 2 * q); }
+                if (M2[q].y > Ms2[q].y && !((fm >> (2 * q + 1)) & 1u)) { ia2[q].y = ive; again &= ~(2u << 2 * q); }
                 T2[q] = __ffma2_rn(make_float2(-2.f, -2.f), dq2[q], M2[q]);
                 const float2 lv = __ffma2_rn(make_float2(-1.f, -1.f), ng2[q], make_float2(level, level));
                 K2[q] = __ffma2_rn(make_float2((float)(U - 1) * 1.00001f, (float)(U - 1) * 1.00001f),
@@ -2049,29 +2057,33 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
         __syncwarp();
         if (longest > 0)
             sweep_rows_skip<CERT_POV, U, false, false, NT>(sp, rows, arrays + ROW_PADL, sp.lgna,
-                                                       (longest + CERT_POV - 1) / CERT_POV, zs_off, wm_off, tab,
+                                                       (longest + CERT_POV - 1) / CERT_POV, 0, 0, zs_off, wm_off, tab,
                                                        nullptr, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
 
-// Barrier of the two warps of pair `pair` (named barrier 1 + pair).
-__device__ __forceinline__ void pair_sync(int pair)
+// Barrier of the 2^lgw warps that share row buffer `row` (named barrier 1 + row).
+__device__ __forceinline__ void row_sync(int row, int lgw)
 {
-    asm volatile("bar.sync %0, %1;" :: "r"(1 + pair), "r"(64) : "memory");
+    asm volatile("bar.sync %0, %1;" :: "r"(1 + row), "r"(32 << lgw) : "memory");
 }
 
-// The certified sweep with one staged row per pair of warps: warp 2k walks
-// every row of the pair forward and warp 2k + 1 walks the same row backward
-// (items 2p and 2p + 1), so a row's double-float samples and end samples are
-// staged once and held once for both directions (half the shared memory per
-// warp of one row per warp, and room for twice the warps at 2000-sample
-// rows).  Both warps stage half of the row; the forward warp computes its
-// suffix maxima, the backward warp its prefix maxima (pruning).  Each warp
-// runs one direction's code only.  Per pair, shared memory holds [Fh
-// half][Fl half][suffix maxima][prefix maxima][window maxima][ends 4][exchange
-// 4][SkipRow per warp]; per warp
-// the long-walk spill.
+// The certified sweep with one staged row per 2^lgw warps, half of which walk
+// it forward (items 2p) and half backward (items 2p + 1), so a row's
+// double-float samples and end samples are staged once and held once for all
+// of them.  The warps of one walk direction take every 2^(lgw - 1)-th group.
+// Two warps per row when that fills the SM (rows of up to about 2600 samples),
+// more beyond (pruned): 4000-sample rows leave room for 4, and with two warps
+// each for 8 warps in all (4000^2, 90 directions, 10 km: 264 ms with two warps
+// per row, 204 with four; 5000^2, 8 directions: 74 and 53).  All of them stage a share of the row; the first
+// computes its suffix maxima, the second its prefix maxima (pruning).  Each
+// warp runs one direction's code only.  Per row, shared memory holds [Fh
+// half][Fl half][suffix maxima][prefix maxima][window maxima][ends 4][item and
+// zmax exchange][a SkipRow per walk direction]; per warp the long-walk spill.
+constexpr int MAX_LGW = 4;
+constexpr int ROW_XCH = 4 + (1 << MAX_LGW);   // floats of the exchange
+
 template <bool PRUNE, bool LONG, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams sp)
 {
@@ -2080,8 +2092,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     Entry* tab = reinterpret_cast<Entry*>(smem);
     int* istart = reinterpret_cast<int*>(smem + sp.tab_floats);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pair = warp >> 1, bwd = warp & 1;
-    const int npairs = blockDim.x >> 6;
+    const int lgw = sp.lgw, nw = 1 << lgw;
+    const int pair = warp >> lgw, part = warp & (nw - 1), bwd = part & 1;
+    const int npairs = blockDim.x >> (5 + lgw);
     float* base = smem + sp.tab_floats + sp.istart_len;
     float* Fh = base + pair * sp.per_pair;
     float* Fl = Fh + sp.half;
@@ -2090,7 +2103,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     float* ends = WM + sp.wm_len;                          // 4 floats
     constexpr int U = PRUNE ? SKIP_UNROLL : CERT_UNROLL;
     float* xch = ends + 4;                                   // item number and the halves' zmax
-    SkipRow* row = reinterpret_cast<SkipRow*>(xch + 4) + bwd;   // this warp's view of the row (pruned)
+    // the row as either walk direction sees it (pruned)
+    SkipRow* row = reinterpret_cast<SkipRow*>(xch + ROW_XCH) + bwd;
     float* own = base + npairs * sp.per_pair + warp * sp.per_warp;
     int* spill = reinterpret_cast<int*>(own) + lane;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
@@ -2103,27 +2117,29 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     const long long t_start = clock64();
 
     for (;;) {
-        if (bwd == 0 && lane == 0) reinterpret_cast<int*>(xch)[0] = (int)atomicAdd(sp.counter, 2u);
-        pair_sync(pair);
+        if (part == 0 && lane == 0) reinterpret_cast<int*>(xch)[0] = (int)atomicAdd(sp.counter, 2u);
+        row_sync(pair, lgw);
         const int pitem = reinterpret_cast<const int*>(xch)[0];   // items pitem (forward), pitem + 1
         if (pitem >= sp.total_items) break;
         ItemRow it;
         const bool nonempty = decode_item(sp, istart, pitem + bwd, &it);
         if (nonempty) {
-            const float zpart = stage_row<true>(sp, it, Fh, Fl, ends, lane, bwd, 2, false);
-            if (lane == 0) xch[1 + bwd] = zpart;
-            pair_sync(pair);   // the staged row is complete
-            if (PRUNE) {   // each warp's own suffix or prefix maxima, half of the window maxima
-                if (bwd) end_max<true>(Fh, ZS, it.L, lane);
-                else end_max<false>(Fh, ZS, it.L, lane);
-                window_max<CERT_POV, U>(Fh, WM, it.L, lane, bwd, 2);
-                pair_sync(pair);
+            const float zpart = stage_row<true>(sp, it, Fh, Fl, ends, lane, part, nw, false);
+            if (lane == 0) xch[1 + part] = zpart;
+            row_sync(pair, lgw);   // the staged row is complete
+            if (PRUNE) {   // suffix and prefix maxima by the first two warps, each a share of the window maxima
+                if (part == 1) end_max<true>(Fh, ZS, it.L, lane);
+                if (part == 0) end_max<false>(Fh, ZS, it.L, lane);
+                window_max<CERT_POV, U>(Fh, WM, it.L, lane, part, nw);
+                row_sync(pair, lgw);
             }
-            const float zmax = fmaxf(xch[1], xch[2]);
+            float zmax = xch[1];
+            for (int m = 2; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
             int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
             if constexpr (PRUNE) {
                 bool ok = true;
                 if (lane == 0) {
+                    // (the warps of one walk direction all write the same)
                     ok = skip_row(sp, it, bwd != 0, zmax, cv, false, LONG, row);
 #pragma unroll
                     for (int m = 0; m < 4; ++m) row->ends[m] = ends[m];
@@ -2134,16 +2150,18 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                 const int groups = ok ? (it.L + CERT_POV - 1) / CERT_POV : 0;
                 const int zs_off = (int)(ZS - H), wm_off = (int)(WM - H);
                 if (bwd)
-                    sweep_rows_skip<CERT_POV, U, LONG, true, SKIP_TESTS>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
+                    sweep_rows_skip<CERT_POV, U, LONG, true, SKIP_TESTS>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
+                                                                     wm_off, tab, spill, lane);
                 else
-                    sweep_rows_skip<CERT_POV, U, LONG, false, SKIP_TESTS>(sp, row, H, 0, groups, zs_off, wm_off, tab, spill, lane);
+                    sweep_rows_skip<CERT_POV, U, LONG, false, SKIP_TESTS>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
+                                                                     wm_off, tab, spill, lane);
             } else {
                 const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, cv, false);
                 if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
                 else sweep_row_cert<CERT_POV, U, LONG, false, true>(sp, r, tab, spill, lane);
             }
         }
-        pair_sync(pair);   // both walks are done with the row (and with the exchange slot)
+        row_sync(pair, lgw);   // both walks are done with the row (and with the exchange slot)
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
@@ -2154,14 +2172,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
 // on samples blended from the DEM as the staging does (the DEM is L2-resident
 // while the sweep runs).  Bound by the latency of those gathers.  A warp takes
 // two entries at a time: two FLAG_BLOCK entries in one go, a half-warp each,
-// what else there is (whole walks, walks with an earlier flagged block, FP64)
+// what else there is (whole walks, walks flagged since their last rise, FP64)
 // with all 32 lanes.  An entry names its row directly (no search of the item
 // table) and the counters stay in registers: 12 mixed tiles (7.3 million
 // blocks) 214 -> 204 ms, 2000^2 (1.26 million) 95.5 -> 92.6 ms.
 // flag_count[0] is the buffer's fill.
 constexpr int EXACT_WARPS = 16;
 
-__global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2) exact_kernel(SweepParams sp)
 {
     const int lane = threadIdx.x & 31;
     const unsigned n = min(sp.flag_count[0], (unsigned)sp.flag_cap);
@@ -2207,39 +2225,35 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32) exact_kernel(SweepParams sp)
 }
 
 // The walks that found the flag buffer full: their measures are negative.
-// Does nothing unless the sweep saw a full buffer; otherwise every row of the
-// launch is searched, a warp per item, and its marked walks are walked exactly.
-__global__ void __launch_bounds__(EXACT_WARPS * 32) exact_scan_kernel(SweepParams sp)
+// Does nothing unless the sweep saw a full buffer; otherwise the measures of
+// the whole launch are searched, 32 samples of an item at a time (a few long
+// rows would leave most warps without one), and the marked walks walked
+// exactly.
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2) exact_scan_kernel(SweepParams sp)
 {
     if (sp.flag_count[2] == 0u) return;
     const int lane = threadIdx.x & 31;
-    const long long step = (long long)gridDim.x * EXACT_WARPS;
     unsigned count[2] = {0u, 0u};
-    for (long long item = (long long)blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); item < sp.total_items;
-         item += step) {
+    const long long units = (long long)sp.total_items * sp.scan_blocks, step = (long long)gridDim.x * EXACT_WARPS;
+    for (long long u = (long long)blockIdx.x * EXACT_WARPS + (threadIdx.x >> 5); u < units; u += step) {
+        const int item = (int)(u / sp.scan_blocks), x0 = (int)(u % sp.scan_blocks) * 32;
         ItemRow it;
-        if (!decode_item(sp, sp.item_start, (int)item, &it)) continue;
+        if (!decode_item(sp, sp.item_start, item, &it) || x0 >= it.L) continue;
         const int* cv = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
-        ExactCtx xc;
-        bool ready = false;                  // xc is set once a marked walk is found
-        for (int x0 = 0; x0 < it.L; x0 += 32) {
-            unsigned marked = __ballot_sync(0xffffffffu, x0 + lane < it.L && cv[x0 + lane] < 0);
-            if (marked && !ready) {
-                ready = true;
-                xc = exact_ctx(sp, it, 0.f);
-                float zmax = 0.f;
-                for (int x = lane; x < it.L; x += 32) {
-                    float va, vb;
-                    unsigned fr;
-                    dem_pair(xc, x, va, vb, fr);
-                    zmax = fmaxf(zmax, fmaxf(fabsf(va), fabsf(vb)));
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-                xc = exact_ctx(sp, it, zmax);
-            }
-            for (; marked; marked &= marked - 1) exact_walk(xc, x0 + __ffs(marked) - 1, lane, count);
+        unsigned marked = __ballot_sync(0xffffffffu, x0 + lane < it.L && cv[x0 + lane] < 0);
+        if (!marked) continue;
+        ExactCtx c = exact_ctx(sp, it, 0.f);
+        float zmax = 0.f;
+        for (int x = lane; x < it.L; x += 32) {
+            float va, vb;
+            unsigned fr;
+            dem_pair(c, x, va, vb, fr);
+            zmax = fmaxf(zmax, fmaxf(fabsf(va), fabsf(vb)));
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+        c = exact_ctx(sp, it, zmax);
+        for (; marked; marked &= marked - 1) exact_walk(c, x0 + __ffs(marked) - 1, lane, count);
     }
     if (lane == 0) {
         if (count[0]) atomicAdd(&g_sweep_stats[0], (unsigned long long)count[0]);
@@ -2317,6 +2331,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     sp.dirs = d_dirs; sp.jobs = d_jobs; sp.item_start = d_item_start; sp.rowlo = rowlo;
     sp.rowhi = rowhi; sp.cv_fwd = cv_fwd; sp.cv_bwd = cv_bwd; sp.counter = counter; sp.ndir = ndir;
     sp.total_items = total_items;
+    sp.scan_blocks = (wmax + 31) / 32;
     if (cert && !flag_count) return cudaErrorInvalidValue;
     sp.flag_buf = flag_buf;
     sp.flag_count = flag_count;
@@ -2332,7 +2347,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     sp.per_row = z.row;
     sp.lgna = 0;
     const bool longw = wmax - 2 > LONG_WALK && dmax - 1 > LONG_WALK;
-    const int lspill = longw ? 32 * LARGE_POV : 0;
+    const int lspill = longw ? 32 * (cert || prune ? CERT_POV : LARGE_POV) : 0;
     // FP32 decisions: one row per warp.  Certified: rows of a warp's own (one,
     // reversed for backward walks, or when pruned up to 2^PACK_MAX_LG) when
     // TVS_CERT_SINGLE_MIN such warps fit, else one row per pair of warps (both
@@ -2353,22 +2368,34 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
                                     (long long)PACK_MIN_CLAIMS * num_sms * PACK_WARPS)
             ++sp.lgna;
     }
-    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 8 + (prune ? 2 * SKIP_ROW_FLOATS : 0) : 0;
+    sp.per_pair = pairs ? 2 * sp.half + 2 * sp.zs_len + sp.wm_len + 4 + ROW_XCH + (prune ? 2 * SKIP_ROW_FLOATS : 0) : 0;
     sp.per_warp = single ? (prune ? (SKIP_ROW_FLOATS + z.row) << sp.lgna : 2 * sp.half + 4)
                 : pairs ? lspill
                         : sp.half + sp.zs_len + sp.wm_len + lspill;
-    // shared memory of one unit: a pair of warps or one warp
-    const int uw = pairs ? 2 : 1;
+    // warps per shared row: more than two where that raises the warps of an SM
+    // by a fifth
+    sp.lgw = 1;
+    if (pairs && prune) {
+        const int most = max_warps > 0 ? std::min(max_warps, SKIP_WARPS) : SKIP_WARPS;
+        auto warps_of = [&](int lgw) {
+            const size_t unit = (size_t)sp.per_pair + ((size_t)sp.per_warp << lgw);
+            return (int)std::min<size_t>(std::max<size_t>(z.room / unit, longw ? 1 : 0), (size_t)(most >> lgw)) << lgw;
+        };
+        for (int lgw = 2; lgw <= MAX_LGW; ++lgw)
+            if (5 * warps_of(lgw) >= 6 * warps_of(sp.lgw)) sp.lgw = lgw;
+    }
+    // shared memory of one unit: the warps that share a row, or one warp
+    const int uw = pairs ? 1 << sp.lgw : 1;
     const size_t unit = (size_t)(sp.per_pair + uw * sp.per_warp) * 4;
     const size_t slack = prune ? WM_SLACK * 4 : 0;   // past the last warp's window maxima
     size_t fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4 + slack;
-    if (longw && fixed + (size_t)(LONG_MIN_WARPS / uw) * unit > (size_t)smem_optin) {
+    if (longw && fixed + (size_t)std::max(1, LONG_MIN_WARPS / uw) * unit > (size_t)smem_optin) {
         // Rows of more than about 10^4 samples: the whole table and several
         // staged rows do not fit together.  Keep LONG_MIN_WARPS warps (or as
         // many as fit) and a table of what is left (at least MIN_TABLE
         // entries); the long-walk sweep computes the entries past its end.
         const size_t base = (size_t)sp.istart_len * 4 + slack;
-        int w = LONG_MIN_WARPS / uw;
+        int w = std::max(1, LONG_MIN_WARPS / uw);
         const size_t min_tab = (size_t)tab_floats_for(MIN_TABLE, prune != 0, cert != 0) * 4;
         while (w > 1 && base + min_tab + (size_t)w * unit > (size_t)smem_optin) --w;
         if (base + 16 * 4 + (size_t)w * unit >= (size_t)smem_optin) return cudaErrorInvalidConfiguration;
@@ -2393,9 +2420,9 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         else kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
     } else if (pairs) {
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = wide ? WW : prune && !longw ? SKIP_WARPS : CW;
+        most = wide ? WW : prune ? SKIP_WARPS : CW;
         if (wide) kern = sweep_pair_kernel<false, false, WW>;
-        else kern = prune ? (longw ? sweep_pair_kernel<true, true, CW> : sweep_pair_kernel<true, false, SKIP_WARPS>)
+        else kern = prune ? (longw ? sweep_pair_kernel<true, true, SKIP_WARPS> : sweep_pair_kernel<true, false, SKIP_WARPS>)
                           : (longw ? sweep_pair_kernel<false, true, CW> : sweep_pair_kernel<false, false, CW>);
     } else {
         most = FW;
