@@ -194,23 +194,23 @@ void tvs_batch_destroy(tvs_batch_handle b);
 
 /* Launch choices of a handle (no effect on results, only on speed, except
  * fp32_decisions).
- * small_pov_below_w: every skewed row of a direction whose walk axis is
- *   shorter than this is swept with 4 POVs per lane group (default 0: none);
- * p4_cost_pct: the other rows pick 4 or 8 POVs per lane group row by row,
+ * small_pov_below_w: unpruned FP32 sweeps take every skewed row of a direction
+ *   whose walk axis is shorter than this with 4 POVs per lane group (default
+ *   0: none; the other sweeps always take 4);
+ * p4_cost_pct: their other rows pick 4 or 8 POVs per lane group row by row,
  *   whichever needs fewer warp items x walk steps x POVs x step cost, where a
  *   4-POV step costs p4_cost_pct percent of an 8-POV step per POV (default
  *   107; 1 << 20 keeps every such row on 8; 0 in tvs_set_tuning = default);
- * sweep_max_warps: warps per sweep CTA, 0 = as many as shared memory allows,
- *   at most 16 (default 0; certified launches whose rows need one staged row
- *   per pair of warps take at most 12 when pruning, where the 12-warp build
- *   runs without register spills and was measured faster);
+ * sweep_max_warps: warps per sweep CTA, at most 16; 0 (default) = as many as
+ *   shared memory allows, up to 16, or 20 in pruned certified launches whose
+ *   warps hold one row each;
  * unskew_ctas_per_sm: a chunk whose DEMs have fewer cell tiles than this many
  *   per SM splits its directions into ranges across CTAs (1 to 4, default 2);
  * prune: exact horizon pruning in the sweep (1, default) or none (0): a group
- *   of POVs stops walking once no remaining target can rise above its running
- *   maximum elevation angle (bounded through the row's suffix maximum with
- *   monotone rounding), which leaves every result bit for bit the same;
- *   the work count (evaluations) stays the unpruned one.
+ *   of POVs skips every block of targets none of which can rise above its
+ *   running maximum elevation angle, and stops once no remaining one can
+ *   (bounded through maxima of the row), which leaves every result bit for bit
+ *   the same; the work count (evaluations) stays the unpruned one.
  * fp32_decisions: 0 (default) takes every visibility decision (Alg. 8's
  *   comparison of a target's elevation angle with the running maximum) as
  *   exact arithmetic on the blended heights takes it -- FP32 decisions proved
@@ -284,7 +284,7 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
                            int32_t* cv, int32_t* R, int32_t* W);
 
 /* Test hook: the sweep checks the indices of its staging, per-block margins,
- * flagged-POV list and exact walks against their buffers; the first violation
+ * flag buffer and exact walks against their buffers; the first violation
  * on the current device (code, index, bound, CTA; all zero when none) is
  * copied to out[0..3] after a device synchronisation, and cleared when
  * `clear` is non-zero.  A violation means a library bug: the access was
@@ -292,12 +292,12 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
 int tvs_debug_sweep_check(int32_t* out, int clear);
 
 /* Test and profiling hook: event counts of the certified sweep on the current
- * device since the last clear, after a device synchronisation: out[0] exact
- * walks (POVs with a decision inside its FP32 margin), out[1] of them walked
- * in FP64 (a decision inside the double-float margin too), out[2] SM clock
- * cycles warps spent walking flagged POVs exactly, out[3] cycles warps spent
- * in the certified sweep in all (out[2] / out[3] is the share of the exact
- * walks).  out holds 4 entries.  Errors: TVS_ERR_ARG, TVS_ERR_CUDA. */
+ * device since the last clear, after a device synchronisation: out[0] walks
+ * (unpruned) or 16-step blocks of walks (pruned) that held a decision inside
+ * its FP32 margin and were decided again exactly, out[1] of them in FP64 (a
+ * decision inside the double-float margin too), out[2] SM clock cycles warps
+ * spent in the exact pass, out[3] in the certified sweep kernels.  out holds 4
+ * entries.  Errors: TVS_ERR_ARG, TVS_ERR_CUDA. */
 int tvs_debug_sweep_stats(uint64_t* out, int clear);
 
 /* Turn per-kernel timing on (1) or off (0); turning it on clears the counters.

@@ -190,8 +190,8 @@ def sweep_check(clear: bool = True) -> list[int]:
 
 def sweep_stats(clear: bool = True) -> dict:
     """tvs_debug_sweep_stats: event counts of the certified sweep on the
-    current device (exact walks, FP64 walks, warp cycles in exact walks and
-    in the sweep)."""
+    current device (walks or blocks decided again exactly, of them in FP64,
+    warp cycles in the exact pass and in the sweep)."""
     out = (C.c_uint64 * 4)()
     _check(load().tvs_debug_sweep_stats(out, int(clear)))
     return {"exact_walks": int(out[0]), "fp64_walks": int(out[1]), "exact_cycles": int(out[2]),

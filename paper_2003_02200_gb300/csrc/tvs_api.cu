@@ -240,7 +240,7 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
     unsigned* d_cnt = reinterpret_cast<unsigned*>(ws + L.counter);
     TVS_CUDA(launch_rowmap(d_dir, 1, v.R, d_lo, d_hi, d_cnt, s), "rowmap launch");
     TVS_CUDA(launch_sweep(d_dir, d_jobs, reinterpret_cast<const int*>(ws + L.istart), 1, c.items, d_lo, d_hi, d_cv,
-                          d_cb, v.W, v.K, h->tuning.prune, !h->tuning.fp32_decisions, d_cnt,
+                          d_cb, v.W, v.K, c.ranged, h->tuning.prune, !h->tuning.fp32_decisions, d_cnt,
                           reinterpret_cast<int4*>(ws + L.flags), d_cnt + FLAG_COUNT, (int)L.flag_cap, h->num_sms, h->smem_optin, h->tuning.sweep_max_warps, s),
              "sweep launch");
     std::vector<int> slab(c.slab_elems), slabb(c.slab_elems), lo(v.R), hi(v.R);
@@ -495,15 +495,17 @@ extern "C" int tvs_total_viewshed_device_noalloc(const float* d_dem, int rows, i
     for (int c = 0; c < nchunks; ++c) {
         const int k0 = chunk_k0[c], nd = chunk_k0[c + 1] - k0;
         int max_R = 0, wmax = 0, dmax = 0;
+        bool ranged = false;
         for (int q = k0; q < k0 + nd; ++q) {
             dmax = std::max(dmax, dirs[q].K);
+            ranged = ranged || walk_limited(dirs[q].K, dirs[q].W);
             max_R = std::max(max_R, dirs[q].R);
             wmax = std::max(wmax, dirs[q].W);
         }
         const DirDev* cd = d_dirs + k0;
         TVS_CUDA(launch_rowmap(cd, nd, max_R, d_rowlo, d_rowhi, d_counter, s), "rowmap launch");
         TVS_CUDA(launch_sweep(cd, d_job, d_istart + at, nd, istart[at + nd], d_rowlo, d_rowhi, d_cvf, d_cvb, wmax,
-                              dmax, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_counter + FLAG_COUNT, flag_cap,
+                              dmax, ranged, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_counter + FLAG_COUNT, flag_cap,
                               num_sms, smem_optin, tn.sweep_max_warps, s),
                  "sweep launch");
         TVS_CUDA(launch_unskew(d_cvf, d_cvb, d_job, cd, d_cj + c, 1, tiles, cjs[c].nsplit, d_part, s),

@@ -111,6 +111,7 @@ struct Chunk {
     long long rows;          // sum of R
     int items;               // sweep warp items
     int max_R, wmax, dmax;
+    bool ranged;             // walk_limited of some direction
     int cj_beg, ncj;         // the chunk's entries of the chunk-job table
     int total_tiles, max_split;
     long long total_cells, part_elems;

@@ -121,6 +121,10 @@ struct ChunkJob {
     int pad_;
 };
 
+// Whether some walk of a direction may end at its range limit (K steps) rather
+// than at its row's end: a row's first sample walks up to W - 1 steps.
+constexpr bool walk_limited(int K, int W) { return K < W - 1; }
+
 // Launchers (tvs_kernels.cu).  All are asynchronous on `stream`.
 // The row tables of a chunk; also clears the COUNTER_WORDS counters of the
 // chunk's other kernels (the sweep's work counter, at FLAG_COUNT its flag
@@ -133,14 +137,15 @@ cudaError_t launch_colmap(const DirDev* d_dir, int* dest, unsigned* frac, cudaSt
 // direction (items 2p and 2p + 1 of a direction are row p forward and
 // backward), its row gathered from the job's DEM; `prune` turns exact horizon
 // pruning on, `cert` certified (exact) visibility decisions instead of FP32
-// ones.  With cert the walks the sweep cannot certify go to the flag buffer
+// ones; `ranged` (some walk may end at its range limit, walk_limited) picks the
+// pruned kernels that can cut a block there.  With cert the walks the sweep cannot certify go to the flag buffer
 // (flag_cap entries, possibly none; flag_count three counters; these and
 // `counter` are zero before the launch) and are walked
 // exactly by a second kernel on the same stream; those that find it full are
 // marked in their measures and found by a third.
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
                          int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
-                         int dmax, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
+                         int dmax, bool ranged, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
                          int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream);
 // Layout class of a certified sweep launch (rows up to wmax samples, walks
 // up to dmax steps, ndir directions): the warps of its one-row-per-warp

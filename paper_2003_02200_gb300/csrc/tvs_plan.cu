@@ -437,6 +437,7 @@ int plan_batch(const std::vector<JobSpec>& jobs, size_t avail, int num_sms, cons
             c.max_R = std::max(c.max_R, d.R);
             c.wmax = std::max(c.wmax, d.W);
             c.dmax = std::max(c.dmax, v.K);
+            c.ranged = c.ranged || walk_limited(v.K, v.W);
             const DirWork w = inst_work[t];
             c.evals += (double)w.evals;
             c.unskew_bytes += 8.0 * (double)w.samples;
@@ -603,7 +604,7 @@ int enqueue_chunks(tvs_ctx* h, const BatchPlan& plan, const Layout& L, char* bas
         {
             Timer t(h, K_SWEEP, s, c.evals);
             TVS_CUDA(launch_sweep(cd, d_jobs, d_istart + c.istart_at, nd, c.items, d_rowlo, d_rowhi, d_cvf, d_cvb,
-                                  c.wmax, c.dmax, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_fcount,
+                                  c.wmax, c.dmax, c.ranged, tn.prune, !tn.fp32_decisions, d_counter, d_flags, d_fcount,
                                   (int)L.flag_cap, num_sms, smem_optin, tn.sweep_max_warps, s),
                      "sweep launch");
         }

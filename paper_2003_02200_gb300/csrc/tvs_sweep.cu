@@ -559,10 +559,24 @@ constexpr int SKIP_RESTART = TVS_SKIP_RESTART;   // finished lanes before a prun
 #endif
 constexpr int SKIP_TESTS = TVS_SKIP_TESTS;
 constexpr int PACK_TESTS = TVS_PACK_TESTS;
+// Steps per pass of a block's evaluation loop: whole blocks save the loop where
+// registers allow (rows of a warp's own, 1000^2: 19.3 ms with 8, 18.3 with 16);
+// the kernel of shared rows, which has code for both walk directions, spills
+// (2000^2: 87.2 and 97.4 ms).
 #ifndef TVS_SKIP_CHUNK
 #define TVS_SKIP_CHUNK 8
 #endif
-constexpr int SKIP_CHUNK = TVS_SKIP_CHUNK;       // steps per pass of a block's evaluation loop
+#ifndef TVS_SINGLE_CHUNK
+#define TVS_SINGLE_CHUNK 16
+#endif
+#ifndef TVS_PACK_CHUNK
+#define TVS_PACK_CHUNK 8
+#endif
+#ifndef TVS_FP32_CHUNK
+#define TVS_FP32_CHUNK 16
+#endif
+constexpr int SKIP_CHUNK = TVS_SKIP_CHUNK, SINGLE_CHUNK = TVS_SINGLE_CHUNK, PACK_CHUNK = TVS_PACK_CHUNK;
+constexpr int FP32_CHUNK = TVS_FP32_CHUNK;
 #ifndef TVS_SKIP_UNROLL
 #define TVS_SKIP_UNROLL 16
 #endif
@@ -1382,6 +1396,13 @@ __device__ __forceinline__ float min3(float a, float b, float c)
 // Floats that a search may read past the last row's window maxima.
 constexpr int WM_SLACK = std::max(SKIP_TESTS, PACK_TESTS) * SKIP_UNROLL / ZS_STRIDE;
 
+// How a pruned walk takes the block that its range limit ends: there is none in
+// the launch; in a masked copy of the block's code beside it; or cut short in
+// the common code, so that its lanes run with the others (one row per warp,
+// 1000^2, 1.5 km: 15.3 ms masked, 14.8 cut; shared rows, 4000^2, 10 km: 205
+// masked, 211 cut).
+enum class RangeEnd { NONE, MASKED, CUT };
+
 // One round of a searching lane: tests NT blocks from step e on
 // against the lines T d + K of its four POVs (see sweep_row_skip) and returns
 // the first step that may hold a visible target (*ready), the walk's end when
@@ -1453,6 +1474,9 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // local memory per lane; 16 warps then lost to 12), form the window as they
 // go, and treat the inner groups of a row apart from its ends (92.6 -> 89.1).
 //
+// END says how the block in which the range limit ends the walks (at the same
+// step for every POV) is walked.
+//
 // Work is done in three warp-wide phases, each with as many lanes as possible:
 // finished groups are written and replaced (SKIP_RESTART lanes at a time, or
 // when no lane has work); lanes without a block test NT blocks at a
@@ -1462,13 +1486,12 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // block is evaluated SKIP_CHUNK steps at a time, with the window formed as it
 // goes: the few registers that takes let 20 warps share an SM, and their
 // number is what hides the latency of the tests.
-template <int P, int U, bool LONG, bool BWD, int NT>
+template <int P, int U, bool LONG, RangeEnd END, bool BWD, int NT, int CH>
 __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const SkipRow* __restrict__ rows,
                                                 const float* H0, int lgna, int groups, int lgs, int gsub, int zs_off,
                                                 int wm_off,
                                                 const float2* __restrict__ tab, int* __restrict__ spill, int lane)
 {
-    constexpr int CH = SKIP_CHUNK;
     static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
     const unsigned FULL = 0xffffffffu;
     const unsigned below = (1u << lane) - 1u;
@@ -1660,11 +1683,23 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                 };
                 quad(0, 0);
                 const int steps = min(dlim - e, U);
+                // RangeEnd::CUT: POV q's last target is element steps + q.
+                // Elements past `steps` are hidden from all POVs and the targets
+                // that POVs 1 to 3 still have among them taken one by one.
+                const bool cut = END == RangeEnd::CUT && klimited && steps < U;
+                if (cut) {
+#pragma unroll
+                    for (int m = 0; m < P; ++m) y[m] = m > steps ? neg_inf() : y[m];
+                }
 #pragma unroll 1
                 for (int c = 0; c < steps; c += CH) {
 #pragma unroll
                     for (int m = P; m < P + CH; m += 4) quad(BWD ? -(c + m) : c + m, m);
-                    if (klimited && c + CH > steps) {
+                    if (cut) {
+#pragma unroll
+                        for (int m = P; m < P + CH; ++m) y[m] = c + m > steps ? neg_inf() : y[m];
+                    }
+                    if (END == RangeEnd::MASKED && klimited && c + CH > steps) {
                         if (far) cert_block<P, CH, true, true, PACK>(y, tab, e + c, ng2, M2, blk2, mn, steps - c);
                         else cert_block<P, CH, true, false, PACK>(y, tb + c, e + c, ng2, M2, blk2, mn, steps - c);
                     } else {
@@ -1673,6 +1708,27 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                     }
 #pragma unroll
                     for (int m = 0; m < P; ++m) y[m] = y[m + CH];
+                }
+                if (cut) {
+#pragma unroll
+                    for (int q = 1; q < P; ++q) {
+                        float2& M = M2[q / 2];
+                        float2& A = blk2[q / 2];
+#pragma unroll
+                        for (int k = 0; k < q; ++k) {
+                            const int w = steps - q + k;     // element steps + 1 + k
+                            if (w < 0) continue;
+                            const int at = BWD ? P - 1 - (steps + 1 + k) : steps + 1 + k;
+                            const float yk = __fadd_rn(__fsub_rn(bh[at], Rh), bl[at]);
+                            const float iv = far ? __frcp_rn((float)(e + w + 1)) : tb[w].x;
+                            const float x = __fmul_rn(__fadd_rn(yk, q % 2 ? ng2[q / 2].y : ng2[q / 2].x), iv);
+                            const float sx = __fsub_rn(x, q % 2 ? M.y : M.x);
+                            const float add = __fmul_rn(sat_pos(sx), (float)(2 * (e + w) + 3));
+                            if (q % 2) { A.y = __fadd_rn(A.y, add); M.y = fmaxf(M.y, x); }
+                            else { A.x = __fadd_rn(A.x, add); M.x = fmaxf(M.x, x); }
+                            mn[q] = fminf(mn[q], fabsf(sx));
+                        }
+                    }
                 }
             }
             // the margin test of sweep_row_cert, and the lines of the next tests
@@ -1729,14 +1785,14 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
 // 1201 x 777, 180 directions: 19.5 -> 13.5 ms against the walk that only
 // stopped (8 POVs and 28 steps per block: larger blocks hold a visible target
 // more often).
-template <int P, int U, bool LONG>
+template <int P, int U, bool LONG, bool RANGED>
 __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const float* __restrict__ F,
                                                  const float* __restrict__ ZS, const float* __restrict__ WM,
                                                  const float2* __restrict__ tab, int* __restrict__ cvrow,
                                                  int* __restrict__ spill, int L, int K, float h0, float zmax,
                                                  bool rev, int lane)
 {
-    constexpr int CH = SKIP_CHUNK;
+    constexpr int CH = FP32_CHUNK;
     static_assert(P == 4 && U % 8 == 0 && U % CH == 0 && CH % 4 == 0, "groups of four, window loads 16-byte aligned");
     const unsigned FULL = 0xffffffffu;
     const unsigned below = (1u << lane) - 1u;
@@ -1819,19 +1875,40 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
             };
             quad(0, 0);
             const int steps = min(dlim - e, U);
+            // the block that the range limit cuts, as in sweep_rows_skip
+            const bool cut = RANGED && klimited && steps < U;
+            if (cut) {
+#pragma unroll
+                for (int m = 0; m < P; ++m) w[m] = m > steps ? NEG : w[m];
+            }
 #pragma unroll 1
             for (int c = 0; c < steps; c += CH) {
 #pragma unroll
                 for (int m = P; m < P + CH; m += 4) quad(c + m, m);
-                if (klimited && c + CH > steps) {
-                    if (far) sweep_block<P, CH, true, true>(w, tab, e + c, h, M, acc2, steps - c);
-                    else sweep_block<P, CH, true, false>(w, tb + c, e + c, h, M, acc2, steps - c);
-                } else {
-                    if (far) sweep_block<P, CH, false, true>(w, tab, e + c, h, M, acc2, CH);
-                    else sweep_block<P, CH, false, false>(w, tb + c, e + c, h, M, acc2, CH);
+                if (cut) {
+#pragma unroll
+                    for (int m = P; m < P + CH; ++m) w[m] = c + m > steps ? NEG : w[m];
                 }
+                if (far) sweep_block<P, CH, false, true>(w, tab, e + c, h, M, acc2, CH);
+                else sweep_block<P, CH, false, false>(w, tb + c, e + c, h, M, acc2, CH);
 #pragma unroll
                 for (int m = 0; m < P; ++m) w[m] = w[m + CH];
+            }
+            if (cut) {
+#pragma unroll
+                for (int q = 1; q < P; ++q) {
+#pragma unroll
+                    for (int k = 0; k < q; ++k) {
+                        const int u = steps - q + k;
+                        if (u < 0) continue;
+                        const float iv = far ? __frcp_rn((float)(e + u + 1)) : tb[u].x;
+                        const float t = __fmul_rn(__fsub_rn(base[steps + 1 + k], h[q]), iv);
+                        const float add = __fmul_rn(fset_gt(t, M[q]), (float)(2 * (e + u) + 3));
+                        if (q % 2) acc2[q / 2].y = __fadd_rn(acc2[q / 2].y, add);
+                        else acc2[q / 2].x = __fadd_rn(acc2[q / 2].x, add);
+                        M[q] = fmaxf(M[q], t);
+                    }
+                }
             }
             rising = true;
 #pragma unroll
@@ -1885,7 +1962,7 @@ static_assert(CERT_MAX_WARPS % 2 == 0 && CERT_WIDE_WARPS % 2 == 0, "certified wa
 // the flushing walk).  Per warp, shared memory holds the staged row (reversed
 // for backward items), its suffix maxima (PRUNE) and the long-walk spill
 // (LONG).
-template <bool PRUNE, bool LONG, int WARPS>
+template <bool PRUNE, bool LONG, bool RANGED, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1925,7 +2002,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
             end_max<false>(Fh, ZS, it.L, lane);
             window_max<SMALL_POV, SKIP_UNROLL>(Fh, WM, it.L, lane);
             __syncwarp();
-            sweep_row_skip32<SMALL_POV, SKIP_UNROLL, LONG>(sp, Fh, ZS, WM, tab, cvrow, spill, it.L, it.K, it.h0, zmax,
+            sweep_row_skip32<SMALL_POV, SKIP_UNROLL, LONG, RANGED>(sp, Fh, ZS, WM, tab, cvrow, spill, it.L, it.K, it.h0, zmax,
                                                            it.rev, lane);
         } else {
             sweep_item<LONG>(it, Fh, tab, sp.inv_len, cvrow, spill, lane);
@@ -1989,7 +2066,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
 // at 20 warps instead of 16: 1000^2 21.9 -> 20.5 ms).  Per warp, shared memory
 // holds the rows' SkipRows and per row [Fh half][Fl half][suffix maxima]
 // [window maxima].
-template <int WARPS, int NT>
+template <bool RANGED, int WARPS, int NT, int CH>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
@@ -2056,7 +2133,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
         }
         __syncwarp();
         if (longest > 0)
-            sweep_rows_skip<CERT_POV, U, false, false, NT>(sp, rows, arrays + ROW_PADL, sp.lgna,
+            sweep_rows_skip<CERT_POV, U, false, RANGED ? RangeEnd::CUT : RangeEnd::NONE, false, NT, CH>(sp, rows, arrays + ROW_PADL, sp.lgna,
                                                        (longest + CERT_POV - 1) / CERT_POV, 0, 0, zs_off, wm_off, tab,
                                                        nullptr, lane);
     }
@@ -2084,7 +2161,7 @@ __device__ __forceinline__ void row_sync(int row, int lgw)
 constexpr int MAX_LGW = 4;
 constexpr int ROW_XCH = 4 + (1 << MAX_LGW);   // floats of the exchange
 
-template <bool PRUNE, bool LONG, int WARPS>
+template <bool PRUNE, bool LONG, bool RANGED, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
@@ -2105,6 +2182,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     float* xch = ends + 4;                                   // item number and the halves' zmax
     // the row as either walk direction sees it (pruned)
     SkipRow* row = reinterpret_cast<SkipRow*>(xch + ROW_XCH) + bwd;
+    constexpr RangeEnd END = RANGED ? RangeEnd::MASKED : RangeEnd::NONE;
     float* own = base + npairs * sp.per_pair + warp * sp.per_warp;
     int* spill = reinterpret_cast<int*>(own) + lane;
     for (int m = threadIdx.x; m < sp.inv_len; m += blockDim.x) {
@@ -2150,10 +2228,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                 const int groups = ok ? (it.L + CERT_POV - 1) / CERT_POV : 0;
                 const int zs_off = (int)(ZS - H), wm_off = (int)(WM - H);
                 if (bwd)
-                    sweep_rows_skip<CERT_POV, U, LONG, true, SKIP_TESTS>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
+                    sweep_rows_skip<CERT_POV, U, LONG, END, true, SKIP_TESTS, SKIP_CHUNK>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
                                                                      wm_off, tab, spill, lane);
                 else
-                    sweep_rows_skip<CERT_POV, U, LONG, false, SKIP_TESTS>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
+                    sweep_rows_skip<CERT_POV, U, LONG, END, false, SKIP_TESTS, SKIP_CHUNK>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
                                                                      wm_off, tab, spill, lane);
             } else {
                 const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, cv, false);
@@ -2323,7 +2401,7 @@ int cert_sweep_class(int wmax, int dmax, int prune, int ndir, int smem_optin)
 
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
                          int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
-                         int dmax, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
+                         int dmax, bool ranged, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
                          int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream)
 {
     if (ndir <= 0 || total_items <= 0) return cudaSuccess;
@@ -2416,18 +2494,24 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
         const bool pack = sp.lgna > 0;
         most = prune ? (pack ? PACK_WARPS : SINGLE_WARPS) : wide ? WW : CW;
-        if (prune) kern = pack ? sweep_pack_kernel<PACK_WARPS, PACK_TESTS> : sweep_pack_kernel<SINGLE_WARPS, SKIP_TESTS>;
-        else kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
+        if (!prune) kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
+        else if (pack) kern = ranged ? sweep_pack_kernel<true, PACK_WARPS, PACK_TESTS, PACK_CHUNK>
+                                     : sweep_pack_kernel<false, PACK_WARPS, PACK_TESTS, PACK_CHUNK>;
+        else kern = ranged ? sweep_pack_kernel<true, SINGLE_WARPS, SKIP_TESTS, SINGLE_CHUNK>
+                           : sweep_pack_kernel<false, SINGLE_WARPS, SKIP_TESTS, SINGLE_CHUNK>;
     } else if (pairs) {
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
         most = wide ? WW : prune ? SKIP_WARPS : CW;
-        if (wide) kern = sweep_pair_kernel<false, false, WW>;
-        else kern = prune ? (longw ? sweep_pair_kernel<true, true, SKIP_WARPS> : sweep_pair_kernel<true, false, SKIP_WARPS>)
-                          : (longw ? sweep_pair_kernel<false, true, CW> : sweep_pair_kernel<false, false, CW>);
+        if (wide) kern = sweep_pair_kernel<false, false, true, WW>;
+        else if (!prune) kern = longw ? sweep_pair_kernel<false, true, true, CW> : sweep_pair_kernel<false, false, true, CW>;
+        else if (longw) kern = sweep_pair_kernel<true, true, true, SKIP_WARPS>;
+        else kern = ranged ? sweep_pair_kernel<true, false, true, SKIP_WARPS>
+                           : sweep_pair_kernel<true, false, false, SKIP_WARPS>;
     } else {
         most = FW;
-        kern = prune ? (longw ? sweep_kernel<true, true, FW> : sweep_kernel<true, false, FW>)
-                     : (longw ? sweep_kernel<false, true, FW> : sweep_kernel<false, false, FW>);
+        if (!prune) kern = longw ? sweep_kernel<false, true, true, FW> : sweep_kernel<false, false, true, FW>;
+        else if (longw) kern = sweep_kernel<true, true, true, FW>;
+        else kern = ranged ? sweep_kernel<true, false, true, FW> : sweep_kernel<true, false, false, FW>;
     }
     const int cap = max_warps > 0 ? std::max(std::min(max_warps, most), uw) : most;
     const int units = (int)std::min<size_t>(fit, (size_t)(cap / uw));

@@ -35,12 +35,12 @@ def _terrain(kind, rows, cols, seed):
     return (z + r.uniform(0.0, 3.0, (rows, cols))).astype(np.float32)
 
 
-def _check(ctx, orc, dem, h0, n, rng, ks):
+def _check(ctx, orc, dem, h0, n, rng, ks, prec=64):
     rows, cols = dem.shape
     for k in ks:
         got = ctx.debug_direction_cv(dem, 10.0, h0, n, rng, k)
         d = orc.direction(n, k, rows, cols)
-        want = np.stack([orc.line_cv(dem, 10.0, h0, n, rng, 64, k, p - d["D"]) for p in range(d["H"] + d["D"])])
+        want = np.stack([orc.line_cv(dem, 10.0, h0, n, rng, prec, k, p - d["D"]) for p in range(d["H"] + d["D"])])
         bad = np.argwhere(got != want)
         assert bad.size == 0, f"k {k}: {len(bad)} samples differ, first {bad[:4].tolist()}"
 
@@ -58,14 +58,33 @@ def test_walk_limits(ctx, orc, kind, rng):
     _check(ctx, orc, _terrain(kind, 6, 150, 5), 2.0, 12, rng, (0, 2, 11))
 
 
-# rows of 1100 to 2300 samples take the paired-warp layout, shorter ones one row per warp
+# rows of more than about 1200 samples are shared by two warps, shorter ones are a warp's own
 @pytest.mark.parametrize("cols", [1000, 1351, 2003, 2300])
 @pytest.mark.parametrize("kind", ["fractal", "valley", "ridge", "sawtooth"])
 def test_long_rows(ctx, orc, kind, cols):
     _check(ctx, orc, _terrain(kind, 3, cols, 9), 1.5, 8, 0.0, (0, 7))
 
 
-@pytest.mark.parametrize("rows,cols", [(260, 300), (3, 2100)])
+@pytest.mark.parametrize("limit", list(range(1, 21)) + [31, 32, 33, 34, 47, 48, 49])
+@pytest.mark.parametrize("cols", [71, 1500])
+def test_every_place_of_a_limit_in_a_block(ctx, orc, cols, limit):
+    """Walks of 1 to 49 steps: the block that the limit ends, for one row per
+    warp and for shared rows, certified and with FP32 decisions."""
+    dem = _terrain("fractal", 3, cols, 40 + limit)
+    _check(ctx, orc, dem, 1.5, 4, 10.0 * limit + 1.0, (0,))
+    with tvs.Context(0) as c:
+        c.set_tuning(fp32_decisions=1)
+        _check(c, orc, dem, 1.5, 4, 10.0 * limit + 1.0, (0,), prec=32)
+
+
+# rows that 2, 4, 8 and 16 warps share, and walks long enough to flush their measures
+@pytest.mark.parametrize("cols,rng", [(2500, 0.0), (3300, 0.0), (3300, 12345.0), (5000, 0.0), (5000, 45678.0),
+                                      (9000, 0.0), (16384, 0.0)])
+def test_rows_shared_by_many_warps(ctx, orc, cols, rng):
+    _check(ctx, orc, _terrain("fractal", 2, cols, 17), 1.5, 4, rng, (0,))
+
+
+@pytest.mark.parametrize("rows,cols", [(260, 300), (3, 2100), (2, 9000)])
 def test_full_flag_buffer(ctx, rows, cols):
     """Level ground seen from its own height: every target ties with the
     running maximum, so nearly every walk is flagged and the buffer (one entry
