@@ -185,12 +185,9 @@ int tvs_debug_plan(const int32_t* rows, const int32_t* cols, const int32_t* n_se
     Tuning tn;
     tn.prune = prune != 0;
     tn.fp32_decisions = fp32_decisions != 0;
-    // the budget split of a batch call (run_batch): fixed parts first, the rest for chunks
-    const size_t budget = (size_t)budget_bytes;
-    const size_t fixed = fixed_bytes(jobs, false, num_sms, budget_flags(budget));
-    if (fixed >= budget) return fail(TVS_ERR_OOM, "the DEMs do not fit the HBM budget");
     BatchPlan plan;
-    const int rc = plan_batch(jobs, budget - fixed, num_sms, tn, &plan, -1, smem_optin);
+    size_t max_flags = 0;
+    const int rc = plan_within(jobs, (size_t)budget_bytes, false, num_sms, tn, &plan, smem_optin, &max_flags);
     if (rc) return rc;
     const int n = (int)plan.inst_job.size();
     for (int q = 0; q < (int)plan.chunks.size(); ++q)
@@ -585,12 +582,10 @@ int tvs_batch_create(tvs_handle h, const tvs_job* jobs, int njobs, size_t hbm_bu
     if (rc) return rc;
     DeviceGuard g(h->device);
     const size_t budget = hbm_budget_bytes ? hbm_budget_bytes : h->budget;
-    const size_t mf = budget_flags(budget);
-    const size_t fixed = fixed_bytes(specs, false, h->num_sms, mf);
-    if (fixed >= budget) return fail(TVS_ERR_OOM, "the DEMs do not fit the HBM budget");
     tvs_batch* b = new tvs_batch();
     b->h = h;
-    rc = plan_batch(specs, budget - fixed, h->num_sms, h->tuning, &b->plan, -1, h->smem_optin);
+    size_t mf = 0;
+    rc = plan_within(specs, budget, false, h->num_sms, h->tuning, &b->plan, h->smem_optin, &mf);
     if (rc) { delete b; return rc; }
     b->L = make_layout(b->plan, false, mf);
     cudaError_t e = cudaMalloc(&b->ws, b->L.total);

@@ -159,6 +159,10 @@ Layout make_layout(const BatchPlan& plan, bool host_io, size_t max_flags = FLAG_
 size_t fixed_bytes(const std::vector<JobSpec>& jobs, bool host_io, int num_sms, size_t max_flags);
 // The flagged-walk buffer entries a scratch budget allows: a sixteenth of it.
 size_t budget_flags(size_t budget);
+// Plans `jobs` within a scratch budget: the fixed parts first, the rest for
+// chunks; *max_flags is what make_layout then takes.
+int plan_within(const std::vector<JobSpec>& jobs, size_t budget, bool host_io, int num_sms, const Tuning& tn,
+                BatchPlan* plan, int smem_optin, size_t* max_flags);
 // Host image of the header for the scratch at `base`.
 void build_header(const BatchPlan& plan, const Layout& L, char* base, bool host_io, std::vector<char>* img);
 

@@ -501,13 +501,13 @@ int plan_batch(const std::vector<JobSpec>& jobs, size_t avail, int num_sms, cons
 // samples and to 1 in 10 at 8000; what finds the buffer full is searched for
 // and walked whole, at a cost), at least 4096, at most `cap` and
 // FLAG_BUF_ENTRIES.
-size_t flag_entries(const std::vector<JobSpec>& jobs, size_t cap)
+size_t flag_entries(const std::vector<JobSpec>& jobs, size_t cap, bool scaled = true)
 {
     double walks = 0.0;
     for (const JobSpec& J : jobs) {
         const int nd = J.k1 > J.k0 ? J.k1 - J.k0 : J.n;   // the job's directions in this call
         walks += 2.0 * (double)J.rows * (double)J.cols * (double)nd *
-                 std::max(1.0, (double)std::max(J.rows, J.cols) / 1024.0);
+                 (scaled ? std::max(1.0, (double)std::max(J.rows, J.cols) / 1024.0) : 1.0);
     }
     return (size_t)std::min<double>((double)std::min<size_t>(cap, FLAG_BUF_ENTRIES), std::max(4096.0, walks / 64.0));
 }
@@ -515,6 +515,22 @@ size_t flag_entries(const std::vector<JobSpec>& jobs, size_t cap)
 size_t budget_flags(size_t budget)
 {
     return std::min<size_t>((size_t)FLAG_BUF_ENTRIES, budget / 16 / FLAG_ENTRY_BYTES);
+}
+
+int plan_within(const std::vector<JobSpec>& jobs, size_t budget, bool host_io, int num_sms, const Tuning& tn,
+                BatchPlan* plan, int smem_optin, size_t* max_flags)
+{
+    int rc = TVS_ERR_OOM;
+    *max_flags = budget_flags(budget);
+    for (int pass = 0; pass < 2 && rc == TVS_ERR_OOM; ++pass) {
+        // second pass: the flag buffer without its allowance for long rows
+        if (pass) *max_flags = std::min(*max_flags, flag_entries(jobs, *max_flags, false));
+        *plan = BatchPlan();
+        const size_t fixed = fixed_bytes(jobs, host_io, num_sms, *max_flags);
+        rc = fixed >= budget ? fail(TVS_ERR_OOM, "the DEMs do not fit the HBM budget")
+                             : plan_batch(jobs, budget - fixed, num_sms, tn, plan, -1, smem_optin);
+    }
+    return rc;
 }
 
 Layout make_layout(const BatchPlan& plan, bool host_io, size_t max_flags)
@@ -654,11 +670,9 @@ int upload_header(tvs_ctx* h, const std::vector<char>& img, void* dst, cudaStrea
 int run_batch(tvs_ctx* h, const std::vector<JobSpec>& jobs, cudaStream_t s, bool host_io, const float* host_dem,
               float* host_out)
 {
-    const size_t mf = budget_flags(h->budget);
-    const size_t fixed = fixed_bytes(jobs, host_io, h->num_sms, mf);
-    if (fixed >= h->budget) return fail(TVS_ERR_OOM, "the DEMs do not fit the HBM budget");
     BatchPlan plan;
-    int rc = plan_batch(jobs, h->budget - fixed, h->num_sms, h->tuning, &plan, -1, h->smem_optin);
+    size_t mf = 0;
+    int rc = plan_within(jobs, h->budget, host_io, h->num_sms, h->tuning, &plan, h->smem_optin, &mf);
     if (rc) return rc;
     const Layout L = make_layout(plan, host_io, mf);
     rc = ensure_scratch(h, L.total);

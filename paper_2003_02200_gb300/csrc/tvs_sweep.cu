@@ -2534,7 +2534,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     exact_kernel<<<xper * num_sms, EXACT_WARPS * 32, 0, stream>>>(sp);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    exact_scan_kernel<<<num_sms, EXACT_WARPS * 32, 0, stream>>>(sp);
+    exact_scan_kernel<<<2 * num_sms, EXACT_WARPS * 32, 0, stream>>>(sp);   // two resident CTAs per SM
     return cudaGetLastError();
 }
 
