@@ -989,7 +989,7 @@ def run_points_bench(args) -> int:
                                        "largest area of the sample and mean over mean; sDEM places the observer "
                                        "on lines blended from neighbouring rows, so the gap grows when the "
                                        "ground between neighbours changes by more than the observer height"},
-            "gpu_launches": 4 * args.steps,
+            "gpu_launches": 3 * args.steps,
         }
         if not args.no_cpu_baseline:
             import oracle

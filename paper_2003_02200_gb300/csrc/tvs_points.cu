@@ -15,16 +15,15 @@
 //                     sDEM value measures the discretisation, as section 5
 //                     compares sDEM with TVS.
 //
-// One warp per (POV, group of FP32_GROUP directions): lane = 4 kk + 2 v + s
-// walks direction 8 g + kk, virtual POV v (hi / lo; DIRECT uses v = 0 only),
-// forward (s = 0) or backward (s = 1).  The walk is the sweep's: targets
-// d = 1 .. n (n = min(usable samples, K)), visible iff the target's slope is
-// strictly above the running maximum -- the exact decision (certified walks,
-// the default) or the FP32 one, (z - h) * rcp(d) (fp32_decisions) -- and
-// cv = 1 + sum_{d < n} v_d (2d + 1) for n >= 1 (the last target only closes a
-// segment).  Lane 0 adds the group's terms g * blend(cv) in direction order in
-// FP32 and stores the group sum as an exact partial; a finalize kernel adds
-// each POV's partials and applies the (pi/(2n)) step^2 scale.
+// One warp per half-line (POV, direction, virtual POV hi / lo, side; DIRECT has
+// one line per direction).  The walk is the sweep's: targets d = 1 .. n (n =
+// min(usable samples, K)), visible iff the target's slope is strictly above the
+// running maximum -- the exact decision (certified walks, the default) or the
+// FP32 one, (z - h) * rcp(d) (fp32_decisions) -- and cv = 1 + sum_{d < n} v_d
+// (2d + 1) for n >= 1 (the last target only closes a segment).  Each
+// direction's term is g * blend(cv); points_sum adds a POV's groups of
+// FP32_GROUP terms in FP32, in direction order, the groups exactly, and applies the
+// (pi/(2n)) step^2 scale.
 #include "tvs.h"
 #include "tvs_host.h"
 #include "tvs_internal.h"
@@ -47,7 +46,6 @@ struct PointsParams {
     const DirDev* dirs;     // the job's n directions (t_fx, frame, H, W, K, g)
     const int* pov;         // npov (row, col) pairs of DEM cells
     float* term;            // npov x n direction terms g * blend(cv)
-    __int128* part;         // npov x ngroups exact group sums
     float* area;            // npov visible areas
     double scale;           // (pi / (2n)) step^2
     int rows, cols, n, ngroups, npov, mode;
@@ -745,27 +743,29 @@ __global__ void __launch_bounds__(128 * POINTS_DIRS, CERT ? POINTS_MIN_CTAS : 1)
     pp.term[(long long)q * pp.n + k] = __fmul_rn(L.d.g, val);
 }
 
-// One thread per (POV, group of FP32_GROUP directions): the FP32 sum of the
-// group's terms in direction order, stored as one exact partial (the total
-// viewshed map's unskew adds its groups the same way).
-__global__ void points_groups(PointsParams pp)
+// One warp per POV: the FP32 sums of its groups of FP32_GROUP directions, in
+// direction order (the total viewshed map's unskew adds its groups the same
+// way), a group per lane at a time, added exactly; integer addition does not
+// depend on the order.  (A kernel for the groups and one for their sum, a
+// thread each, took 3.4 and 6.5 us of dependent loads and a launch.)
+__global__ void __launch_bounds__(128) points_sum(PointsParams pp)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)pp.npov * pp.ngroups) return;
-    const int q = (int)(t / pp.ngroups), grp = (int)(t % pp.ngroups);
+    const int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (q >= pp.npov) return;                    // warp-uniform
     const float* term = pp.term + (long long)q * pp.n;
-    float acc = 0.f;
-    for (int k = grp * FP32_GROUP; k < min(pp.n, (grp + 1) * FP32_GROUP); ++k) acc = __fadd_rn(acc, term[k]);
-    pp.part[t] = acc_of(acc);
-}
-
-__global__ void points_finalize(PointsParams pp)
-{
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= pp.npov) return;
     __int128 tot = 0;
-    for (int g = 0; g < pp.ngroups; ++g) tot += pp.part[(long long)q * pp.ngroups + g];
-    pp.area[q] = area_of(tot, pp.scale);
+    for (int grp = lane; grp < pp.ngroups; grp += 32) {
+        float acc = 0.f;
+        for (int k = grp * FP32_GROUP; k < min(pp.n, (grp + 1) * FP32_GROUP); ++k) acc = __fadd_rn(acc, term[k]);
+        tot += acc_of(acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)tot, o);
+        const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(tot >> 64), o);
+        tot += ((__int128)hi << 64) | (__int128)lo;
+    }
+    if (lane == 0) pp.area[q] = area_of(tot, pp.scale);
 }
 
 // ------------------------------------------------------------ visibility map --
@@ -818,18 +818,39 @@ __global__ void __launch_bounds__(256, CERT ? POINTS_MIN_CTAS : 1) map_flags_ker
     }
 }
 
+// Angle of (y, x), not both 0, in (-pi, pi], within 6e-7: the arctangent of
+// the smaller over the larger by Hastings' polynomial (Abramowitz and Stegun
+// 4.4.49, |error| <= 2e-8 on [0, 1]) in single precision, then the octant.
+__device__ __forceinline__ float angle_of(int y, int x)
+{
+    const float ay = (float)abs(y), ax = (float)abs(x);
+    const float t = __fdividef(fminf(ay, ax), fmaxf(ay, ax));
+    const float u = t * t;
+    float p = -0.0040540580f;
+    p = __fmaf_rn(p, u, 0.0218612288f);
+    p = __fmaf_rn(p, u, -0.0559098861f);
+    p = __fmaf_rn(p, u, 0.0964200441f);
+    p = __fmaf_rn(p, u, -0.1390853351f);
+    p = __fmaf_rn(p, u, 0.1994653599f);
+    p = __fmaf_rn(p, u, -0.3332985605f);
+    p = __fmaf_rn(p, u, 0.9999993329f);
+    float a = t * p;
+    if (ay > ax) a = 1.57079637f - a;
+    if (x < 0) a = 3.14159274f - a;
+    return y < 0 ? -a : a;
+}
+
 // One thread per cell: the sector of each POV it falls in (nearest of the 2n
 // half-line axes k' pi / n to the direction of the cell, the double-precision
 // decision kp = floor(atan2(di, dj) n / pi + 1/2) mod 2n) and the flag of the
 // target at the cell's walk-axis column.  The decision is taken from a
-// single-precision angle when it is far from a sector boundary: atan2f is
-// within a few ulp of the angle (|angle| <= pi, ulp 2^-22), so with the three
-// roundings of q = angle (n / pi) + 1/2 the single-precision q is within
-// about 4.1e-7 n of the double one; a cell whose q lies within
-// 1e-6 n + 1e-6 of a boundary takes the double-precision angle instead (a
-// warp takes that path, hundreds of FP64 instructions, when one of its 32
-// cells does, so the margin is kept tight: 4e-6 n sent 4.5 % of the warps
-// there at n = 180).
+// single-precision angle when it is far from a sector boundary: that angle is
+// within 6e-7 (angle_of), so with the three roundings of q = angle (n / pi) +
+// 1/2 (1.8e-7 n together) the single-precision q is within about 3.8e-7 n of
+// the double one; a cell whose q lies within 1e-6 n + 1e-6 of a boundary takes
+// the double-precision angle instead (a warp takes that path, hundreds of FP64
+// instructions, when one of its 32 cells does, so the margin is kept tight:
+// 4e-6 n sent 4.5 % of the warps there at n = 180).
 // A warp takes 8 x 4 cells and a CTA RASTER_X x RASTER_Y: seen from a POV such a
 // patch lies in a few sectors and a few distances, so the flags its cells
 // read fall in a few 32-byte sectors (a row of 32 cells reads up to 32 of
@@ -848,11 +869,13 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
     const float scale = (float)((double)mp.n / 3.141592653589793);
     const float margin = 1e-6f * (float)mp.n + 1e-6f;
     int seen = 0;
-    for (int q = 0; q < mp.npov; ++q) {
+    const unsigned char* flags = mp.flags;       // of POV q
+    const long long per_pov = (long long)2 * mp.n * mp.cap;
+    for (int q = 0; q < mp.npov; ++q, flags += per_pov) {
         const int i0 = mp.pov[2 * q], j0 = mp.pov[2 * q + 1];
         if (iD == i0 && jD == j0) { ++seen; continue; }
         const int di = iD - i0, dj = jD - j0;
-        const float x = __fadd_rn(__fmul_rn(atan2f((float)di, (float)dj), scale), 0.5f);
+        const float x = __fadd_rn(__fmul_rn(angle_of(di, dj), scale), 0.5f);
         const float fl = floorf(x);
         const float fx = x - fl;                  // exact
         int kp;
@@ -878,7 +901,7 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
         int dd = along_cols ? dj : first2 ? di : -di;
         if (!plus) dd = -dd;
         if (dd >= 1 && dd < mp.cap)
-            seen += mp.flags[((long long)q * 2 * mp.n + (plus ? k : mp.n + k)) * mp.cap + dd];
+            seen += flags[(long long)(plus ? k : mp.n + k) * mp.cap + dd];
     }
     mp.count[c] = seen;
 }
@@ -1070,8 +1093,7 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
     }
     const size_t o_dirs = 0, o_pov = align256((size_t)n_sectors * sizeof(DirDev));
     const size_t hdr = o_pov + align256((size_t)npov * 8);
-    const size_t o_part = hdr;
-    const size_t o_term = o_part + align256((size_t)npov * ngroups * 16);
+    const size_t o_term = hdr;
     const size_t o_tiles = o_term + align256((size_t)npov * n_sectors * 4);
     const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs);
     const size_t total = o_tiles + (tiles ? tile_bytes(rows, cols) : 0);
@@ -1086,7 +1108,6 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
     pp.dem = d_dem;
     pp.dirs = reinterpret_cast<const DirDev*>(h->ws + o_dirs);
     pp.pov = reinterpret_cast<const int*>(h->ws + o_pov);
-    pp.part = reinterpret_cast<__int128*>(h->ws + o_part);
     pp.term = reinterpret_cast<float*>(h->ws + o_term);
     pp.area = d_area;
     pp.scale = (M_PI / (2.0 * (double)n_sectors)) * (step_m * step_m);
@@ -1112,9 +1133,7 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
             TVS_CUDA(launch_tile_max(d_dem, rows, cols, reinterpret_cast<float*>(h->ws + o_tiles), s), "tile maxima");
         const long long ctas = (long long)npov * ((n_sectors + POINTS_DIRS - 1) / POINTS_DIRS);
         walk_kernel<<<(unsigned)ctas, 128 * POINTS_DIRS, rtab_bytes, s>>>(pp);
-        const long long groups = (long long)npov * ngroups;
-        points_groups<<<(unsigned)((groups + 127) / 128), 128, 0, s>>>(pp);
-        points_finalize<<<(npov + 127) / 128, 128, 0, s>>>(pp);
+        points_sum<<<(npov + 3) / 4, 128, 0, s>>>(pp);
     }
     TVS_CUDA(cudaGetLastError(), "points launch");
     return TVS_OK;

@@ -596,6 +596,10 @@ constexpr int SKIP_WARPS = TVS_SKIP_WARPS;       // most warps of a pruned certi
 #define TVS_PACK_WARPS 16
 #endif
 constexpr int SINGLE_WARPS = TVS_SINGLE_WARPS, PACK_WARPS = TVS_PACK_WARPS;
+#ifndef TVS_FP32_WARPS
+#define TVS_FP32_WARPS 20
+#endif
+constexpr int FP32_WARPS = TVS_FP32_WARPS;       // pruned FP32 decisions
 constexpr int SKIP_UNROLL = TVS_SKIP_UNROLL;   // steps per block of a pruned walk
 static_assert(SKIP_UNROLL <= ROW_PADL && CERT_POV + SKIP_UNROLL <= ROW_PADR && FLUSH_STEPS % SKIP_UNROLL == 0,
               "pads and flushes of a pruned walk");
@@ -2508,10 +2512,10 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         else kern = ranged ? sweep_pair_kernel<true, false, true, SKIP_WARPS>
                            : sweep_pair_kernel<true, false, false, SKIP_WARPS>;
     } else {
-        most = FW;
+        most = prune ? FP32_WARPS : FW;
         if (!prune) kern = longw ? sweep_kernel<false, true, true, FW> : sweep_kernel<false, false, true, FW>;
-        else if (longw) kern = sweep_kernel<true, true, true, FW>;
-        else kern = ranged ? sweep_kernel<true, false, true, FW> : sweep_kernel<true, false, false, FW>;
+        else if (longw) kern = sweep_kernel<true, true, true, FP32_WARPS>;
+        else kern = ranged ? sweep_kernel<true, false, true, FP32_WARPS> : sweep_kernel<true, false, false, FP32_WARPS>;
     }
     const int cap = max_warps > 0 ? std::max(std::min(max_warps, most), uw) : most;
     const int units = (int)std::min<size_t>(fit, (size_t)(cap / uw));
