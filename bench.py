@@ -313,9 +313,9 @@ def run_ours(args) -> int:
                  "fp64_walks_per_step": cert["fp64_walks"] / args.steps,
                  "exact_walk_fraction": cert["exact_walks"] / walks,
                  "exact_share_of_sweep_time": cert["exact_cycles"] / max(cert["sweep_cycles"], 1),
-                 "note": "walks (POV x direction x side) whose FP32 fast path had a decision inside its proven "
-                         "margin and were walked again exactly (double-float, FP64 past its margin); the share "
-                         "is of the warps' SM cycles in the sweep"}
+                 "note": "blocks of walks (POV x direction x side) with an FP32 decision inside its proven margin, "
+                         "decided again exactly (double-float, FP64 past its margin), per step and per walk; the "
+                         "share is of the warps' SM cycles in the sweep"}
     step_ms = [s.elapsed_time(e) for s, e in zip(starts, ends)]
     local_s = sum(step_ms) / 1e3
     total_evals, max_s = aggregate(float(E) * args.steps, local_s, dist, device)

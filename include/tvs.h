@@ -292,10 +292,10 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
 int tvs_debug_sweep_check(int32_t* out, int clear);
 
 /* Test and profiling hook: event counts of the certified sweep on the current
- * device since the last clear, after a device synchronisation: out[0] walks
- * (unpruned) or 16-step blocks of walks (pruned) that held a decision inside
- * its FP32 margin and were decided again exactly, out[1] of them in FP64 (a
- * decision inside the double-float margin too), out[2] SM clock cycles warps
+ * device since the last clear, after a device synchronisation: out[0]
+ * blocks of walks that held a decision inside its FP32 margin and were decided
+ * again exactly, out[1] of them in FP64 (a decision inside the double-float
+ * margin too), out[2] SM clock cycles warps
  * spent in the exact pass, out[3] in the certified sweep kernels.  out holds 4
  * entries.  Errors: TVS_ERR_ARG, TVS_ERR_CUDA. */
 int tvs_debug_sweep_stats(uint64_t* out, int clear);

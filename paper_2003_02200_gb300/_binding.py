@@ -190,7 +190,7 @@ def sweep_check(clear: bool = True) -> list[int]:
 
 def sweep_stats(clear: bool = True) -> dict:
     """tvs_debug_sweep_stats: event counts of the certified sweep on the
-    current device (walks or blocks decided again exactly, of them in FP64,
+    current device (blocks of walks decided again exactly, of them in FP64,
     warp cycles in the exact pass and in the sweep)."""
     out = (C.c_uint64 * 4)()
     _check(load().tvs_debug_sweep_stats(out, int(clear)))

@@ -840,6 +840,13 @@ __device__ __forceinline__ float angle_of(int y, int x)
     return y < 0 ? -a : a;
 }
 
+// floor(atan2(y, x) n / pi + 1/2) in double precision.
+__device__ __noinline__ int exact_sector(int y, int x, int n)
+{
+    const double q = atan2((double)y, (double)x) * (double)n / 3.141592653589793;
+    return (int)floor(q + 0.5);
+}
+
 // One thread per cell: the sector of each POV it falls in (nearest of the 2n
 // half-line axes k' pi / n to the direction of the cell, the double-precision
 // decision kp = floor(atan2(di, dj) n / pi + 1/2) mod 2n) and the flag of the
@@ -855,8 +862,9 @@ __device__ __forceinline__ float angle_of(int y, int x)
 // patch lies in a few sectors and a few distances, so the flags its cells
 // read fall in a few 32-byte sectors (a row of 32 cells reads up to 32 of
 // them).  Bound by instructions, the angle's above all: 10 POVs on 2000^2 take
-// 0.167 ms (0.174 a row of cells per warp; 0.26 with the margin of 4e-6 n;
-// 0.42 before, with the direction table read and 64-bit remainders per cell).
+// 0.154 ms (0.167 with atan2f; 0.174 also a row of cells per warp; 0.26 with
+// the margin of 4e-6 n; 0.42 with the direction table read and 64-bit
+// remainders per cell).
 constexpr int RASTER_X = 32, RASTER_Y = 8;
 
 __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapParams mp)
@@ -871,6 +879,7 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
     int seen = 0;
     const unsigned char* flags = mp.flags;       // of POV q
     const long long per_pov = (long long)2 * mp.n * mp.cap;
+#pragma unroll 2
     for (int q = 0; q < mp.npov; ++q, flags += per_pov) {
         const int i0 = mp.pov[2 * q], j0 = mp.pov[2 * q + 1];
         if (iD == i0 && jD == j0) { ++seen; continue; }
@@ -879,12 +888,8 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
         const float fl = floorf(x);
         const float fx = x - fl;                  // exact
         int kp;
-        if (fx > margin && fx < 1.0f - margin) {
-            kp = (int)fl;
-        } else {
-            const double qq = atan2((double)di, (double)dj) * (double)mp.n / 3.141592653589793;
-            kp = (int)floor(qq + 0.5);
-        }
+        if (fx > margin && fx < 1.0f - margin) kp = (int)fl;
+        else kp = exact_sector(di, dj, mp.n);
         // kp mod 2n: the angle lies in [-pi, pi], so kp in [-n, n]
         if (kp < 0) kp += 2 * mp.n;
         const bool half = kp < mp.n;
@@ -894,9 +899,9 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
         // the column in views 0 and 3, the row in view 1 and the reversed row in
         // view 2; +j of the view points along theta_k in views 0 and 1, along
         // theta_k + pi in views 2 and 3
-        const long long k4 = 4ll * k;
-        const bool first2 = k4 < 2ll * mp.n;
-        const bool along_cols = k4 < mp.n || k4 >= 3ll * mp.n;
+        const int k4 = 4 * k;                    // n <= 2^20
+        const bool first2 = k4 < 2 * mp.n;
+        const bool along_cols = k4 < mp.n || k4 >= 3 * mp.n;
         const bool plus = first2 == half;
         int dd = along_cols ? dj : first2 ? di : -di;
         if (!plus) dd = -dd;

@@ -511,8 +511,8 @@ __device__ __forceinline__ void window_max(const float* __restrict__ F, float* _
 // its end)), 1/(e+1) >= 1/d_t, ia >= 1/d_a (1/(e'+1) of the last block e' in
 // which M rose; 1 at first), Eg' >= Eg from the group's largest |g_q|.
 // Induction over the targets then makes every unflagged decision the exact
-// one.  A POV with a step inside its margin is flagged: its fast-path
-// measure is discarded and it is walked again exactly.
+// one.  A POV with a step inside its margin leaves the block to the exact pass
+// (flag_block); its M, the largest x whatever was decided, goes on.
 constexpr float CERT_REL = 10.2f * 0x1p-24f * 1.01f;
 constexpr float CERT_ABS = 1.03f * 1.01f;
 constexpr float CERT_FLOOR = 0x1p-99f;
@@ -599,7 +599,8 @@ constexpr int SINGLE_WARPS = TVS_SINGLE_WARPS, PACK_WARPS = TVS_PACK_WARPS;
 #ifndef TVS_FP32_WARPS
 #define TVS_FP32_WARPS 20
 #endif
-constexpr int FP32_WARPS = TVS_FP32_WARPS;       // pruned FP32 decisions
+// Pruned FP32 decisions (1201 x 777: 12.5 ms with 16 warps, 11.8 with 20).
+constexpr int FP32_WARPS = TVS_FP32_WARPS;
 constexpr int SKIP_UNROLL = TVS_SKIP_UNROLL;   // steps per block of a pruned walk
 static_assert(SKIP_UNROLL <= ROW_PADL && CERT_POV + SKIP_UNROLL <= ROW_PADR && FLUSH_STEPS % SKIP_UNROLL == 0,
               "pads and flushes of a pruned walk");
@@ -630,10 +631,10 @@ size_t tab_entries_fit(size_t floats, bool prune, bool cert)
     return cert ? (floats / 4 < 2 ? 0 : (floats / 4 - 2) * TAB_SKEW_MIN / (TAB_SKEW_MIN + 1)) : floats / 4;
 }
 // Far from the POV one margin serves several window blocks: from step
-// CERT_NEAR on a margin block is 2 window blocks long, from CERT_FAR on 4 and
-// from CERT_FAR2 on 8 (while the group's walks have that many steps left), so
-// that the finish vote, the margins and the last-rise update are taken once
-// per 32, 64 or 128 steps.  Near the POV, where the margin's 1/(e+1) terms
+// CERT_NEAR on a margin block is 2 window blocks long, from CERT_FAR on 4
+// (while the group's walks have that many steps left), so that the finish
+// vote, the margins and the last-rise update are taken once per 32 or 64
+// steps.  Near the POV, where the margin's 1/(e+1) terms
 // fall fastest, every window block takes its own.  The lanes of a warp run
 // as many window blocks as the longest of their margin blocks (the others
 // wait), which pays only on long rows: the paired-warp kernel takes these
@@ -647,15 +648,11 @@ size_t tab_entries_fit(size_t floats, bool prune, bool cert)
 #ifndef TVS_CERT_FAR
 #define TVS_CERT_FAR 256
 #endif
-#ifndef TVS_CERT_FAR2
-#define TVS_CERT_FAR2 (1 << 30)
-#endif
 #ifndef TVS_CERT_PACKADD
 #define TVS_CERT_PACKADD 1
 #endif
 constexpr int CERT_NEAR = TVS_CERT_NEAR;
 constexpr int CERT_FAR = TVS_CERT_FAR;
-constexpr int CERT_FAR2 = TVS_CERT_FAR2;
 
 // Targets per lane per chunk of an exact walk.
 constexpr int XW_KPL = 8;
@@ -725,29 +722,12 @@ __device__ __forceinline__ void pov_hl(const CertRow& r, int x, float& hi, float
     else { hi = r.H[x]; lo = r.Lo[x]; }
 }
 
-// Hands the flagged walks of one group (bits of fm, staged samples x0 + bit)
-// to the exact pass; returns the bits that found the buffer full.
-__device__ __forceinline__ unsigned flag_walks(const SweepParams& sp, const CertRow& r, unsigned fm, int x0)
-{
-    // a full buffer's fill no longer counts, so it cannot wrap
-    const unsigned cap = (unsigned)sp.flag_cap;
-    unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
-    if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)__popc(fm));
-    for (; fm && at < cap; fm &= fm - 1, ++at) {
-        const int xs = x0 + __ffs(fm) - 1;   // staged sample; the entry holds the row's
-        sp.flag_buf[at] = make_int4(r.key, r.rev_staged ? r.L - 1 - xs : xs, __float_as_int(r.zmax), 0);
-    }
-    if (fm) sp.flag_count[2] = 1u;
-    return fm;
-}
-
-// The sample field of a flag entry holds the entry's kind above bit 16: a
-// whole walk to take again, or one block of a walk.  The fourth field of a
-// block entry is the block's first step e0 and p0, the first step of the block
-// in which the maximum last rose for certain: the walk's running maximum
-// before e0 lies in that block, or (FLAG_PREFIX, when a block after it was
-// flagged) anywhere from there on.
-constexpr int FLAG_WALK = 0, FLAG_BLOCK = 1, FLAG_PREFIX = 2;
+// The sample field of a flag entry holds the entry's kind above bit 16: the
+// block's running maximum before its first step e0 lies in the block p0 in
+// which the walk's maximum last rose for certain, or (FLAG_PREFIX, when a block
+// after it was flagged) anywhere from there on; above that the lengths of both
+// blocks in eighths.  The fourth field holds e0 and p0.
+constexpr int FLAG_BLOCK = 1, FLAG_PREFIX = 2;
 static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 
 // A staged row as the pruned certified walks see it (in shared memory, so that
@@ -775,15 +755,17 @@ constexpr int PACK_MAX_LG = TVS_PACK_MAX_LG;           // at most 8 staged rows 
 #endif
 constexpr int PACK_MIN_CLAIMS = TVS_PACK_MIN_CLAIMS;   // packs per warp that packing must leave
 
-// Hands block e0 of staged sample x's walk to the exact pass, p0 the block of
-// its last rise; false when the buffer is full.
-__device__ __forceinline__ bool flag_block(const SweepParams& sp, const SkipRow& r, int x, int e0, int p0, int kind)
+// Hands the len-step block at e0 of row sample x's walk to the exact pass, p0
+// (plen steps) the block of its last rise; false when the buffer is full.
+__device__ __forceinline__ bool flag_block(const SweepParams& sp, int key, float zmax, int x, int e0, int len, int p0,
+                                           int plen, int kind)
 {
     const unsigned cap = (unsigned)sp.flag_cap;
     unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
     if (at < cap) at = atomicAdd(sp.flag_count, 1u);
     if (at >= cap) return false;
-    sp.flag_buf[at] = make_int4(r.key, (r.rev ? r.L - 1 - x : x) | kind << 16, __float_as_int(r.zmax), e0 | p0 << 14);
+    sp.flag_buf[at] = make_int4(key, x | kind << 16 | (len >> 3) << 18 | (plen >> 3) << 22, __float_as_int(zmax),
+                                e0 | p0 << 14);
     return true;
 }
 
@@ -810,21 +792,18 @@ __device__ __forceinline__ bool skip_row(const SweepParams& sp, const ItemRow& i
 }
 
 // Writes the measures of a finished group of P POVs (pov_x(q): staged sample
-// of POV q; mask: its flagged POVs).
-template <int P, bool LONG, bool BWD, class X, class N, class S>
-__device__ __forceinline__ void finish_group(const SweepParams& sp, const CertRow& r, int x0, unsigned mask,
-                                             X pov_x, N walk_n, S measure, const int* spill)
+// of POV q; lost: POVs whose walk is taken again whole).
+template <int P, bool LONG, class X, class N, class S>
+__device__ __forceinline__ void finish_group(const SweepParams& sp, const CertRow& r, unsigned lost, X pov_x, N walk_n,
+                                             S measure, const int* spill)
 {
-    unsigned full = 0u;                      // bits by sample
-    if (mask) full = flag_walks(sp, r, BWD ? __brev(mask) >> (32 - P) : mask, x0);
+    if (lost) sp.flag_count[2] = 1u;
 #pragma unroll
     for (int q = 0; q < P; ++q) {
         const int x = pov_x(q);
         if (x >= r.L) continue;
-        const bool lost = (full >> (x - x0)) & 1u;
-        if (((mask >> q) & 1u) && !lost) continue;   // the exact pass writes it
         const int cv = walk_n(x) >= 1 ? 1 + (int)measure(q) + (LONG ? spill[32 * q] : 0) : 0;
-        r.cvrow[r.rev_staged ? r.L - 1 - x : x] = lost ? CV_FLAGGED : cv;
+        r.cvrow[r.rev_staged ? r.L - 1 - x : x] = (lost >> q) & 1u ? CV_FLAGGED : cv;
     }
 }
 
@@ -1045,41 +1024,39 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane, unsi
     if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
 }
 
-// Adds to POV x's measure what the targets of block e0 (U steps) add, decided
-// exactly; kind and p0 as in the flag entry.
-template <int U>
-__device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int p0, int kind, int lane,
-                                         unsigned* count)
+// Adds to POV x's measure what the targets of block e0 (len steps) add, decided
+// exactly; kind, p0 and plen as in the flag entry.
+__device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int len, int p0, int plen, int kind,
+                                         int lane, unsigned* count)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
-    const int last = min(n - 1, e0 + U);
+    const int last = min(n - 1, e0 + len);
     if (last <= e0) return;
     bool esc = false;
     const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, p0, e0, e0, last, lane, &esc)
-                                      : df_walk<1>(c, x, p0, min(p0 + U, e0), e0, last, lane, &esc);
+                                      : df_walk<4>(c, x, p0, min(p0 + plen, e0), e0, last, lane, &esc);
     const int add = esc ? fp64_walk(c, x, e0, last, lane) : s;
     if (lane == 0 && in_range(x, c.L, 14) && add) atomicAdd(c.cvrow + x, add);
     ++count[0];
     if (esc) ++count[1];
 }
 
-// The same for one FLAG_BLOCK entry per half-warp (h: the lane's place in its
+// The same for one FLAG_BLOCK entry of at most 16 steps in either block per half-warp (h: the lane's place in its
 // half; valid: the half has an entry): one target of the earlier block and one
 // of the flagged block per lane.  The maximum of the earlier block is one of
 // its near-tied largest slopes, so its error is taken at that block's first
 // distance.  Returns whether the half's decisions need the FP64 walk (nothing
 // is added then).
-template <int U>
-__device__ __forceinline__ bool exact_half(const ExactCtx& c, bool valid, int x, int e0, int p0, int lane)
+__device__ __forceinline__ bool exact_half(const ExactCtx& c, bool valid, int x, int e0, int len, int p0, int plen,
+                                           int lane)
 {
-    static_assert(U <= 16, "a lane per target");
     const unsigned FULL = 0xffffffffu;
     const float NEG = neg_inf();
     const int h = lane & 15, dir = c.bwd ? -1 : 1;
     int da = 0, db = 0;
     if (valid) {
-        const int last = min(min(c.bwd ? x : c.L - 1 - x, c.K) - 1, e0 + U);
-        if (p0 + 1 + h <= min(p0 + U, e0)) da = p0 + 1 + h;
+        const int last = min(min(c.bwd ? x : c.L - 1 - x, c.K) - 1, e0 + len);
+        if (p0 + 1 + h <= min(p0 + plen, e0)) da = p0 + 1 + h;
         if (e0 + 1 + h <= last) db = e0 + 1 + h;
     }
     float ah = NEG, al = 0.f, bh = NEG, bl = 0.f, iv = 1.f;
@@ -1204,7 +1181,7 @@ __device__ __forceinline__ void cert_block(const float* y, const T* __restrict__
 // w meets the window's element q + w + 1: a backward block's window is
 // loaded from x0 - e - U and stored reversed.  Backward groups are taken
 // from the row's end (the longest walks first).
-template <int P, int U, bool LONG, bool BWD, bool TIERS>
+template <int P, int U, bool LONG, bool RANGED, bool BWD, bool TIERS>
 __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const CertRow& r,
                                                const float4* __restrict__ tab, int* __restrict__ spill, int lane)
 {
@@ -1226,7 +1203,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
 #define CERT_M(q) ((q) % 2 ? M2[(q) / 2].y : M2[(q) / 2].x)
 #define CERT_NG(q) ((q) % 2 ? ng2[(q) / 2].y : ng2[(q) / 2].x)
     float Rh = 0.f, c2e = 0.f;
-    unsigned mask = 0u;
+    unsigned lost = 0u, again = 0u;  // as in sweep_rows_skip
     int gi = lane, next = 32;
     int x0 = 0, e = 0, dlim = -1, seg = FLUSH_STEPS;
     bool klimited = false;
@@ -1243,7 +1220,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
         klimited = klim < rowlim;
         e = 0;
         seg = FLUSH_STEPS;
-        mask = 0u;
+        lost = again = 0u;
 #pragma unroll
         for (int q = 0; q < P / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
         if (LONG) {
@@ -1259,8 +1236,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
         if (!in_range(ROW_PADL + wlo, sp.half, 19) || !in_range(ROW_PADL + whi + P + U - 1, sp.half, 19) ||
             (!(LONG && elast + U > tabn) && !in_range(elast + U - 1, tabn, 11))) {
             dlim = 0;
-            const unsigned all = L - x0 >= P ? (1u << P) - 1u : (1u << (L - x0)) - 1u;   // bits by sample
-            mask = BWD ? __brev(all) >> (32 - P) : all;                                   // bits by POV q
+            lost = (1u << P) - 1u;
             return;
         }
         float Rl;
@@ -1303,8 +1279,8 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
         const unsigned need = __ballot_sync(FULL, fin);
         if (need) {
             if (fin) {
-                finish_group<P, LONG, BWD>(sp, r, x0, mask, pov_x, walk_n,
-                                           [&](int q) { return q % 2 ? acc2[q / 2].y : acc2[q / 2].x; }, spill);
+                finish_group<P, LONG>(sp, r, lost, pov_x, walk_n,
+                                      [&](int q) { return q % 2 ? acc2[q / 2].y : acc2[q / 2].x; }, spill);
                 gi = next + __popc(need & below);
                 if (gi < G) start(); else gi = G;
             }
@@ -1326,10 +1302,15 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
             // before the group's last needed step (e + nh U <= dlim), so none
             // of its window blocks is masked and every window and table entry
             // it reads lies in the ranges start() checked.
-            const int nh = (!TIERS || LONG || e < CERT_NEAR) ? 1
-                         : (e >= CERT_FAR2 && e + 8 * U <= dlim) ? 8
-                         : (e >= CERT_FAR && e + 4 * U <= dlim) ? 4
-                         : (e + 2 * U <= dlim) ? 2 : 1;
+            auto blocks_at = [&](int e) {
+                return (!TIERS || LONG || e < CERT_NEAR) ? 1
+                     : (e >= CERT_FAR && e + 4 * U <= dlim) ? 4
+                     : (e + 2 * U <= dlim) ? 2 : 1;
+            };
+            const int nh = blocks_at(e);
+            float2 before[P / 2];    // the measures before the block
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) before[q] = acc2[q];
             const float4* __restrict__ tb = tab + e + e / U;
             const float ive = (LONG && e >= tabn) ? __frcp_rn((float)(e + 1)) : tb->x;
             float Ms[P], mn[P];
@@ -1361,7 +1342,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
                         for (int i = 0; i < 4; ++i) y[BWD ? P + U - 1 - (m + i) : m + i] = v[i];
                     }
                 }
-                const bool masked = klimited && eh + U > dlim;
+                const bool masked = RANGED && klimited && eh + U > dlim;
                 if (masked) {
                     if (far) cert_block<P, U, true, true, PACK>(y, tab, eh, ng2, M2, acc2, mn, dlim - eh);
                     else cert_block<P, U, true, false, PACK>(y, tbh, eh, ng2, M2, acc2, mn, dlim - eh);
@@ -1374,14 +1355,29 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
             // within the block, so max(|M| at its start, |M| at its end)
             // bounds |M| at every one of its steps
             const float ce = __fmaf_rn(c2e, ive, CERT_FLOOR);
+            unsigned fm = 0u;
 #pragma unroll
             for (int q = 0; q < P; ++q) {
                 const float dq =
                     __fmaf_rn(CERT_REL, fmaxf(fabsf(Ms[q]), fabsf(CERT_M(q))), __fmaf_rn(c2e, ia[q], ce));
-                mask |= mn[q] < dq ? 1u << q : 0u;
+                fm |= mn[q] < dq ? 1u << q : 0u;
+            }
+            if (fm) {
+                // flagged POVs leave the block to the exact pass
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    if (!((fm >> q) & 1u)) continue;
+                    (q % 2 ? acc2[q / 2].y : acc2[q / 2].x) = q % 2 ? before[q / 2].y : before[q / 2].x;
+                    const int x = pov_x(q), p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
+                    if (!flag_block(sp, r.key, r.zmax, r.rev_staged ? L - 1 - x : x, e, nh * U, p0, blocks_at(p0) * U,
+                                    (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                        lost |= 1u << q;
+                }
+                again |= fm;
             }
 #pragma unroll
-            for (int q = 0; q < P; ++q) ia[q] = CERT_M(q) > Ms[q] ? ive : ia[q];
+            for (int q = 0; q < P; ++q)
+                if (CERT_M(q) > Ms[q] && !((fm >> q) & 1u)) { ia[q] = ive; again &= ~(1u << q); }
             e += nh * U;
         }
     }
@@ -1755,7 +1751,9 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                     fm |= 1u << q;
                     (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
                     const int p0 = __float2int_rn(__frcp_rn(q % 2 ? ia2[q / 2].y : ia2[q / 2].x)) - 1;
-                    if (!flag_block(sp, *r, pov_x(q), e, p0, (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                    const int x = pov_x(q);
+                    if (!flag_block(sp, r->key, r->zmax, r->rev ? r->L - 1 - x : x, e, U, p0, U,
+                                    (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
                 }
                 again |= fm;
@@ -2019,7 +2017,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
 // 12): a backward item's row is staged reversed and walked forward, like the
 // FP32 sweep's.  Per warp, shared memory holds
 // [Fh half][Fl half][ends 4].
-template <bool LONG, int WARPS>
+template <bool LONG, bool RANGED, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams sp)
 {
     extern __shared__ __align__(16) float smem[];
@@ -2054,7 +2052,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
         __syncwarp();   // the staged row is visible to every lane
         const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
-        sweep_row_cert<CERT_POV, U, LONG, false, false>(sp, r, tab, spill, lane);
+        sweep_row_cert<CERT_POV, U, LONG, RANGED, false, false>(sp, r, tab, spill, lane);
     }
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
@@ -2239,8 +2237,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
                                                                      wm_off, tab, spill, lane);
             } else {
                 const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, cv, false);
-                if (bwd) sweep_row_cert<CERT_POV, U, LONG, true, true>(sp, r, tab, spill, lane);
-                else sweep_row_cert<CERT_POV, U, LONG, false, true>(sp, r, tab, spill, lane);
+                if (bwd) sweep_row_cert<CERT_POV, U, LONG, RANGED, true, true>(sp, r, tab, spill, lane);
+                else sweep_row_cert<CERT_POV, U, LONG, RANGED, false, true>(sp, r, tab, spill, lane);
             }
         }
         row_sync(pair, lgw);   // both walks are done with the row (and with the exchange slot)
@@ -2248,14 +2246,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
     if (lane == 0) atomicAdd(&g_sweep_stats[3], (unsigned long long)(clock64() - t_start));
 }
 
-// The exact pass of a certified launch: every walk or block the sweep flagged
+// The exact pass of a certified launch: every block the sweep flagged
 // (a row key, the sample and its entry's kind, the row's |elevation| bound and
 // the blocks) is decided again exactly, double-float or FP64 past its margin,
 // on samples blended from the DEM as the staging does (the DEM is L2-resident
 // while the sweep runs).  Bound by the latency of those gathers.  A warp takes
-// two entries at a time: two FLAG_BLOCK entries in one go, a half-warp each,
-// what else there is (whole walks, walks flagged since their last rise, FP64)
-// with all 32 lanes.  An entry names its row directly (no search of the item
+// two entries at a time: two FLAG_BLOCK entries of 16 steps in one go, a
+// half-warp each, what else there is (longer blocks, walks flagged since their
+// last rise, FP64) with all 32 lanes.  An entry names its row directly (no search of the item
 // table) and the counters stay in registers: 12 mixed tiles (7.3 million
 // blocks) 214 -> 204 ms, 2000^2 (1.26 million) 95.5 -> 92.6 ms.
 // flag_count[0] is the buffer's fill.
@@ -2280,11 +2278,11 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32, 2) exact_kernel(SweepParams 
         }
         ExactCtx c{};
         if (ok) c = exact_ctx(sp, it, __int_as_float(en.z));
-        const int x = en.y & 0xffff, kind = en.y >> 16, e0 = en.w & 0x3fff, p0 = en.w >> 14;
-        const bool half = ok && kind == FLAG_BLOCK;
+        const int x = en.y & 0xffff, kind = en.y >> 16 & 3, e0 = en.w & 0x3fff, p0 = en.w >> 14;
+        const bool half = ok && kind == FLAG_BLOCK && (en.y >> 18 & 15) <= 2 && (en.y >> 22) <= 2;
         bool left = ok;                       // the half's entry is still to do
         if (__any_sync(0xffffffffu, half)) {
-            const bool esc = exact_half<SKIP_UNROLL>(c, half, x, e0, p0, lane);
+            const bool esc = exact_half(c, half, x, e0, (en.y >> 18 & 15) * 8, p0, (en.y >> 22) * 8, lane);
             if (half && !esc) left = false;
             count[0] += __popc(__ballot_sync(0xffffffffu, half && !esc) & 0x00010001u);
         }
@@ -2295,8 +2293,8 @@ __global__ void __launch_bounds__(EXACT_WARPS * 32, 2) exact_kernel(SweepParams 
             const int z = __shfl_sync(0xffffffffu, en.z, src), w = __shfl_sync(0xffffffffu, en.w, src);
             decode_row(sp, key >> 16, key >> 1 & 0x7fff, (key & 1) != 0, &it);
             const ExactCtx cc = exact_ctx(sp, it, __int_as_float(z));
-            if (y >> 16 == FLAG_WALK) exact_walk(cc, y & 0xffff, lane, count);
-            else exact_block<SKIP_UNROLL>(cc, y & 0xffff, w & 0x3fff, w >> 14, y >> 16, lane, count);
+            exact_block(cc, y & 0xffff, w & 0x3fff, (y >> 18 & 15) * 8, w >> 14, (y >> 22) * 8, y >> 16 & 3, lane,
+                        count);
         }
     }
     if (lane == 0) {
@@ -2498,7 +2496,8 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
         const bool pack = sp.lgna > 0;
         most = prune ? (pack ? PACK_WARPS : SINGLE_WARPS) : wide ? WW : CW;
-        if (!prune) kern = wide ? sweep_cert_kernel<false, WW> : sweep_cert_kernel<false, CW>;
+        if (!prune) kern = ranged ? (wide ? sweep_cert_kernel<false, true, WW> : sweep_cert_kernel<false, true, CW>)
+                                  : (wide ? sweep_cert_kernel<false, false, WW> : sweep_cert_kernel<false, false, CW>);
         else if (pack) kern = ranged ? sweep_pack_kernel<true, PACK_WARPS, PACK_TESTS, PACK_CHUNK>
                                      : sweep_pack_kernel<false, PACK_WARPS, PACK_TESTS, PACK_CHUNK>;
         else kern = ranged ? sweep_pack_kernel<true, SINGLE_WARPS, SKIP_TESTS, SINGLE_CHUNK>
@@ -2506,7 +2505,7 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     } else if (pairs) {
         const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
         most = wide ? WW : prune ? SKIP_WARPS : CW;
-        if (wide) kern = sweep_pair_kernel<false, false, true, WW>;
+        if (wide) kern = ranged ? sweep_pair_kernel<false, false, true, WW> : sweep_pair_kernel<false, false, false, WW>;
         else if (!prune) kern = longw ? sweep_pair_kernel<false, true, true, CW> : sweep_pair_kernel<false, false, true, CW>;
         else if (longw) kern = sweep_pair_kernel<true, true, true, SKIP_WARPS>;
         else kern = ranged ? sweep_pair_kernel<true, false, true, SKIP_WARPS>
