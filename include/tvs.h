@@ -283,8 +283,8 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
                            double obs_height_m, int n_sectors, double max_range_m, int k,
                            int32_t* cv, int32_t* R, int32_t* W);
 
-/* Test hook: the sweep checks the indices of its staging, per-block margins,
- * flag buffer and exact walks against their buffers; the first violation
+/* Test hook: the sweep checks the indices of its staging, blocks and exact
+ * walks against their buffers; the first violation
  * on the current device (code, index, bound, CTA; all zero when none) is
  * copied to out[0..3] after a device synchronisation, and cleared when
  * `clear` is non-zero.  A violation means a library bug: the access was

@@ -1,8 +1,9 @@
 // tvs_sweep.cu -- the sweep of the sDEM total viewshed (Kernel-2, Alg. 7 and
 // 8) with the relocation of Kernel-1 (Alg. 6) fused into its row staging.
 //
-// A warp item is one skewed row and one walk direction.  The warp gathers the
-// row's samples straight from the DEM (section 4.1 step 1(a): sample j of
+// A work item is one skewed row and one walk direction; a warp takes one, both
+// directions of several short rows, or a share of a long one.  The row's
+// samples are gathered straight from the DEM (section 4.1 step 1(a): sample j of
 // line b blends view rows a = b + dest(j) and a + 1 with weights 1 - r(j) and
 // r(j)), so the skewed DEM never reaches HBM, then every usable sample of the
 // row walks it (forward items walk the row, backward items its reverse).
@@ -20,9 +21,12 @@
 //    row is staged as a double-float (hi + lo) pair per sample.  The fast
 //    path still decides in FP32, on height differences formed against a
 //    per-group reference, and proves each decision with a margin derived
-//    below; a decision inside the margin flags its POV, and flagged POVs are
-//    walked again exactly (double-float slopes with their own margin, and the
-//    FP64 definition itself for what that margin cannot settle).
+//    below; a decision inside its margin leaves its block of the walk to an
+//    exact pass (double-float slopes with their own margin, and the FP64
+//    definition itself for what that margin cannot settle).
+//
+// Pruned launches (the default) evaluate only the blocks of a walk that can
+// hold a visible target; unpruned ones evaluate every target.
 #include "tvs.h"
 #include "tvs_internal.h"
 #include "tvs_df.cuh"
@@ -34,16 +38,16 @@
 
 namespace tvs {
 
-// Index checks of the sweep.  Every index the staging, the per-block margins,
-// the flagged-POV list and the exact walks use is checked against its buffer
-// (not the inner step loop, whose indices follow from the block's): a
+// Index checks of the sweep.  The indices of the staging, of the blocks and
+// tests (once per row or group) and of the exact walks are checked against
+// their buffers (not the inner step loop, whose indices follow): a
 // violation records the first offending index in g_sweep_check (code, index,
 // bound, CTA) and skips the access instead of faulting.  Read and cleared by
 // tvs_debug_sweep_check.
 __device__ int g_sweep_check[4];
-// Event counts of the certified sweep: exact walks (flagged POVs), of them
-// FP64 walks, SM clock cycles warps spent in exact walks, and cycles warps
-// spent in the certified sweep kernels in all.
+// Event counts of the certified sweep: blocks (or whole walks) decided again
+// exactly, of them in FP64, SM clock cycles warps spent in the exact pass, and
+// cycles warps spent in the certified sweep kernels.
 __device__ unsigned long long g_sweep_stats[4];
 
 __device__ __forceinline__ bool in_range(long long idx, long long bound, int code)
@@ -1298,10 +1302,10 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
                     acc2[q / 2] = make_float2(0.f, 0.f);
                 }
             }
-            // a margin block of nh window blocks of U steps.  A margin block of several window blocks lies wholly
-            // before the group's last needed step (e + nh U <= dlim), so none
-            // of its window blocks is masked and every window and table entry
-            // it reads lies in the ranges start() checked.
+            // a margin block of nh window blocks of U steps.  One of several
+            // window blocks lies wholly before the group's last needed step (e +
+            // nh U <= dlim), so none of them is masked and every window and
+            // table entry it reads lies in the ranges start() checked.
             auto blocks_at = [&](int e) {
                 return (!TIERS || LONG || e < CERT_NEAR) ? 1
                      : (e >= CERT_FAR && e + 4 * U <= dlim) ? 4
@@ -1938,7 +1942,7 @@ __device__ __forceinline__ void sweep_item(const ItemRow& it, const float* F, co
 }
 
 
-// Warps per CTA of the certified kernels (pairs of warps, below): their
+// Warps per CTA of the unpruned certified kernels: their
 // per-lane state (4 POVs' maxima, heights, margins and last-visible bounds,
 // the window relative to the group) takes about 160 registers, which 12 warps
 // still leave every thread.  When shared memory holds CERT_WIDE_WARPS warps, a
