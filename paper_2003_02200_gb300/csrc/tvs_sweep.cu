@@ -730,7 +730,13 @@ __device__ __forceinline__ void pov_hl(const CertRow& r, int x, float& hi, float
 // block's running maximum before its first step e0 lies in the block p0 in
 // which the walk's maximum last rose for certain, or (FLAG_PREFIX, when a block
 // after it was flagged) anywhere from there on; above that the lengths of both
-// blocks in eighths.  The fourth field holds e0 and p0.
+// blocks in eighths.  The fourth field holds e0 and p0.  A FLAG_PREFIX entry
+// is all that is left of its walk from e0 on, not one block: where a walk is
+// flagged all along (ties, elevations so large that no margin settles
+// anything) each of its entries would walk again from p0 (one cell of -3.4e38
+// in a 220 x 310 map, 24 directions: 2.9 ms block by block, 1.0 so).  Rare
+// elsewhere (90 of 7.3 million entries of 12 mixed tiles), where it costs a
+// little (4000^2, 10 km: 204.9 and 206.9 ms; 100 x 16384: 27.8 and 28.8).
 constexpr int FLAG_BLOCK = 1, FLAG_PREFIX = 2;
 static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 
@@ -1028,13 +1034,13 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane, unsi
     if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
 }
 
-// Adds to POV x's measure what the targets of block e0 (len steps) add, decided
-// exactly; kind, p0 and plen as in the flag entry.
+// Adds to POV x's measure what the targets of block e0 (len steps; FLAG_PREFIX:
+// and all after it) add, decided exactly; kind, p0 and plen as in the flag entry.
 __device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int len, int p0, int plen, int kind,
                                          int lane, unsigned* count)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
-    const int last = min(n - 1, e0 + len);
+    const int last = kind == FLAG_PREFIX ? n - 1 : min(n - 1, e0 + len);
     if (last <= e0) return;
     bool esc = false;
     const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, p0, e0, e0, last, lane, &esc)
@@ -1376,6 +1382,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
                     if (!flag_block(sp, r.key, r.zmax, r.rev_staged ? L - 1 - x : x, e, nh * U, p0, blocks_at(p0) * U,
                                     (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
+                    if ((again >> q) & 1u) CERT_M(q) = pos_inf();   // nothing more is visible to it, or flagged
                 }
                 again |= fm;
             }
@@ -1759,6 +1766,8 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                     if (!flag_block(sp, r->key, r->zmax, r->rev ? r->L - 1 - x : x, e, U, p0, U,
                                     (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
+                    if ((again >> q) & 1u)   // nothing more is visible to it, or flagged
+                        (q % 2 ? M2[q / 2].y : M2[q / 2].x) = pos_inf();
                 }
                 again |= fm;
             }
@@ -2256,8 +2265,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
 // on samples blended from the DEM as the staging does (the DEM is L2-resident
 // while the sweep runs).  Bound by the latency of those gathers.  A warp takes
 // two entries at a time: two FLAG_BLOCK entries of 16 steps in one go, a
-// half-warp each, what else there is (longer blocks, walks flagged since their
-// last rise, FP64) with all 32 lanes.  An entry names its row directly (no search of the item
+// half-warp each, what else there is (longer blocks, the rest of walks flagged
+// twice since their last rise, FP64) with all 32 lanes.  An entry names its row directly (no search of the item
 // table) and the counters stay in registers: 12 mixed tiles (7.3 million
 // blocks) 214 -> 204 ms, 2000^2 (1.26 million) 95.5 -> 92.6 ms.
 // flag_count[0] is the buffer's fill.

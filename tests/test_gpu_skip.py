@@ -113,3 +113,18 @@ def test_packed_rows(ctx, kind, rows, cols, n, rng):
     with tvs.Context(0) as c:
         c.set_tuning(prune=0)
         np.testing.assert_array_equal(got, c.total_viewshed(dem, 10.0, 2.5, n, rng))
+
+
+@pytest.mark.parametrize("rows,cols", [(40, 61), (5, 300), (4, 900), (3, 2100)])
+@pytest.mark.parametrize("value", [-3.4028234663852886e38, 1e30, -1e9])
+@pytest.mark.parametrize("h0,rng", [(1.5, 0.0), (0.0, 700.0)])
+def test_rest_of_a_walk(ctx, orc, rows, cols, value, h0, rng):
+    """One cell so high or low that no margin settles anything on its rows:
+    block after block of a walk is flagged, and its second flag hands over all
+    that is left of it, pruned and unpruned."""
+    dem = _terrain("fractal", rows, cols, 33)
+    dem[rows // 2, cols // 3] = value
+    _check(ctx, orc, dem, h0, 8, rng, (0, 3))
+    with tvs.Context(0) as c:
+        c.set_tuning(prune=0)
+        _check(c, orc, dem, h0, 8, rng, (0, 3))
