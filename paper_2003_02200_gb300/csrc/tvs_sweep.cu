@@ -2220,27 +2220,24 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
             const float zpart = stage_row<true>(sp, it, Fh, Fl, ends, lane, part, nw, false);
             if (lane == 0) xch[1 + part] = zpart;
             row_sync(pair, lgw);   // the staged row is complete
-            if (PRUNE) {   // suffix and prefix maxima by the first two warps, each a share of the window maxima
+            int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
+            float zmax = xch[1];
+            for (int m = 2; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
+            if (PRUNE) {   // suffix and prefix maxima and the rows' records by the first two warps (one of each
+                           // walk direction), a share of the window maxima by each
+                if (part < 2 && lane == 0) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) row->ends[m] = ends[m];
+                    if (!skip_row(sp, it, bwd != 0, zmax, cv, false, LONG, row)) row->L = 0;
+                }
                 if (part == 1) end_max<true>(Fh, ZS, it.L, lane);
                 if (part == 0) end_max<false>(Fh, ZS, it.L, lane);
                 window_max<CERT_POV, U>(Fh, WM, it.L, lane, part, nw);
-                row_sync(pair, lgw);
+                row_sync(pair, lgw);   // every warp sees them
             }
-            float zmax = xch[1];
-            for (int m = 2; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
-            int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
             if constexpr (PRUNE) {
-                bool ok = true;
-                if (lane == 0) {
-                    // (the warps of one walk direction all write the same)
-                    ok = skip_row(sp, it, bwd != 0, zmax, cv, false, LONG, row);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) row->ends[m] = ends[m];
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                __syncwarp();
                 const float* H = Fh + ROW_PADL;
-                const int groups = ok ? (it.L + CERT_POV - 1) / CERT_POV : 0;
+                const int groups = (row->L + CERT_POV - 1) / CERT_POV;
                 const int zs_off = (int)(ZS - H), wm_off = (int)(WM - H);
                 if (bwd)
                     sweep_rows_skip<CERT_POV, U, LONG, END, true, SKIP_TESTS, SKIP_CHUNK>(sp, row, H, 0, groups, lgw - 1, part >> 1, zs_off,
