@@ -9,6 +9,14 @@
 namespace tvs {
 namespace df {
 
+// Heights (and observer heights) from here on are no ground elevations but
+// no-data values (-3.4e38, 1e20, 1e30): a double-float height errs by 2^-42 of
+// the largest elevation near it, 2^18 m here, so no margin settles a decision
+// on the ground around one, and near FLT_MAX differences overflow, which the
+// margins do not cover.  Walks that meet one are decided in FP64.
+constexpr float BEYOND = 0x1p60f;
+__device__ __forceinline__ bool beyond(float zmax, float h0) { return !(zmax + fabsf(h0) < BEYOND); }
+
 // Error-free transformations in round-to-nearest single precision.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 {

@@ -732,12 +732,13 @@ __device__ __forceinline__ void pov_hl(const CertRow& r, int x, float& hi, float
 // after it was flagged) anywhere from there on; above that the lengths of both
 // blocks in eighths.  The fourth field holds e0 and p0.  A FLAG_PREFIX entry
 // is all that is left of its walk from e0 on, not one block: where a walk is
-// flagged all along (ties, elevations so large that no margin settles
-// anything) each of its entries would walk again from p0 (one cell of -3.4e38
-// in a 220 x 310 map, 24 directions: 2.9 ms block by block, 1.0 so).  Rare
-// elsewhere (90 of 7.3 million entries of 12 mixed tiles), where it costs a
-// little (4000^2, 10 km: 204.9 and 206.9 ms; 100 x 16384: 27.8 and 28.8).
-constexpr int FLAG_BLOCK = 1, FLAG_PREFIX = 2;
+// flagged all along (ties) each of its entries would walk again from p0 (400^2,
+// 36 directions: level ground seen from its own height 247 ms block by block,
+// 242 so; steps of whole metres 39.2 and 37.0).  Rare elsewhere (90 of 7.3
+// million entries of 12 mixed tiles), where it costs a little (4000^2, 10 km:
+// 204.9 and 206.9 ms; 100 x 16384: 27.8 and 28.8).
+// FLAG_WALK is a whole walk, decided in FP64 (hand_over_row).
+constexpr int FLAG_BLOCK = 1, FLAG_PREFIX = 2, FLAG_WALK = 3;
 static_assert(2 * 14 < 32, "e0 and p0 (< 16384) share a word");
 
 // A staged row as the pruned certified walks see it (in shared memory, so that
@@ -777,6 +778,29 @@ __device__ __forceinline__ bool flag_block(const SweepParams& sp, int key, float
     sp.flag_buf[at] = make_int4(key, x | kind << 16 | (len >> 3) << 18 | (plen >> 3) << 22, __float_as_int(zmax),
                                 e0 | p0 << 14);
     return true;
+}
+
+// Hands every walk of a row to the exact pass, which walks it in FP64: rows
+// that hold a height beyond what the margins cover (df::beyond).  Flagged block
+// by block such a row's walks were wrong where differences overflowed, and
+// walked in single precision, double-float and twice in FP64 (220 x 310, 24
+// directions, one cell of -3.4e38: 0.97 ms, 0.53 so; 0.58 when every flag sent
+// its whole walk to the exact pass).  Lanes take samples first, first + step, ...
+__device__ __forceinline__ void hand_over_row(const SweepParams& sp, const ItemRow& it, bool back, float zmax, int* cv,
+                                              int first, int step)
+{
+    int* cvrow = cv + it.rowbase;
+    const int key = row_key(it.dir, it.p, back);
+#pragma unroll 1
+    for (int x = first; x < it.L; x += step) {
+        const int n = min(back ? x : it.L - 1 - x, it.K);
+        int m = n >= 1 ? 1 : 0;
+        if (n >= 2 && !flag_block(sp, key, zmax, x, 0, 0, 0, 0, FLAG_WALK)) {
+            m = CV_FLAGGED;
+            sp.flag_count[2] = 1u;
+        }
+        cvrow[x] = m;
+    }
 }
 
 // Fills a staged row's SkipRow (the ends are there already), walked backward
@@ -1025,8 +1049,8 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane, unsi
     if (n < 2) {
         cv = n < 1 ? 0 : 1;
     } else {
-        bool esc = false;
-        const int s = df_walk<XW_KPL>(c, x, 0, 0, 0, n - 1, lane, &esc);
+        bool esc = c.eta >= 0x1p-42f * df::BEYOND;
+        const int s = esc ? 0 : df_walk<XW_KPL>(c, x, 0, 0, 0, n - 1, lane, &esc);
         cv = 1 + (esc ? fp64_walk(c, x, 0, n - 1, lane) : s);
         ++count[0];
         if (esc) ++count[1];
@@ -1034,16 +1058,16 @@ __device__ __noinline__ void exact_walk(const ExactCtx& c, int x, int lane, unsi
     if (lane == 0 && in_range(x, c.L, 14)) c.cvrow[x] = cv;
 }
 
-// Adds to POV x's measure what the targets of block e0 (len steps; FLAG_PREFIX:
-// and all after it) add, decided exactly; kind, p0 and plen as in the flag entry.
+// Adds to POV x's measure what the targets of block e0 (len steps; FLAG_PREFIX
+// and FLAG_WALK: and all after it) add, decided exactly; kind, p0 and plen as in the flag entry.
 __device__ __noinline__ void exact_block(const ExactCtx& c, int x, int e0, int len, int p0, int plen, int kind,
                                          int lane, unsigned* count)
 {
     const int n = min(c.bwd ? x : c.L - 1 - x, c.K);
-    const int last = kind == FLAG_PREFIX ? n - 1 : min(n - 1, e0 + len);
+    const int last = kind == FLAG_BLOCK ? min(n - 1, e0 + len) : n - 1;
     if (last <= e0) return;
-    bool esc = false;
-    const int s = kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, p0, e0, e0, last, lane, &esc)
+    bool esc = kind == FLAG_WALK;
+    const int s = kind == FLAG_WALK ? 0 : kind == FLAG_PREFIX ? df_walk<XW_KPL>(c, x, p0, e0, e0, last, lane, &esc)
                                       : df_walk<4>(c, x, p0, min(p0 + plen, e0), e0, last, lane, &esc);
     const int add = esc ? fp64_walk(c, x, e0, last, lane) : s;
     if (lane == 0 && in_range(x, c.L, 14) && add) atomicAdd(c.cvrow + x, add);
@@ -2063,6 +2087,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         if (!nonempty) continue;
         __syncwarp();
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
+        if (df::beyond(zmax, it.h0)) {
+            hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32);
+            continue;
+        }
         __syncwarp();   // the staged row is visible to every lane
         const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
         sweep_row_cert<CERT_POV, U, LONG, RANGED, false, false>(sp, r, tab, spill, lane);
@@ -2125,6 +2153,15 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
             const bool both = na > 1;
             const float zmax = stage_row<true>(sp, it, Fh, Fh + sp.half, r->ends, lane, 0, 1, true,
                                                both ? Fb : nullptr, Fb + sp.half);
+            if (df::beyond(zmax, it.h0)) {
+                hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32);
+                if (both) hand_over_row(sp, it, true, zmax, sp.cv_bwd, lane, 32);
+                if (lane == 0) {
+                    r->L = 0;
+                    if (both) r[1].L = 0;
+                }
+                continue;
+            }
             __syncwarp();   // the staged rows are visible to every lane
             if (lane == 0) {
                 const bool ok = skip_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev, false, r);
@@ -2216,13 +2253,17 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
         if (pitem >= sp.total_items) break;
         ItemRow it;
         const bool nonempty = decode_item(sp, istart, pitem + bwd, &it);
+        float zmax = 0.f;
+        int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
         if (nonempty) {
             const float zpart = stage_row<true>(sp, it, Fh, Fl, ends, lane, part, nw, false);
             if (lane == 0) xch[1 + part] = zpart;
             row_sync(pair, lgw);   // the staged row is complete
-            int* cv = bwd ? sp.cv_bwd : sp.cv_fwd;
-            float zmax = xch[1];
-            for (int m = 2; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
+            for (int m = 1; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
+        }
+        if (nonempty && df::beyond(zmax, it.h0)) {
+            hand_over_row(sp, it, bwd != 0, zmax, cv, (part >> 1) * 32 + lane, 16 << lgw);
+        } else if (nonempty) {
             if (PRUNE) {   // suffix and prefix maxima and the rows' records by the first two warps (one of each
                            // walk direction), a share of the window maxima by each
                 if (part < 2 && lane == 0) {
@@ -2263,7 +2304,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
 // while the sweep runs).  Bound by the latency of those gathers.  A warp takes
 // two entries at a time: two FLAG_BLOCK entries of 16 steps in one go, a
 // half-warp each, what else there is (longer blocks, the rest of walks flagged
-// twice since their last rise, FP64) with all 32 lanes.  An entry names its row directly (no search of the item
+// twice since their last rise, whole walks, FP64) with all 32 lanes.  An entry names its row directly (no search of the item
 // table) and the counters stay in registers: 12 mixed tiles (7.3 million
 // blocks) 214 -> 204 ms, 2000^2 (1.26 million) 95.5 -> 92.6 ms.
 // flag_count[0] is the buffer's fill.

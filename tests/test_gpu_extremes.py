@@ -1,0 +1,80 @@
+"""Finite elevations so large that single-precision differences overflow: any
+finite DEM is accepted, so every decision on it is the FP64 definition's."""
+import numpy as np
+import pytest
+
+import paper_2003_02200_gb300 as tvs
+from paper_2003_02200_gb300 import terrain
+
+pytestmark = pytest.mark.gpu
+
+BIG = np.float32(3.4028234663852886e38)
+
+
+@pytest.fixture(scope="module", params=[1, 0], ids=["pruned", "unpruned"])
+def ctx(request):
+    with tvs.Context(0) as c:
+        c.set_tuning(prune=request.param)
+        yield c
+
+
+def _check(ctx, orc, dem, h0, n, rng, ks):
+    rows, cols = dem.shape
+    for k in ks:
+        got = ctx.debug_direction_cv(dem, 10.0, h0, n, rng, k)
+        d = orc.direction(n, k, rows, cols)
+        want = np.stack([orc.line_cv(dem, 10.0, h0, n, rng, 64, k, p - d["D"]) for p in range(d["H"] + d["D"])])
+        bad = np.argwhere(got != want)
+        assert bad.size == 0, f"k {k}: {len(bad)} samples differ, first {bad[:4].tolist()}"
+
+
+def _towers(rows, cols, seed):
+    """Fractal ground with cells of either sign whose differences pass FLT_MAX."""
+    r = np.random.default_rng(seed)
+    dem = terrain.fractal_dem(rows, cols, 0.7, 1200.0, seed)
+    for v in (-3e38, 0.5e38, 3.4e38, -1e38, 2e38, -3.4e38, 3e38, -0.25e38):
+        dem[r.integers(rows), r.integers(cols)] = v
+    return dem
+
+
+def test_rise_after_an_overflowed_slope(ctx, orc):
+    """From -3e38, 0.5e38 at 20 steps overflows a single-precision difference;
+    3.4e38 at 34 steps is higher still, and 3.3e38 at 35 is not."""
+    dem = np.zeros((2, 96), np.float32)
+    dem[:, 8] = -3e38
+    dem[:, 28], dem[:, 42], dem[:, 43] = 0.5e38, 3.4e38, 3.3e38
+    _check(ctx, orc, dem, 1.5, 4, 0.0, (0,))
+
+
+def test_falls_past_the_lowest_float(ctx, orc):
+    """From 3e38, a near target at 2e38 and farther ones below -0.5e38: their
+    differences overflow downward, their slopes lie above the near one's."""
+    dem = np.full((2, 96), -1e38, np.float32)
+    dem[:, 8], dem[:, 9] = 3e38, 2e38
+    dem[:, 28:40] = -0.5e38
+    _check(ctx, orc, dem, 1.5, 4, 0.0, (0,))
+
+
+# packed rows, one row per warp, rows shared by 2, 4 and 16 warps
+@pytest.mark.parametrize("rows,cols", [(40, 61), (5, 300), (4, 900), (3, 2100), (2, 3300), (2, 9000)])
+@pytest.mark.parametrize("h0,rng", [(1.5, 0.0), (0.0, 405.0)])
+def test_towers(ctx, orc, rows, cols, h0, rng):
+    _check(ctx, orc, _towers(rows, cols, 70 + cols), h0, 8, rng, (0, 3))
+
+
+@pytest.mark.parametrize("value", [-BIG, np.float32(1e20), np.float32(-(2.0 ** 59))])
+@pytest.mark.parametrize("rows,cols", [(40, 61), (9, 700), (3, 2100)])
+def test_no_data_cells(ctx, orc, rows, cols, value):
+    """One cell in fifty holds a no-data value, so that most rows do (and the
+    flag buffer fills), two neighbours of a blend among them; the last value
+    is just below where rows are handed over whole."""
+    r = np.random.default_rng(cols)
+    dem = terrain.fractal_dem(rows, cols, 0.7, 1200.0, 8)
+    dem[r.random(dem.shape) < 0.02] = value
+    dem[:2, 11] = value
+    _check(ctx, orc, dem, 1.5, 8, 0.0, (0, 3))
+
+
+@pytest.mark.parametrize("h0", [2.0 ** 60, 3e38, 1e300])
+def test_huge_observer_heights(ctx, orc, h0):
+    _check(ctx, orc, terrain.fractal_dem(5, 130, 0.7, 1200.0, 7), h0, 8, 0.0, (0, 3))
