@@ -281,8 +281,9 @@ __device__ __forceinline__ int walk_half_line(const float* __restrict__ dem, int
 // double-float heights (the blend of Alg. 6 to about 2^-43 of the heights) and
 // double-float slopes, warp-cooperatively as walk_half_line does; each
 // decision is proved by a margin (slope errors <= 2^-45 |theta| + 2 eta / d),
-// and when one is not, the warp walks the half-line again in FP64 exactly as
-// the FP64 definition does ((1 - r) a + r b, h = z + h0, (z - h) / d, strict
+// and when one is not, or a height is beyond what the margins cover
+// (df::beyond), the warp walks the half-line again in FP64 exactly as the FP64
+// definition does ((1 - r) a + r b, h = z + h0, (z - h) / d, strict
 // comparison with the running maximum).  Either way every decision is the one
 // exact arithmetic takes (up to FP64 rounding, which the FP64 walk shares with
 // the definition), so an sDEM point's area is the certified map's value.
@@ -419,6 +420,7 @@ __device__ __noinline__ int walk_df(const LineRef& L, float hh, float hl, float 
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(FULL, zmax, o));
         const float eta = 0x1p-42f * (zmax + h0abs) + 0x1p-126f;
+        if (df::beyond(zmax, h0abs)) esc = true;
         float mh = NEG, ml = 0.f;
         int md = 1;
 #pragma unroll
@@ -530,6 +532,8 @@ __device__ __forceinline__ int line_targets(const LineRef& L)
 // (run = rh + rl at distance rd: eta / rd, and 2^-21 |rh| for rl and the
 // rounding of the test), is at most the running maximum: its targets are then
 // not visible, by more than walk_df's margin, and leave the maximum as it is.
+// (The bound cannot overflow: the observer's height is below df::BEYOND here,
+// and taking it from an elevation near FLT_MAX rounds back to it.)
 __device__ __noinline__ int walk_tiles(const LineRef& L, const float* __restrict__ tiles, int tpitch, float hh,
                                        float hl, float zobs, float h0abs, unsigned char* flags, int cap, int lane,
                                        bool* esc_out)
@@ -572,6 +576,7 @@ __device__ __noinline__ int walk_tiles(const LineRef& L, const float* __restrict
         // the largest |elevation| so far (floats >= 0 order like their bits)
         zmax = fmaxf(zmax, __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(za))));
         eta = 0x1p-42f * (zmax + h0abs) + 0x1p-126f;
+        if (df::beyond(zmax, h0abs)) esc = true;
         float ph = th, pl = tl;
         int pd = d;
 #pragma unroll
@@ -672,10 +677,11 @@ __device__ __forceinline__ int walk_exact(const LineRef& L, long long a0, unsign
         e = __fadd_rn(e, __fadd_rn(zl, h0_lo));
         df::two_sum(s, e, hh, hl);
     }
-    bool esc = false;
     const float zobs = fmaxf(fabsf(va), fabsf(vb));
-    const int cv = tiles ? walk_tiles(L, tiles, tpitch, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc)
-                         : walk_df(L, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc);
+    bool esc = df::beyond(zobs, h0);
+    const int cv = esc     ? 0
+                   : tiles ? walk_tiles(L, tiles, tpitch, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc)
+                           : walk_df(L, hh, hl, zobs, fabsf(h0), flags, cap, lane, &esc);
     if (!esc) return cv;
     return walk_fp64(L, __dadd_rn(z64_of(L, a0, fr0, L.j0), h0d), flags, cap, lane);
 }

@@ -78,3 +78,52 @@ def test_no_data_cells(ctx, orc, rows, cols, value):
 @pytest.mark.parametrize("h0", [2.0 ** 60, 3e38, 1e300])
 def test_huge_observer_heights(ctx, orc, h0):
     _check(ctx, orc, terrain.fractal_dem(5, 130, 0.7, 1200.0, 7), h0, 8, 0.0, (0, 3))
+
+
+def _points(ctx, orc, dem, povs, n, h0=1.5):
+    """Areas in both readings and the map of each POV."""
+    import torch
+    cols = dem.shape[1]
+    d = torch.tensor(dem, device="cuda")
+    p = np.asarray(povs, np.int32)
+    want = ctx.total_viewshed(dem, 10.0, h0, n)[p[:, 0], p[:, 1]]
+    np.testing.assert_array_equal(ctx.viewshed_points(d, 10.0, h0, n, 0.0, p).cpu().numpy(), want)
+    want = orc.direct_viewshed(dem, 10.0, h0, n, 0.0, cells=p[:, 0].astype(np.int64) * cols + p[:, 1])
+    got = ctx.viewshed_points(d, 10.0, h0, n, 0.0, p, mode="direct").cpu().numpy()
+    # FP32 blend and sums of 8 directions
+    np.testing.assert_allclose(got, want, rtol=4e-6, atol=4e-4)
+    for q in p:
+        seen = ctx.visibility_map(d, 10.0, h0, n, 0.0, q[None]).cpu().numpy()
+        ref = orc.visibility_map(dem, 10.0, h0, n, 0.0, povs=q[None])
+        # cells on a sector boundary may fall to either side (two atan2 implementations)
+        assert np.mean(seen != ref) < 1e-3
+
+
+@pytest.mark.parametrize("rows,cols", [(40, 61), (130, 170)])
+def test_points_among_towers(ctx, orc, rows, cols):
+    """Short walks and walks by tile maxima, from the towers and beside them."""
+    dem = _towers(rows, cols, 5)
+    ii, jj = np.nonzero(np.abs(dem) > 1e37)
+    p = np.concatenate([np.stack([ii, jj], 1), np.stack([ii, (jj + 1) % cols], 1), [[0, 0], [rows - 1, cols - 1]]])
+    _points(ctx, orc, dem, p, 7)
+
+
+def test_points_above_a_fall_past_the_lowest_float(ctx, orc):
+    """A tile's bound overflows downward: from 3e38 over 2e38 the ground at
+    -1e38 is hidden at first and rises into view far out."""
+    dem = np.full((40, 300), -1e38, np.float32)
+    dem[:, :48] = 2e38        # three whole tiles
+    dem[20, 8] = 3e38
+    _points(ctx, orc, dem, [(20, 8), (20, 7), (3, 299)], 4)
+
+
+def test_points_beside_a_fall_at_the_first_target(ctx, orc):
+    """The first target's slope overflows in double-float."""
+    dem = np.full((9, 60), 100.0, np.float32)
+    dem[4, 8], dem[4, 9], dem[4, 10], dem[4, 11] = -3.4e38, 3.4e38, 1e37, 3.4e38
+    _points(ctx, orc, dem, [(4, 8), (4, 9), (4, 10), (4, 7)], 4)
+
+
+@pytest.mark.parametrize("h0", [2.0 ** 60, 3e38, 1e300])
+def test_points_at_huge_observer_heights(ctx, orc, h0):
+    _points(ctx, orc, terrain.fractal_dem(60, 150, 0.7, 1200.0, 7), [(0, 0), (30, 60), (59, 149)], 4, h0)
