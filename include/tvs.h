@@ -267,6 +267,16 @@ int tvs_debug_plan(const int32_t* rows, const int32_t* cols, const int32_t* n_se
                    int prune, int fp32_decisions, int32_t* inst_job, int32_t* inst_k, int32_t* inst_chunk,
                    int inst_cap, int32_t* ninst, int32_t* nchunks);
 
+/* Host only (needs no GPU): the CTAs of a sweep launch with rows of up to wmax
+ * samples, walks of up to dmax steps, ndir directions and `items` work items
+ * (one per skewed row and walk direction) on a GPU of num_sms SMs with
+ * smem_optin bytes of shared memory per CTA, under the tuning's prune,
+ * fp32_decisions and sweep_max_warps: out[0] = warps of a CTA, out[1] = warps
+ * that share a staged row (1: each has its own), out[2] = rows staged per warp
+ * at a time.  Errors: TVS_ERR_ARG; TVS_ERR_OOM when a row does not fit. */
+int tvs_debug_sweep_layout(int wmax, int dmax, int ndir, int items, int prune, int fp32_decisions, int max_warps,
+                           int num_sms, int smem_optin, int32_t* out);
+
 /* Row map of direction k computed by the device kernel that the sweep uses,
  * copied to host arrays: dest[j], frac[j] for j < W (integer row shift and
  * 32-bit fraction of j*t), jlo[p], jhi[p] for p < R (usable columns of skewed

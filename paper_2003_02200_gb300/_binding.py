@@ -132,6 +132,7 @@ def load(build_if_missing: bool = True) -> C.CDLL:
                                       C.c_int64),
             "tvs_debug_plan": ([vp, vp, vp, vp, vp, C.c_int, C.c_uint64, C.c_int, C.c_int, C.c_int, C.c_int, vp, vp,
                                 vp, C.c_int, i32p, i32p], C.c_int),
+            "tvs_debug_sweep_layout": ([C.c_int] * 9 + [i32p], C.c_int),
             "tvs_debug_rowmap": ([vp, C.c_int, C.c_int, C.c_int, C.c_int, vp, vp, vp, vp, i32p], C.c_int),
             "tvs_debug_direction_cv": ([vp, vp, C.c_int, C.c_int, C.c_double, C.c_double, C.c_int,
                                         C.c_double, C.c_int, vp, i32p, i32p], C.c_int),
@@ -225,6 +226,16 @@ def debug_plan(jobs, budget_bytes: int, num_sms: int = 152, smem_optin: int = 0,
                                  C.byref(ninst), C.byref(nchunks)))
     n = ninst.value
     return ij[:n].copy(), ik[:n].copy(), ic[:n].copy()
+
+
+def debug_sweep_layout(wmax: int, dmax: int, ndir: int, items: int, prune: int = 1, fp32_decisions: int = 0,
+                       max_warps: int = 0, num_sms: int = 152, smem_optin: int = 232448) -> tuple[int, int, int]:
+    """tvs_debug_sweep_layout: warps per sweep CTA, warps per staged row and
+    rows per warp of a launch (host only)."""
+    out = (C.c_int32 * 3)()
+    _check(load().tvs_debug_sweep_layout(wmax, dmax, ndir, items, prune, fp32_decisions, max_warps, num_sms,
+                                         smem_optin, out))
+    return int(out[0]), int(out[1]), int(out[2])
 
 
 def count_point_evals(rows: int, cols: int, n_sectors: int, povs, step_m: float = 1.0, max_range_m: float = 0.0,

@@ -2452,22 +2452,24 @@ int cert_sweep_class(int wmax, int dmax, int prune, int ndir, int smem_optin)
     return CERT_WIDE_WARPS << (prune ? pack_fit(z) : 0);
 }
 
-cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
-                         int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
-                         int dmax, bool ranged, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
-                         int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream)
+// Layout of a launch's CTAs in shared memory.
+struct SweepLayout {
+    bool single, pairs, longw;   // certified: rows of a warp's own, or shared ones; walks of more than LONG_WALK steps
+    size_t single_fit;           // certified warps that could hold a row of their own
+    size_t fit;                  // units that fit: warps, or the groups of warps that share a row
+    int most;                    // most warps of its kernel
+    int units, warps;            // units and warps of a CTA
+    size_t smem;                 // its bytes
+};
+
+// Fills the sizes of sp (ndir and total_items are set) and the layout of a
+// launch with rows of up to wmax samples and walks of up to dmax steps; false
+// when they do not fit.
+static bool sweep_layout(SweepParams& sp, int wmax, int dmax, bool prune, bool cert, int num_sms, int smem_optin,
+                         int max_warps, SweepLayout* lay)
 {
-    if (ndir <= 0 || total_items <= 0) return cudaSuccess;
-    SweepParams sp;
-    sp.dirs = d_dirs; sp.jobs = d_jobs; sp.item_start = d_item_start; sp.rowlo = rowlo;
-    sp.rowhi = rowhi; sp.cv_fwd = cv_fwd; sp.cv_bwd = cv_bwd; sp.counter = counter; sp.ndir = ndir;
-    sp.total_items = total_items;
-    sp.scan_blocks = (wmax + 31) / 32;
-    if (cert && !flag_count) return cudaErrorInvalidValue;
-    sp.flag_buf = flag_buf;
-    sp.flag_count = flag_count;
-    sp.flag_cap = flag_buf ? flag_cap : 0;
-    const SweepSizes z = sweep_sizes(wmax, dmax, prune != 0, cert != 0, ndir, smem_optin);
+    const int ndir = sp.ndir, total_items = sp.total_items;
+    const SweepSizes z = sweep_sizes(wmax, dmax, prune, cert, ndir, smem_optin);
     sp.inv_len = z.inv_len;
     sp.tab_floats = z.tab;
     sp.istart_len = z.istart;
@@ -2485,11 +2487,13 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     // staged arrays, the maxima, the end samples, an exchange slot and pruned
     // each warp's SkipRow), and per warp its spill: a row's samples are then
     // held once for both walk directions.
-    const size_t single_fit = cert ? cert_single_fit(z, prune != 0) : 0;
+    lay->single_fit = cert ? cert_single_fit(z, prune) : 0;
     const int single_min = TVS_CERT_SINGLE_MIN;
-    const bool single = cert && !longw && (max_warps == 0 || max_warps >= single_min) &&
-                        single_fit >= (size_t)single_min;
-    const bool pairs = cert && !single;
+    lay->longw = longw;
+    lay->single = cert && !longw && (max_warps == 0 || max_warps >= single_min) &&
+                  lay->single_fit >= (size_t)single_min;
+    lay->pairs = cert && !lay->single;
+    const bool single = lay->single, pairs = lay->pairs;
     if (single && prune) {
         // as many rows as fit, while every warp still finds several packs to
         // claim: the last packs of a launch run alone (100 x 100, 180
@@ -2507,13 +2511,13 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
     // by a fifth
     sp.lgw = 1;
     if (pairs && prune) {
-        const int most = max_warps > 0 ? std::min(max_warps, SKIP_WARPS) : SKIP_WARPS;
+        const int most = max_warps > 0 ? std::max(std::min(max_warps, SKIP_WARPS), 2) : SKIP_WARPS;
         auto warps_of = [&](int lgw) {
             const size_t unit = (size_t)sp.per_pair + ((size_t)sp.per_warp << lgw);
             return (int)std::min<size_t>(std::max<size_t>(z.room / unit, longw ? 1 : 0), (size_t)(most >> lgw)) << lgw;
         };
         for (int lgw = 2; lgw <= MAX_LGW; ++lgw)
-            if (5 * warps_of(lgw) >= 6 * warps_of(sp.lgw)) sp.lgw = lgw;
+            if (warps_of(lgw) > 0 && 5 * warps_of(lgw) >= 6 * warps_of(sp.lgw)) sp.lgw = lgw;
     }
     // shared memory of one unit: the warps that share a row, or one warp
     const int uw = pairs ? 1 << sp.lgw : 1;
@@ -2527,57 +2531,83 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
         // entries); the long-walk sweep computes the entries past its end.
         const size_t base = (size_t)sp.istart_len * 4 + slack;
         int w = std::max(1, LONG_MIN_WARPS / uw);
-        const size_t min_tab = (size_t)tab_floats_for(MIN_TABLE, prune != 0, cert != 0) * 4;
+        const size_t min_tab = (size_t)tab_floats_for(MIN_TABLE, prune, cert) * 4;
         while (w > 1 && base + min_tab + (size_t)w * unit > (size_t)smem_optin) --w;
-        if (base + 16 * 4 + (size_t)w * unit >= (size_t)smem_optin) return cudaErrorInvalidConfiguration;
+        if (base + 16 * 4 + (size_t)w * unit >= (size_t)smem_optin) return false;
         // floats that fit, and the most entries whose slots do
         const size_t room = ((size_t)smem_optin - base - (size_t)w * unit) / 16 * 4;
-        sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, tab_entries_fit(room, prune != 0, cert != 0)) & ~1;
-        sp.tab_floats = tab_floats_for(sp.inv_len, prune != 0, cert != 0);
+        sp.inv_len = (int)std::min<size_t>((size_t)sp.inv_len, tab_entries_fit(room, prune, cert)) & ~1;
+        sp.tab_floats = tab_floats_for(sp.inv_len, prune, cert);
         fixed = (size_t)(sp.tab_floats + sp.istart_len) * 4 + slack;
     }
-    if (fixed + unit > (size_t)smem_optin) return cudaErrorInvalidConfiguration;
+    if (fixed + unit > (size_t)smem_optin) return false;
     // As many resident units as shared memory and registers allow, in one CTA
     // per SM (the 1/d table is shared by the CTA).
-    const size_t fit = (smem_optin - fixed) / unit;
+    lay->fit = (smem_optin - fixed) / unit;
+    // (unpruned certified launches take 16 warps, of 128 registers, where that many
+    // fit, else 12)
+    const bool wide = max_warps == 0 || max_warps >= CERT_WIDE_WARPS;
+    if (single)
+        lay->most = prune ? (sp.lgna > 0 ? PACK_WARPS : SINGLE_WARPS)
+                    : wide && lay->single_fit >= (size_t)CERT_WIDE_WARPS ? CERT_WIDE_WARPS : CERT_MAX_WARPS;
+    else if (pairs)
+        lay->most = prune ? SKIP_WARPS
+                    : wide && !longw && lay->fit * 2 >= (size_t)CERT_WIDE_WARPS ? CERT_WIDE_WARPS : CERT_MAX_WARPS;
+    else
+        lay->most = prune ? FP32_WARPS : SWEEP_MAX_WARPS;
+    const int cap = max_warps > 0 ? std::max(std::min(max_warps, lay->most), uw) : lay->most;
+    lay->units = (int)std::min<size_t>(lay->fit, (size_t)(cap / uw));
+    lay->warps = lay->units * uw;
+    lay->smem = fixed + (size_t)lay->units * unit;
+    return true;
+}
+
+cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
+                         int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
+                         int dmax, bool ranged, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
+                         int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream)
+{
+    if (ndir <= 0 || total_items <= 0) return cudaSuccess;
+    SweepParams sp;
+    sp.dirs = d_dirs; sp.jobs = d_jobs; sp.item_start = d_item_start; sp.rowlo = rowlo;
+    sp.rowhi = rowhi; sp.cv_fwd = cv_fwd; sp.cv_bwd = cv_bwd; sp.counter = counter; sp.ndir = ndir;
+    sp.total_items = total_items;
+    sp.scan_blocks = (wmax + 31) / 32;
+    if (cert && !flag_count) return cudaErrorInvalidValue;
+    sp.flag_buf = flag_buf;
+    sp.flag_count = flag_count;
+    sp.flag_cap = flag_buf ? flag_cap : 0;
+    SweepLayout lay;
+    if (!sweep_layout(sp, wmax, dmax, prune != 0, cert != 0, num_sms, smem_optin, max_warps, &lay))
+        return cudaErrorInvalidConfiguration;
     constexpr int CW = CERT_MAX_WARPS, WW = CERT_WIDE_WARPS, FW = SWEEP_MAX_WARPS;
+    const bool wide = lay.most == WW, longw = lay.longw;
     void (*kern)(SweepParams);
-    int most;
-    if (single) {
-        const bool wide = single_fit >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        const bool pack = sp.lgna > 0;
-        most = prune ? (pack ? PACK_WARPS : SINGLE_WARPS) : wide ? WW : CW;
+    if (lay.single) {
         if (!prune) kern = ranged ? (wide ? sweep_cert_kernel<false, true, WW> : sweep_cert_kernel<false, true, CW>)
                                   : (wide ? sweep_cert_kernel<false, false, WW> : sweep_cert_kernel<false, false, CW>);
-        else if (pack) kern = ranged ? sweep_pack_kernel<true, PACK_WARPS, PACK_TESTS, PACK_CHUNK>
-                                     : sweep_pack_kernel<false, PACK_WARPS, PACK_TESTS, PACK_CHUNK>;
+        else if (sp.lgna > 0) kern = ranged ? sweep_pack_kernel<true, PACK_WARPS, PACK_TESTS, PACK_CHUNK>
+                                            : sweep_pack_kernel<false, PACK_WARPS, PACK_TESTS, PACK_CHUNK>;
         else kern = ranged ? sweep_pack_kernel<true, SINGLE_WARPS, SKIP_TESTS, SINGLE_CHUNK>
                            : sweep_pack_kernel<false, SINGLE_WARPS, SKIP_TESTS, SINGLE_CHUNK>;
-    } else if (pairs) {
-        const bool wide = !longw && !prune && fit * 2 >= (size_t)WW && (max_warps == 0 || max_warps >= WW);
-        most = wide ? WW : prune ? SKIP_WARPS : CW;
-        if (wide) kern = ranged ? sweep_pair_kernel<false, false, true, WW> : sweep_pair_kernel<false, false, false, WW>;
-        else if (!prune) kern = longw ? sweep_pair_kernel<false, true, true, CW> : sweep_pair_kernel<false, false, true, CW>;
-        else if (longw) kern = sweep_pair_kernel<true, true, true, SKIP_WARPS>;
-        else kern = ranged ? sweep_pair_kernel<true, false, true, SKIP_WARPS>
-                           : sweep_pair_kernel<true, false, false, SKIP_WARPS>;
+    } else if (lay.pairs) {
+        if (prune && longw) kern = sweep_pair_kernel<true, true, true, SKIP_WARPS>;
+        else if (prune) kern = ranged ? sweep_pair_kernel<true, false, true, SKIP_WARPS>
+                                      : sweep_pair_kernel<true, false, false, SKIP_WARPS>;
+        else if (wide) kern = ranged ? sweep_pair_kernel<false, false, true, WW> : sweep_pair_kernel<false, false, false, WW>;
+        else kern = longw ? sweep_pair_kernel<false, true, true, CW> : sweep_pair_kernel<false, false, true, CW>;
     } else {
-        most = prune ? FP32_WARPS : FW;
         if (!prune) kern = longw ? sweep_kernel<false, true, true, FW> : sweep_kernel<false, false, true, FW>;
         else if (longw) kern = sweep_kernel<true, true, true, FP32_WARPS>;
         else kern = ranged ? sweep_kernel<true, false, true, FP32_WARPS> : sweep_kernel<true, false, false, FP32_WARPS>;
     }
-    const int cap = max_warps > 0 ? std::max(std::min(max_warps, most), uw) : most;
-    const int units = (int)std::min<size_t>(fit, (size_t)(cap / uw));
-    const int warps = units * uw;
-    const size_t smem = fixed + (size_t)units * unit;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, lay.warps * 32, lay.smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    kern<<<per_sm * num_sms, warps * 32, smem, stream>>>(sp);
+    kern<<<per_sm * num_sms, lay.warps * 32, lay.smem, stream>>>(sp);
     err = cudaGetLastError();
     if (err != cudaSuccess || !cert) return err;
     // the exact pass: no shared memory, as many warps as registers allow
@@ -2593,6 +2623,22 @@ cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* 
 }
 
 }  // namespace tvs
+
+extern "C" int tvs_debug_sweep_layout(int wmax, int dmax, int ndir, int items, int prune, int fp32_decisions,
+                                      int max_warps, int num_sms, int smem_optin, int32_t* out)
+{
+    if (!out || wmax < 2 || dmax < 1 || ndir < 1 || items < 1 || max_warps < 0 || num_sms < 1) return TVS_ERR_ARG;
+    tvs::SweepParams sp{};
+    sp.ndir = ndir;
+    sp.total_items = items;
+    tvs::SweepLayout lay;
+    if (!tvs::sweep_layout(sp, wmax, dmax, prune != 0, !fp32_decisions, num_sms, smem_optin, max_warps, &lay))
+        return TVS_ERR_OOM;
+    out[0] = lay.warps;
+    out[1] = lay.pairs ? 1 << sp.lgw : 1;
+    out[2] = 1 << sp.lgna;
+    return TVS_OK;
+}
 
 extern "C" int tvs_debug_sweep_stats(uint64_t* out, int clear)
 {

@@ -128,3 +128,13 @@ def test_rest_of_a_walk(ctx, orc, rows, cols, value, h0, rng):
     with tvs.Context(0) as c:
         c.set_tuning(prune=0)
         _check(c, orc, dem, h0, 8, rng, (0, 3))
+
+
+@pytest.mark.parametrize("rows,cols,rng", [(60, 90, 0.0), (9, 1500, 0.0), (2, 3300, 9000.0), (2, 6000, 0.0)])
+def test_every_cta_size_gives_the_same_map(ctx, rows, cols, rng):
+    dem = _terrain("fractal", rows, cols, 4)
+    want = ctx.total_viewshed(dem, 10.0, 1.5, 8, rng)
+    with tvs.Context(0) as c:
+        for most in (1, 2, 3, 5, 11, 13):
+            c.set_tuning(sweep_max_warps=most)
+            np.testing.assert_array_equal(c.total_viewshed(dem, 10.0, 1.5, 8, rng), want, err_msg=f"{most} warps")

@@ -222,3 +222,15 @@ def test_plan_errors():
                             1 << 30, 152, 0, 1, 0, out.ctypes.data, out.ctypes.data, out.ctypes.data, 15,
                             C.byref(cnt), C.byref(cnt))
     assert rc == tvs._binding.TVS_ERR_ARG               # inst_cap below the number of directions
+
+
+@pytest.mark.parametrize("prune,fp32", [(1, 0), (0, 0), (1, 1), (0, 1)])
+@pytest.mark.parametrize("w", [64, 300, 1000, 1400, 2000, 2600, 3300, 4000, 4500, 9000, 16384])
+def test_sweep_max_warps_bounds_the_cta(w, prune, fp32):
+    """A sweep CTA holds at most sweep_max_warps warps (two where the walk
+    directions of a row share it), and the default fits shared memory."""
+    layout = tvs._binding.debug_sweep_layout
+    for most in (0, 1, 2, 3, 5, 8, 11, 12, 13, 16):
+        warps, per_row, rows = layout(w, w, 8, 2 * 8 * (w + w // 2), prune, fp32, most)
+        assert warps >= 1 and warps % per_row == 0 and per_row in (1, 2, 4, 8, 16) and rows in (1, 2, 4, 8)
+        assert warps <= (max(most, per_row if per_row == 2 else 1) if most else 20)
