@@ -670,6 +670,14 @@ __device__ __forceinline__ float sat_pos(float s)
     return v;
 }
 
+// Whether a flagged POV's whole walk will be flagged: its group's error bound
+// (c2e, a height at distance 1, at least a millimetre) exceeds the running
+// maximum.  That is so beside a cell kilometres and more above or below the
+// ground (-1e9), which spoils its group's reference; on even ground the bound is
+// some 10^-10 m.  Such a walk's rest is handed over at its first flag, not at
+// its second.
+__device__ __forceinline__ bool beside_outlier(float c2e, float M) { return c2e > fmaxf(fabsf(M), 0x1p-10f); }
+
 // What names a walk's row in the flag buffer: direction (< 4096), skewed row
 // (< 32768) and walk direction.
 __device__ __forceinline__ int row_key(int dir, int p, bool back) { return dir << 16 | p << 1 | (back ? 1 : 0); }
@@ -1403,10 +1411,11 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
                     if (!((fm >> q) & 1u)) continue;
                     (q % 2 ? acc2[q / 2].y : acc2[q / 2].x) = q % 2 ? before[q / 2].y : before[q / 2].x;
                     const int x = pov_x(q), p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
+                    const bool rest = (again >> q) & 1u || beside_outlier(c2e, CERT_M(q));
                     if (!flag_block(sp, r.key, r.zmax, r.rev_staged ? L - 1 - x : x, e, nh * U, p0, blocks_at(p0) * U,
-                                    (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                                    rest ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
-                    if ((again >> q) & 1u) CERT_M(q) = pos_inf();   // nothing more is visible to it, or flagged
+                    if (rest) CERT_M(q) = pos_inf();   // nothing more is visible to it, or flagged
                 }
                 again |= fm;
             }
@@ -1787,11 +1796,12 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                     (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
                     const int p0 = __float2int_rn(__frcp_rn(q % 2 ? ia2[q / 2].y : ia2[q / 2].x)) - 1;
                     const int x = pov_x(q);
+                    float& M = q % 2 ? M2[q / 2].y : M2[q / 2].x;
+                    const bool rest = (again >> q) & 1u || beside_outlier(c2e, M);
                     if (!flag_block(sp, r->key, r->zmax, r->rev ? r->L - 1 - x : x, e, U, p0, U,
-                                    (again >> q) & 1u ? FLAG_PREFIX : FLAG_BLOCK))
+                                    rest ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
-                    if ((again >> q) & 1u)   // nothing more is visible to it, or flagged
-                        (q % 2 ? M2[q / 2].y : M2[q / 2].x) = pos_inf();
+                    if (rest) M = pos_inf();   // nothing more is visible to it, or flagged
                 }
                 again |= fm;
             }

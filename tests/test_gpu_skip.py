@@ -138,3 +138,23 @@ def test_every_cta_size_gives_the_same_map(ctx, rows, cols, rng):
         for most in (1, 2, 3, 5, 11, 13):
             c.set_tuning(sweep_max_warps=most)
             np.testing.assert_array_equal(c.total_viewshed(dem, 10.0, 1.5, 8, rng), want, err_msg=f"{most} warps")
+
+
+@pytest.mark.parametrize("prune", [1, 0])
+def test_walks_beside_an_outlier_are_handed_over_once(orc, prune):
+    """A cell of -1e9 spoils the reference of the groups around its samples:
+    every decision of their walks is inside its margin.  The cell enters one
+    sample of two rows per direction, so a group of four POVs in each, walked
+    both ways; each of those walks reaches the exact pass once."""
+    n, rows, cols = 8, 60, 90
+    dem = _terrain("fractal", rows, cols, 12)
+    with tvs.Context(0) as c:
+        c.set_tuning(prune=prune)
+        c.total_viewshed(dem, 10.0, 1.5, n)
+        tvs.sweep_stats(clear=True)
+        c.total_viewshed(dem, 10.0, 1.5, n)
+        usual = tvs.sweep_stats(clear=True)["exact_walks"]
+        dem[rows // 2, cols // 2] = -1e9
+        c.total_viewshed(dem, 10.0, 1.5, n)
+        assert tvs.sweep_stats(clear=True)["exact_walks"] <= usual + n * 2 * 4 * 2
+        _check(c, orc, dem, 1.5, n, 0.0, (0, 1, 3))
