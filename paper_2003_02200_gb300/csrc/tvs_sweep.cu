@@ -774,15 +774,45 @@ constexpr int PACK_MAX_LG = TVS_PACK_MAX_LG;           // at most 8 staged rows 
 #endif
 constexpr int PACK_MIN_CLAIMS = TVS_PACK_MIN_CLAIMS;   // packs per warp that packing must leave
 
-// Hands the len-step block at e0 of row sample x's walk to the exact pass, p0
-// (plen steps) the block of its last rise; false when the buffer is full.
-__device__ __forceinline__ bool flag_block(const SweepParams& sp, int key, float zmax, int x, int e0, int len, int p0,
-                                           int plen, int kind)
+// The staged lo array's first word, before the samples that any window reads:
+// zero when a row is staged, and set once the row's walks found the flag buffer
+// full.  (Warps that share a row may set it together; volatile, as nothing
+// orders them.)
+__device__ __forceinline__ volatile int* full_mark(const float* lo)
+{
+    static_assert(CERT_UNROLL < ROW_PADL && SKIP_UNROLL < ROW_PADL, "the pad is longer than a window");
+    return reinterpret_cast<volatile int*>(const_cast<float*>(lo) - ROW_PADL);
+}
+
+// Reserves `count` entries of the flag buffer; returns the first.  Each flag used
+// to ask the counter, also once the buffer was full, and where many walks are
+// flagged they queued on its address (100 x 100 with 1 % cells of -1e9, 60
+// directions: sweep 706 us with as many instructions as level ground's 64; the
+// call 1.35 -> 0.76 ms so, 220 x 310 4.25 -> 2.08).  One reservation for all lanes
+// of a warp was no better (0.85, 2.16) and cost the other walks more (4000^2, 10
+// km: 205.5 before, 208.2 so, 213.5).  A launch that fills the buffer says so in
+// the third counter.
+__device__ __forceinline__ unsigned flag_slots(const SweepParams& sp, int count, volatile int* full)
 {
     const unsigned cap = (unsigned)sp.flag_cap;
+    if (*full) return cap;
+    // (a full buffer's counter stays where it is)
     unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
-    if (at < cap) at = atomicAdd(sp.flag_count, 1u);
-    if (at >= cap) return false;
+    if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)count);
+    if (at + (unsigned)count > cap) {
+        *full = 1;
+        sp.flag_count[2] = 1u;
+    }
+    return at;
+}
+
+// Hands the len-step block at e0 of row sample x's walk to the exact pass in
+// entry `at`, p0 (plen steps) the block of its last rise; false when that is
+// past the buffer.
+__device__ __forceinline__ bool flag_block(const SweepParams& sp, unsigned at, int key, float zmax, int x, int e0,
+                                           int len, int p0, int plen, int kind)
+{
+    if (at >= (unsigned)sp.flag_cap) return false;
     sp.flag_buf[at] = make_int4(key, x | kind << 16 | (len >> 3) << 18 | (plen >> 3) << 22, __float_as_int(zmax),
                                 e0 | p0 << 14);
     return true;
@@ -795,7 +825,7 @@ __device__ __forceinline__ bool flag_block(const SweepParams& sp, int key, float
 // directions, one cell of -3.4e38: 0.97 ms, 0.53 so; 0.58 when every flag sent
 // its whole walk to the exact pass).  Lanes take samples first, first + step, ...
 __device__ __forceinline__ void hand_over_row(const SweepParams& sp, const ItemRow& it, bool back, float zmax, int* cv,
-                                              int first, int step)
+                                              int first, int step, const float* lo)
 {
     int* cvrow = cv + it.rowbase;
     const int key = row_key(it.dir, it.p, back);
@@ -803,10 +833,8 @@ __device__ __forceinline__ void hand_over_row(const SweepParams& sp, const ItemR
     for (int x = first; x < it.L; x += step) {
         const int n = min(back ? x : it.L - 1 - x, it.K);
         int m = n >= 1 ? 1 : 0;
-        if (n >= 2 && !flag_block(sp, key, zmax, x, 0, 0, 0, 0, FLAG_WALK)) {
+        if (n >= 2 && !flag_block(sp, flag_slots(sp, 1, full_mark(lo)), key, zmax, x, 0, 0, 0, 0, FLAG_WALK))
             m = CV_FLAGGED;
-            sp.flag_count[2] = 1u;
-        }
         cvrow[x] = m;
     }
 }
@@ -839,7 +867,6 @@ template <int P, bool LONG, class X, class N, class S>
 __device__ __forceinline__ void finish_group(const SweepParams& sp, const CertRow& r, unsigned lost, X pov_x, N walk_n,
                                              S measure, const int* spill)
 {
-    if (lost) sp.flag_count[2] = 1u;
 #pragma unroll
     for (int q = 0; q < P; ++q) {
         const int x = pov_x(q);
@@ -1279,6 +1306,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
             (!(LONG && elast + U > tabn) && !in_range(elast + U - 1, tabn, 11))) {
             dlim = 0;
             lost = (1u << P) - 1u;
+            sp.flag_count[2] = 1u;
             return;
         }
         float Rl;
@@ -1406,14 +1434,15 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
             }
             if (fm) {
                 // flagged POVs leave the block to the exact pass
+                unsigned at = flag_slots(sp, __popc(fm), full_mark(r.Lo));
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     if (!((fm >> q) & 1u)) continue;
                     (q % 2 ? acc2[q / 2].y : acc2[q / 2].x) = q % 2 ? before[q / 2].y : before[q / 2].x;
                     const int x = pov_x(q), p0 = __float2int_rn(__frcp_rn(ia[q])) - 1;
                     const bool rest = (again >> q) & 1u || beside_outlier(c2e, CERT_M(q));
-                    if (!flag_block(sp, r.key, r.zmax, r.rev_staged ? L - 1 - x : x, e, nh * U, p0, blocks_at(p0) * U,
-                                    rest ? FLAG_PREFIX : FLAG_BLOCK))
+                    if (!flag_block(sp, at++, r.key, r.zmax, r.rev_staged ? L - 1 - x : x, e, nh * U, p0,
+                                    blocks_at(p0) * U, rest ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
                     if (rest) CERT_M(q) = pos_inf();   // nothing more is visible to it, or flagged
                 }
@@ -1661,7 +1690,6 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
                 } else
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
-                    if (q == 0 && lost) sp.flag_count[2] = 1u;
                     const int x = pov_x(q);
                     if (x >= L) continue;
                     const int n = min(BWD ? x : L - 1 - x, K);
@@ -1790,15 +1818,17 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
             if (min3(fminf(ex2[0].x, ex2[0].y), ex2[1].x, ex2[1].y) < 0.f) {
                 // flagged POVs leave the block to the exact pass
 #pragma unroll
+                for (int q = 0; q < P; ++q) fm |= (q % 2 ? ex2[q / 2].y : ex2[q / 2].x) < 0.f ? 1u << q : 0u;
+                unsigned at = flag_slots(sp, __popc(fm), full_mark(H + sp.half));
+#pragma unroll
                 for (int q = 0; q < P; ++q) {
-                    if (!((q % 2 ? ex2[q / 2].y : ex2[q / 2].x) < 0.f)) continue;
-                    fm |= 1u << q;
+                    if (!((fm >> q) & 1u)) continue;
                     (q % 2 ? blk2[q / 2].y : blk2[q / 2].x) = 0.f;
                     const int p0 = __float2int_rn(__frcp_rn(q % 2 ? ia2[q / 2].y : ia2[q / 2].x)) - 1;
                     const int x = pov_x(q);
                     float& M = q % 2 ? M2[q / 2].y : M2[q / 2].x;
                     const bool rest = (again >> q) & 1u || beside_outlier(c2e, M);
-                    if (!flag_block(sp, r->key, r->zmax, r->rev ? r->L - 1 - x : x, e, U, p0, U,
+                    if (!flag_block(sp, at++, r->key, r->zmax, r->rev ? r->L - 1 - x : x, e, U, p0, U,
                                     rest ? FLAG_PREFIX : FLAG_BLOCK))
                         lost |= 1u << q;
                     if (rest) M = pos_inf();   // nothing more is visible to it, or flagged
@@ -2097,11 +2127,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_cert_kernel(SweepParams s
         if (!nonempty) continue;
         __syncwarp();
         const float zmax = stage_row<true>(sp, it, Fh, Fl, ends, lane);
+        __syncwarp();   // the staged row is visible to every lane
         if (df::beyond(zmax, it.h0)) {
-            hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32);
+            hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32, Fl + ROW_PADL);
             continue;
         }
-        __syncwarp();   // the staged row is visible to every lane
         const CertRow r = cert_row(sp, it, Fh, Fl, ends, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev);
         sweep_row_cert<CERT_POV, U, LONG, RANGED, false, false>(sp, r, tab, spill, lane);
     }
@@ -2163,16 +2193,17 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pack_kernel(SweepParams s
             const bool both = na > 1;
             const float zmax = stage_row<true>(sp, it, Fh, Fh + sp.half, r->ends, lane, 0, 1, true,
                                                both ? Fb : nullptr, Fb + sp.half);
+            __syncwarp();   // the staged rows are visible to every lane
             if (df::beyond(zmax, it.h0)) {
-                hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32);
-                if (both) hand_over_row(sp, it, true, zmax, sp.cv_bwd, lane, 32);
+                const float* lo = Fh + sp.half + ROW_PADL;
+                hand_over_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, lane, 32, lo);
+                if (both) hand_over_row(sp, it, true, zmax, sp.cv_bwd, lane, 32, lo);
                 if (lane == 0) {
                     r->L = 0;
                     if (both) r[1].L = 0;
                 }
                 continue;
             }
-            __syncwarp();   // the staged rows are visible to every lane
             if (lane == 0) {
                 const bool ok = skip_row(sp, it, it.rev, zmax, it.rev ? sp.cv_bwd : sp.cv_fwd, it.rev, false, r);
                 if (both) {
@@ -2272,7 +2303,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_pair_kernel(SweepParams s
             for (int m = 1; m <= nw; ++m) zmax = fmaxf(zmax, xch[m]);
         }
         if (nonempty && df::beyond(zmax, it.h0)) {
-            hand_over_row(sp, it, bwd != 0, zmax, cv, (part >> 1) * 32 + lane, 16 << lgw);
+            hand_over_row(sp, it, bwd != 0, zmax, cv, (part >> 1) * 32 + lane, 16 << lgw, Fl + ROW_PADL);
         } else if (nonempty) {
             if (PRUNE) {   // suffix and prefix maxima and the rows' records by the first two warps (one of each
                            // walk direction), a share of the window maxima by each
