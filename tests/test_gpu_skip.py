@@ -158,3 +158,21 @@ def test_walks_beside_an_outlier_are_handed_over_once(orc, prune):
         c.total_viewshed(dem, 10.0, 1.5, n)
         assert tvs.sweep_stats(clear=True)["exact_walks"] <= usual + n * 2 * 4 * 2
         _check(c, orc, dem, 1.5, n, 0.0, (0, 1, 3))
+
+
+@pytest.mark.parametrize("cols", [33, 34, 65, 97, 129, 256, 257, 258, 259, 289, 513, 515, 2100, 9000])
+@pytest.mark.parametrize("kind", ["level", "steps"])
+def test_exact_walks_of_every_length(ctx, orc, kind, cols):
+    """Ties block after block at lengths around the exact walks' chunks (32 to
+    256 targets), with more flagged walks than the buffer has entries (one per
+    64 walks, more for long rows, 4096 at least): the rest are found by the scan
+    and walked whole.  Per sample against the FP64 oracle."""
+    rows = 2 if cols > 2000 else 5000 // cols + 4
+    dem = np.zeros((rows, cols), np.float32)
+    if kind == "steps":
+        dem += (2 * np.random.default_rng(cols).integers(0, 3, (rows, cols))).astype(np.float32)
+    tvs.sweep_stats(clear=True)
+    _check(ctx, orc, dem, 0.0, 4, 0.0, (0,))
+    if kind == "level":
+        cap = max(4096, 2 * rows * cols * max(1.0, max(rows, cols) / 1024) / 64)
+        assert tvs.sweep_stats(clear=True)["exact_walks"] > cap
