@@ -165,8 +165,8 @@ __device__ __forceinline__ bool decode_item(const SweepParams& sp, const int* is
 // a sentinel that is never visible.  With CERT the first sample and the
 // ROW_PADL samples before it are sentinels too (the last target of a backward
 // walk), and the real hi and lo parts of the two end samples, which are POVs,
-// go to ends[0..3] (first hi, first lo, last hi, last lo).  Returns the row's
-// largest |elevation| read, for the error bounds.
+// go to ends[0..3] (first hi, first lo, last hi, last lo).  Returns (with CERT)
+// the row's largest |elevation| read, for the error bounds.
 template <bool CERT>
 __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow& it, float* Fh, float* Fl,
                                            float* ends, int lane, int part = 0, int parts = 1, bool rev_ok = true,
@@ -219,7 +219,6 @@ __device__ __forceinline__ float stage_row(const SweepParams& sp, const ItemRow&
                 zmax = fmaxf(zmax, fmaxf(fabsf(va[k]), fabsf(vb[k])));
             } else {
                 Fh[ROW_PADL + x] = x == it.L - 1 ? NEG : blend32(va[k], vb[k], fr[k]);
-                zmax = fmaxf(zmax, fmaxf(fabsf(va[k]), fabsf(vb[k])));
             }
         }
     }
@@ -439,7 +438,16 @@ __device__ __forceinline__ float quad_max(const float* __restrict__ F, int q)
     return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
 }
 
-// The maxima a pruned walk tests its blocks against, one entry per
+// A maximum as the tests of a pruned walk take it: raised by 2^-20 of itself, for
+// the roundings of the line it is compared with and the lo parts of the samples
+// (-inf, of windows without samples, as the lowest float).
+__device__ __forceinline__ float raised(float m)
+{
+    m = fmaxf(m, -3.4028234663852886e38f);
+    return __fmaf_rn(0x1p-20f, fabsf(m), m);
+}
+
+// The maxima a pruned walk tests its blocks against (raised), one entry per
 // ZS_STRIDE samples of the staged row F (L samples, -inf beyond them).
 // warp-scans of 32 quads at a time: consecutive lanes read consecutive quads.
 //
@@ -462,7 +470,7 @@ __device__ __forceinline__ void end_max(const float* __restrict__ F, float* __re
             if (PREFIX ? lane >= o : lane + o < 32) m = fmaxf(m, t);
         }
         m = fmaxf(m, carry);
-        if (q < nq) ZS[q] = m;
+        if (q < nq) ZS[q] = raised(m);
         carry = __shfl_sync(FULL, m, PREFIX ? 31 : 0);
     }
 }
@@ -481,7 +489,7 @@ __device__ __forceinline__ void window_max(const float* __restrict__ F, float* _
         float m = quad_max(F, j - U / 4);
 #pragma unroll
         for (int k = 1; k < (P + U) / 4; ++k) m = fmaxf(m, quad_max(F, j - U / 4 + k));
-        WM[j] = m;
+        WM[j] = raised(m);
     }
 }
 
@@ -1543,10 +1551,12 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // min_q limit_q.  The walk is over when every thr_q >= 0 (the lines only
 // rise) and the maximum of all remaining targets (ZS: suffix maxima, or
 // prefix maxima walking backward) is at most that minimum too.  slack covers
-// the hi / lo split, the rounding of g_q (Eg) and of the line: the line's own
-// three roundings are relative to values no larger than the heights it is
-// compared with (where it is larger it is not close), 2^-20 of the row's
-// largest elevation and of |g_q| each; the (U - 1) term is taken 2^-17 larger.
+// the rounding of g_q (Eg) and, 2^-20 of |R| and of |g_q|, of the line's start;
+// the line's last rounding is relative to its own height, which is that of the
+// maximum it is compared with where the two are close: the maxima are raised by
+// 2^-20 of themselves, which covers the samples' lo parts too.  The (U - 1) term
+// is taken 2^-17 larger.  (A slack of the row's largest |elevation| let one cell
+// of -1e9 keep its rows from skipping.)
 // A POV with no target that adds area has M = +inf and thr NaN, which the
 // minimum drops.
 //
@@ -1643,7 +1653,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
         const float2 y1 = __fadd2_rn(__fadd2_rn(make_float2(a.z, a.w), nRh), make_float2(b.z, b.w));
         const float yt = __fadd_rn(__fsub_rn(ht[0], Rh), ht[sp.half]);
         const float ys[P + 1] = {BWD ? y1.y : y0.x, BWD ? y1.x : y0.y, BWD ? y0.y : y1.x, BWD ? y0.x : y1.y, yt};
-        const float4 rh = *reinterpret_cast<const float4*>(&r->h0);   // h0, eg0, zmax
+        const float2 rh = *reinterpret_cast<const float2*>(&r->h0);   // h0, eg0
         float gq[P];
         bool area[P];
 #pragma unroll
@@ -1663,7 +1673,7 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
         }
         const float gmax = fmaxf(fmaxf(fabsf(gq[0]), fabsf(gq[1])), fmaxf(fabsf(gq[2]), fabsf(gq[3])));
         c2e = CERT_ABS * __fmaf_rn(5.1f * 0x1p-24f, gmax, rh.y);
-        level = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(3.f, rh.z, gmax), __fmul_rn(2.f, c2e)));
+        level = __fsub_rn(Rh, __fmaf_rn(0x1p-20f, __fmaf_rn(2.f, fabsf(Rh), gmax), __fmul_rn(2.f, c2e)));
         const float c0 = __fmaf_rn(4.f, c2e, 0x1p-16f);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
@@ -1865,11 +1875,12 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
 }
 
 // Pruned FP32-decision sweep of one staged row (backward rows staged
-// reversed), in the phases of sweep_row_skip.  A skipped target must be one
+// reversed), in the phases of sweep_rows_skip.  A skipped target must be one
 // whose single-precision slope fl(fl(z - h) fl(1/d)) is at most M_q, which the
 // maximum then keeps: three roundings move a slope by less than 2^-22 of
 // itself, so with thr_q = M_q - 2^-21 |M_q| every target no higher than
-// h_q + thr_q d qualifies; slack covers the line's own rounding as there.
+// h_q + thr_q d qualifies; the line starts 2^-19 of |h_q| lower and the maxima
+// are raised for the line's own rounding, as there.
 // Every measure is bit for bit the unpruned walk's.  A POV without targets
 // has thr = -inf, which keeps its (short) group from skipping.
 // 1201 x 777, 180 directions: 19.5 -> 13.5 ms against the walk that only
@@ -1879,7 +1890,7 @@ template <int P, int U, bool LONG, bool RANGED>
 __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const float* __restrict__ F,
                                                  const float* __restrict__ ZS, const float* __restrict__ WM,
                                                  const float2* __restrict__ tab, int* __restrict__ cvrow,
-                                                 int* __restrict__ spill, int L, int K, float h0, float zmax,
+                                                 int* __restrict__ spill, int L, int K, float h0,
                                                  bool rev, int lane)
 {
     constexpr int CH = FP32_CHUNK;
@@ -2004,7 +2015,7 @@ __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const fl
 #pragma unroll
             for (int q = 0; q < P; ++q) {
                 const float thr = __fmaf_rn(-0x1p-21f, fabsf(M[q]), M[q]);
-                const float base0 = __fsub_rn(h[q], 0x1p-20f * __fmaf_rn(3.f, zmax, fabsf(h[q])));
+                const float base0 = __fmaf_rn(-0x1p-19f, fabsf(h[q]), h[q]);
                 (q % 2 ? T2[q / 2].y : T2[q / 2].x) = thr;
                 (q % 2 ? K2[q / 2].y : K2[q / 2].x) =
                     __fmaf_rn((float)(U - 1) * 1.00001f, fminf(thr, 0.f), base0);
@@ -2085,14 +2096,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) sweep_kernel(SweepParams sp)
         next = __shfl_sync(0xffffffffu, next, 0);
         if (!nonempty) continue;
         __syncwarp();
-        const float zmax = stage_row<false>(sp, it, Fh, nullptr, nullptr, lane);
+        stage_row<false>(sp, it, Fh, nullptr, nullptr, lane);
         __syncwarp();   // the staged row is visible to every lane
         int* cvrow = (it.rev ? sp.cv_bwd : sp.cv_fwd) + it.rowbase;
         if constexpr (PRUNE) {
             end_max<false>(Fh, ZS, it.L, lane);
             window_max<SMALL_POV, SKIP_UNROLL>(Fh, WM, it.L, lane);
             __syncwarp();
-            sweep_row_skip32<SMALL_POV, SKIP_UNROLL, LONG, RANGED>(sp, Fh, ZS, WM, tab, cvrow, spill, it.L, it.K, it.h0, zmax,
+            sweep_row_skip32<SMALL_POV, SKIP_UNROLL, LONG, RANGED>(sp, Fh, ZS, WM, tab, cvrow, spill, it.L, it.K, it.h0,
                                                            it.rev, lane);
         } else {
             sweep_item<LONG>(it, Fh, tab, sp.inv_len, cvrow, spill, lane);

@@ -127,3 +127,21 @@ def test_points_beside_a_fall_at_the_first_target(ctx, orc):
 @pytest.mark.parametrize("h0", [2.0 ** 60, 3e38, 1e300])
 def test_points_at_huge_observer_heights(ctx, orc, h0):
     _points(ctx, orc, terrain.fractal_dem(60, 150, 0.7, 1200.0, 7), [(0, 0), (30, 60), (59, 149)], 4, h0)
+
+
+@pytest.mark.parametrize("value", [-BIG, BIG, np.float32(1e30), np.float32(-1e9), np.float32(-9999.0), np.float32(1e-30)])
+@pytest.mark.parametrize("rows,cols,rng", [(40, 61, 0.0), (6, 900, 0.0), (3, 2100, 4567.0), (2, 5000, 0.0)])
+@pytest.mark.parametrize("base", [0.0, -3e6])
+def test_skipping_beside_no_data_changes_no_bit(rows, cols, rng, value, base):
+    """The lines that blocks are tested against, on ground whose heights are far
+    below (or above) the row's largest: FP32 and certified decisions, skipping
+    or not."""
+    r = np.random.default_rng(cols)
+    dem = terrain.fractal_dem(rows, cols, 0.7, 1200.0, 8) + np.float32(base)
+    dem[r.random(dem.shape) < 0.02] = value
+    with tvs.Context(0) as c:
+        for fp32 in (1, 0):
+            c.set_tuning(fp32_decisions=fp32, prune=1)
+            got = c.total_viewshed(dem, 10.0, 1.5, 8, rng)
+            c.set_tuning(prune=0)
+            np.testing.assert_array_equal(got, c.total_viewshed(dem, 10.0, 1.5, 8, rng))
