@@ -920,15 +920,18 @@ __global__ void __launch_bounds__(RASTER_X * RASTER_Y) map_raster_kernel(MapPara
 // Whether a call's certified walks go by tile maxima.  The tile kernel reads
 // the DEM once (6 us on 2000^2, of memory bandwidth beyond), the walks then
 // skip most targets: 10 POVs on 2000^2 take 72 us instead of 113, 2000 POVs
-// 2.8 ms instead of 15.7.  Walks of fewer than 128 targets have little to
-// skip, and the DEM may be larger than what the walks save: a walk_df pass
-// (256 targets) takes some 15 us, the time to read 2^24 cells, so a call has to
-// walk at least one target per 2^16 cells.
-bool use_tiles(bool cert, int rows, int cols, const std::vector<DirDev>& dirs)
+// 2.8 ms instead of 15.7.  Walks of fewer than 128 targets have little to skip;
+// nor have a few lines' of up to 768, which pay for the launch (1 POV, 4
+// directions, 128 to 300 targets: 46 us, 49 with tiles).  And the DEM may be
+// larger than what the walks save: a walk_df pass (256 targets) takes some 15
+// us, the time to read 2^24 cells, so the longest walk has to visit one target
+// per 2^16 cells at least (what many POVs walk together is not counted).
+bool use_tiles(bool cert, int rows, int cols, const std::vector<DirDev>& dirs, int npov)
 {
     int reach = 0;
     for (const DirDev& d : dirs) reach = std::max(reach, std::min(d.K, d.W));
-    return cert && reach >= 128 && (long long)rows * cols <= (long long)reach << 16;
+    return cert && (reach >= 768 || (reach >= 128 && (long long)npov * (long long)dirs.size() >= 512)) &&
+           (long long)rows * cols <= (long long)reach << 16;
 }
 
 int tile_pitch(int cols) { return (cols + TILE - 1) / TILE; }
@@ -1025,7 +1028,7 @@ extern "C" int tvs_visibility_map(tvs_handle h, const float* d_dem, int rows, in
     const size_t hdr = o_pov + align256((size_t)npov * 8);
     const size_t o_flags = hdr;
     const size_t o_tiles = o_flags + align256(flag_bytes);
-    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs);
+    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs, npov);
     const size_t total = o_tiles + (tiles ? tile_bytes(rows, cols) : 0);
     rc = ensure_scratch(h, total);
     if (rc) return rc;
@@ -1106,7 +1109,7 @@ extern "C" int tvs_viewshed_points(tvs_handle h, const float* d_dem, int rows, i
     const size_t hdr = o_pov + align256((size_t)npov * 8);
     const size_t o_term = hdr;
     const size_t o_tiles = o_term + align256((size_t)npov * n_sectors * 4);
-    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs);
+    const bool tiles = use_tiles(!h->tuning.fp32_decisions, rows, cols, dirs, npov);
     const size_t total = o_tiles + (tiles ? tile_bytes(rows, cols) : 0);
     rc = ensure_scratch(h, total);
     if (rc) return rc;

@@ -145,3 +145,13 @@ def test_skipping_beside_no_data_changes_no_bit(rows, cols, rng, value, base):
             got = c.total_viewshed(dem, 10.0, 1.5, 8, rng)
             c.set_tuning(prune=0)
             np.testing.assert_array_equal(got, c.total_viewshed(dem, 10.0, 1.5, 8, rng))
+
+
+@pytest.mark.parametrize("value", [-BIG, np.float32(-1e9), np.float32(1e20)])
+@pytest.mark.parametrize("rows,cols", [(40, 61), (60, 600)])
+def test_points_beside_no_data(ctx, orc, rows, cols, value):
+    """From inside a corner without data, its edge and beyond it."""
+    dem = terrain.fractal_dem(rows, cols, 0.7, 600.0, 3)
+    dem[:rows // 3, :cols // 3] = value
+    i, j = rows // 3, cols // 3
+    _points(ctx, orc, dem, [(0, 0), (i - 1, j - 1), (i - 1, 3), (i, 3), (i + 1, j + 1), (rows - 1, cols - 1)], 7)

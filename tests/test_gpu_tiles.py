@@ -63,3 +63,23 @@ def test_direct_points_and_visibility_map(ctx, orc, kind, h0, rows, cols, n, rng
     ref = orc.visibility_map(dem, 10.0, h0, n, rng, povs=q)
     # cells on a sector boundary may fall to either side (two atan2 implementations)
     assert np.mean(seen != ref) < 1e-3
+
+
+@pytest.mark.parametrize("npov,n", [(1, 4), (63, 8), (64, 8)])
+@pytest.mark.parametrize("rows,cols", [(40, 767), (40, 768), (769, 40), (127, 128), (128, 90), (120, 127)])
+def test_either_side_of_the_rule(ctx, orc, npov, n, rows, cols):
+    """Walks of 127, 128, 767, 768 targets of fewer and more lines than the tile
+    maxima are taken for, in both readings, and their visibility map."""
+    import torch
+    dem = _dem("fractal", rows, cols)
+    d = torch.tensor(dem, device="cuda")
+    p = np.random.default_rng(rows + cols).integers(0, (rows, cols), (npov, 2)).astype(np.int32)
+    want = ctx.total_viewshed(dem, 10.0, 1.5, n)[p[:, 0], p[:, 1]]
+    np.testing.assert_array_equal(ctx.viewshed_points(d, 10.0, 1.5, n, 0.0, p).cpu().numpy(), want)
+    want = orc.direct_viewshed(dem, 10.0, 1.5, n, 0.0, cells=p[:, 0].astype(np.int64) * cols + p[:, 1])
+    got = ctx.viewshed_points(d, 10.0, 1.5, n, 0.0, p, mode="direct").cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=RTOL, atol=RTOL * 100.0)
+    seen = ctx.visibility_map(d, 10.0, 1.5, n, 0.0, p).cpu().numpy()
+    ref = orc.visibility_map(dem, 10.0, 1.5, n, 0.0, povs=p)
+    # cells on a sector boundary may fall to either side (two atan2 implementations)
+    assert np.mean(seen != ref) < 1e-3 * npov
