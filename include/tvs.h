@@ -201,9 +201,11 @@ void tvs_batch_destroy(tvs_batch_handle b);
  *   whichever needs fewer warp items x walk steps x POVs x step cost, where a
  *   4-POV step costs p4_cost_pct percent of an 8-POV step per POV (default
  *   107; 1 << 20 keeps every such row on 8; 0 in tvs_set_tuning = default);
- * sweep_max_warps: warps per sweep CTA, at most 16; 0 (default) = as many as
- *   shared memory allows, up to 16, or 20 in pruned certified launches whose
- *   warps hold one row each;
+ * sweep_max_warps: warps per sweep CTA, at most 16 (two where the walk
+ *   directions of a row share it, at least); 0 (default) = as many as shared
+ *   memory allows, up to 16, or 20 in pruned launches whose warps hold one row
+ *   each (certified rows too long to pack and too short to share; FP32
+ *   decisions);
  * unskew_ctas_per_sm: a chunk whose DEMs have fewer cell tiles than this many
  *   per SM splits its directions into ranges across CTAs (1 to 4, default 2);
  * prune: exact horizon pruning in the sweep (1, default) or none (0): a group
@@ -302,12 +304,13 @@ int tvs_debug_direction_cv(tvs_handle h, const float* dem, int rows, int cols, d
 int tvs_debug_sweep_check(int32_t* out, int clear);
 
 /* Test and profiling hook: event counts of the certified sweep on the current
- * device since the last clear, after a device synchronisation: out[0]
- * blocks of walks that held a decision inside its FP32 margin and were decided
- * again exactly, out[1] of them in FP64 (a decision inside the double-float
- * margin too), out[2] SM clock cycles warps
- * spent in the exact pass, out[3] in the certified sweep kernels.  out holds 4
- * entries.  Errors: TVS_ERR_ARG, TVS_ERR_CUDA. */
+ * device since the last clear, after a device synchronisation: out[0] blocks of
+ * walks that held a decision inside its FP32 margin, rests of walks and whole
+ * walks (heights of 2^60 m and more, flags that found their buffer full) that
+ * were decided again exactly, out[1] of them in FP64 (a decision inside the
+ * double-float margin too), out[2] SM clock cycles warps spent in the exact
+ * pass, out[3] in the certified sweep kernels.  out holds 4 entries.  Errors:
+ * TVS_ERR_ARG, TVS_ERR_CUDA. */
 int tvs_debug_sweep_stats(uint64_t* out, int clear);
 
 /* Turn per-kernel timing on (1) or off (0); turning it on clears the counters.

@@ -138,20 +138,23 @@ cudaError_t launch_colmap(const DirDev* d_dir, int* dest, unsigned* frac, cudaSt
 // backward), its row gathered from the job's DEM; `prune` turns exact horizon
 // pruning on, `cert` certified (exact) visibility decisions instead of FP32
 // ones; `ranged` (some walk may end at its range limit, walk_limited) picks the
-// pruned kernels that can cut a block there.  With cert the walks the sweep cannot certify go to the flag buffer
-// (flag_cap entries, possibly none; flag_count three counters; these and
-// `counter` are zero before the launch) and are walked
-// exactly by a second kernel on the same stream; those that find it full are
-// marked in their measures and found by a third.
+// pruned kernels that can cut a block there.  With cert the blocks of walks that
+// the sweep cannot certify (or the rest of a walk, or all of it) go to the flag
+// buffer (flag_cap entries, possibly none; flag_count three counters: its fill,
+// one unused, whether a flag found it full; these and `counter` are zero before
+// the launch) and are decided exactly by a second kernel on the same stream;
+// walks that find the buffer full are marked in their measures, found by a third
+// kernel and walked exactly, whole.
 cudaError_t launch_sweep(const DirDev* d_dirs, const JobDev* d_jobs, const int* d_item_start, int ndir,
                          int total_items, const int* rowlo, const int* rowhi, int* cv_fwd, int* cv_bwd, int wmax,
                          int dmax, bool ranged, int prune, int cert, unsigned* counter, int4* flag_buf, unsigned* flag_count,
                          int flag_cap, int num_sms, int smem_optin, int max_warps, cudaStream_t stream);
 // Layout class of a certified sweep launch (rows up to wmax samples, walks
-// up to dmax steps, ndir directions): the warps of its one-row-per-warp
-// kernel (16 or 12), or 0 when its rows go to warp pairs.  Chunks of a batch
-// are cut where the class changes, so that short rows do not run in a launch
-// sized for long ones.
+// up to dmax steps, ndir directions): equal numbers mean equal layouts.  0: its
+// rows are shared by warps; otherwise each warp has rows of its own, as many as
+// the class says (pruned launches of short rows stage up to 8 per warp: 16, 32,
+// 64 or 128; else 16 or 12 rows per CTA).  Chunks of a batch are cut where the
+// class changes, so that short rows do not run in a launch sized for long ones.
 int cert_sweep_class(int wmax, int dmax, int prune, int ndir, int smem_optin);
 // Entries of a launch's flagged-walk buffer (16 bytes each), at most.
 constexpr int FLAG_BUF_ENTRIES = 1 << 24;

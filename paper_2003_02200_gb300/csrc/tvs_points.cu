@@ -691,7 +691,8 @@ constexpr int POINTS_DIRS = 2;
 // CTAs of 8 warps per SM that a certified walk kernel's registers leave room
 // for: the walks wait on their gathers one after another, so warps in flight
 // decide (2000 POVs on 2000^2: 4.5, 3.6, 3.1 and 2.8 ms with 24, 32, 40 and 48
-// warps, the last at 40 registers with a few spills).
+// warps, the last at 40 registers with spills: 52 bytes of loads in the kernel, 76
+// to 92 in walk_tiles, 240 to 380 in the walks of escapes and short lines).
 constexpr int POINTS_MIN_CTAS = 6;
 
 // One CTA of 4 POINTS_DIRS warps per (POV q, POINTS_DIRS consecutive
@@ -825,8 +826,10 @@ __global__ void __launch_bounds__(256, CERT ? POINTS_MIN_CTAS : 1) map_flags_ker
 }
 
 // Angle of (y, x), not both 0, in (-pi, pi], within 6e-7: the arctangent of
-// the smaller over the larger by Hastings' polynomial (Abramowitz and Stegun
-// 4.4.49, |error| <= 2e-8 on [0, 1]) in single precision, then the octant.
+// the smaller over the larger by Hastings' polynomial of eight terms
+// (Approximations for Digital Computers, 1955; its error on [0, 1] is 3.8e-8) in
+// single precision, then the octant (4.3e-7 in all, emulated over [0, 1] with 2
+// ulp on the quotient).
 __device__ __forceinline__ float angle_of(int y, int x)
 {
     const float ay = (float)abs(y), ax = (float)abs(x);

@@ -45,7 +45,7 @@ namespace tvs {
 // bound, CTA) and skips the access instead of faulting.  Read and cleared by
 // tvs_debug_sweep_check.
 __device__ int g_sweep_check[4];
-// Event counts of the certified sweep: blocks (or whole walks) decided again
+// Event counts of the certified sweep: blocks (or rests of walks, or whole walks) decided again
 // exactly, of them in FP64, SM clock cycles warps spent in the exact pass, and
 // cycles warps spent in the certified sweep kernels.
 __device__ unsigned long long g_sweep_stats[4];
@@ -76,7 +76,7 @@ struct SweepParams {
     int* cv_bwd;       // backward measure of every sample (slab layout)
     unsigned* counter;
     int4* flag_buf;    // certified: flagged walks for the exact pass
-    unsigned* flag_count;   // its fill, the exact pass's claims, and whether a walk found it full
+    unsigned* flag_count;   // its fill, one unused, and whether a flag found it full
     int flag_cap;
     int ndir;
     int total_items;
@@ -830,7 +830,7 @@ __device__ __forceinline__ bool flag_block(const SweepParams& sp, unsigned at, i
 // that hold a height beyond what the margins cover (df::beyond).  Flagged block
 // by block such a row's walks were wrong where differences overflowed, and
 // walked in single precision, double-float and twice in FP64 (220 x 310, 24
-// directions, one cell of -3.4e38: 0.97 ms, 0.53 so; 0.58 when every flag sent
+// directions, one cell of -3.4e38: 0.97 ms, 0.45 so; 0.58 when every flag sent
 // its whole walk to the exact pass).  Lanes take samples first, first + step, ...
 __device__ __forceinline__ void hand_over_row(const SweepParams& sp, const ItemRow& it, bool back, float zmax, int* cv,
                                               int first, int step, const float* lo)
@@ -1260,7 +1260,7 @@ __device__ __forceinline__ void cert_block(const float* y, const T* __restrict__
 }
 
 // Certified sweep of one staged row (the lane queue of sweep_row).  Every
-// target is walked; pruned launches take sweep_row_skip.
+// target is walked; pruned launches take sweep_rows_skip.
 //
 // The row is staged in row order for both walk directions.  A group covers
 // the samples x0 .. x0 + P - 1 (x0 a multiple of 4, so that every window is
@@ -1496,7 +1496,7 @@ constexpr int WM_SLACK = std::max(SKIP_TESTS, PACK_TESTS) * SKIP_UNROLL / ZS_STR
 enum class RangeEnd { NONE, MASKED, CUT };
 
 // One round of a searching lane: tests NT blocks from step e on
-// against the lines T d + K of its four POVs (see sweep_row_skip) and returns
+// against the lines T d + K of its four POVs (see sweep_rows_skip) and returns
 // the first step that may hold a visible target (*ready), the walk's end when
 // no remaining target can be visible, or the step after the tested blocks.
 // x0 and e are multiples of 4.  Blocks past the walk's end are tested against
