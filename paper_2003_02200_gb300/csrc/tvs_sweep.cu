@@ -792,25 +792,32 @@ __device__ __forceinline__ volatile int* full_mark(const float* lo)
     return reinterpret_cast<volatile int*>(const_cast<float*>(lo) - ROW_PADL);
 }
 
-// Reserves `count` entries of the flag buffer; returns the first.  Each flag used
-// to ask the counter, also once the buffer was full, and where many walks are
-// flagged they queued on its address (100 x 100 with 1 % cells of -1e9, 60
-// directions: sweep 706 us with as many instructions as level ground's 64; the
-// call 1.35 -> 0.76 ms so, 220 x 310 4.25 -> 2.08).  One reservation for all lanes
-// of a warp was no better (0.85, 2.16) and cost the other walks more (4000^2, 10
-// km: 205.5 before, 208.2 so, 213.5).  A launch that fills the buffer says so in
-// the third counter.
+// Reserves `count` entries of the flag buffer; returns the first, past its end
+// (and says in the third counter that a flag found it full) when there are none.
+__device__ __forceinline__ unsigned reserve_flags(const SweepParams& sp, int count)
+{
+    const unsigned cap = (unsigned)sp.flag_cap;
+    // (a full buffer's counter stays where it is)
+    unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
+    if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)count);
+    if (at + (unsigned)count > cap) sp.flag_count[2] = 1u;
+    return at;
+}
+
+// The same for a pruned walk, by its row's mark.  Each flag used to ask the
+// counter, also once the buffer was full, and where many walks are flagged they
+// queued on its address (100 x 100 with 1 % cells of -1e9, 60 directions: sweep 706
+// us with as many instructions as level ground's 64; the call 1.35 -> 0.76 ms so,
+// 220 x 310 4.25 -> 2.08).  One reservation for all lanes of a warp was no better
+// (0.85, 2.16) and cost the other walks more (4000^2, 10 km: 205.5 before, 208.2
+// so, 213.5).  Unpruned walks go by whether their group has lost a flag: the mark
+// costs them more (2000^2, 48 directions: 87.5 before, 88.3 so, 90.1 with it).
 __device__ __forceinline__ unsigned flag_slots(const SweepParams& sp, int count, volatile int* full)
 {
     const unsigned cap = (unsigned)sp.flag_cap;
     if (*full) return cap;
-    // (a full buffer's counter stays where it is)
-    unsigned at = *reinterpret_cast<volatile unsigned*>(sp.flag_count);
-    if (at < cap) at = atomicAdd(sp.flag_count, (unsigned)count);
-    if (at + (unsigned)count > cap) {
-        *full = 1;
-        sp.flag_count[2] = 1u;
-    }
+    const unsigned at = reserve_flags(sp, count);
+    if (at + (unsigned)count > cap) *full = 1;
     return at;
 }
 
@@ -1453,7 +1460,7 @@ __device__ __forceinline__ void sweep_row_cert(const SweepParams& sp, const Cert
             }
             if (fm) {
                 // flagged POVs leave the block to the exact pass
-                unsigned at = flag_slots(sp, __popc(fm), full_mark(r.Lo));
+                unsigned at = lost ? (unsigned)sp.flag_cap : reserve_flags(sp, __popc(fm));
 #pragma unroll
                 for (int q = 0; q < P; ++q) {
                     if (!((fm >> q) & 1u)) continue;
