@@ -986,12 +986,11 @@ __device__ __noinline__ int fp64_walk(const ExactCtx& c, int x, int from, int la
         const int kpl = chunk_targets<XW_KPL>(last - base + 1);
         double th[XW_KPL];
         double m = run;
-        const int d0 = base + lane * kpl;
+        const int d0 = base + lane * kpl, dl = min(d0 + kpl - 1, last);   // the lane's targets
 #pragma unroll
         for (int k = 0; k < XW_KPL; ++k) {
             const int d = d0 + k;
-            th[k] = run;
-            if (k < kpl && d <= last) th[k] = __ddiv_rn(__dsub_rn(z64_at(c, x + dir * d), h), (double)d);
+            th[k] = d <= dl ? __ddiv_rn(__dsub_rn(z64_at(c, x + dir * d), h), (double)d) : run;
             m = fmax(m, th[k]);
         }
         double incl = m;
@@ -1006,7 +1005,8 @@ __device__ __noinline__ int fp64_walk(const ExactCtx& c, int x, int from, int la
 #pragma unroll
         for (int k = 0; k < XW_KPL; ++k) {
             const int d = d0 + k;
-            if (k < kpl && d <= last && th[k] > cur) { acc += d > from ? 2 * d + 1 : 0; cur = th[k]; }
+            if (d > dl) break;
+            if (th[k] > cur) { acc += d > from ? 2 * d + 1 : 0; cur = th[k]; }
         }
         run = fmax(run, __shfl_sync(0xffffffffu, incl, 31));
         base += 32 * kpl;
@@ -1045,13 +1045,13 @@ __device__ __forceinline__ int df_walk(const ExactCtx& c, int x, int a0, int a1,
         float th[KPL], tl[KPL], iv[KPL];
         float mh = NEG, ml = 0.f;
         int md = 1;
-        const int i0 = base + lane * kpl;
+        const int i0 = base + lane * kpl, il = min(i0 + kpl, total);   // the lane's targets
         auto dist = [&](int i) { return i < na ? a0 + 1 + i : b0 + 1 + i - na; };
 #pragma unroll
         for (int k = 0; k < KPL; ++k) {
             const int i = i0 + k, d = dist(i);
             th[k] = NEG; tl[k] = 0.f; iv[k] = 1.f;
-            if (k < kpl && i < total) {
+            if (i < il) {
                 iv[k] = __frcp_rn((float)d);
                 float zh, zl;
                 dem_hl(c, x + dir * d, zh, zl);
@@ -1077,7 +1077,7 @@ __device__ __forceinline__ int df_walk(const ExactCtx& c, int x, int a0, int a1,
 #pragma unroll
         for (int k = 0; k < KPL; ++k) {
             const int i = i0 + k, d = dist(i);
-            if (k >= kpl || i >= total) break;
+            if (i >= il) break;
             bool v = true;                           // the first target (no earlier one) is visible
             if (ch > NEG) {
                 float s, e;
@@ -1568,7 +1568,11 @@ __device__ __forceinline__ int skip_blocks(const float2* T2, const float2* K2, b
 // minimum drops.
 //
 // Measured (whole maps, against the walk that only stopped): 2000^2 199 ->
-// 88.0 ms, 1000^2 32.7 -> 19.4 ms.  Bound by the FMA and ALU pipes and by what
+// 85.1 ms, 1000^2 32.7 -> 18.6 ms.  Where every target is visible nothing can be
+// skipped and each block pays its tests and lines (level ground from 1.5 m, 8
+// directions: 2000^2 16.4 -> 19.6 ms, 4000^2, 2 directions, 47.5 -> 45.0); leaving
+// tests out after blocks that were needed gave 18.0 and cost 2000^2 fractal ground
+// 85 -> 90.  Bound by the FMA and ALU pipes and by what
 // the lanes wait for each other (22 of 32 active, issue slots 67 to 75 %
 // used): registers decide how many warps hide the tests' latency, so the
 // kernels keep no exact walks of their own (their context cost 200 bytes of
@@ -1890,9 +1894,10 @@ __device__ __forceinline__ void sweep_rows_skip(const SweepParams& sp, const Ski
 // are raised for the line's own rounding, as there.
 // Every measure is bit for bit the unpruned walk's.  A POV without targets
 // has thr = -inf, which keeps its (short) group from skipping.
-// 1201 x 777, 180 directions: 19.5 -> 13.5 ms against the walk that only
+// 1201 x 777, 180 directions: 19.5 -> 11.5 ms against the walk that only
 // stopped (8 POVs and 28 steps per block: larger blocks hold a visible target
-// more often).
+// more often, but cost less where all are: level ground, 2000^2, 8 directions 9.8
+// ms then, 13.7 so).
 template <int P, int U, bool LONG, bool RANGED>
 __device__ __forceinline__ void sweep_row_skip32(const SweepParams& sp, const float* __restrict__ F,
                                                  const float* __restrict__ ZS, const float* __restrict__ WM,
