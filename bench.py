@@ -425,8 +425,8 @@ def run_ours(args) -> int:
         "pruned": {"value": p_evals / p_max / 1e9, "unit": UNIT, "dems_per_s": args.steps * world / p_max,
                    "ms_per_step": statistics.mean(p_ms), "speedup": statistics.mean(step_ms) / statistics.mean(p_ms),
                    "identical_output": same_pruned,
-                   "note": "exact horizon pruning on (the library default): walks stop once no remaining target "
-                           "can rise above the running maximum; evaluations counted unpruned, output bit-identical"},
+                   "note": "exact horizon pruning on (the library default): blocks of targets none of which "
+                           "can rise above the running maximum are skipped; evaluations counted unpruned, output bit-identical"},
         "fp32_decisions": {"value": f_evals / f_max / 1e9, "unit": UNIT, "dems_per_s": args.steps * world / f_max,
                            "ms_per_step": statistics.mean(f_ms), "sweep_geval_per_s": f_sweep_rate / 1e9,
                            "sweep_frac_of_roofline": f_sweep_rate / peak_evals, **f32_cells,
