@@ -174,7 +174,8 @@ int tvs_total_viewshed_batch(tvs_handle h, const tvs_job* jobs, int njobs, void*
  * once in a CUDA graph.  tvs_batch_launch replays the graph on a stream; the
  * caller may change the contents of the jobs' d_dem between launches, not the
  * pointers or parameters.  Launches of one prepared batch must not overlap on
- * the GPU (they share its scratch).  tvs_batch_destroy is NULL-safe. */
+ * the GPU (they share its scratch).  A batch may outlive its handle.
+ * tvs_batch_destroy is NULL-safe. */
 typedef struct tvs_batch* tvs_batch_handle;
 
 typedef struct {

@@ -540,7 +540,7 @@ int check_jobs(const tvs_job* jobs, int njobs, std::vector<JobSpec>* out)
 }  // namespace
 
 struct tvs_batch {
-    tvs_ctx* h = nullptr;
+    int device = 0;          // of the handle it was created with (which may be gone by now)
     BatchPlan plan;
     Layout L{};
     char* ws = nullptr;
@@ -564,7 +564,7 @@ int tvs_total_viewshed_batch(tvs_handle h, const tvs_job* jobs, int njobs, void*
 void tvs_batch_destroy(tvs_batch_handle b)
 {
     if (!b) return;
-    DeviceGuard g(b->h->device);
+    DeviceGuard g(b->device);
     cudaDeviceSynchronize();
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
@@ -583,7 +583,7 @@ int tvs_batch_create(tvs_handle h, const tvs_job* jobs, int njobs, size_t hbm_bu
     DeviceGuard g(h->device);
     const size_t budget = hbm_budget_bytes ? hbm_budget_bytes : h->budget;
     tvs_batch* b = new tvs_batch();
-    b->h = h;
+    b->device = h->device;
     size_t mf = 0;
     rc = plan_within(specs, budget, false, h->num_sms, h->tuning, &b->plan, h->smem_optin, &mf);
     if (rc) { delete b; return rc; }
@@ -621,7 +621,7 @@ int tvs_batch_create(tvs_handle h, const tvs_job* jobs, int njobs, size_t hbm_bu
 int tvs_batch_launch(tvs_batch_handle b, void* cuda_stream)
 {
     if (!b) return fail(TVS_ERR_ARG, "batch is NULL");
-    DeviceGuard g(b->h->device);
+    DeviceGuard g(b->device);
     TVS_CUDA(cudaGraphLaunch(b->exec, reinterpret_cast<cudaStream_t>(cuda_stream)), "graph launch");
     return TVS_OK;
 }

@@ -142,3 +142,20 @@ def test_group_size_choice_does_not_change_results(ctx, pov_below, p4_cost):
         torch.cuda.synchronize()
     for j, w in zip(jobs, want):
         np.testing.assert_array_equal(j["out"].cpu().numpy(), w)
+
+
+def test_a_prepared_batch_outlives_its_handle():
+    """The batch keeps what it needs of the handle it was created with."""
+    import torch
+    c = tvs.Context(0)
+    jobs = _jobs(SPECS[:3], seed=50)
+    want = _singles(c, jobs)
+    b = c.prepare_batch(jobs)
+    c.close()
+    for j in jobs:
+        j["out"].fill_(-1.0)
+    b.launch()
+    torch.cuda.synchronize()
+    for j, w in zip(jobs, want):
+        np.testing.assert_array_equal(j["out"].cpu().numpy(), w)
+    b.close()
